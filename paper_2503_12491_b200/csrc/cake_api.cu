@@ -696,14 +696,18 @@ int32_t cake_decode_begin(cake_ctx* ctx, const void* const* k_layers, const void
     CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->h_budget_stage, ctx->d_budget[(c.n_layers - 1) & 1], nb,
                                   cudaMemcpyDeviceToHost, st));
     CAKE_CUDA_TRY(cudaStreamSynchronize(st));
+    for (int l = 0; l < c.n_layers; ++l) ctx->h_dec_cap[l] = 1;
     for (int i = 0; i < ctx->n_req * c.n_layers; ++i) {
-      const int64_t cap = (int64_t)ctx->h_budget_stage[i] + c.window + 1;
+      const int32_t cap = ctx->h_budget_stage[i] + c.window + 1;
+      int32_t& layer_cap = ctx->h_dec_cap[i % c.n_layers];
+      if (cap > layer_cap) layer_cap = cap;
       if (cap > ctx->dec_max_cap) ctx->dec_max_cap = cap;
     }
   }
   const int32_t rc = launch_decode_begin(ctx, ptrs, k_cache, v_cache, row_offsets_out, st);
   if (rc != CAKE_OK) return rc;
   ctx->dec_update_mode = update_mode;
+  ctx->dec_last_layer = -1;
   ctx->dec_ready = true;
   return CAKE_OK;
 }

@@ -172,6 +172,8 @@ struct cake_ctx {
   int32_t* d_dec_order;           // per head: rank in ascending position -> slot
   int4* d_dec_meta;               // [max_lists] (len, free slot, next position, frozen budget)
   int32_t* h_budget_stage;        // pinned [max_requests*L] read-back of the final budgets
+  int32_t dec_last_layer;         // layer of the latest decode step on the cluster form, -1 = none yet
+  int32_t h_dec_cap[CAKE_MAX_LAYERS];   // slots of the largest head of every layer
   int64_t wait_limit_cycles;      // bound of every device-side wait (0 = the default, about 2 s)
   int32_t debug_epoch_skew;       // test hook: added to the launch count the cross-CTA waits expect
   int32_t n_tc_asegs, n_tc_bsegs;          // pass-A / pass-B segments per layer

@@ -17,16 +17,16 @@
 #include <algorithm>
 #include <cstdlib>
 
-#include <cooperative_groups.h>
-
 #include <math_constants.h>
 
 namespace cake {
 namespace {
 
 constexpr int DEC_THREADS = 512;
-constexpr int DEC_CLUSTER = 8;    // CTAs that share a head in the cluster form of the step kernel
-constexpr int DEC_CLUSTER_MIN_CAP = 512;   // smaller heads stay on one CTA
+constexpr int DEC_CLUSTER = 8;    // most CTAs that share a head in the cluster form of the step kernel,
+constexpr int DEC_CLUSTER_WIDE = 16;   //   and the most (beyond the portable 8) where the grid is small
+constexpr int DEC_CTA_ENTRIES = 256;       // entries per CTA up to which a head is spread no further
+constexpr size_t kDecSmemMax = 200 * 1024;
 constexpr int DEC_ROWS = 4;       // cache rows a half-warp has in flight in the logit loop
 
 __device__ __forceinline__ float key_to_float(uint32_t key) {
@@ -319,227 +319,364 @@ decode_step_kernel(const DecodeArgs A) {
   }
 }
 
-// The same step with a head spread over a thread-block cluster of DEC_CLUSTER CTAs: the head's
-// slots (logits, softmax) and then its ranks (pooling, score update, list shift) are cut into
-// DEC_CLUSTER contiguous parts, the per-head maxima, sums and the eviction candidate are exchanged
-// through distributed shared memory, and the group-mean attention passes from slot order to rank
-// order through the context's work area.  Every cluster barrier is reached by all CTAs of the
-// cluster: what decides the control flow (cap, the evicted rank) is the same in all of them.
-// Dynamic shared memory: G * part floats (logits by slot), reused for the pooled window and the
-// list shift.
-template <typename T, int G>
-__global__ void __launch_bounds__(DEC_THREADS)
-decode_step_cluster_kernel(const DecodeArgs A) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  extern __shared__ float sh[];
-  __shared__ float red_v[DEC_THREADS / 32];
-  __shared__ int red_i[DEC_THREADS / 32];
-  __shared__ float x_m[G], x_z[G];                   // this CTA's partial maximum / sum per head
-  __shared__ float x_worst;                          // this CTA's eviction candidate
-  __shared__ int x_worst_r;
-  __shared__ float s_m[G], s_z[G];
-  const int crank = (int)cluster.block_rank();
-  const int g = blockIdx.x / DEC_CLUSTER, req = blockIdx.y;
+// ---------------------------------------------------------------- the step on a cluster of CTAs
+__device__ __forceinline__ uint32_t dec_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Stores into the shared memory of CTA `rank` of the cluster, at the place `p` has in this CTA's.
+__device__ __forceinline__ uint32_t remote_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(dec_smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(remote_addr(p, rank)), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, uint4 v) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(remote_addr(p, rank)), "r"(v.x), "r"(v.y),
+               "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
+// 32 bytes in one load: with four lanes to a row a load covers whole 128-byte lines, half the L1 tag
+// look-ups of 16-byte loads.
+__device__ __forceinline__ void ld_32b(const void* p, uint4& a, uint4& b) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+               : "l"(p)
+               : "memory");
+}
+
+// D[16 rows][8 heads] += A[16][16] B[16][8], bf16 operands, fp32 accumulators.
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Logits (base 2) of the G query heads against the rows of ranks w_lo .. w_lo + n_win - 1 into
+// lg[h * stride + i], and every warp's maximum per head.  `ord` holds the ranks' slots; the last rank of the head (`new_i`, if it lies
+// in the window) is the new token, whose row comes from k_new.  bf16: a warp takes 16 rows at a
+// time, every lane loads whole 16-byte pieces of two rows and uses them as the A operand of
+// m16n8k16 MMAs with the contraction index permuted (the query operand has the same permutation),
+// so a row costs no conversion, no shuffle and no shared memory.
+template <int G>
+__device__ __forceinline__ void window_logits(const __nv_bfloat16* kc, const __nv_bfloat16* kn, const __nv_bfloat16* q,
+                                              int d, int n_win, const int* ord, int new_i, float scale2, float* lg,
+                                              int stride, float (*warp_max)[G]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int blk = req * A.L + A.layer;
-  const size_t lid = (size_t)blk * A.Hkv + g;
-  const int4 mt = A.meta[lid];
-  const int len = mt.x, fre = mt.y, next_pos = mt.z, budget = mt.w;
-  const int cap = len + 1;
-  const int64_t base = A.dec_off[blk] + (int64_t)g * cap;
-  const int part = (cap + DEC_CLUSTER - 1) / DEC_CLUSTER;
-  const int s_lo = min(cap, crank * part), s_hi = min(cap, s_lo + part);
-  float* p = sh;                                     // [G][part], slot s at s - s_lo
-  float* aslot = A.tmp + (size_t)(G + 1) * ((size_t)g * (size_t)(A.T + A.n_req) + (size_t)A.reqs[req].cu + req);
-  T* kc = reinterpret_cast<T*>(A.k_cache) + (size_t)base * A.d;
-  T* vc = reinterpret_cast<T*>(A.v_cache) + (size_t)base * A.d;
-  const T* kn = reinterpret_cast<const T*>(A.k_new) + ((size_t)req * A.Hkv + g) * A.d;
-  const T* vn = reinterpret_cast<const T*>(A.v_new) + ((size_t)req * A.Hkv + g) * A.d;
-  // 1. the new token takes the free slot and the last rank (first CTA of the cluster)
-  if (crank == 0) {
-    for (int e = threadIdx.x; e < A.d; e += DEC_THREADS) {
-      kc[(size_t)fre * A.d + e] = kn[e];
-      vc[(size_t)fre * A.d + e] = vn[e];
+  const int r8 = lane >> 2, t = lane & 3;
+  float m0 = -CUDART_INF_F, m1 = -CUDART_INF_F;
+  const int n_c = d / 64;                            // 32-byte pieces of a row per lane: 1 or 2
+  uint4 qv[4];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    qv[2 * c] = qv[2 * c + 1] = make_uint4(0, 0, 0, 0);
+    if (r8 < G && c < n_c) ld_32b(q + (size_t)r8 * d + (4 * c + t) * 16, qv[2 * c], qv[2 * c + 1]);
+  }
+  for (int i0 = warp * 16; i0 < n_win; i0 += (DEC_THREADS / 32) * 16) {
+    uint4 x[2][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int i = i0 + r8 + 8 * u;
+      const __nv_bfloat16* row = i == new_i ? kn : kc + (size_t)ord[min(i, n_win - 1)] * d;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        x[u][2 * c] = x[u][2 * c + 1] = make_uint4(0, 0, 0, 0);
+        if (c < n_c) ld_32b(row + (4 * c + t) * 16, x[u][2 * c], x[u][2 * c + 1]);
+      }
     }
-    if (threadIdx.x == 0) {
-      A.order[base + len] = fre;
-      A.pos[base + fre] = next_pos;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      mma_bf16(acc, x[0][c].x, x[1][c].x, x[0][c].y, x[1][c].y, qv[c].x, qv[c].y);
+      mma_bf16(acc, x[0][c].z, x[1][c].z, x[0][c].w, x[1][c].w, qv[c].z, qv[c].w);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int i = i0 + r8 + 8 * u;
+      if (i < n_win) {
+        const float l0 = acc[2 * u] * scale2, l1 = acc[2 * u + 1] * scale2;
+        m0 = fmaxf(m0, l0);
+        m1 = fmaxf(m1, l1);
+        if (2 * t < G) lg[(2 * t) * stride + i] = l0;
+        if (2 * t + 1 < G) lg[(2 * t + 1) * stride + i] = l1;
+      }
     }
   }
-  // 2. logits of the G query heads against this CTA's slots
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+    m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+  }
+  if (r8 == 0) {
+    if (2 * t < G) warp_max[warp][2 * t] = m0;
+    if (2 * t + 1 < G) warp_max[warp][2 * t + 1] = m1;
+  }
+}
+// fp32: 16 lanes per row, fp32 FMAs.
+template <int G>
+__device__ __forceinline__ void window_logits(const float* kc, const float* kn, const float* q, int d, int n_win,
+                                              const int* ord, int new_i, float scale2, float* lg, int stride,
+                                              float (*warp_max)[G]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int sub = lane >> 4, l16 = lane & 15;
-  const int per = A.d / 16;
-  float qv[G][8];
+  float m[G];
+#pragma unroll
+  for (int h = 0; h < G; ++h) m[h] = -CUDART_INF_F;
+  const int n4 = d / 64;                             // 16-byte pieces per lane: 1 or 2
+  float4 qv[G][2];
 #pragma unroll
   for (int h = 0; h < G; ++h)
 #pragma unroll
-    for (int e = 0; e < 8; ++e)
-      qv[h][e] = e < per ? to_f32(reinterpret_cast<const T*>(A.q_new)[((size_t)req * A.Hq + g * G + h) * A.d +
-                                                                     l16 * per + e]) : 0.f;
-  const int n8 = per * (int)sizeof(T) / 8;
+    for (int c = 0; c < 2; ++c)
+      qv[h][c] = c < n4 ? reinterpret_cast<const float4*>(q + (size_t)h * d)[16 * c + l16] : make_float4(0.f, 0.f, 0.f, 0.f);
   constexpr int kStep = (DEC_THREADS / 32) * 2;
-  for (int s0 = s_lo + warp * 2; s0 < s_hi; s0 += kStep * DEC_ROWS) {
-    uint2 raw[DEC_ROWS][4];
+  for (int i0 = warp * 2 + sub; i0 - sub < n_win; i0 += kStep * DEC_ROWS) {
+    float4 x[DEC_ROWS][2];
 #pragma unroll
     for (int u = 0; u < DEC_ROWS; ++u) {
-      const int s = s0 + u * kStep + sub;
-      const T* row = s == fre ? kn : kc + (size_t)s * A.d;
+      const int i = i0 + u * kStep;
+      const float* row = i == new_i ? kn : kc + (size_t)ord[min(i, n_win - 1)] * d;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        raw[u][i] = (s < s_hi && i < n8) ? reinterpret_cast<const uint2*>(row + l16 * per)[i] : make_uint2(0u, 0u);
+      for (int c = 0; c < 2; ++c)
+        x[u][c] = c < n4 ? reinterpret_cast<const float4*>(row)[16 * c + l16] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < DEC_ROWS; ++u) {
-      const int s = s0 + u * kStep + sub;
-      float kv[8];
-      unpack_row<T>(raw[u], kv);
+      const int i = i0 + u * kStep;
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         float acc = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc = fmaf(qv[h][e], kv[e], acc);
+        for (int c = 0; c < 2; ++c) {
+          acc = fmaf(qv[h][c].x, x[u][c].x, acc);
+          acc = fmaf(qv[h][c].y, x[u][c].y, acc);
+          acc = fmaf(qv[h][c].z, x[u][c].z, acc);
+          acc = fmaf(qv[h][c].w, x[u][c].w, acc);
+        }
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (l16 == 0 && s < s_hi) p[(size_t)h * part + (s - s_lo)] = acc * A.scale2;
+        if (i < n_win) {
+          m[h] = fmaxf(m[h], acc * scale2);
+          if (l16 == 0) lg[h * stride + i] = acc * scale2;
+        }
       }
     }
   }
-  __syncthreads();
-  // 3. softmax per head over all cap slots (base 2): partial maxima, then partial sums, each
-  //    combined over the cluster in rank order
-  const int n_loc = s_hi - s_lo;
+#pragma unroll
   for (int h = 0; h < G; ++h) {
-    float m = -CUDART_INF_F;
-    for (int i = threadIdx.x; i < n_loc; i += DEC_THREADS) m = fmaxf(m, p[(size_t)h * part + i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) red_v[warp] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float t = red_v[0];
-      for (int w = 1; w < DEC_THREADS / 32; ++w) t = fmaxf(t, red_v[w]);
-      x_m[h] = t;
-    }
-    __syncthreads();
+    m[h] = fmaxf(m[h], __shfl_xor_sync(0xffffffffu, m[h], 16));
+    if (lane == 0) warp_max[warp][h] = m[h];
   }
-  cluster.sync();
-  if (threadIdx.x < G) {
-    float t = -CUDART_INF_F;
-    for (int c = 0; c < DEC_CLUSTER; ++c) t = fmaxf(t, *cluster.map_shared_rank(&x_m[threadIdx.x], c));
-    s_m[threadIdx.x] = t;
-  }
+}
+
+// (score, rank) as one integer whose minimum is the entry that goes: the lowest score, among equal
+// scores the highest rank.  -0 and +0 are equal.
+__device__ __forceinline__ unsigned long long evict_key(float score, int rank) {
+  uint32_t b = __float_as_uint(score);
+  if (b == 0x80000000u) b = 0u;
+  b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+  return ((unsigned long long)b << 32) | (uint32_t)(0x7FFFFFFF - rank);
+}
+constexpr unsigned long long kNoKey = ~0ull;
+
+// The same step with a head spread over a cluster of `csize` CTAs by RANK: a CTA owns a contiguous
+// run of the head's entries in ascending token position and, besides, computes the logits of the
+// pool_kernel / 2 neighbours on either side, so pooling needs nothing from the other CTAs.  The
+// softmax sums are taken against the CTA's own maximum and corrected once the maxima and sums of
+// the cluster are known, so a step meets the cluster twice: (maximum, sum) per
+// head, then (score, rank, slot) of the eviction candidate.  The old list of slots stays in shared
+// memory from the first read on, so its shift needs no further meeting.
+//
+// Bound: the latency of one chain per layer and token (state -> slots -> key rows -> two cluster
+// barriers -> stores), about 8 us of it with heads of up to 256 entries per CTA; the keys of a layer
+// (8 MB at budgets of 4096) take 1.3 us at the copy rate.  Cut by slot with a third meeting for the
+// pooled window, a fourth for the list shift, and shuffles for the dot products it was 22 us per
+// launch at budgets of 4096 and 37 us for four requests at 768; now 12 and 10.
+// Dynamic shared memory: (G + 3) words per entry of the largest window (logits, mean, slot, score).
+template <typename T, int G>
+__global__ void __launch_bounds__(DEC_THREADS, 2)
+decode_step_cluster_kernel(const DecodeArgs A, int csize, int cap_words) {
+  extern __shared__ __align__(16) float sh[];
+  __shared__ __align__(16) float2 x_mz[DEC_CLUSTER_WIDE][G];      // (maximum, sum) of every CTA of the cluster
+  __shared__ __align__(16) uint4 x_cand[DEC_CLUSTER_WIDE];        // eviction candidate of every CTA: key, slot
+  __shared__ float red[DEC_THREADS / 32][G], red_z[DEC_THREADS / 32][G];
+  __shared__ float s_m[G];
+  __shared__ unsigned long long red_k[DEC_THREADS / 32];
+  const int crank = (int)cluster_rank();
+  if (csize > 1) cluster_arrive();                   // peers may be written only once they run: waited for below
+  const int g = blockIdx.x / csize, req = blockIdx.y;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int blk = req * A.L + A.layer;
+  const size_t lid = (size_t)blk * A.Hkv + g;
+  const int4 mt = A.meta[lid];
+  const int64_t off = A.dec_off[blk];
+  const int len = mt.x, fre = mt.y, next_pos = mt.z, budget = mt.w;
+  const int cap = len + 1;
+  const int64_t base = off + (int64_t)g * cap;
+  const int part = (cap + csize - 1) / csize;
+  const int r_lo = min(cap, crank * part), r_hi = min(cap, r_lo + part);
+  const int rad = A.kp >> 1;
+  const int w_lo = max(0, r_lo - rad), w_hi = r_hi > r_lo ? min(cap, r_hi + max(rad, 1)) : w_lo;
+  const int n_win = w_hi - w_lo, own = r_lo - w_lo, n_own = r_hi - r_lo;
+  float* lg = sh;                                    // [G][cap_words] logits
+  float* abar = lg + (size_t)G * cap_words;          // group-mean attention
+  int* ord = reinterpret_cast<int*>(abar + cap_words);
+  float* old = reinterpret_cast<float*>(ord + cap_words);
+  T* kc = reinterpret_cast<T*>(A.k_cache) + (size_t)base * A.d;
+  T* vc = reinterpret_cast<T*>(A.v_cache) + (size_t)base * A.d;
+  const T* kn = reinterpret_cast<const T*>(A.k_new) + ((size_t)req * A.Hkv + g) * A.d;
+  const T* vn = reinterpret_cast<const T*>(A.v_new) + ((size_t)req * A.Hkv + g) * A.d;
+  // 1. slots of the window
+  for (int i = threadIdx.x; i < n_win; i += DEC_THREADS) ord[i] = w_lo + i == len ? fre : A.order[base + w_lo + i];
   __syncthreads();
-  for (int h = 0; h < G; ++h) {
-    const float m = s_m[h];
-    float z = 0.f;
-    for (int i = threadIdx.x; i < n_loc; i += DEC_THREADS) {
-      const float e = exp2f(p[(size_t)h * part + i] - m);
-      p[(size_t)h * part + i] = e;
-      z += e;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    if (lane == 0) red_v[warp] = z;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float t = 0.f;
-      for (int w = 0; w < DEC_THREADS / 32; ++w) t += red_v[w];
-      x_z[h] = t;
-    }
-    __syncthreads();
-  }
-  cluster.sync();
-  if (threadIdx.x < G) {
-    float t = 0.f;
-    for (int c = 0; c < DEC_CLUSTER; ++c) t += *cluster.map_shared_rank(&x_z[threadIdx.x], c);
-    s_z[threadIdx.x] = t;
-  }
-  __syncthreads();
-  // 4. group-mean attention of this CTA's slots into the work area (by slot)
-  {
-    float inv_z[G];
-#pragma unroll
-    for (int h = 0; h < G; ++h) inv_z[h] = s_z[h];
-    for (int i = threadIdx.x; i < n_loc; i += DEC_THREADS) {
-      float a = 0.f;
-#pragma unroll
-      for (int h = 0; h < G; ++h) a += p[(size_t)h * part + i] / inv_z[h];
-      aslot[s_lo + i] = a * (1.f / (float)G);
-    }
-  }
-  cluster.sync();                                    // every slot's value is written; sh is free
-  // 5. this CTA's ranks: pooling along the rank order, score update, eviction candidate
+  const int new_i = (w_lo <= len && len < w_hi) ? len - w_lo : -1;
+  // the rows on their way to L2 before the first pass over them waits
+  for (int i = threadIdx.x; i < n_win; i += DEC_THREADS)
+    if (i != new_i)
+      for (int b = 0; b < A.d * (int)sizeof(T); b += 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(kc + (size_t)ord[i] * A.d) + b));
   const int n_obs = cap - A.Sw;                      // entries outside the recent window
   const int n_old = len - A.Sw;                      // of which these already carry a score
-  const int rad = A.kp >> 1;
-  const int rpart = (n_obs + DEC_CLUSTER - 1) / DEC_CLUSTER;
-  const int r_lo = min(n_obs, crank * rpart), r_hi = min(n_obs, r_lo + rpart);
-  const int w_lo = max(0, r_lo - rad), w_hi = min(n_obs, r_hi + rad);
-  float* abar = sh;                                  // ranks w_lo .. w_hi - 1
-#pragma unroll 4
-  for (int i = threadIdx.x; i < w_hi - w_lo; i += DEC_THREADS) abar[i] = aslot[A.order[base + w_lo + i]];
+  for (int i = threadIdx.x; i < n_own; i += DEC_THREADS) old[i] = r_lo + i < n_old ? A.score[base + ord[own + i]] : 0.f;
+  // Everything up to here reads the context's own state of this layer; the caller's tensors may
+  // come from the kernel before this one in the stream.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // 2. logits of the window's rows
+  window_logits<G>(kc, kn, reinterpret_cast<const T*>(A.q_new) + ((size_t)req * A.Hq + g * G) * A.d, A.d, n_win, ord, new_i,
+                   A.scale2, lg, cap_words, red);
   __syncthreads();
-  float worst = CUDART_INF_F;
-  int worst_r = -1;
-#pragma unroll 2
-  for (int r = r_lo + threadIdx.x; r < r_hi; r += DEC_THREADS) {
-    const int lo = max(0, r - rad), hi = min(n_obs, r + rad + 1);
-    float v = abar[lo - w_lo];
-    for (int x = lo + 1; x < hi; ++x) v = A.pool_mode == CAKE_POOL_MAX ? fmaxf(v, abar[x - w_lo]) : v + abar[x - w_lo];
+  // the new token takes the free slot and the last rank
+  if (r_lo <= len && len < r_hi) {
+    const int n16 = A.d * (int)sizeof(T) / 16;
+    if (threadIdx.x < n16)
+      reinterpret_cast<uint4*>(kc + (size_t)fre * A.d)[threadIdx.x] = reinterpret_cast<const uint4*>(kn)[threadIdx.x];
+    else if (threadIdx.x < 2 * n16)
+      reinterpret_cast<uint4*>(vc + (size_t)fre * A.d)[threadIdx.x - n16] = reinterpret_cast<const uint4*>(vn)[threadIdx.x - n16];
+    if (threadIdx.x == 0) A.pos[base + fre] = next_pos;
+  }
+  // 3. maximum of the window and sum of the CTA's own entries, per head (base 2)
+  {
+    float m[G], z[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      float t = red[lane % (DEC_THREADS / 32)][h];
+#pragma unroll
+      for (int o = DEC_THREADS / 64; o > 0; o >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, o));
+      m[h] = t;
+      z[h] = 0.f;
+    }
+    for (int i = own + threadIdx.x; i < own + n_own; i += DEC_THREADS)
+#pragma unroll
+      for (int h = 0; h < G; ++h) z[h] += exp2f(lg[h * cap_words + i] - m[h]);
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) z[h] += __shfl_xor_sync(0xffffffffu, z[h], o);
+      if (lane == h) red_z[warp][h] = z[h];
+      if (threadIdx.x == h) s_m[h] = m[h];
+    }
+  }
+  __syncthreads();
+  if (csize > 1) cluster_wait();                     // every CTA of the cluster runs
+  if (threadIdx.x < csize * G) {
+    const int h = threadIdx.x % G, peer = threadIdx.x / G;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < DEC_THREADS / 32; ++w) t += red_z[w][h];
+    const float2 v = make_float2(s_m[h], t);
+    if (csize > 1) st_remote(&x_mz[crank][h], (uint32_t)peer, v);
+    else x_mz[0][h] = v;
+  }
+  if (csize > 1) { cluster_arrive(); cluster_wait(); } else __syncthreads();
+  // 4. group-mean attention along the window, pooling, score update, eviction candidate
+  //    (every CTA takes the probabilities from the same maximum and sum: entries that share the
+  //    largest neighbour tie exactly, on whichever side of a CTA boundary they lie)
+  float gm[G], fac[G];
+  {
+    // a lane takes head lane % G of every (32 / G)-th CTA
+    const int h = lane % G;
+    float m = -CUDART_INF_F, z = 0.f;
+    for (int c = lane / G; c < csize; c += 32 / G) m = fmaxf(m, x_mz[c][h].x);
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int c = lane / G; c < csize; c += 32 / G) {
+      const float2 v = x_mz[c][h];
+      if (v.y > 0.f) z += v.y * exp2f(v.x - m);
+    }
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    const float f = 1.f / (z * (float)G);
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      gm[k] = __shfl_sync(0xffffffffu, m, k);
+      fac[k] = __shfl_sync(0xffffffffu, f, k);
+    }
+  }
+  for (int i = threadIdx.x; i < n_win; i += DEC_THREADS) {
+    float a = 0.f;
+#pragma unroll
+    for (int h = 0; h < G; ++h) a = fmaf(exp2f(lg[h * cap_words + i] - gm[h]), fac[h], a);
+    abar[i] = a;
+  }
+  __syncthreads();
+  unsigned long long best = kNoKey;
+  for (int i = threadIdx.x; i < n_own; i += DEC_THREADS) {
+    const int r = r_lo + i;
+    if (r >= n_obs) break;
+    const int lo = max(0, r - rad) - w_lo, hi = min(n_obs, r + rad + 1) - w_lo;
+    float v = abar[lo];
+    for (int x = lo + 1; x < hi; ++x) v = A.pool_mode == CAKE_POOL_MAX ? fmaxf(v, abar[x]) : v + abar[x];
     if (A.pool_mode != CAKE_POOL_MAX) v /= (float)A.kp;
-    const int s = A.order[base + r];
     float sc = v;
     if (r < n_old) {
-      const float old = A.score[base + s];
-      sc = A.update_mode == CAKE_DECODE_ADD ? old + v : A.update_mode == CAKE_DECODE_MAX ? fmaxf(old, v) : v;
+      const float o = old[i];
+      sc = A.update_mode == CAKE_DECODE_ADD ? o + v : A.update_mode == CAKE_DECODE_MAX ? fmaxf(o, v) : v;
     }
-    A.score[base + s] = sc;
-    worse_of(worst, worst_r, sc, r);
+    A.score[base + ord[own + i]] = sc;
+    best = min(best, evict_key(sc, r));
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, worst, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, worst_r, o);
-    if (oi >= 0 && (worst_r < 0 || ov < worst || (ov == worst && oi > worst_r))) { worst = ov; worst_r = oi; }
-  }
-  if (lane == 0) { red_v[warp] = worst; red_i[warp] = worst_r; }
+  for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
+  if (lane == 0) red_k[warp] = best;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float bv = CUDART_INF_F;
-    int bi = -1;
-    for (int w = 0; w < DEC_THREADS / 32; ++w)
-      if (red_i[w] >= 0 && (bi < 0 || red_v[w] < bv || (red_v[w] == bv && red_i[w] > bi))) { bv = red_v[w]; bi = red_i[w]; }
-    x_worst = bv;
-    x_worst_r = bi;
+  if (warp == 0) {
+    best = lane < DEC_THREADS / 32 ? red_k[lane] : kNoKey;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
+    const int r = 0x7FFFFFFF - (int)(uint32_t)best;
+    const uint4 v = make_uint4((uint32_t)(best >> 32), (uint32_t)best, best == kNoKey ? 0u : (uint32_t)ord[r - w_lo], 0u);
+    if (csize == 1) { if (lane == 0) x_cand[0] = v; }
+    else if (lane < csize) st_remote(&x_cand[crank], (uint32_t)lane, v);
   }
-  cluster.sync();
-  int ev = -1;
-  if (n_obs > budget) {
-    float bv = CUDART_INF_F;
-    for (int c = 0; c < DEC_CLUSTER; ++c) {
-      const float cv = *cluster.map_shared_rank(&x_worst, c);
-      const int ci = *cluster.map_shared_rank(&x_worst_r, c);
-      if (ci >= 0 && (ev < 0 || cv < bv || (cv == bv && ci > ev))) { bv = cv; ev = ci; }
-    }
+  if (csize > 1) { cluster_arrive(); cluster_wait(); } else __syncthreads();
+  // 5. evict back to the frozen budget: ranks after the evicted one move down by one, its slot
+  //    becomes the free one
+  best = kNoKey;
+  int ev_slot = 0;
+  for (int c = 0; c < csize; ++c) {
+    const uint4 v = x_cand[c];
+    const unsigned long long k = ((unsigned long long)v.x << 32) | v.y;
+    if (k < best) { best = k; ev_slot = (int)v.z; }
   }
-  if (ev < 0) {                                      // below the budget: the cache would have to grow
+  if (best == kNoKey || n_obs <= budget) {           // below the budget: the cache would have to grow
     if (crank == 0 && threadIdx.x == 0) atomicCAS(A.status, 0, CAKE_ERR_CAPACITY);
-    cluster.sync();                                  // nobody leaves while its candidate may still be read
     return;
   }
-  // 6. ranks after the evicted one move down by one; its slot becomes the free one.  Every CTA
-  //    reads the successors of its part of the list, the cluster meets, then it writes them.
-  const int ev_slot = A.order[base + ev];
-  const int m_lo = max(ev, min(cap - 1, crank * part)), m_hi = max(m_lo, min(cap - 1, crank * part + part));
-  int* nxt = reinterpret_cast<int*>(sh);
-#pragma unroll 4
-  for (int i = threadIdx.x; i < m_hi - m_lo; i += DEC_THREADS) nxt[i] = A.order[base + m_lo + i + 1];
-  cluster.sync();
-#pragma unroll 4
-  for (int i = threadIdx.x; i < m_hi - m_lo; i += DEC_THREADS) A.order[base + m_lo + i] = nxt[i];
+  const int ev = 0x7FFFFFFF - (int)(uint32_t)best;
+  for (int i = max(0, ev - r_lo) + (int)threadIdx.x; i < n_own; i += DEC_THREADS) {
+    const int r = r_lo + i;
+    A.order[base + r] = r < len ? ord[own + i + 1] : ev_slot;
+  }
   if (crank == 0 && threadIdx.x == 0) {
-    A.order[base + cap - 1] = ev_slot;
     A.pos[base + ev_slot] = -1;
     A.meta[lid] = make_int4(len, ev_slot, next_pos + 1, budget);
   }
@@ -594,39 +731,45 @@ decode_gather(LayerPtrs ptrs, const int64_t* __restrict__ packed_off, const int6
 }
 
 template <typename T, int G>
-cudaError_t launch_step_cluster_g(dim3 grid, size_t smem, cudaStream_t st, const DecodeArgs& A) {
+cudaError_t launch_step_cluster_g(dim3 grid, int csize, int cap_words, bool early, size_t smem, cudaStream_t st,
+                                  const DecodeArgs& A) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid.x * DEC_CLUSTER, grid.y, 1);
+  cfg.gridDim = dim3(grid.x * csize, grid.y, 1);
   cfg.blockDim = dim3(DEC_THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = DEC_CLUSTER;
+  at[0].val.clusterDim.x = csize;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_step_cluster_kernel<T, G>, A);
+  cfg.numAttrs = early ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, decode_step_cluster_kernel<T, G>, A, csize, cap_words);
 }
 
 template <typename T>
-cudaError_t launch_step_cluster(int device, int G, dim3 grid, size_t smem, cudaStream_t st, const DecodeArgs& A) {
+cudaError_t launch_step_cluster(int device, int G, dim3 grid, int csize, int cap_words, bool early, cudaStream_t st,
+                                const DecodeArgs& A) {
   static PerDeviceOnce attr;
   if (attr.need(device)) {
     cudaError_t e = cudaSuccess;
 #define CAKE_DEC_ATTR(GG) \
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemMax); \
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
     CAKE_DEC_ATTR(1); CAKE_DEC_ATTR(2); CAKE_DEC_ATTR(4); CAKE_DEC_ATTR(8);
 #undef CAKE_DEC_ATTR
     if (e != cudaSuccess) return e;
     attr.mark(device);
   }
+  const size_t smem = (size_t)(G + 3) * cap_words * sizeof(float);
   switch (G) {
-    case 1: return launch_step_cluster_g<T, 1>(grid, smem, st, A);
-    case 2: return launch_step_cluster_g<T, 2>(grid, smem, st, A);
-    case 4: return launch_step_cluster_g<T, 4>(grid, smem, st, A);
-    case 8: return launch_step_cluster_g<T, 8>(grid, smem, st, A);
+    case 1: return launch_step_cluster_g<T, 1>(grid, csize, cap_words, early, smem, st, A);
+    case 2: return launch_step_cluster_g<T, 2>(grid, csize, cap_words, early, smem, st, A);
+    case 4: return launch_step_cluster_g<T, 4>(grid, csize, cap_words, early, smem, st, A);
+    case 8: return launch_step_cluster_g<T, 8>(grid, csize, cap_words, early, smem, st, A);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -706,17 +849,33 @@ int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, cons
   A.smem_cap = (int)cap;
   A.tmp = ctx->d_dec_tmp; A.reqs = ctx->d_req; A.T = ctx->total_tokens; A.n_req = ctx->n_req;
   const dim3 grid(c.n_kv_heads, ctx->n_req);
-  // Large heads are spread over a cluster of DEC_CLUSTER CTAs each (CAKE_DECODE_CLUSTER=0 keeps
-  // every head on one CTA): G floats per slot of a CTA's part, reused for the pooled window.
-  const int64_t part = (ctx->dec_max_cap + DEC_CLUSTER - 1) / DEC_CLUSTER;
-  const size_t smem_cl = ((size_t)G * part + (size_t)c.pool_kernel + 8) * sizeof(float);
+  // A head is spread over the fewest CTAs that leave each at most DEC_CTA_ENTRIES entries (one
+  // pass of its sixteen warps over 16 key rows each), up to DEC_CLUSTER, or up to DEC_CLUSTER_WIDE
+  // while the grid still fits the SMs (at one request of eight heads 64 CTAs would leave half of
+  // them idle).  Heads whose share does not fit a CTA's shared memory even then, tensors that do
+  // not start on a 32-byte boundary, and all heads with CAKE_DECODE_CLUSTER=0, stay on one CTA of
+  // the form that reads 8 bytes at a time and can work in global memory.
+  const int64_t max_cap = ctx->h_dec_cap[layer];
+  const int64_t heads = (int64_t)c.n_kv_heads * ctx->n_req;
+  int csize = 1;
+  while (max_cap > (int64_t)csize * DEC_CTA_ENTRIES &&
+         (csize < DEC_CLUSTER || (csize < DEC_CLUSTER_WIDE && heads * csize * 2 <= ctx->n_sm)))
+    csize *= 2;
+  const int64_t words = (max_cap + csize - 1) / csize + 2 * (c.pool_kernel / 2) + 2;
+  const bool aligned = (((uintptr_t)q_new | (uintptr_t)k_new | (uintptr_t)v_new | (uintptr_t)k_cache | (uintptr_t)v_cache) & 31) == 0;
   const char* env = getenv("CAKE_DECODE_CLUSTER");
-  const bool use_cluster = ctx->dec_max_cap >= DEC_CLUSTER_MIN_CAP && smem_cl <= 200 * 1024 &&
-                           !(env && env[0] == '0');
+  const bool use_cluster = aligned && (size_t)(G + 3) * words * sizeof(float) <= kDecSmemMax && !(env && env[0] == '0');
+  // A step may start while the kernel before it in the stream still runs, read its layer's state and
+  // bring the layer's keys towards the SMs, and then wait.  That state was last written by the same
+  // layer's previous step.  A step lets its successor start only after its own predecessor has
+  // finished, so everything but that one predecessor is complete by then; hence not when the
+  // predecessor may be this layer's own previous step, or the set-up of the cache.
+  const bool early = ctx->dec_last_layer >= 0 && ctx->dec_last_layer != layer;
+  ctx->dec_last_layer = use_cluster ? layer : -1;
   cudaError_t e;
   if (use_cluster)
-    e = c.dtype == CAKE_DTYPE_FP32 ? launch_step_cluster<float>(ctx->device, G, grid, smem_cl, st, A)
-                                   : launch_step_cluster<__nv_bfloat16>(ctx->device, G, grid, smem_cl, st, A);
+    e = c.dtype == CAKE_DTYPE_FP32 ? launch_step_cluster<float>(ctx->device, G, grid, csize, (int)words, early, st, A)
+                                   : launch_step_cluster<__nv_bfloat16>(ctx->device, G, grid, csize, (int)words, early, st, A);
   else
     e = c.dtype == CAKE_DTYPE_FP32 ? launch_step<float>(ctx->device, G, grid, smem, st, A)
                                    : launch_step<__nv_bfloat16>(ctx->device, G, grid, smem, st, A);

@@ -150,3 +150,34 @@ def test_decode_requires_a_finished_prefill():
         cake.decode_begin(ks, vs)
     assert e.value.code == CAKE_ERR_STATE
     cake.destroy()
+
+
+@pytest.mark.parametrize("layers,budget,heads", [(1, 130, (4, 4)), (2, 255, (8, 2)), (2, 256, (8, 1)), (2, 513, (8, 2)),
+                                                 (2, 2055, (4, 2)), (3, 4097, (2, 1))])
+def test_decode_heads_at_the_edges_of_a_cta_share(layers, budget, heads):
+    """Heads just below and above the entries one CTA takes, and above the clusters of 8 and 16; with
+    two or more layers a step starts while the other layer's step still runs."""
+    w = synth.scaled(synth.workload(3), n_layers=layers, n_q_heads=heads[0], n_kv_heads=heads[1],
+                     window=16, seq_lens=(budget * 2 + 77,), total_budget=layers * budget)
+    ties = run_decode(w, steps=4)
+    assert ties <= 1
+
+
+def test_decode_tensors_off_a_32_byte_boundary_give_the_same_state():
+    w = synth.scaled(synth.workload(3), n_layers=1, n_q_heads=8, n_kv_heads=2, seq_lens=(900,), total_budget=300)
+    qs, ks, vs = harness.device_inputs(w)
+    gen = torch.Generator().manual_seed(5)
+    vals = [torch.randn(n * w.head_dim, generator=gen).to(w.torch_dtype).cuda() for n in (8, 2, 2)]
+    states = []
+    for off in (0, 8):                               # 8 bf16 elements: 16 bytes
+        cake = harness.cake_for(w)
+        cake.run(qs, ks, vs, w.cu_seqlens)
+        k_cache, v_cache, _ = cake.decode_begin(ks, vs)
+        q, k, v = (torch.zeros(x.numel() + 8, dtype=x.dtype, device="cuda")[off:off + x.numel()].copy_(x) for x in vals)
+        cake.decode_step(0, q, k, v, k_cache, v_cache)
+        assert cake.status() == 0
+        states.append([x.clone() for x in cake.decode_get_state(0, 0, 300)] + [k_cache.clone(), v_cache.clone()])
+        cake.destroy()
+    assert torch.equal(states[0][0], states[1][0]) and torch.equal(states[0][2], states[1][2])
+    assert torch.allclose(states[0][1], states[1][1], rtol=1e-4, atol=1e-9)
+    assert torch.equal(states[0][3], states[1][3]) and torch.equal(states[0][4], states[1][4])
