@@ -1,8 +1,9 @@
-"""ctypes binding of libcake.so: argument marshalling only.
+"""Binding of libcake.so: argument marshalling only.
 
 Every step of the eviction path runs inside the CUDA library; this module turns
 torch tensors into device pointers, passes the current CUDA stream, and raises
-`CakeError` on a non-zero status.  There is no CPU fallback: if the shared
+`CakeError` on a non-zero status.  The calls of the path go through a small
+extension module (csrc/py_args.cpp), the rest through ctypes.  There is no CPU fallback: if the shared
 library is missing or a tensor is not on a CUDA device the call fails.
 """
 from __future__ import annotations
@@ -58,11 +59,12 @@ class CakeError(RuntimeError):
 
 
 _lib: Optional[ctypes.CDLL] = None
+_fast = None                       # the extension module, bound to the same library
 
 
 def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     """dlopen libcake.so and declare the signatures.  Raises if it is missing."""
-    global _lib
+    global _lib, _fast
     if _lib is not None:
         return _lib
     if not os.path.exists(path):
@@ -110,7 +112,9 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         if name not in ("cake_packed_rows_bound", "cake_strerror", "cake_launch_count",
                         "cake_decode_rows_bound"):
             fn.restype = i32
-    _lib = lib
+    from . import _cake_py
+    _cake_py.init(path)
+    _lib, _fast = lib, _cake_py
     return lib
 
 
@@ -154,9 +158,9 @@ def select_positions_static(values: torch.Tensor, keep: int,
     if out is None:
         out = torch.empty(n_heads, max(keep, 1), dtype=torch.int32, device=values.device)[:, :keep]
         out = out.contiguous()
-    _check(load_library().cake_select_positions_static(
-        _ptr(values, torch.float32), n_heads, n, keep, _ptr(out, torch.int32) if keep > 0 else None,
-        _stream()), "cake_select_positions_static")
+    if _fast is None:
+        load_library()
+    _check(_fast.select(values, n_heads, n, keep, out if keep > 0 else None), "cake_select_positions_static")
     return out
 
 
@@ -176,8 +180,11 @@ class Cake:
                               gamma, tau1, tau2, total_budget, max_requests, max_total_tokens,
                               indicator_mode, alloc_mode, pyramid_slope)
         self.dtype = dtype
+        self._fp32 = dtype == torch.float32
+        self._a = 0                        # address of the context, 0 once destroyed
         self._h = ctypes.c_void_p()
         _check(self.lib.cake_create(ctypes.byref(self.cfg), ctypes.byref(self._h)), "cake_create")
+        self._a = self._h.value
         self.n_req = 0
         self.total_tokens = 0
         self.seq_lens: List[int] = []
@@ -187,6 +194,7 @@ class Cake:
         if getattr(self, "_h", None) and self._h.value:
             self.lib.cake_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._a = 0
 
     def __del__(self):
         try:
@@ -197,22 +205,20 @@ class Cake:
     # -- the path
     def begin(self, cu_seqlens: Sequence[int]) -> None:
         n_req = len(cu_seqlens) - 1
-        arr = (ctypes.c_int64 * (n_req + 1))(*[int(x) for x in cu_seqlens])
-        _check(self.lib.cake_begin(self._h, n_req, arr, _stream()), "cake_begin")
+        _check(_fast.begin(self._a, cu_seqlens), "cake_begin")
         self.n_req = n_req
         self.total_tokens = int(cu_seqlens[-1]) if n_req > 0 else 0
         self.seq_lens = [int(cu_seqlens[r + 1] - cu_seqlens[r]) for r in range(n_req)]
 
     def score_layer(self, layer: int, q_win: torch.Tensor, k: torch.Tensor,
                     lse: Optional[torch.Tensor] = None) -> None:
-        _check(self.lib.cake_score_layer(self._h, layer, _ptr(q_win, self.dtype), _ptr(k, self.dtype),
-                                         _ptr(lse, torch.float32), _stream()), "cake_score_layer")
+        _check(_fast.score_layer(self._a, layer, self._fp32, q_win, k, lse), "cake_score_layer")
 
     def allocate(self, stage: int) -> None:
-        _check(self.lib.cake_allocate(self._h, stage, _stream()), "cake_allocate")
+        _check(_fast.allocate(self._a, stage), "cake_allocate")
 
     def evict(self, stage: int) -> None:
-        _check(self.lib.cake_evict(self._h, stage, _stream()), "cake_evict")
+        _check(_fast.evict(self._a, stage), "cake_evict")
 
     def packed_rows_bound(self) -> int:
         v = int(self.lib.cake_packed_rows_bound(self._h))
@@ -238,13 +244,8 @@ class Cake:
             row_offsets = torch.empty(self.n_req * L + 1, dtype=torch.int64, device=dev)
         if positions is None and want_positions:
             positions = torch.empty(max(rows, 1), dtype=torch.int32, device=dev)
-        # K/V of a layer may also live in pinned host memory: the gather then fetches only the
-        # retained rows over the bus
-        kp = (ctypes.c_void_p * L)(*[(_ptr(t, self.dtype, True) if t is not None else None) for t in k_layers])
-        vp = (ctypes.c_void_p * L)(*[(_ptr(t, self.dtype, True) if t is not None else None) for t in v_layers])
-        _check(self.lib.cake_compact(self._h, layer_lo, hi, kp, vp, _ptr(k_out), _ptr(v_out),
-                                     _ptr(row_offsets, torch.int64), _ptr(positions, torch.int32),
-                                     _stream()), "cake_compact")
+        _check(_fast.compact(self._a, L, self._fp32, layer_lo, hi, k_layers, v_layers, k_out, v_out, row_offsets, positions),
+               "cake_compact")
         return k_out, v_out, row_offsets, positions
 
     def compact_int4(self, k_layers, v_layers, group: int = 32):
@@ -262,12 +263,7 @@ class Cake:
                    row_offsets=torch.empty(self.n_req * L + 1, dtype=torch.int64, device=dev),
                    kgroup_offsets=torch.empty(self.n_req * L + 1, dtype=torch.int64, device=dev),
                    positions=torch.empty(rows, dtype=torch.int32, device=dev))
-        kp = (ctypes.c_void_p * L)(*[_ptr(t, self.dtype) for t in k_layers])
-        vp = (ctypes.c_void_p * L)(*[_ptr(t, self.dtype) for t in v_layers])
-        _check(self.lib.cake_compact_int4(
-            self._h, 0, L, kp, vp, group, _ptr(out["k_codes"]), _ptr(out["k_scale"]), _ptr(out["k_zero"]),
-            _ptr(out["v_codes"]), _ptr(out["v_scale"]), _ptr(out["v_zero"]), _ptr(out["row_offsets"]),
-            _ptr(out["kgroup_offsets"]), _ptr(out["positions"]), _stream()), "cake_compact_int4")
+        _check(_fast.compact_int4(self._a, L, self._fp32, group, k_layers, v_layers, *out.values()), "cake_compact_int4")
         return out
 
     # -- getters / hooks
@@ -329,9 +325,9 @@ class Cake:
         return k_cache, v_cache, off
 
     def decode_step(self, layer: int, q_new, k_new, v_new, k_cache, v_cache) -> None:
-        _check(self.lib.cake_decode_step(self._h, layer, _ptr(q_new, self.dtype), _ptr(k_new, self.dtype),
-                                         _ptr(v_new, self.dtype), _ptr(k_cache), _ptr(v_cache),
-                                         _stream()), "cake_decode_step")
+        rc = _fast.decode_step(self._a, layer, self._fp32, q_new, k_new, v_new, k_cache, v_cache)
+        if rc:
+            raise CakeError(rc, "cake_decode_step")
 
     def decode_get_state(self, req: int, layer: int, length: int):
         """(positions, scores, slots), each [H_kv][length], entries in ascending token position."""
@@ -339,8 +335,7 @@ class Cake:
         pos = torch.empty(H, length, dtype=torch.int32, device="cuda")
         sc = torch.empty(H, length, dtype=torch.float32, device="cuda")
         sl = torch.empty(H, length, dtype=torch.int32, device="cuda")
-        _check(self.lib.cake_decode_get_state(self._h, req, layer, _ptr(pos), _ptr(sc), _ptr(sl),
-                                              _stream()), "cake_decode_get_state")
+        _check(_fast.decode_get_state(self._a, req, layer, pos, sc, sl), "cake_decode_get_state")
         return pos, sc, sl
 
     def set_wait_limit(self, cycles: int) -> None:
@@ -374,8 +369,5 @@ class Cake:
             v_layers: Sequence[torch.Tensor], cu_seqlens: Sequence[int], **compact_kw):
         """begin; for every layer score -> allocate -> evict; compact once at the end."""
         self.begin(cu_seqlens)
-        for l in range(self.cfg.n_layers):
-            self.score_layer(l, q_layers[l], k_layers[l])
-            self.allocate(l)
-            self.evict(l)
+        _check(_fast.prefill(self._a, self.cfg.n_layers, self._fp32, q_layers, k_layers), "cake_score_layer / allocate / evict")
         return self.compact(k_layers, v_layers, **compact_kw)

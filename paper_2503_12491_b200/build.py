@@ -1,4 +1,4 @@
-"""Builds libcake.so (sm_100a only) in-tree with nvcc.
+"""Builds libcake.so (sm_100a only, nvcc) and _cake_py.so (the binding's native half, g++) in-tree.
 
     python -m paper_2503_12491_b200.build [--force] [--verbose]
 """
@@ -8,6 +8,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from typing import List
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +16,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libcake.so")
+PY_SOURCE = os.path.join(CSRC, "py_args.cpp")
+PY_LIB = os.path.join(PKG, "_cake_py.so")
 
 SOURCES = ["cake_api.cu", "score_simt.cu", "score_tc.cu", "cascade.cu", "compact.cu",
            "decode.cu", "quant.cu", "select_static.cu"]
@@ -41,8 +44,33 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _inputs())
 
 
+def _run(cmd: List[str], what: str, verbose: bool) -> None:
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError(f"compiler failed building {what}")
+
+
+def build_binding(force: bool = False, verbose: bool = False) -> None:
+    """Compiles the native half of binding.py against this interpreter and its torch."""
+    deps = [PY_SOURCE, os.path.join(INCLUDE, "cake.h")]
+    if not force and os.path.exists(PY_LIB) and all(os.path.getmtime(f) <= os.path.getmtime(PY_LIB) for f in deps):
+        return
+    import torch
+    home = os.path.dirname(torch.__file__)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+    libs = os.path.join(home, "lib")
+    _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", INCLUDE,
+          "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(home, "include"), "-isystem", cuda,
+          PY_SOURCE, "-o", PY_LIB, "-L", libs, f"-Wl,-rpath,{libs}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
+          "-lc10_cuda", "-ldl"], "_cake_py.so", verbose)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compiles every CUDA source for sm_100a into one shared library."""
+    """Compiles every CUDA source for sm_100a into one shared library, and the binding's native half."""
+    build_binding(force, verbose)
     if not force and not is_stale():
         return LIB
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3",
@@ -51,11 +79,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         cmd += ["-Xptxas", "-v"]
     cmd += [os.path.join(CSRC, s) for s in SOURCES] + ["-o", LIB]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed building libcake.so")
+    _run(cmd, "libcake.so", verbose)
     return LIB
 
 
