@@ -207,6 +207,14 @@ int32_t cake_compact_int4(cake_ctx* ctx, int32_t layer_lo, int32_t layer_hi,
                           int64_t* row_offsets_out, int64_t* kgroup_offsets_out,
                           int32_t* positions_out, void* stream);
 
+/* Zeroes what the calls above leave unwritten at the end of buffers allocated by an upper bound:
+ * rows used_rows[i][0] .. rows[i]-1 of buffer i, a row being row_bytes[i] bytes.  bufs, row_bytes,
+ * rows and used_rows are HOST arrays of n <= CAKE_CLEAR_MAX entries; used_rows[i] is a DEVICE pointer
+ * to the count (the last entry of an offsets array). */
+#define CAKE_CLEAR_MAX 8
+int32_t cake_clear_unused(int32_t n, void* const* bufs, const int64_t* row_bytes, const int64_t* rows,
+                          const int64_t* const* used_rows, void* stream);
+
 /* Upper bound on the rows cake_compact writes for the current batch:
  * H_kv * sum_r min(B_total, L*N_r).  Returns the bound or a negative error. */
 int64_t cake_packed_rows_bound(const cake_ctx* ctx);

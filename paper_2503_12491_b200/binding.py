@@ -32,7 +32,7 @@ EXPORTS = [
     "cake_profile_enable", "cake_profile_read", "cake_uses_tensor_cores",
     "cake_select_positions_static", "cake_plan_info", "cake_set_wait_limit", "cake_debug_skew_sync",
     "cake_decode_rows_bound", "cake_decode_begin", "cake_decode_step", "cake_decode_get_state",
-    "cake_compact_int4", "cake_plan_check",
+    "cake_compact_int4", "cake_plan_check", "cake_clear_unused",
 ]
 PROF_KINDS = ["score", "finalize", "allocate", "evict", "compact"]
 
@@ -80,6 +80,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.cake_compact.argtypes = [vp, i32, i32, ctypes.POINTER(vp), ctypes.POINTER(vp), vp, vp, vp, vp, vp]
     lib.cake_compact_int4.argtypes = [vp, i32, i32, ctypes.POINTER(vp), ctypes.POINTER(vp), i32,
                                       vp, vp, vp, vp, vp, vp, vp, vp, vp, vp]
+    lib.cake_clear_unused.argtypes = [i32, ctypes.POINTER(vp), ctypes.POINTER(i64), ctypes.POINTER(i64),
+                                      ctypes.POINTER(vp), vp]
     lib.cake_packed_rows_bound.argtypes = [vp]
     lib.cake_packed_rows_bound.restype = i64
     lib.cake_get_indicators.argtypes = [vp, i32, vp, vp]
@@ -254,16 +256,20 @@ class Cake:
         dev = torch.device("cuda", torch.cuda.current_device())
         rows = max(self.packed_rows_bound(), 1)
         kg = rows // group + self.n_req * L * self.cfg.n_kv_heads + 1
-        out = dict(k_codes=torch.zeros(rows, d // 2, dtype=torch.uint8, device=dev),
-                   k_scale=torch.zeros(kg, d, dtype=torch.float32, device=dev),
-                   k_zero=torch.zeros(kg, d, dtype=torch.float32, device=dev),
-                   v_codes=torch.zeros(rows, d // 2, dtype=torch.uint8, device=dev),
-                   v_scale=torch.zeros(rows, d // group, dtype=torch.float32, device=dev),
-                   v_zero=torch.zeros(rows, d // group, dtype=torch.float32, device=dev),
+        # rows beyond the retained ones read as zero
+        out = dict(k_codes=torch.empty(rows, d // 2, dtype=torch.uint8, device=dev),
+                   k_scale=torch.empty(kg, d, dtype=torch.float32, device=dev),
+                   k_zero=torch.empty(kg, d, dtype=torch.float32, device=dev),
+                   v_codes=torch.empty(rows, d // 2, dtype=torch.uint8, device=dev),
+                   v_scale=torch.empty(rows, d // group, dtype=torch.float32, device=dev),
+                   v_zero=torch.empty(rows, d // group, dtype=torch.float32, device=dev),
                    row_offsets=torch.empty(self.n_req * L + 1, dtype=torch.int64, device=dev),
                    kgroup_offsets=torch.empty(self.n_req * L + 1, dtype=torch.int64, device=dev),
                    positions=torch.empty(rows, dtype=torch.int32, device=dev))
         _check(_fast.compact_int4(self._a, L, self._fp32, group, k_layers, v_layers, *out.values()), "cake_compact_int4")
+        ro, ko = out["row_offsets"], out["kgroup_offsets"]
+        _check(_fast.clear_unused((out["k_codes"], out["k_scale"], out["k_zero"], out["v_codes"], out["v_scale"], out["v_zero"]),
+                                  (ro, ko, ko, ro, ro, ro)), "cake_clear_unused")
         return out
 
     # -- getters / hooks

@@ -9,18 +9,53 @@
 namespace cake {
 namespace {
 
-// row_offsets[r*L + l] = first packed row of block (r, l); lengths of layers
-// outside [lo, hi) or not yet evicted count as zero.
-__global__ void packed_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ offsets,
-                               int n_req, int L, int lo, int hi, int Hkv, int Sw) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int64_t acc = 0;
-  for (int r = 0; r < n_req; ++r)
-    for (int l = 0; l < L; ++l) {
-      offsets[(size_t)r * L + l] = acc;
-      if (l >= lo && l < hi) acc += (int64_t)Hkv * (budget[(size_t)r * L + l] + Sw);
+// First row of every block (r, l) = index r*L + l in the packed cache, and, where asked for, its
+// first key group of the 4-bit layout and its first row of the decode cache (one spare row per
+// head).  Layers outside [lo, hi) have no rows.  One CTA, block scans over the blocks (one thread
+// that walked them took 4 us at 64 blocks, 11 us at 256).
+constexpr int OFF_THREADS = 1024;
+__global__ void __launch_bounds__(OFF_THREADS)
+block_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ row_off, int64_t* __restrict__ key_off,
+              int64_t* __restrict__ dec_off, int nblk, int L, int lo, int hi, int Hkv, int Sw, int group) {
+  __shared__ int64_t tot[2][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = (int)blockDim.x >> 5;
+  int64_t base0 = 0, base1 = 0;                       // rows and key groups (or heads) so far
+  for (int i0 = 0; i0 < nblk; i0 += (int)blockDim.x) {
+    const int i = i0 + (int)threadIdx.x, l = i % L;
+    int64_t a = 0, b = 0;
+    if (i < nblk && l >= lo && l < hi) {
+      const int len = budget[i] + Sw;
+      a = (int64_t)Hkv * len;
+      b = key_off ? (int64_t)Hkv * ((len + group - 1) / group) : (int64_t)Hkv;
     }
-  offsets[(size_t)n_req * L] = acc;
+    int64_t sa = a, sb = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t na = __shfl_up_sync(0xffffffffu, sa, o), nb = __shfl_up_sync(0xffffffffu, sb, o);
+      if (lane >= o) { sa += na; sb += nb; }
+    }
+    if (lane == 31) { tot[0][warp] = sa; tot[1][warp] = sb; }
+    __syncthreads();
+    int64_t pa = base0, pb = base1;
+    for (int w = 0; w < n_warps; ++w) {
+      if (w < warp) { pa += tot[0][w]; pb += tot[1][w]; }
+      base0 += tot[0][w];
+      base1 += tot[1][w];
+    }
+    pa += sa - a;
+    pb += sb - b;
+    if (i < nblk) {
+      row_off[i] = pa;
+      if (key_off) key_off[i] = pb;
+      if (dec_off) dec_off[i] = pa + pb;             // a spare row per head
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    row_off[nblk] = base0;
+    if (key_off) key_off[nblk] = base1;
+    if (dec_off) dec_off[nblk] = base0 + base1;
+  }
 }
 
 constexpr int POS_THREADS = 1024;
@@ -155,6 +190,19 @@ gather_rows(LayerPtrs ptrs, const int64_t* __restrict__ offsets, const int32_t* 
   }
 }
 
+}  // namespace
+
+int32_t run_offsets(cake_ctx* ctx, int lo, int hi, int64_t* row_off, int64_t* key_off, int group, int64_t* dec_off,
+                    cudaStream_t st) {
+  const cake_config& c = ctx->cfg;
+  const int nblk = ctx->n_req * c.n_layers;
+  const int threads = nblk >= OFF_THREADS ? OFF_THREADS : nblk > 32 ? (nblk + 31) / 32 * 32 : 32;
+  block_offsets<<<1, threads, 0, st>>>(ctx->n_req > 0 ? ctx->d_budget[(ctx->n_evicted - 1) & 1] : nullptr, row_off, key_off,
+                                       dec_off, nblk, c.n_layers, lo, hi, c.n_kv_heads, c.window, group);
+  count_launch();
+  return cuda_status(cudaGetLastError());
+}
+
 int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi, const int64_t* offsets,
                              int32_t* out, int64_t capacity, cudaStream_t st) {
   const cake_config& c = ctx->cfg;
@@ -182,19 +230,15 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
   return cuda_status(cudaGetLastError());
 }
 
-}  // namespace
-
 int32_t launch_compact(cake_ctx* ctx, int32_t lo, int32_t hi, const LayerPtrs& ptrs, void* k_out,
                        void* v_out, int64_t* row_offsets, int32_t* positions, cudaStream_t st) {
   const cake_config& c = ctx->cfg;
   const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
-  packed_offsets<<<1, 32, 0, st>>>(budget, row_offsets, ctx->n_req, c.n_layers, lo, hi,
-                                   c.n_kv_heads, c.window);
-  count_launch();
-  if (ctx->n_req == 0 || hi <= lo) return cuda_status(cudaGetLastError());
+  int32_t rc = run_offsets(ctx, lo, hi, row_offsets, nullptr, 1, nullptr, st);
+  if (rc != CAKE_OK || ctx->n_req == 0 || hi <= lo) return rc;
   // positions in packed row order: into the caller's buffer if there is one
   int32_t* pos = positions ? positions : ctx->d_pos_packed;
-  int32_t rc = run_sorted_positions(ctx, 0, ctx->n_req, lo, hi, row_offsets, pos, 0, st);
+  rc = run_sorted_positions(ctx, 0, ctx->n_req, lo, hi, row_offsets, pos, 0, st);
   if (rc != CAKE_OK) return rc;
   const int esize = c.dtype == CAKE_DTYPE_FP32 ? 4 : 2;
   const int cpr = c.head_dim * esize / 16;
@@ -205,33 +249,52 @@ int32_t launch_compact(cake_ctx* ctx, int32_t lo, int32_t hi, const LayerPtrs& p
   return cuda_status(cudaGetLastError());
 }
 
-// Packed row offsets and positions of layers [lo, hi): the first half of a compaction.
-int32_t run_packed_positions(cake_ctx* ctx, int32_t lo, int32_t hi, int64_t* row_offsets, int32_t* positions,
-                             cudaStream_t st) {
-  const cake_config& c = ctx->cfg;
-  const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
-  packed_offsets<<<1, 32, 0, st>>>(budget, row_offsets, ctx->n_req, c.n_layers, lo, hi, c.n_kv_heads,
-                                   c.window);
-  count_launch();
-  if (ctx->n_req == 0 || hi <= lo) return cuda_status(cudaGetLastError());
-  return run_sorted_positions(ctx, 0, ctx->n_req, lo, hi, row_offsets, positions, 0, st);
-}
-
-// Packed row offsets and positions of every layer into context scratch (decode-time set-up).
-int32_t run_sorted_positions_packed(cake_ctx* ctx, const int64_t* offsets_c, int32_t* out, cudaStream_t st) {
-  const cake_config& c = ctx->cfg;
-  int64_t* offsets = const_cast<int64_t*>(offsets_c);
-  const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
-  packed_offsets<<<1, 32, 0, st>>>(budget, offsets, ctx->n_req, c.n_layers, 0, c.n_layers, c.n_kv_heads,
-                                   c.window);
-  count_launch();
-  return run_sorted_positions(ctx, 0, ctx->n_req, 0, c.n_layers, offsets, out, 0, st);
-}
-
 int32_t launch_get_positions(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* out,
                              int64_t capacity, cudaStream_t st) {
   if (capacity < 0) return CAKE_ERR_ARG;
   return run_sorted_positions(ctx, req, 1, layer, layer + 1, nullptr, out, capacity, st);
 }
 
+namespace {
+struct ClearArgs {
+  uint8_t* buf[CAKE_CLEAR_MAX];
+  const int64_t* used[CAKE_CLEAR_MAX];
+  int64_t row_bytes[CAKE_CLEAR_MAX], rows[CAKE_CLEAR_MAX];
+};
+// Rows [*used, rows) of every buffer; blockIdx.y = buffer.  Usually a few rows or none.
+__global__ void clear_unused(const ClearArgs A) {
+  const int b = blockIdx.y;
+  const int64_t lo = *A.used[b] * A.row_bytes[b], hi = A.rows[b] * A.row_bytes[b];
+  uint8_t* p = A.buf[b];
+  const int64_t mid = min(hi, (lo + 15) & ~(int64_t)15), last = max(mid, hi & ~(int64_t)15);   // 16-byte part, if aligned
+  const bool vec = ((uintptr_t)p & 15) == 0;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+  if (vec) {
+    for (int64_t i = lo + t; i < mid; i += nt) p[i] = 0;
+    for (int64_t i = mid / 16 + t; i < last / 16; i += nt) reinterpret_cast<uint4*>(p)[i] = make_uint4(0, 0, 0, 0);
+    for (int64_t i = last + t; i < hi; i += nt) p[i] = 0;
+  } else {
+    for (int64_t i = lo + t; i < hi; i += nt) p[i] = 0;
+  }
+}
+}  // namespace
+
 }  // namespace cake
+
+extern "C" int32_t cake_clear_unused(int32_t n, void* const* bufs, const int64_t* row_bytes, const int64_t* rows,
+                                     const int64_t* const* used_rows, void* stream) {
+  using namespace cake;
+  if (n < 0 || n > CAKE_CLEAR_MAX || (n > 0 && (!bufs || !row_bytes || !rows || !used_rows))) return CAKE_ERR_ARG;
+  if (n == 0) return CAKE_OK;
+  ClearArgs A;
+  for (int i = 0; i < n; ++i) {
+    if (!bufs[i] || !used_rows[i] || row_bytes[i] < 0 || rows[i] < 0) return CAKE_ERR_ARG;
+    A.buf[i] = (uint8_t*)bufs[i];
+    A.used[i] = used_rows[i];
+    A.row_bytes[i] = row_bytes[i];
+    A.rows[i] = rows[i];
+  }
+  clear_unused<<<dim3(64, n), 256, 0, (cudaStream_t)stream>>>(A);
+  count_launch();
+  return cuda_status(cudaGetLastError());
+}

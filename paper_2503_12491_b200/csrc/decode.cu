@@ -34,18 +34,6 @@ __device__ __forceinline__ float key_to_float(uint32_t key) {
   return __uint_as_float(b);
 }
 
-// Decode row offsets: block (r, l) occupies H_kv * (len + 1) rows.
-__global__ void decode_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ offsets,
-                               int n_req, int L, int Hkv, int Sw) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int64_t acc = 0;
-  for (int i = 0; i < n_req * L; ++i) {
-    offsets[i] = acc;
-    acc += (int64_t)Hkv * (budget[i] + Sw + 1);
-  }
-  offsets[(size_t)n_req * L] = acc;
-}
-
 // One CTA per (head, layer, request): positions (ascending, from the packed order), identity
 // slot order, and the stored indicator of every survivor, found by binary search of its position.
 __global__ void __launch_bounds__(DEC_THREADS)
@@ -798,20 +786,18 @@ cudaError_t launch_step(int device, int G, dim3 grid, size_t smem, cudaStream_t 
 
 }  // namespace
 
-int32_t run_sorted_positions_packed(cake_ctx* ctx, const int64_t* offsets, int32_t* out, cudaStream_t st);
-
 int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache, void* v_cache,
                             int64_t* row_offsets, cudaStream_t st) {
   const cake_config& c = ctx->cfg;
   const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
-  decode_offsets<<<1, 32, 0, st>>>(budget, ctx->d_dec_off, ctx->n_req, c.n_layers, c.n_kv_heads, c.window);
-  count_launch();
+  int32_t rc = run_offsets(ctx, 0, c.n_layers, ctx->d_dec_packed_off, nullptr, 1, ctx->d_dec_off, st);
+  if (rc != CAKE_OK) return rc;
   if (row_offsets)
     CAKE_CUDA_TRY(cudaMemcpyAsync(row_offsets, ctx->d_dec_off, sizeof(int64_t) * (ctx->n_req * c.n_layers + 1),
                                   cudaMemcpyDeviceToDevice, st));
-  if (ctx->n_req == 0) return cuda_status(cudaGetLastError());
+  if (ctx->n_req == 0) return CAKE_OK;
   // positions in packed order (context scratch), then the decode state and the rows
-  int32_t rc = run_sorted_positions_packed(ctx, ctx->d_dec_packed_off, ctx->d_pos_packed, st);
+  rc = run_sorted_positions(ctx, 0, ctx->n_req, 0, c.n_layers, ctx->d_dec_packed_off, ctx->d_pos_packed, 0, st);
   if (rc != CAKE_OK) return rc;
   const dim3 grid(c.n_kv_heads, c.n_layers, ctx->n_req);
   decode_build<<<grid, DEC_THREADS, 0, st>>>(ctx->d_lists, ctx->d_prefix, ctx->d_lstate, ctx->d_req, budget,

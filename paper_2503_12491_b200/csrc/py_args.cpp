@@ -26,6 +26,7 @@ struct Lib {
   decltype(&cake_evict) evict;
   decltype(&cake_compact) compact;
   decltype(&cake_compact_int4) compact_int4;
+  decltype(&cake_clear_unused) clear_unused;
   decltype(&cake_decode_step) decode_step;
   decltype(&cake_decode_get_state) decode_get_state;
   decltype(&cake_select_positions_static) select_positions_static;
@@ -162,8 +163,8 @@ PyObject* init(PyObject*, PyObject* path) {
     PyErr_SetString(PyExc_ImportError, "libcake lacks cake_" #name); \
     return nullptr;                                                \
   }
-  SYM(begin) SYM(score_layer) SYM(allocate) SYM(evict) SYM(compact) SYM(compact_int4) SYM(decode_step)
-  SYM(decode_get_state) SYM(select_positions_static)
+  SYM(begin) SYM(score_layer) SYM(allocate) SYM(evict) SYM(compact) SYM(compact_int4) SYM(clear_unused)
+  SYM(decode_step) SYM(decode_get_state) SYM(select_positions_static)
 #undef SYM
   Py_RETURN_NONE;
 }
@@ -259,6 +260,30 @@ PyObject* compact_int4(PyObject*, PyObject* const* a, Py_ssize_t n) {
                         (float*)o[4], (float*)o[5], (int64_t*)o[6], (int64_t*)o[7], (int32_t*)o[8], st));
 }
 
+// clear_unused(tensors, offsets): zeroes the rows of every tensor beyond the last entry of its offsets
+PyObject* clear_unused(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (!arity(n, 2)) return nullptr;
+  std::vector<const void*> t, off;
+  if (!ptrs(a[0], kAny, false, t) || !ptrs(a[1], at::ScalarType::Long, false, off)) return nullptr;
+  const int32_t m = (int32_t)t.size();
+  void* bufs[CAKE_CLEAR_MAX];
+  const int64_t* used[CAKE_CLEAR_MAX];
+  int64_t bytes[CAKE_CLEAR_MAX], rows[CAKE_CLEAR_MAX];
+  if (m > CAKE_CLEAR_MAX || off.size() != t.size()) {
+    PyErr_SetString(PyExc_ValueError, "clear_unused: too many tensors");
+    return nullptr;
+  }
+  for (int32_t i = 0; i < m; ++i) {
+    const at::Tensor& x = THPVariable_Unpack(PySequence_Fast_GET_ITEM(a[0], i));
+    const at::Tensor& o = THPVariable_Unpack(PySequence_Fast_GET_ITEM(a[1], i));
+    bufs[i] = const_cast<void*>(t[i]);
+    rows[i] = x.size(0);
+    bytes[i] = rows[i] > 0 ? (int64_t)x.nbytes() / rows[i] : 0;
+    used[i] = (const int64_t*)off[i] + (o.numel() - 1);
+  }
+  DONE(lib.clear_unused(m, bufs, bytes, rows, used, st));
+}
+
 // decode_step(ctx, layer, is_fp32, q_new, k_new, v_new, k_cache, v_cache)
 PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void *q, *k, *v, *kc, *vc;
@@ -293,7 +318,7 @@ PyObject* select(PyObject*, PyObject* const* a, Py_ssize_t n) {
 #define FAST(f) {#f, (PyCFunction)(void (*)(void))f, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {{"init", init, METH_O, nullptr},
                          FAST(begin), FAST(score_layer), FAST(allocate), FAST(evict), FAST(prefill), FAST(compact),
-                         FAST(compact_int4), FAST(decode_step), FAST(decode_get_state), FAST(select),
+                         FAST(compact_int4), FAST(clear_unused), FAST(decode_step), FAST(decode_get_state), FAST(select),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_cake_py", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -76,3 +76,38 @@ def test_int4_compaction_rejects_bad_groups():
             cake.compact_int4(ks, vs, group=group)
         assert e.value.code == CAKE_ERR_ARG
     cake.destroy()
+
+
+@pytest.mark.parametrize("dtype,d,group,budget,shift", [("bf16", 64, 32, 65, 0), ("bf16", 64, 64, 63, 0), ("bf16", 128, 32, 33, 1),
+                                                        ("fp32", 128, 128, 129, 0), ("fp32", 128, 64, 47, 1), ("fp32", 64, 32, 96, 0)])
+def test_int4_rows_at_the_edges_of_a_group_and_off_the_vector_boundary(dtype, d, group, budget, shift):
+    """Heads a row longer or shorter than whole groups and than a warp's 32 rows, every head size and
+    type of the row kernel, values at exact half-steps, and K/V that start off a 16-byte boundary."""
+    w = synth.scaled(synth.workload(1 if dtype == "fp32" else 3), n_layers=2, n_q_heads=4, n_kv_heads=2, head_dim=d,
+                     window=16 if dtype == "fp32" else 32, seq_lens=(301, 150), total_budget=2 * budget)
+    L = w.n_layers
+    qs, ks, vs = harness.device_inputs(w)
+    for t in ks + vs:                                # coarse values: many quotients lie half-way between codes
+        t[:, ::3] = (t[:, ::3].float() * 4).round().div(4).to(t.dtype)
+    cake = harness.cake_for(w)
+    k_out, v_out, off, _ = cake.run(qs, ks, vs, w.cu_seqlens)
+    odd = lambda t: torch.zeros(t.numel() + 8, dtype=t.dtype, device="cuda")[shift:shift + t.numel()].view(t.shape).copy_(t)
+    out = cake.compact_int4([odd(t) for t in ks], [odd(t) for t in vs], group=group)
+    assert cake.status() == 0
+    n_rows, off_h, kg = int(off[-1]), off.cpu().numpy(), out["kgroup_offsets"].cpu().numpy()
+    got = {k: v.cpu().numpy() for k, v in out.items()}
+    k_rows, v_rows = to_f32(k_out[:n_rows]), to_f32(v_out[:n_rows])
+    q, s, z = O.quantize_values_per_token(v_rows, group)
+    assert np.array_equal(got["v_codes"][:n_rows], O.pack_nibbles(q))
+    assert np.array_equal(got["v_scale"][:n_rows], s) and np.array_equal(got["v_zero"][:n_rows], z)
+    for blk in range(len(w.seq_lens) * L):
+        length = (off_h[blk + 1] - off_h[blk]) // w.n_kv_heads
+        gpb = (length + group - 1) // group
+        for g in range(w.n_kv_heads):
+            a, ga = off_h[blk] + g * length, kg[blk] + g * gpb
+            q, s, z = O.quantize_keys_per_channel(k_rows[a:a + length], group)
+            assert np.array_equal(got["k_codes"][a:a + length], O.pack_nibbles(q)), (blk, g)
+            assert np.array_equal(got["k_scale"][ga:ga + gpb], s) and np.array_equal(got["k_zero"][ga:ga + gpb], z)
+    for name, used in (("k_codes", n_rows), ("v_codes", n_rows), ("v_scale", n_rows), ("k_scale", kg[-1]), ("k_zero", kg[-1])):
+        assert not got[name][used:].any(), name      # beyond the retained rows: zero
+    cake.destroy()
