@@ -320,14 +320,16 @@ class Cake:
         if rows < 0:
             raise CakeError(rows, "cake_decode_rows_bound")
         dev = torch.device("cuda", torch.cuda.current_device())
-        k_cache = torch.zeros(max(rows, 1), self.cfg.head_dim, dtype=self.dtype, device=dev)
-        v_cache = torch.zeros(max(rows, 1), self.cfg.head_dim, dtype=self.dtype, device=dev)
+        # spare rows, and rows beyond the last head's, read as zero
+        k_cache = torch.empty(max(rows, 1), self.cfg.head_dim, dtype=self.dtype, device=dev)
+        v_cache = torch.empty(max(rows, 1), self.cfg.head_dim, dtype=self.dtype, device=dev)
         off = torch.empty(self.n_req * L + 1, dtype=torch.int64, device=dev)
         kp = (ctypes.c_void_p * L)(*[_ptr(t, self.dtype) for t in k_layers])
         vp = (ctypes.c_void_p * L)(*[_ptr(t, self.dtype) for t in v_layers])
         _check(self.lib.cake_decode_begin(self._h, kp, vp, _ptr(k_cache), _ptr(v_cache),
                                           _ptr(off, torch.int64), update_mode, _stream()),
                "cake_decode_begin")
+        _check(_fast.clear_unused((k_cache, v_cache), (off, off)), "cake_clear_unused")
         return k_cache, v_cache, off
 
     def decode_step(self, layer: int, q_new, k_new, v_new, k_cache, v_cache) -> None:

@@ -229,6 +229,8 @@ int32_t launch_compact(cake_ctx* ctx, int32_t lo, int32_t hi, const LayerPtrs& p
                        void* v_out, int64_t* row_offsets, int32_t* positions, cudaStream_t st);
 int32_t run_offsets(cake_ctx* ctx, int lo, int hi, int64_t* row_off, int64_t* key_off, int group, int64_t* dec_off,
                     cudaStream_t st);
+int32_t run_gather(cake_ctx* ctx, const LayerPtrs& ptrs, const int64_t* row_off, const int64_t* dec_off, const int32_t* pos,
+                   void* k_out, void* v_out, cudaStream_t st);
 int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi, const int64_t* offsets,
                              int32_t* out, int64_t capacity, cudaStream_t st);
 int32_t launch_get_positions(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* out,

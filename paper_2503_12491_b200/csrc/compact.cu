@@ -140,51 +140,65 @@ sorted_positions(const uint2* __restrict__ lists, const int32_t* __restrict__ pr
     if (b + t < room) dst[b + t] = rq.n + t;
 }
 
-constexpr int GA_THREADS = 256;
+constexpr int GA_THREADS = 128;
+constexpr int GA_BATCH = 8;                          // passes of K and of V loads a warp has in flight
 
-// Persistent grid: each warp copies whole rows, `rpp` rows per pass, 16 bytes per lane.
+// Copies the retained rows, one warp per 32 consecutive packed rows: every lane finds the source of
+// one row, then the warp copies them CPR lanes (16 bytes each) to a row.  With dec_off the rows go into
+// the decode layout, one spare row (written as zero) behind every head's rows.
+//
+// Bound: memory; rows of 256 bytes at random places.  One lookup (a binary search and a 64-bit division) per
+// row and four rows in flight took 210 us for 1.05 M rows of 256 bytes in K and V (5.1 TB/s).
+template <int CPR, bool kDecode>
 __global__ void __launch_bounds__(GA_THREADS)
-gather_rows(LayerPtrs ptrs, const int64_t* __restrict__ offsets, const int32_t* __restrict__ budget,
-            const int32_t* __restrict__ pos_packed, const ReqInfo* __restrict__ reqs,
-            uint4* __restrict__ k_out, uint4* __restrict__ v_out, int n_req, int L, int Hkv, int Sw,
-            int64_t T, int cpr /* 16-byte chunks per row */) {
-  const int64_t total = offsets[(size_t)n_req * L];
+gather_rows(const LayerPtrs ptrs, const int64_t* __restrict__ offsets, const int64_t* __restrict__ dec_off,
+            const int32_t* __restrict__ budget, const int32_t* __restrict__ pos_packed, const ReqInfo* __restrict__ reqs,
+            uint4* __restrict__ k_out, uint4* __restrict__ v_out, int n_req, int L, int Hkv, int Sw, int64_t T) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  constexpr int RPP = 32 / CPR, NIT = 32 / RPP, NB = NIT < GA_BATCH ? NIT : GA_BATCH;
   const int nblk = n_req * L;
-  const int lane = threadIdx.x & 31;
-  const int rpp = 32 / cpr;
-  const int sub = lane / cpr, chunk = lane - sub * cpr;
-  const int64_t warp_global = ((int64_t)blockIdx.x * GA_THREADS + threadIdx.x) >> 5;
+  const int64_t total = offsets[nblk];
+  const int lane = threadIdx.x & 31, sub = lane / CPR, chunk = lane % CPR;
   const int64_t n_warps = ((int64_t)gridDim.x * GA_THREADS) >> 5;
-  for (int64_t base = warp_global * rpp * 4; base < total; base += n_warps * rpp * 4) {
-    uint4 kv[4], vv[4];
-    int64_t dst[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t row = base + (int64_t)u * rpp + sub;
-      dst[u] = -1;
-      if (row < total) {
-        int lo = 0, hi = nblk - 1;                   // last block with offset <= row
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (offsets[mid] <= row) lo = mid; else hi = mid - 1;
-        }
-        const int r = lo / L, l = lo - r * L;
-        const ReqInfo rq = reqs[r];
-        const int len = budget[lo] + Sw;
-        const int64_t rel = row - offsets[lo];
-        const int g = (int)(rel / len);
-        const int pos = pos_packed[row];
-        const size_t srow = ((size_t)g * T + rq.cu + pos) * cpr + chunk;
-        kv[u] = reinterpret_cast<const uint4*>(ptrs.k[l])[srow];
-        vv[u] = reinterpret_cast<const uint4*>(ptrs.v[l])[srow];
-        dst[u] = row;
-      }
+  for (int64_t base = (((int64_t)blockIdx.x * GA_THREADS + threadIdx.x) >> 5) * 32; base < total; base += n_warps * 32) {
+    // the block of the first row, 32 probes at a time; a lane's own row lies there or shortly after
+    int blk = 0, hi = nblk;
+    while (hi - blk > 1) {
+      const int step = (hi - blk + 31) / 32, at = blk + lane * step;
+      const unsigned below = __ballot_sync(kAll, at < hi && offsets[at] <= base);
+      blk += (31 - __clz(below)) * step;
+      hi = min(hi, blk + step);
     }
+    const int64_t row = min(base + lane, total - 1);
+    while (offsets[blk + 1] <= row) ++blk;
+    const int r = blk / L, l = blk - r * L, len = budget[blk] + Sw;
+    const int rel = (int)(row - offsets[blk]), g = rel / len;
+    const size_t src = ((size_t)g * T + reqs[r].cu + pos_packed[row]) * CPR;
+    const unsigned long long ks = (unsigned long long)(reinterpret_cast<const uint4*>(ptrs.k[l]) + src);
+    const unsigned long long vs = (unsigned long long)(reinterpret_cast<const uint4*>(ptrs.v[l]) + src);
+    // where the row goes; in the decode layout also whether a spare row follows it
+    long long dst = kDecode ? dec_off[blk] + rel + g : row;
+    if (kDecode && rel - g * len == len - 1) dst = ~dst;
+    const int n_rows = (int)min((int64_t)32, total - base);
+#pragma unroll 1
+    for (int b = 0; b < NIT && b * RPP < n_rows; b += NB) {
+      uint4 kv[NB], vv[NB];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (dst[u] >= 0) {
-        k_out[(size_t)dst[u] * cpr + chunk] = kv[u];
-        v_out[(size_t)dst[u] * cpr + chunk] = vv[u];
+      for (int j = 0; j < NB; ++j) {
+        const int from = (b + j) * RPP + sub;
+        kv[j] = __ldcs(reinterpret_cast<const uint4*>(__shfl_sync(kAll, ks, from)) + chunk);
+        vv[j] = __ldcs(reinterpret_cast<const uint4*>(__shfl_sync(kAll, vs, from)) + chunk);
+      }
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const int from = (b + j) * RPP + sub;
+        const long long d = __shfl_sync(kAll, dst, from);
+        if (from < n_rows) {
+          const size_t o = (size_t)(d < 0 ? ~d : d) * CPR + chunk;
+          k_out[o] = kv[j];
+          v_out[o] = vv[j];
+          if (kDecode && d < 0) k_out[o + CPR] = v_out[o + CPR] = make_uint4(0, 0, 0, 0);
+        }
       }
     }
   }
@@ -230,23 +244,40 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
   return cuda_status(cudaGetLastError());
 }
 
-int32_t launch_compact(cake_ctx* ctx, int32_t lo, int32_t hi, const LayerPtrs& ptrs, void* k_out,
-                       void* v_out, int64_t* row_offsets, int32_t* positions, cudaStream_t st) {
+// Rows of the packed order into k_out / v_out (dec_off: into the decode layout).
+int32_t run_gather(cake_ctx* ctx, const LayerPtrs& ptrs, const int64_t* row_off, const int64_t* dec_off, const int32_t* pos,
+                   void* k_out, void* v_out, cudaStream_t st) {
   const cake_config& c = ctx->cfg;
   const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
+  const int grid = ctx->n_sm * 5;
+#define CAKE_GATHER(CPR)                                                                                                 \
+  if (dec_off)                                                                                                           \
+    gather_rows<CPR, true><<<grid, GA_THREADS, 0, st>>>(ptrs, row_off, dec_off, budget, pos, ctx->d_req, (uint4*)k_out,  \
+                                                        (uint4*)v_out, ctx->n_req, c.n_layers, c.n_kv_heads, c.window,   \
+                                                        ctx->total_tokens);                                              \
+  else                                                                                                                   \
+    gather_rows<CPR, false><<<grid, GA_THREADS, 0, st>>>(ptrs, row_off, dec_off, budget, pos, ctx->d_req, (uint4*)k_out, \
+                                                         (uint4*)v_out, ctx->n_req, c.n_layers, c.n_kv_heads, c.window,  \
+                                                         ctx->total_tokens)
+  switch (c.head_dim * (c.dtype == CAKE_DTYPE_FP32 ? 4 : 2) / 16) {
+    case 8: CAKE_GATHER(8); break;
+    case 16: CAKE_GATHER(16); break;
+    default: CAKE_GATHER(32); break;
+  }
+#undef CAKE_GATHER
+  count_launch();
+  return cuda_status(cudaGetLastError());
+}
+
+int32_t launch_compact(cake_ctx* ctx, int32_t lo, int32_t hi, const LayerPtrs& ptrs, void* k_out,
+                       void* v_out, int64_t* row_offsets, int32_t* positions, cudaStream_t st) {
   int32_t rc = run_offsets(ctx, lo, hi, row_offsets, nullptr, 1, nullptr, st);
   if (rc != CAKE_OK || ctx->n_req == 0 || hi <= lo) return rc;
   // positions in packed row order: into the caller's buffer if there is one
   int32_t* pos = positions ? positions : ctx->d_pos_packed;
   rc = run_sorted_positions(ctx, 0, ctx->n_req, lo, hi, row_offsets, pos, 0, st);
   if (rc != CAKE_OK) return rc;
-  const int esize = c.dtype == CAKE_DTYPE_FP32 ? 4 : 2;
-  const int cpr = c.head_dim * esize / 16;
-  gather_rows<<<ctx->n_sm * 8, GA_THREADS, 0, st>>>(
-      ptrs, row_offsets, budget, pos, ctx->d_req, (uint4*)k_out, (uint4*)v_out, ctx->n_req,
-      c.n_layers, c.n_kv_heads, c.window, ctx->total_tokens, cpr);
-  count_launch();
-  return cuda_status(cudaGetLastError());
+  return run_gather(ctx, ptrs, row_offsets, nullptr, pos, k_out, v_out, st);
 }
 
 int32_t launch_get_positions(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* out,

@@ -671,7 +671,7 @@ decode_step_cluster_kernel(const DecodeArgs A, int csize, int cap_words) {
 }
 
 // Entries of one (request, layer) in ascending position: positions, scores (window entries 0),
-// slots.  One CTA per head.
+// slots.  One thread per entry, a row of CTAs per head.
 __global__ void decode_read_state(const int64_t* __restrict__ dec_off, const float* __restrict__ score,
                                   const int32_t* __restrict__ pos, const int32_t* __restrict__ order,
                                   const int4* __restrict__ meta, int32_t* __restrict__ pos_out,
@@ -680,41 +680,11 @@ __global__ void decode_read_state(const int64_t* __restrict__ dec_off, const flo
   const int g = blockIdx.x;
   const int len = meta[(size_t)blk * Hkv + g].x;
   const int64_t base = dec_off[blk] + (int64_t)g * (len + 1);
-  for (int r = threadIdx.x; r < len; r += blockDim.x) {
+  for (int r = blockIdx.y * blockDim.x + threadIdx.x; r < len; r += gridDim.y * blockDim.x) {
     const int s = order[base + r];
     if (pos_out) pos_out[(size_t)g * len + r] = pos[base + s];
     if (slot_out) slot_out[(size_t)g * len + r] = s;
     if (score_out) score_out[(size_t)g * len + r] = r < len - Sw ? score[base + s] : 0.f;
-  }
-}
-
-// Rows of the packed order into the decode layout (one spare row per head).
-__global__ void __launch_bounds__(256)
-decode_gather(LayerPtrs ptrs, const int64_t* __restrict__ packed_off, const int64_t* __restrict__ dec_off,
-              const int32_t* __restrict__ budget, const int32_t* __restrict__ pos_packed,
-              const ReqInfo* __restrict__ reqs, uint4* __restrict__ k_out, uint4* __restrict__ v_out,
-              int n_req, int L, int Hkv, int Sw, int64_t T, int cpr) {
-  const int64_t total = packed_off[(size_t)n_req * L];
-  const int nblk = n_req * L;
-  const int64_t n_chunks = total * cpr;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_chunks;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = i / cpr;
-    const int chunk = (int)(i - row * cpr);
-    int lo = 0, hi = nblk - 1;                       // last block with offset <= row
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (packed_off[mid] <= row) lo = mid; else hi = mid - 1;
-    }
-    const int r = lo / L, l = lo - r * L;
-    const int len = budget[lo] + Sw;
-    const int64_t rel = row - packed_off[lo];
-    const int g = (int)(rel / len);
-    const int idx = (int)(rel - (int64_t)g * len);
-    const size_t srow = ((size_t)g * T + reqs[r].cu + pos_packed[row]) * cpr + chunk;
-    const size_t drow = (size_t)(dec_off[lo] + (int64_t)g * (len + 1) + idx) * cpr + chunk;
-    k_out[drow] = reinterpret_cast<const uint4*>(ptrs.k[l])[srow];
-    v_out[drow] = reinterpret_cast<const uint4*>(ptrs.v[l])[srow];
   }
 }
 
@@ -805,14 +775,8 @@ int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache,
                                              ctx->d_dec_score, ctx->d_dec_pos, ctx->d_dec_order,
                                              ctx->d_dec_meta, c.n_layers, c.n_kv_heads, c.window);
   count_launch();
-  const int esize = c.dtype == CAKE_DTYPE_FP32 ? 4 : 2;
-  const int cpr = c.head_dim * esize / 16;
-  decode_gather<<<ctx->n_sm * 8, 256, 0, st>>>(ptrs, ctx->d_dec_packed_off, ctx->d_dec_off, budget,
-                                               ctx->d_pos_packed, ctx->d_req, (uint4*)k_cache, (uint4*)v_cache,
-                                               ctx->n_req, c.n_layers, c.n_kv_heads, c.window,
-                                               ctx->total_tokens, cpr);
-  count_launch();
-  return cuda_status(cudaGetLastError());
+  CAKE_CUDA_TRY(cudaGetLastError());
+  return run_gather(ctx, ptrs, ctx->d_dec_packed_off, ctx->d_dec_off, ctx->d_pos_packed, k_cache, v_cache, st);
 }
 
 int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, const void* k_new,
@@ -872,7 +836,8 @@ int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, cons
 int32_t launch_decode_read(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* positions, float* scores,
                            int32_t* slots, cudaStream_t st) {
   const cake_config& c = ctx->cfg;
-  decode_read_state<<<c.n_kv_heads, 256, 0, st>>>(ctx->d_dec_off, ctx->d_dec_score, ctx->d_dec_pos,
+  const dim3 grid(c.n_kv_heads, (unsigned)std::min<int64_t>(64, (ctx->h_dec_cap[layer] + 255) / 256));
+  decode_read_state<<<grid, 256, 0, st>>>(ctx->d_dec_off, ctx->d_dec_score, ctx->d_dec_pos,
                                                   ctx->d_dec_order, ctx->d_dec_meta, positions, scores, slots,
                                                   req * c.n_layers + layer, c.n_kv_heads, c.window);
   count_launch();
