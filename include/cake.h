@@ -357,16 +357,12 @@ int32_t cake_plan_check(const cake_config* cfg, int32_t n_sm, int32_t reserved_s
  * cake_evict -- and writes their positions in ascending order.
  *   values        device fp32 [n_heads][n]
  *   positions_out device int32 [n_heads][keep]
- * It calls no cudaMalloc, cudaFree or other allocating routine.  Its working memory (two
- * bitmaps per head) is a fixed 256 KB array inside the library, present on every GPU that
- * loads the library until the process exits, which bounds the problem size:
+ * It calls no cudaMalloc, cudaFree or other allocating routine; its working memory is the shared
+ * memory of its kernel, so calls may overlap on the GPU.  Problem size:
  *   n_heads * ceil(n / 32) <= 32768      (about one million values per call);
  * anything larger returns CAKE_ERR_CAPACITY and does nothing.  0 <= keep <= n, else
- * CAKE_ERR_ARG.  All calls share that array and the array keeps the previous call's
- * contents; the kernel clears what it needs first, but two calls that overlap on the GPU
- * (different streams, or different host threads without ordering) race on it: serialise them.
- * The first call on each device looks up the array's device address (once per device, with
- * that device current); make that first call outside any stream capture. */
+ * CAKE_ERR_ARG.  The first call on each device sets the kernel's attributes there; make that first
+ * call outside any stream capture. */
 int32_t cake_select_positions_static(const float* values, int32_t n_heads, int32_t n, int32_t keep,
                                      int32_t* positions_out, void* stream);
 

@@ -1,129 +1,216 @@
 // A stand-alone per-head top-k selection that allocates nothing: the entry point for
-// callers that must not touch the device allocator.  Its scratch (two bitmaps per head) lives
-// in a fixed array inside the library instead of in memory obtained from cudaMalloc.
+// callers that must not touch the device allocator.  All its working memory is the shared memory of
+// the CTAs that do the work.
 #include "cake_internal.cuh"
+
+#include <algorithm>
 
 namespace cake {
 namespace {
 
-constexpr int SEL_THREADS = 1024;
-constexpr int kSelMaxWords = 32768;            // 32-bit bitmap words: heads * ceil(n/32) at most
-
-// Scratch shared by every call in the process: [2][kSelMaxWords] words = 256 KB per GPU that
-// loads the library.  Half 0: keys above the threshold; half 1: keys equal to it.
-static __device__ __align__(256) uint32_t g_select_scratch[2 * kSelMaxWords];
+constexpr int SEL_THREADS = 512;
+constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr int kSelMaxWords = 32768;            // limit of the entry point: heads * ceil(n/32)
+constexpr int SEL_BINS = 2048;                 // digits of 11, 11 and 10 bits
+constexpr int SEL_CLUSTER = 8;                 // most CTAs per head; SEL_CLUSTER_WIDE where few heads leave SMs idle
+constexpr int SEL_CLUSTER_WIDE = 16;
+constexpr int kSelShare = 2048;                // values per CTA below which a head is spread no further
+constexpr int kSelSmemKeys = 40 * 1024;        // keys a CTA holds in shared memory; a larger share is read again
 
 // Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
-__device__ inline uint32_t sel_key(float v) {
+__device__ __forceinline__ uint32_t sel_key(float v) {
   uint32_t b = __float_as_uint(v);
   if (b == 0x80000000u) b = 0u;
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
-
-// Exclusive scan of two counters packed as (hi: a, lo: b) over the block.
-__device__ inline unsigned long long sel_scan(unsigned long long v, unsigned long long* warp_tot) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  if (lane == 31) warp_tot[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    const unsigned long long w = warp_tot[lane];
-    unsigned long long winc = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long n = __shfl_up_sync(0xffffffffu, winc, o);
-      if (lane >= o) winc += n;
-    }
-    warp_tot[lane] = winc - w;
-  }
-  __syncthreads();
-  return warp_tot[warp] + inc - v;
+__device__ __forceinline__ uint32_t sel_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t sel_remote(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ uint2 sel_ld_remote(const void* p, uint32_t rank) {
+  uint2 v;
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(sel_remote(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sel_st_remote(const void* p, uint32_t rank, uint2 v) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(sel_remote(p, rank)), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void sel_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// One CTA per head: keeps the `keep` entries that come first in the order (value descending,
-// position ascending) -- the TopK of Eq. 12 -- and writes their positions in ascending order.
+// A cluster of `csize` CTAs per head keeps the `keep` entries that come first in the order (value
+// descending, position ascending) -- the TopK of Eq. 12 -- and writes their positions in ascending
+// order.  Every CTA owns a run of the head's values and holds their keys in shared memory, so the
+// values are read once.  Three digit histograms find the key of the keep-th largest entry.  A
+// histogram is summed over the cluster by sections: a CTA fetches its section of the bins from every
+// CTA's shared memory, adds them up and stores the sums into every CTA's (fetching all bins of all
+// CTAs moves csize times as much and took 6 us per histogram at 16 CTAs).  A warp then counts and places
+// a run of its own.
+//
+// Bound: latency (three rounds of histogram, cluster barrier and scan).  One CTA per head that read the
+// values from L2 six times and walked its histograms with one thread took 101 us for 8 heads of
+// 131 040 values.
 __global__ void __launch_bounds__(SEL_THREADS)
-select_positions_static(const float* __restrict__ values, int n, int keep,
-                        int32_t* __restrict__ out, uint32_t* __restrict__ scratch, int words) {
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t s_prefix, s_krem;
-  __shared__ unsigned long long warp_tot[32];
-  const int head = blockIdx.x;
-  const float* v = values + (size_t)head * n;
-  uint32_t* gt = scratch + (size_t)head * words;
-  uint32_t* eq = scratch + kSelMaxWords + (size_t)head * words;
-  int32_t* dst = out + (size_t)head * keep;
-  // the array keeps whatever the previous call left in it
-  for (int w = threadIdx.x; w < words; w += SEL_THREADS) { gt[w] = 0; eq[w] = 0; }
-  // radix select of the keep-th largest key, 8 bits per pass from the top
+select_positions_static(const float* __restrict__ values, int n, int keep, int32_t* __restrict__ out, int csize, int share) {
+  extern __shared__ uint32_t keys[];
+  __shared__ __align__(16) uint32_t hist[3][SEL_BINS], sums[SEL_BINS];
+  __shared__ __align__(16) uint2 parts[SEL_BINS / 2];
+  __shared__ uint32_t s_warp[SEL_WARPS];
+  __shared__ uint2 s_warp2[SEL_WARPS];
+  __shared__ uint32_t s_digit, s_rem;
+  __shared__ uint2 x_count[SEL_CLUSTER_WIDE];        // (above, equal) of every CTA of the cluster
+  const int rank = (int)sel_cluster_rank();
+  const int head = blockIdx.x / csize;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lo = min(n, rank * share), cnt = min(n, lo + share) - lo;
+  const float* v = values + (size_t)head * n + lo;
+  const bool held = cnt <= kSelSmemKeys;
+  for (int i = threadIdx.x; i < 3 * SEL_BINS; i += SEL_THREADS) (&hist[0][0])[i] = 0;
+  __syncthreads();
   uint32_t prefix = 0, mask = 0, krem = (uint32_t)keep;
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int b = threadIdx.x; b < 256; b += SEL_THREADS) hist[b] = 0;
-    __syncthreads();
-    for (int j = threadIdx.x; j < n; j += SEL_THREADS) {
-      const uint32_t key = sel_key(v[j]);
-      if ((key & mask) == prefix) {
-        atomicAdd(&hist[(key >> shift) & 255u], 1u);
+#pragma unroll 1
+  for (int round = 0; round < 3; ++round) {
+    const int shift = round == 0 ? 21 : round == 1 ? 10 : 0;
+    uint32_t* h = hist[round];
+    for (int i0 = 0; i0 < cnt; i0 += SEL_THREADS * 8) {
+      uint32_t k[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + u * SEL_THREADS + (int)threadIdx.x;
+        k[u] = i < cnt ? (round > 0 && held ? keys[i] : sel_key(__ldg(&v[i]))) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + u * SEL_THREADS + (int)threadIdx.x;
+        if (round == 0 && held && i < cnt) keys[i] = k[u];
+        // pooled values repeat: a run of equal digits in neighbouring lanes is counted once
+        const uint32_t digit = i < cnt && (k[u] & mask) == prefix ? (k[u] >> shift) & (SEL_BINS - 1) : SEL_BINS;
+        if (!__any_sync(0xffffffffu, digit < SEL_BINS)) continue;
+        const uint32_t before = __shfl_up_sync(0xffffffffu, digit, 1);
+        const bool first = lane == 0 || digit != before;
+        const uint32_t firsts = __ballot_sync(0xffffffffu, first);
+        if (first && digit < SEL_BINS) {
+          const uint32_t later = lane < 31 ? firsts >> (lane + 1) : 0u;
+          atomicAdd(&h[digit], later ? (uint32_t)__ffs(later) : 32u - lane);
+        }
       }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t above = 0;
-      int dsel = 0;
-      for (int dg = 255; dg >= 0; --dg) {
-        const uint32_t h = hist[dg];
-        if (above + h >= krem) { dsel = dg; break; }
-        above += h;
+    const uint32_t* sum = h;
+    if (csize > 1) {
+      sum = sums;
+      sel_cluster_sync();
+      const int pairs = SEL_BINS / 2 / csize;        // pairs of bins in a section
+      for (int i = threadIdx.x; i < SEL_BINS / 2; i += SEL_THREADS)
+        parts[i] = sel_ld_remote(&h[2 * (rank * pairs + i % pairs)], (uint32_t)(i / pairs));
+      __syncthreads();
+      if ((int)threadIdx.x < pairs) {
+        uint2 t = make_uint2(0, 0);
+        for (int p = 0; p < csize; ++p) { t.x += parts[p * pairs + threadIdx.x].x; t.y += parts[p * pairs + threadIdx.x].y; }
+        parts[threadIdx.x] = t;
       }
-      s_prefix = prefix | ((uint32_t)dsel << shift);
-      s_krem = krem - above;
+      __syncthreads();
+      for (int i = threadIdx.x; i < SEL_BINS / 2; i += SEL_THREADS)
+        sel_st_remote(&sums[2 * (rank * pairs + i % pairs)], (uint32_t)(i / pairs), parts[i % pairs]);
+      sel_cluster_sync();
+    } else {
+      __syncthreads();
+    }
+    // digits from the top: thread t owns 2047 - 4t .. 2044 - 4t
+    constexpr int kOwn = SEL_BINS / SEL_THREADS;
+    static_assert(kOwn == 4, "one vector load per thread");
+    const int d0 = SEL_BINS - kOwn - kOwn * (int)threadIdx.x;
+    const uint4 c = *reinterpret_cast<const uint4*>(&sum[d0]);
+    const uint32_t own = c.x + c.y + c.z + c.w;
+    uint32_t inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    uint32_t w = lane < SEL_WARPS ? s_warp[lane] : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += t;
+    }
+    const uint32_t base = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+    uint32_t above = (warp ? base : 0u) + inc - own;                 // entries with a larger digit than this thread's
+    const uint32_t bins[4] = {c.w, c.z, c.y, c.x};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (above < krem && above + bins[q] >= krem) { s_digit = (uint32_t)(d0 + 3 - q); s_rem = krem - above; }
+      above += bins[q];
     }
     __syncthreads();
-    prefix = s_prefix;
-    krem = s_krem;
-    mask |= 255u << shift;
-    __syncthreads();
+    prefix |= s_digit << shift;
+    krem = s_rem;
+    mask |= (uint32_t)(SEL_BINS - 1) << shift;
   }
   const uint32_t thr = prefix;        // key of the keep-th largest entry
   const uint32_t need_eq = krem;      // entries equal to it that are kept: the lowest positions
-  for (int j = threadIdx.x; j < n; j += SEL_THREADS) {
-    const uint32_t key = sel_key(v[j]);
-    if (key > thr) atomicOr(&gt[j >> 5], 1u << (j & 31));
-    else if (key == thr) atomicOr(&eq[j >> 5], 1u << (j & 31));
+  // every warp owns a run of the CTA's values: count, then place
+  const int per = (cnt + SEL_THREADS - 1) / SEL_THREADS * 32;        // values per warp, whole ballots
+  const int w_lo = min(cnt, warp * per), w_hi = min(cnt, w_lo + per);
+  uint2 mine = make_uint2(0, 0);
+  auto key_at = [&](int i) { return i < w_hi ? (held ? keys[i] : sel_key(__ldg(&v[i]))) : 0u; };
+  for (int i0 = w_lo; i0 < w_hi; i0 += 128) {
+    uint32_t k[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) k[u] = key_at(i0 + 32 * u + lane);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool in = i0 + 32 * u + lane < w_hi;
+      mine.x += in && k[u] > thr ? 1u : 0u;
+      mine.y += in && k[u] == thr ? 1u : 0u;
+    }
   }
-  __threadfence_block();
+  mine.x = __reduce_add_sync(0xffffffffu, mine.x);
+  mine.y = __reduce_add_sync(0xffffffffu, mine.y);
+  if (lane == 0) s_warp2[warp] = mine;
   __syncthreads();
-  // ranks: every thread owns a run of words
-  const int per = (words + SEL_THREADS - 1) / SEL_THREADS;
-  const int w0 = min(words, (int)threadIdx.x * per), w1 = min(words, w0 + per);
-  uint32_t cg = 0, ce = 0;
-  for (int w = w0; w < w1; ++w) { cg += __popc(gt[w]); ce += __popc(eq[w]); }
-  const unsigned long long ex = sel_scan(((unsigned long long)cg << 32) | ce, warp_tot);
-  uint32_t g_before = (uint32_t)(ex >> 32), e_before = (uint32_t)(ex & 0xffffffffu);
-  for (int w = w0; w < w1; ++w) {
-    const uint32_t mg = gt[w], me = eq[w];
-    uint32_t m = mg | me;
-    while (m) {
-      const int bit = __ffs(m) - 1;
-      m &= m - 1;
-      if ((mg >> bit) & 1u) {
-        dst[g_before + min(e_before, need_eq)] = (w << 5) + bit;
-        ++g_before;
-      } else {
-        if (e_before < need_eq) dst[g_before + e_before] = (w << 5) + bit;
-        ++e_before;
+  uint2 before, total = lane < SEL_WARPS ? s_warp2[lane] : make_uint2(0, 0);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, total.x, o), y = __shfl_up_sync(0xffffffffu, total.y, o);
+    if (lane >= o) { total.x += x; total.y += y; }
+  }
+  before = make_uint2(__shfl_sync(0xffffffffu, total.x, warp) - mine.x, __shfl_sync(0xffffffffu, total.y, warp) - mine.y);
+  total = make_uint2(__shfl_sync(0xffffffffu, total.x, 31), __shfl_sync(0xffffffffu, total.y, 31));
+  if (csize > 1) {
+    if ((int)threadIdx.x < csize) sel_st_remote(&x_count[rank], threadIdx.x, total);
+    sel_cluster_sync();               // also: nobody leaves while its histograms may still be read
+    for (int p = 0; p < rank; ++p) { before.x += x_count[p].x; before.y += x_count[p].y; }
+  }
+  int32_t* dst = out + (size_t)head * keep;
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int i0 = w_lo; i0 < w_hi; i0 += 128) {
+    uint32_t k[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) k[u] = key_at(i0 + 32 * u + lane);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + 32 * u + lane;
+      const uint32_t gt = __ballot_sync(0xffffffffu, i < w_hi && k[u] > thr);
+      const uint32_t eq = __ballot_sync(0xffffffffu, i < w_hi && k[u] == thr);
+      if (gt | eq) {
+        const uint32_t g = before.x + __popc(gt & lt), e = before.y + __popc(eq & lt);
+        if ((gt >> lane) & 1u) dst[g + min(e, need_eq)] = lo + i;
+        else if (((eq >> lane) & 1u) && e < need_eq) dst[g + e] = lo + i;
+        before.x += __popc(gt);
+        before.y += __popc(eq);
       }
     }
   }
 }
-
-constexpr int kMaxDevices = 64;
-uint32_t* g_scratch_ptr[kMaxDevices];     // device address of the scratch, per device ordinal
 
 }  // namespace
 }  // namespace cake
@@ -138,15 +225,30 @@ extern "C" int32_t cake_select_positions_static(const float* values, int32_t n_h
   if ((int64_t)n_heads * words > kSelMaxWords) return CAKE_ERR_CAPACITY;
   int dev = -1;
   CAKE_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) return CAKE_ERR_ARG;
-  if (!g_scratch_ptr[dev]) {
-    // In host code the array's name is only a handle; the kernel needs its device address.
-    uint32_t* p = nullptr;
-    CAKE_CUDA_TRY(cudaGetSymbolAddress((void**)&p, g_select_scratch));
-    g_scratch_ptr[dev] = p;
+  static PerDeviceOnce attr;
+  if (attr.need(dev)) {
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(select_positions_static, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemKeys * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(select_positions_static, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    attr.mark(dev);
   }
-  select_positions_static<<<n_heads, SEL_THREADS, 0, (cudaStream_t)stream>>>(
-      values, n, keep, positions_out, g_scratch_ptr[dev], words);
+  // as many CTAs per head as leave each kSelShare values, up to 8, or 16 where that still fits the
+  // device side by side (one 1024-thread CTA per SM)
+  int csize = 1;
+  while ((int64_t)csize * kSelShare < n && (csize < SEL_CLUSTER || (csize < SEL_CLUSTER_WIDE && n_heads * csize * 2 <= 128))) csize *= 2;
+  const int share = ((n + csize - 1) / csize + 31) / 32 * 32;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_heads * csize), 1, 1);
+  cfg.blockDim = dim3(SEL_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)std::min(share, kSelSmemKeys) * 4;
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = csize;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, select_positions_static, values, n, keep, positions_out, csize, share);
   count_launch();
-  return cuda_status(cudaGetLastError());
+  return cuda_status(e);
 }

@@ -76,3 +76,19 @@ def test_static_selection_rejects_what_does_not_fit():
     binding.select_positions_static(vals, 64, out=out)
     assert torch.equal(out[0].cpu(), torch.arange(64, dtype=torch.int32))
     assert binding.select_positions_static(vals, 0).shape == (1, 0)
+
+
+@pytest.mark.parametrize("heads,n,keep", [(1, 1, 1), (3, 31, 7), (2, 2048, 1), (2, 2049, 2048), (5, 16385, 900), (8, 32769, 4096),
+                                          (1, 700001, 30000), (1, 1 << 20, 77), (33, 30001, 30001)])
+@pytest.mark.parametrize("coarse", [False, True])
+def test_static_selection_at_the_edges_of_a_ctas_share(heads, n, keep, coarse):
+    """One CTA per head, clusters of 2 to 16, and shares too large for shared memory; with `coarse` the
+    threshold is one of many equal values spread over the CTAs."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    vals = torch.randn(heads, n, generator=g, device="cuda")
+    if coarse:
+        vals = torch.round(vals * 2) / 2
+    got = binding.select_positions_static(vals, keep).cpu().numpy()
+    v = vals.cpu().numpy().astype(np.float64)
+    for h in range(min(heads, 3)):
+        assert np.array_equal(got[h], O.topk_keep(v[h], keep)), h
