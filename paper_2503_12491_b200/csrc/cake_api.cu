@@ -62,7 +62,7 @@ void free_ctx(cake_ctx* c) {
   cudaFree(c->d_budget[0]); cudaFree(c->d_budget[1]); cudaFree(c->d_status);
   cudaFree(c->d_raw[0]); cudaFree(c->d_raw[1]);
   cudaFree(c->d_fresh[0]); cudaFree(c->d_fresh[1]); cudaFree(c->d_lists); cudaFree(c->d_prefix); cudaFree(c->d_lstate);
-  cudaFree(c->d_hist); cudaFree(c->d_fill); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
+  cudaFree(c->d_hist); cudaFree(c->d_fill[0]); cudaFree(c->d_fill[1]); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
   cudaFree(c->d_rowpart); cudaFree(c->d_colpart[0]); cudaFree(c->d_colpart[1]);
   cudaFree(c->d_tc_ops); cudaFree(c->d_tc_index); cudaFree(c->d_tc_sync);
@@ -81,15 +81,9 @@ void free_ctx(cake_ctx* c) {
     if (c->ev_score[i]) cudaEventDestroy(c->ev_score[i]);
     if (c->ev_pool[i]) cudaEventDestroy(c->ev_pool[i]);
   }
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_pool_side) cudaEventDestroy(c->ev_pool_side);
   for (int i = 0; i < 2; ++i) if (c->ev_evict[i]) cudaEventDestroy(c->ev_evict[i]);
-  for (int i = 0; i < 2; ++i) if (c->ev_alloc[i]) cudaEventDestroy(c->ev_alloc[i]);
-  if (c->ev_alloc_main) cudaEventDestroy(c->ev_alloc_main);
-  if (c->alloc_st) cudaStreamDestroy(c->alloc_st);
   if (c->pool_st) cudaStreamDestroy(c->pool_st);
-  if (c->side2) cudaStreamDestroy(c->side2);
   if (c->side) cudaStreamDestroy(c->side);
   if (c->prof.spans) {
     for (int i = 0; i < c->prof.cap; ++i) {
@@ -107,7 +101,6 @@ cudaError_t side_after(cake_ctx* c, cudaStream_t st) {
   cudaError_t e = cudaEventRecord(c->ev_main, st);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_main, 0);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->pool_st, c->ev_main, 0);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->alloc_st, c->ev_main, 0);
   return e;
 }
 // Orders the caller's stream after everything enqueued so far on the internal streams.
@@ -116,8 +109,6 @@ cudaError_t main_after_side(cake_ctx* c, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_side, 0);
   if (e == cudaSuccess) e = cudaEventRecord(c->ev_pool_side, c->pool_st);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_pool_side, 0);
-  if (e == cudaSuccess) e = cudaEventRecord(c->ev_alloc_main, c->alloc_st);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_alloc_main, 0);
   return e;
 }
 
@@ -158,6 +149,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   x->sel_budget = c.total_budget - (int64_t)c.n_layers * c.window;
   x->alloc_of_buf[0] = x->alloc_of_buf[1] = -1;
   x->last_alloc = -1;
+  x->arrived_budgets = -1;
   cudaError_t e = cudaGetDevice(&x->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&x->n_sm, cudaDevAttrMultiProcessorCount, x->device);
   if (e != cudaSuccess) { free_ctx(x); return CAKE_ERR_CUDA; }
@@ -194,17 +186,10 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && cudaMallocHost((void**)&x->h_units, sizeof(ScoreUnit) * x->max_units) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->upload_done, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaStreamCreateWithFlags(&x->side, cudaStreamNonBlocking) == cudaSuccess;
-  ok = ok && cudaStreamCreateWithFlags(&x->side2, cudaStreamNonBlocking) == cudaSuccess;
   ok = ok && cudaStreamCreateWithFlags(&x->pool_st, cudaStreamNonBlocking) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_pool_side, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && cudaStreamCreateWithFlags(&x->alloc_st, cudaStreamNonBlocking) == cudaSuccess;
-  ok = ok && cudaEventCreateWithFlags(&x->ev_alloc_main, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 2; ++i)
-    ok = ok && cudaEventCreateWithFlags(&x->ev_alloc[i], cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < 2; ++i)
     ok = ok && cudaEventCreateWithFlags(&x->ev_evict[i], cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && cudaEventCreateWithFlags(&x->ev_fork, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && cudaEventCreateWithFlags(&x->ev_join, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_main, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_side, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < 2; ++i) {
@@ -227,14 +212,14 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && dev_alloc(&x->d_prefix, (size_t)x->max_lists * (kBins + 1)) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_lstate, (size_t)x->max_lists) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_hist, (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_fill, (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_arrivals, 2 * (size_t)R * c.n_kv_heads + R) == cudaSuccess;
+  ok = ok && dev_alloc(&x->d_fill[0], (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
+  ok = ok && dev_alloc(&x->d_fill[1], (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
+  ok = ok && dev_alloc(&x->d_arrivals, (size_t)R * c.n_kv_heads) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_headsum, (size_t)R * c.n_q_heads * 2) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_pos_packed, (size_t)x->pos_packed_cap) == cudaSuccess;
   if (x->bitmap_words > 0) ok = ok && dev_alloc(&x->d_bitmap, (size_t)x->bitmap_words) == cudaSuccess;
   ok = ok && cudaMemset(x->d_hist, 0, sizeof(uint32_t) * R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && cudaMemset(x->d_fill, 0, sizeof(uint32_t) * R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && cudaMemset(x->d_arrivals, 0, sizeof(uint32_t) * (2 * R * c.n_kv_heads + R)) == cudaSuccess;
+  ok = ok && cudaMemset(x->d_arrivals, 0, sizeof(uint32_t) * R * c.n_kv_heads) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_lse2, (size_t)R * c.n_q_heads * c.window) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_rowpart, (size_t)x->max_units * c.n_kv_heads * x->rows) == cudaSuccess;
   {
@@ -322,12 +307,8 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       ctx->upload_pending = false;
     }
     const int32_t unit_keys = choose_unit_keys(T, c.n_kv_heads, ctx->n_sm);
-    int32_t nu = 0, max_split = 0;
-    // the pooling / scatter kernels run on the SMs the score kernel leaves free: about two CTAs
-    // per such SM over all (request, head) pairs
-    const int reserve = ctx->n_sm - ctx->n_sm_score;
-    int want_split = (2 * (reserve > 0 ? reserve : 8)) / (n_req * c.n_kv_heads);
-    if (want_split < 1) want_split = 1;
+    int32_t nu = 0;
+    ctx->max_n_tokens = 0;
     int64_t list_off = 0, bound = 0;
     for (int r = 0; r < n_req; ++r) {
       ReqInfo& q = ctx->h_req[r];
@@ -337,13 +318,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       q.keep_all = q.N <= c.total_budget / c.n_layers ? 1 : 0;
       q.list_off = list_off;
       list_off += (int64_t)q.n * c.n_layers * c.n_kv_heads;
-      {
-        const int chunks = (q.N + kChunkKeys - 1) / kChunkKeys;
-        int ns = chunks < want_split ? chunks : want_split;
-        q.span = ((chunks + ns - 1) / ns) * kChunkKeys;
-        q.nsplit = (q.N + q.span - 1) / q.span;
-        if (q.nsplit > max_split) max_split = q.nsplit;
-      }
+      if (q.N > ctx->max_n_tokens) ctx->max_n_tokens = q.N;
       q.unit0 = nu;
       for (int32_t k0 = 0; k0 < q.N; k0 += unit_keys) {
         ScoreUnit& u = ctx->h_units[nu++];
@@ -354,7 +329,6 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       bound += (int64_t)c.n_kv_heads * (c.total_budget < full ? c.total_budget : full);
     }
     if (list_off > ctx->list_elems || nu > ctx->max_units) return CAKE_ERR_CAPACITY;
-    ctx->n_split = max_split;
     if (ctx->use_tc) {
       const int32_t prc = tc_build_plan(ctx, n_req);
       if (prc != CAKE_OK) return prc;
@@ -377,7 +351,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
     CAKE_CUDA_TRY(cudaEventRecord(ctx->upload_done, st));
     ctx->upload_pending = true;
   }
-  if (n_req == 0) { ctx->n_units = 0; ctx->n_split = 0; ctx->packed_rows_bound = 0; ctx->n_tc_ctas = 0; }
+  if (n_req == 0) { ctx->n_units = 0; ctx->packed_rows_bound = 0; ctx->n_tc_ctas = 0; }
   if (ctx->use_tc) {
     ctx->tc_epoch = 0;
     CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_tc_sync, 0, sizeof(uint32_t) * 2 * ctx->max_pairs, st));
@@ -389,6 +363,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
   ctx->n_ind = ctx->n_pref = ctx->n_evicted = 0;
   ctx->alloc_of_buf[0] = ctx->alloc_of_buf[1] = -1;
   ctx->last_alloc = -1;
+  ctx->arrived_budgets = -1;
   CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int32_t), st));
   ctx->pool_recorded[0] = ctx->pool_recorded[1] = false;
   ctx->evict_recorded[0] = ctx->evict_recorded[1] = false;
@@ -410,20 +385,22 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   int32_t rc = ctx->use_tc ? launch_score_tc(ctx, layer, q_win, k, lse, st)
                            : launch_score_simt(ctx, layer, q_win, k, lse, st);
   if (rc != CAKE_OK) return rc;
-  // Pooling and the preference run on their own stream beside the next layer's scoring and
-  // beside the budgets and eviction of the layer before; the pooled buffer of this parity was
-  // last read by the eviction of layer - 2.
+  // Pooling, the preference and the stage's budgets run on their own stream beside the next layer's
+  // scoring and beside the eviction of the layer before; the pooled buffer, the scatter cursors and the
+  // budgets of this parity were last read by the eviction of layer - 2.
   CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_score[par], st));
   CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_score[par], 0));
   if (ctx->evict_recorded[par]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_evict[par], 0));
   const int sp = prof_begin(ctx, CAKE_PROF_FINALIZE, ctx->pool_st);
-  rc = launch_pool(ctx, layer, true, true, ctx->pool_st);
+  const bool budgets = ctx->last_alloc < layer;      // nobody has asked for a later stage's before
+  rc = launch_arrive(ctx, layer, true, true, budgets, ctx->pool_st);
   prof_end(ctx, sp, ctx->pool_st);
   if (rc != CAKE_OK) return rc;
   CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[par], ctx->pool_st));
   ctx->pool_recorded[par] = true;
   ctx->n_ind = layer + 1;
   if (ctx->n_pref < layer + 1) ctx->n_pref = layer + 1;
+  ctx->arrived_budgets = budgets ? layer : -1;
   return CAKE_OK;
 }
 
@@ -432,18 +409,20 @@ int32_t cake_allocate(cake_ctx* ctx, int32_t stage, void* stream) {
   if (stage < 0 || stage >= ctx->cfg.n_layers) return CAKE_ERR_ARG;
   if (stage >= ctx->n_pref) return CAKE_ERR_STATE;
   (void)stream;                      // ordered by the internal streams
-  // The budgets have a stream of their own, so that those of stage m are computed beside the
-  // eviction of stage m-1.  They need the newest layer's preference (pooling stream), and their
-  // buffer was last read by the eviction of stage m-2; the budgets of stage m-1, which they fall
-  // back to, were written on this stream.
-  cudaStream_t ast = ctx->alloc_st;
-  if (ctx->pool_recorded[stage & 1]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ast, ctx->ev_pool[stage & 1], 0));
-  if (ctx->evict_recorded[stage & 1]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ast, ctx->ev_evict[stage & 1], 0));
-  const int sp = prof_begin(ctx, CAKE_PROF_ALLOCATE, ast);
-  int32_t rc = launch_allocate(ctx, stage, ast);
-  prof_end(ctx, sp, ast);
-  if (rc != CAKE_OK) return rc;
-  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_alloc[stage & 1], ast));
+  // The scores' launch has already computed the budgets of its own stage, unless preferences were set
+  // since; any other stage is computed here.  Its buffer was last read by the eviction of stage - 2,
+  // and the budgets of stage - 1, which it falls back to, were written on this stream.
+  if (ctx->arrived_budgets != stage) {
+    cudaStream_t ast = ctx->pool_st;
+    if (ctx->evict_recorded[stage & 1]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ast, ctx->ev_evict[stage & 1], 0));
+    const int sp = prof_begin(ctx, CAKE_PROF_ALLOCATE, ast);
+    const int32_t rc = launch_allocate(ctx, stage, ast);
+    prof_end(ctx, sp, ast);
+    if (rc != CAKE_OK) return rc;
+    CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[stage & 1], ast));
+    ctx->pool_recorded[stage & 1] = true;
+    if (ctx->arrived_budgets >= 0 && ((ctx->arrived_budgets ^ stage) & 1) == 0) ctx->arrived_budgets = -1;   // overwritten
+  }
   ctx->alloc_of_buf[stage & 1] = stage;
   ctx->last_alloc = stage;
   return CAKE_OK;
@@ -456,7 +435,7 @@ int32_t cake_evict(cake_ctx* ctx, int32_t stage, void* stream) {
   if (ctx->alloc_of_buf[stage & 1] != stage) return CAKE_ERR_STATE;
   if (stage > 0 && ctx->alloc_of_buf[(stage + 1) & 1] != stage - 1) return CAKE_ERR_STATE;
   (void)stream;
-  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_alloc[stage & 1], 0));
+  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_pool[stage & 1], 0));
   const int sp = prof_begin(ctx, CAKE_PROF_EVICT, ctx->side);
   int32_t rc = launch_evict(ctx, stage, ctx->side);
   prof_end(ctx, sp, ctx->side);
@@ -567,10 +546,13 @@ int32_t cake_set_indicators(cake_ctx* ctx, int32_t layer, const float* in, void*
                                   sizeof(float) * ctx->cfg.n_kv_heads * ctx->total_tokens,
                                   cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
   CAKE_CUDA_TRY(side_after(ctx, (cudaStream_t)stream));
-  // bucket histogram of the supplied values (they are taken as already pooled)
-  const int32_t rc = launch_pool(ctx, layer, false, false, ctx->side);
+  // bucket histogram of the supplied values (they are taken as already pooled); the cursors of this
+  // parity were last used by the eviction of layer - 2, which `stream` has waited for
+  const int32_t rc = launch_arrive(ctx, layer, false, false, false, ctx->pool_st);
   if (rc != CAKE_OK) return rc;
-  ctx->pool_recorded[layer & 1] = false;             // same stream as the budgets: nothing to wait for
+  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[layer & 1], ctx->pool_st));
+  ctx->pool_recorded[layer & 1] = true;
+  ctx->arrived_budgets = -1;
   ctx->n_ind = layer + 1;
   return CAKE_OK;
 }
@@ -590,6 +572,7 @@ int32_t cake_set_preferences(cake_ctx* ctx, int32_t n_set, const double* P, void
     CAKE_CUDA_TRY(side_after(ctx, (cudaStream_t)stream));
   }
   if (ctx->n_pref < n_set) ctx->n_pref = n_set;
+  ctx->arrived_budgets = -1;
   return CAKE_OK;
 }
 

@@ -27,8 +27,7 @@ struct ReqInfo {
   int32_t N;         // prompt length
   int32_t n;         // N - S_w non-window tokens
   int32_t keep_all;  // 1: N <= floor(B_total/L), nothing is evicted
-  int32_t nsplit;    // CTAs of the pooling / scatter kernels that share the prompt's tokens
-  int32_t span;      // tokens per such CTA (a multiple of kChunkKeys)
+  int32_t pad;
   int64_t list_off;  // first entry of this request's lists; list (layer, head) holds n entries
   int32_t unit0;     // first score unit of the request
   int32_t nunits;    // number of score units of the request
@@ -58,13 +57,14 @@ struct ScoreOp {
   int32_t pad;
 };
 
-// Retained set of one (request, layer, head) list, whose entries (ordered key, position) are
-// stored by bucket.
+// Retained set of one (request, layer, head) list, whose entries (ordered key, position) are stored by
+// bucket.  The first three fields are derived from the list and the budgets of the moment when the
+// retained set is read out (sorted_positions).
 struct ListState {
   int32_t bucket;        // threshold bucket d; all buckets before it are kept; -1: nothing kept
   uint32_t thr_key;      // inside bucket d an entry is kept if key > thr_key,
   int32_t pos_cut;       //   or key == thr_key and position <= pos_cut
-  int32_t kept;          // number of retained non-window tokens
+  int32_t kept;          // budget the list arrived with: entries beyond it are not stored
 };
 
 struct LayerPtrs {
@@ -93,18 +93,13 @@ struct cake_ctx {
   // The cascade of layer l (pooling, preference, budgets, eviction) runs on an internal side
   // stream while the caller's stream already scores layer l+1; events order the two.
   cudaStream_t side;
-  cudaStream_t side2;               // older layers' thresholds of a stage, beside the newest layer's scatter
-  cudaStream_t pool_st;             // pooling + preference of layer l+1, beside the budgets and eviction of layer l
-  cudaStream_t alloc_st;            // budgets of stage m, beside the eviction of stage m-1
-  cudaEvent_t ev_alloc[2];          // budgets of a stage of that parity are written
-  cudaEvent_t ev_alloc_main;        // scratch event: budget stream -> caller's
+  cudaStream_t pool_st;             // pooling, preference and budgets of layer l+1, beside the eviction of layer l
   cudaEvent_t ev_main, ev_side;     // scratch events: caller's stream -> side, side -> caller's
-  cudaEvent_t ev_fork, ev_join;     // side -> side2 and back
   cudaEvent_t ev_pool_side;         // scratch event: pooling stream -> caller's
   cudaEvent_t ev_evict[2];          // eviction stage of that parity has finished (it reads d_fresh of that parity)
   bool evict_recorded[2];
   cudaEvent_t ev_score[2];          // score kernel of a layer of that parity has finished
-  cudaEvent_t ev_pool[2];           // pooling (the last reader of the score outputs) of that parity has finished
+  cudaEvent_t ev_pool[2];           // pooling (the last reader of the score outputs) and budgets of that parity have finished
   bool pool_recorded[2];
   int32_t rows;            // R = G * S_w
   int64_t sel_budget;      // B' = B_total - L * S_w
@@ -117,6 +112,9 @@ struct cake_ctx {
   int32_t n_evicted;       // stages completed
   int32_t alloc_of_buf[2]; // stage whose budgets live in budget buffer 0/1 (-1 none)
   int32_t last_alloc;      // most recent stage passed to cake_allocate
+  int32_t arrived_budgets; // stage whose budgets were computed when its layer was scored (-1: none, or a
+                           // preference was set since)
+  int32_t max_n_tokens;    // longest prompt of the batch
   int64_t packed_rows_bound;
   int64_t* h_cu;           // host copy of cu_seqlens [max_requests+1]
   // ---- pinned staging ----
@@ -141,12 +139,9 @@ struct cake_ctx {
   cake::ListState* d_lstate;   // [max_lists]
   int64_t max_lists;
   uint32_t* d_hist;        // [max_pairs][kBins] bucket histogram of the arriving layer (zero at rest)
-  uint32_t* d_fill;        // [max_pairs][kBins] scatter cursors (zero at rest)
-  uint32_t* d_arrivals;    // zero at rest: [max_pairs] split counters of the scatter, [max_requests] head
-                           // counters of the preference, [max_pairs] split counters of the pooling (the
-                           // pooling of layer l+1 runs beside the scatter of layer l: separate counters)
+  int32_t* d_fill[2];      // [max_pairs][kBins] scatter cursors of the arriving layer, by layer parity
+  uint32_t* d_arrivals;    // [max_pairs] counters of a list's finished runs in the pooling (zero at rest)
   double* d_headsum;       // [max_requests][H_q][2] per-head entropy / variance sums of the layer
-  int32_t n_split;         // largest nsplit of the batch
   int32_t* d_pos_packed;   // [packed rows bound] positions in packed row order
   int64_t pos_packed_cap;
   uint32_t* d_bitmap;      // global bitmaps for requests too long for shared memory (or null)
@@ -209,7 +204,7 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
 int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const void* k,
                         const float* lse, cudaStream_t st);
 // cascade.cu
-int32_t launch_pool(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize, cudaStream_t st);
+int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize, bool budgets, cudaStream_t st);
 int32_t launch_allocate(cake_ctx* ctx, int32_t stage, cudaStream_t st);
 int32_t launch_evict(cake_ctx* ctx, int32_t stage, cudaStream_t st);
 // decode.cu
@@ -245,6 +240,34 @@ __device__ __forceinline__ float combine_indicator(int mode, float gamma, float 
          : mode == CAKE_IND_VAR         ? var
          : mode == CAKE_IND_WINDOW_SUM  ? mean * sw
                                         : mean * var;
+}
+
+// Exclusive block scan (blockDim.x <= 1024) of one int per thread; *total gets the sum.
+__device__ inline int block_excl_scan(int v, int* warp_tot, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += n;
+  }
+  if (lane == 31) warp_tot[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const int w = lane < nw ? warp_tot[lane] : 0;
+    int winc = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xffffffffu, winc, o);
+      if (lane >= o) winc += n;
+    }
+    warp_tot[lane] = winc - w;
+    if (lane == 31) *total = winc;
+  }
+  __syncthreads();
+  const int r = warp_tot[warp] + inc - v;
+  __syncthreads();
+  return r;
 }
 
 // Function attributes (the dynamic shared-memory limit) belong to a device: a flag per device,

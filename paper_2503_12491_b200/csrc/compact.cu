@@ -58,19 +58,138 @@ block_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ row_off,
   }
 }
 
-constexpr int POS_THREADS = 1024;
+constexpr int kTieCap = 2048;
 
-// One CTA per (head, layer in [lo, hi), request): the retained positions of the list in
-// ascending order, then the window, written at out[base + g*len ...].  `bitmap` is dynamic
+struct EvictSmem {
+  uint32_t hist[1024];
+  int32_t ties[kTieCap];
+  int warp_tot[32];
+  int total;
+  uint32_t sel_digit, sel_rem, sel_cnt;
+  int32_t tie_count, pos_cut;
+};
+
+// Among `cnt` entries (all in one bucket), finds the digit (10 bits at `shift`) that holds the
+// krem-th largest key among the entries whose bits above shift+10 equal `prefix_bits`.
+__device__ inline void radix_digit(const uint2* __restrict__ e, int cnt, uint32_t mask,
+                                   uint32_t prefix_bits, int shift, uint32_t krem, EvictSmem& S) {
+  for (int b = threadIdx.x; b < 1024; b += blockDim.x) S.hist[b] = 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+    const uint32_t key = __ldcg(&e[i]).x;
+    if ((key & mask) == prefix_bits) atomicAdd(&S.hist[(key >> shift) & 1023u], 1u);
+  }
+  __syncthreads();
+  // digits from the top: thread t owns digits 1023-4t .. 1020-4t
+  const int per = 1024 / blockDim.x;
+  int mine = 0;
+  for (int q = 0; q < per; ++q) mine += (int)S.hist[1023 - (threadIdx.x * per + q)];
+  int above = block_excl_scan(mine, S.warp_tot, &S.total);
+  for (int q = 0; q < per; ++q) {
+    const int dg = 1023 - (threadIdx.x * per + q);
+    const int h = (int)S.hist[dg];
+    if ((uint32_t)above < krem && (uint32_t)(above + h) >= krem) {
+      S.sel_digit = (uint32_t)dg;
+      S.sel_rem = krem - (uint32_t)above;
+      S.sel_cnt = (uint32_t)h;
+    }
+    above += h;
+  }
+  __syncthreads();
+}
+
+// Where the budget b cuts one list: the retained set is its first b entries in the order (indicator
+// descending, position ascending)  (Section 4.2 EVICT, Eq. 12).
+__device__ void list_threshold(const int32_t* __restrict__ pf, const uint2* __restrict__ list, int b, ListState* out,
+                               EvictSmem& S) {
+  if (b <= 0) {
+    if (threadIdx.x == 0) *out = ListState{-1, 0xFFFFFFFFu, -1, 0};
+    return;
+  }
+  // threshold bucket d: first bucket with prefix[d+1] >= b
+  int less = 0;
+  for (int i = threadIdx.x; i < kBins; i += blockDim.x) less += __ldcg(&pf[i + 1]) < b ? 1 : 0;
+  block_excl_scan(less, S.warp_tot, &S.total);
+  const int d = S.total;
+  __syncthreads();
+  if (d >= kBins) {                                  // b exceeds the stored entries: keep all
+    if (threadIdx.x == 0) *out = ListState{kBins - 1, 0u, 0x7FFFFFFF, __ldcg(&pf[kBins])};
+    return;
+  }
+  const int start = __ldcg(&pf[d]), cnt = __ldcg(&pf[d + 1]) - start;
+  const uint32_t rem = (uint32_t)(b - start);
+  if ((int)rem >= cnt) {
+    if (threadIdx.x == 0) *out = ListState{d, 0u, 0x7FFFFFFF, b};
+    return;
+  }
+  const uint2* e = list + start;
+  constexpr int low = 32 - kBinBits;                 // key bits below the bucket bits (20)
+  radix_digit(e, cnt, 0u, 0u, low - 10, rem, S);
+  uint32_t pre = S.sel_digit << (low - 10);
+  uint32_t krem = S.sel_rem;
+  __syncthreads();
+  radix_digit(e, cnt, 1023u << (low - 10), pre, 0, krem, S);
+  pre |= S.sel_digit;
+  const uint32_t need_eq = S.sel_rem, n_eq = S.sel_cnt;
+  __syncthreads();
+  // full key of the threshold: bucket bits + the 20 selected bits
+  const uint32_t thr = ((uint32_t)(kBins - 1 - d) << low) | pre;
+  int32_t pos_cut = 0x7FFFFFFF;
+  if (need_eq < n_eq) {
+    // ties at the threshold: the need_eq lowest positions win
+    if (threadIdx.x == 0) { S.tie_count = 0; S.pos_cut = 0x7FFFFFFF; }
+    __syncthreads();
+    if (n_eq <= (uint32_t)kTieCap) {
+      for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+        const uint2 v = __ldcg(&e[i]);
+        if (v.x == thr) S.ties[atomicAdd(&S.tie_count, 1)] = (int32_t)v.y;
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < (int)n_eq; i += blockDim.x) {
+        const int32_t p = S.ties[i];
+        uint32_t r = 0;
+        for (int o = 0; o < (int)n_eq; ++o) r += S.ties[o] < p ? 1u : 0u;
+        if (r == need_eq - 1) S.pos_cut = p;
+      }
+      __syncthreads();
+    } else {
+      // many ties: bisect the position (positions are distinct)
+      int lo = 0, hi = 0x7FFFFFFF;                   // smallest cut with count(pos <= cut) >= need_eq
+      while (lo < hi) {
+        const int mid = lo + ((hi - lo) >> 1);
+        int c = 0;
+        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+          const uint2 v = __ldcg(&e[i]);
+          c += (v.x == thr && (int32_t)v.y <= mid) ? 1 : 0;
+        }
+        block_excl_scan(c, S.warp_tot, &S.total);
+        const int tot = S.total;
+        __syncthreads();
+        if ((uint32_t)tot >= need_eq) hi = mid; else lo = mid + 1;
+      }
+      if (threadIdx.x == 0) S.pos_cut = lo;
+      __syncthreads();
+    }
+    pos_cut = S.pos_cut;
+  }
+  if (threadIdx.x == 0) *out = ListState{d, thr, pos_cut, b};
+}
+
+
+// One CTA per (head, layer in [lo, hi), request): where the current budget cuts the list (kept in
+// its state for whoever needs the stored indicators too), then the retained positions in ascending order, then the window, written at out[base + g*len ...].  `bitmap` is dynamic
 // shared memory when the request's n bits fit, else a slice of global scratch.
+template <int POS_THREADS>
 __global__ void __launch_bounds__(POS_THREADS)
 sorted_positions(const uint2* __restrict__ lists, const int32_t* __restrict__ prefix_all,
-                 const ListState* __restrict__ states, const ReqInfo* __restrict__ reqs,
+                 ListState* __restrict__ states, const ReqInfo* __restrict__ reqs,
                  const int32_t* __restrict__ budget, const int64_t* __restrict__ offsets,
                  int32_t* __restrict__ out, uint32_t* __restrict__ scratch, int64_t scratch_words,
                  int req0, int lo, int L, int Hkv, int Sw, int smem_words, int64_t capacity) {
   extern __shared__ uint32_t sh_bits[];
   __shared__ int warp_tot[32];
+  __shared__ EvictSmem S;
+  __shared__ ListState st;
   const int g = blockIdx.x, layer = lo + blockIdx.y, req = req0 + blockIdx.z;
   const ReqInfo rq = reqs[req];
   const size_t lid = ((size_t)req * L + layer) * Hkv + g;
@@ -88,10 +207,14 @@ sorted_positions(const uint2* __restrict__ lists, const int32_t* __restrict__ pr
   }
   for (int wi = threadIdx.x; wi < words; wi += POS_THREADS) bits[wi] = 0;
   if (in_smem) __syncthreads(); else { __threadfence_block(); __syncthreads(); }
-  const ListState st = states[lid];
+  const int32_t* pf = prefix_all + lid * (kBins + 1);
+  const uint2* list = lists + rq.list_off + ((size_t)layer * Hkv + g) * rq.n;
+  // a list never grows again (Proposition 1): entries beyond the budget it arrived with were not stored
+  const int arrived = states[lid].kept;
+  list_threshold(pf, list, min(min(b, rq.n), arrived), &st, S);
+  __syncthreads();
+  if (threadIdx.x == 0) states[lid] = ListState{st.bucket, st.thr_key, st.pos_cut, arrived};
   if (st.bucket >= 0 && b > 0) {
-    const int32_t* pf = prefix_all + lid * (kBins + 1);
-    const uint2* list = lists + rq.list_off + ((size_t)layer * Hkv + g) * rq.n;
     const int start = pf[st.bucket], end = pf[st.bucket + 1];
     for (int i = threadIdx.x; i < end; i += POS_THREADS) {
       const uint2 e = list[i];
@@ -116,7 +239,7 @@ sorted_positions(const uint2* __restrict__ lists, const int32_t* __restrict__ pr
   if (lane == 31) warp_tot[warp] = inc;
   __syncthreads();
   if (warp == 0) {
-    const int w = warp_tot[lane];
+    const int w = lane < POS_THREADS / 32 ? warp_tot[lane] : 0;
     int winc = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -228,18 +351,25 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
   int smem_words = need_words < kBitmapSmemWords ? need_words : kBitmapSmemWords;
   static PerDeviceOnce attr;
   if (attr.need(ctx->device)) {
-    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kBitmapSmemWords * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitmapSmemWords * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitmapSmemWords * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitmapSmemWords * 4));
     attr.mark(ctx->device);
   }
   const int64_t ctas = (int64_t)c.n_kv_heads * (hi - lo) * n_req;
   if (need_words > kBitmapSmemWords &&
       (!ctx->d_bitmap || ctas * (int64_t)need_words > ctx->bitmap_words)) return CAKE_ERR_CAPACITY;
   const dim3 grid(c.n_kv_heads, hi - lo, n_req);
-  sorted_positions<<<grid, POS_THREADS, (size_t)smem_words * 4, st>>>(
-      ctx->d_lists, ctx->d_prefix, ctx->d_lstate, ctx->d_req,
-      budget, offsets, out, ctx->d_bitmap, need_words, req0, lo, c.n_layers, c.n_kv_heads, c.window,
-      smem_words, capacity);
+  // A list is a chain of scans and short passes: with more lists than the device holds CTAs of 1024
+  // threads, smaller ones keep more chains in flight (1024 lists of 4K tokens: 42 us with 1024 threads).
+#define CAKE_POSITIONS(NT)                                                                                                \
+  sorted_positions<NT><<<grid, NT, (size_t)smem_words * 4, st>>>(                                                         \
+      ctx->d_lists, ctx->d_prefix, ctx->d_lstate, ctx->d_req, budget, offsets, out, ctx->d_bitmap, need_words, req0, lo,  \
+      c.n_layers, c.n_kv_heads, c.window, smem_words, capacity)
+  if (ctas <= 2 * ctx->n_sm) CAKE_POSITIONS(1024);
+  else if (ctas <= 4 * ctx->n_sm) CAKE_POSITIONS(512);
+  else CAKE_POSITIONS(256);
+#undef CAKE_POSITIONS
   count_launch();
   return cuda_status(cudaGetLastError());
 }
