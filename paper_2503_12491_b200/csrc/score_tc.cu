@@ -61,6 +61,7 @@ constexpr long long kSpinLimit = 4000000000ll;   // default cycles (~2 s) before
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kChunkSumMax = 65536.f;   // a pass-A chunk sum beyond this moves the row's reference
 constexpr int64_t kWaveBytes = 32ll << 20;
+constexpr int kDirectSegs = 40;       // segments of a pair up to which every CTA merges its rows for itself
 constexpr int kWaveDepth = 1;         // pass B of a wave follows pass A of the wave this far ahead
 
 struct TcParams {
@@ -85,6 +86,7 @@ struct TcParams {
   float scale2, inv_scale2, gamma, bessel;
   int ind_mode;                 // CAKE_IND_*
   int merge_ways;               // rows the merger warp merges side by side: 1, or 2 to 32 when pairs are short
+  int reps, rep_shift;          // copies of the window rows in a pass-A tile: 128 / rows for 32 and 64 rows, else 1
 };
 
 // ------------------------------------------------------------------ PTX
@@ -314,17 +316,20 @@ struct Smem {
   uint64_t* q_empty;   // [2]
   uint64_t* lse_full;  // [2]
   uint64_t* lse_free;  // [2]
+  uint64_t* parts;     // [2] direct merge: the pair's partial rows are all delivered
   uint32_t* tmem_holder;
   uint32_t* a_done;    // [NSTATW] pass-A ops whose partial rows each statistics warp has written
   uint8_t* ext_a;      // the constant key-side operand of the extra K step of pass B
   uint8_t* ext_b;      // [2] its row-side operand: -lse/scale of the current / next pass-B op
+  float4* xrow;        // [2][NWG][128] direct merge: a group's merged rows of the current / next pass-B op
   ScoreOp* ops;        // [kSmemOps] the first ops of this CTA's program
 };
 
 constexpr size_t kQBytes = 2 * SLAB_BYTES;
 constexpr int kSmemOps = 128;        // ops of a CTA's program kept in shared memory
 constexpr size_t kSmemBytes = 1024 /*align*/ + 2 * kQBytes + (size_t)STAGES * 2 * SLAB_BYTES + 320 +
-                              128 + 3 * kExtBytes + kSmemOps * sizeof(ScoreOp) + 64;
+                              128 + 3 * kExtBytes + 2 * NWG * 128 * sizeof(float4) + kSmemOps * sizeof(ScoreOp) + 64;
+static_assert(kSmemBytes <= 227 * 1024, "a CTA has 227 KB of shared memory");
 
 __device__ __forceinline__ Smem carve(uint8_t* base) {
   Smem s;
@@ -339,12 +344,14 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   s.q_empty = (uint64_t*)p;   p += 16;
   s.lse_full = (uint64_t*)p;  p += 16;
   s.lse_free = (uint64_t*)p;  p += 16;
+  s.parts = (uint64_t*)p;     p += 16;
   s.tmem_holder = (uint32_t*)p; p += 8;
   s.a_done = (uint32_t*)p;    p += 4 * 16;
   p = (uint8_t*)(((uintptr_t)p + 15) & ~(uintptr_t)15);
   p = (uint8_t*)(((uintptr_t)p + 127) & ~(uintptr_t)127);
   s.ext_a = p;                p += kExtBytes;
   s.ext_b = p;                p += 2 * kExtBytes;
+  s.xrow = (float4*)p;        p += 2 * NWG * 128 * sizeof(float4);
   s.ops = (ScoreOp*)p;
   return s;
 }
@@ -364,8 +371,43 @@ __device__ __forceinline__ float4 merge_rows(float4 a, float4 b) {
   return o;
 }
 
+// The same for a batch at once: the largest reference first, then independent terms.
+template <int K>
+__device__ __forceinline__ float4 merge_batch(float4 acc, const float4 (&v)[K]) {
+  float m = acc.x;
+#pragma unroll
+  for (int u = 0; u < K; ++u) m = fmaxf(m, v[u].x);
+  if (m == -CUDART_INF_F) return acc;
+  auto term = [&](const float4& t, float4& o) {
+    const float d = t.x == -CUDART_INF_F ? 0.f : t.x - m, f = t.x == -CUDART_INF_F ? 0.f : exp2f(d);
+    o.y = fmaf(t.y, f, o.y);
+    o.z = fmaf(t.z, f, o.z);
+    o.w = fmaf(f, fmaf(d, t.y - t.z, t.w), o.w);
+  };
+  float4 o = make_float4(m, 0.f, 0.f, 0.f);
+  term(acc, o);
+#pragma unroll
+  for (int u = 0; u < K; ++u) term(v[u], o);
+  return o;
+}
+
+// -lse / scale as three bf16 terms (24 bits) in columns 0..2 of the rows' operand of the extra K step.
+__device__ __forceinline__ void put_ext_row(uint8_t* ext, int r, int rows, float lse2, float inv_scale2) {
+  const float t = -lse2 * inv_scale2;
+  const __nv_bfloat16 hi = __float2bfloat16_rn(t);
+  const float r1 = t - __bfloat162float(hi);
+  const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
+  const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+  const uint32_t w0 = (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16);
+  const uint32_t w1 = (uint32_t)__bfloat16_as_ushort(lo);
+  *reinterpret_cast<uint2*>(ext + ext_row_offset(r)) = r < rows ? make_uint2(w0, w1) : make_uint2(0u, 0u);
+}
+
 // ------------------------------------------------------------------ kernel
-template <int G, bool kEntropyB>
+// kCopies: the window has 32 or 64 rows and a pass-A tile holds them 4 or 2 times, so that every
+// statistics warp has rows to work on: copy c sums the c-th part of a key tile's columns.
+// kDirect: one wave; every CTA merges the partial rows of its own pass-B ops (see tc_build_plan).
+template <int G, bool kEntropyB, bool kCopies, bool kDirect>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                    const TcParams P) {
@@ -381,7 +423,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     for (int i = 0; i < STAGES; ++i) { mbar_init(&S.full[i], 1); mbar_init(&S.empty[i], 1); }
     for (int i = 0; i < NBUF; ++i) { mbar_init(&S.acc_full[i], 1); mbar_init(&S.acc_empty[i], 4); }
     for (int i = 0; i < 2; ++i) { mbar_init(&S.q_full[i], 1); mbar_init(&S.q_empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&S.lse_full[i], 1); mbar_init(&S.lse_free[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&S.lse_full[i], kDirect ? 4 : 1); mbar_init(&S.lse_free[i], 1); mbar_init(&S.parts[i], 1); }
     for (int i = 0; i < NSTATW; ++i) S.a_done[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -433,10 +475,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         ok = mbar_wait(&S.q_empty[qb], ((qn >> 1) & 1) ^ 1, P.status, P.spin_limit);
         ++qn;
         if (!ok) break;
-        mbar_expect_tx(&S.q_full[qb], (uint32_t)(P.rows * P.d * 2));
-        for (int sl = 0; sl < n_slab; ++sl)
-          tma_load_4d(S.q + qb * kQBytes + sl * SLAB_BYTES, &q_map, &S.q_full[qb], sl * 64, op.g * G,
-                      0, op.req);
+        const int reps = kCopies && !op.phase ? P.reps : 1;
+        mbar_expect_tx(&S.q_full[qb], (uint32_t)(reps * P.rows * P.d * 2));
+        for (int rp = 0; rp < reps; ++rp)
+          for (int sl = 0; sl < n_slab; ++sl)
+            tma_load_4d(S.q + qb * kQBytes + sl * SLAB_BYTES + rp * P.rows * 128, &q_map, &S.q_full[qb], sl * 64, op.g * G,
+                        0, op.req);
         const int64_t row0 = op.base + op.key0;
         const int ntiles = (op.nkeys + TILE - 1) / TILE;
         for (int it = 0; it < ntiles; ++it, ++t) {
@@ -567,7 +611,15 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         return true;
       };
-      if (P.merge_ways > 1) {
+      // partial `pi` of row r: (segment, group) pi / reps, copy pi % reps of the row
+      const int reps = kCopies ? P.reps : 1;
+      auto part_at = [&](int pi, int r) -> size_t {
+        if constexpr (kCopies) return (size_t)(pi >> P.rep_shift) * 128 + (pi & (P.reps - 1)) * P.rows + r;
+        else return (size_t)pi * 128 + r;
+      };
+      if constexpr (kDirect) {
+        // nothing to merge here: the statistics warps do it
+      } else if (P.merge_ways > 1) {
         // Short pairs (a ragged batch, MHA): a wave holds several pairs whose rows have few
         // partials each, so the rows of `ways` (2 to 32) consecutive pairs are merged side by side,
         // by 32 / ways lanes each, and the wave's denominators are ready that much sooner.
@@ -598,13 +650,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
             float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
             if (active) {
-              for (int base = s_lo; base < s_hi; base += 8 * lpr) {
+              for (int base = s_lo * reps; base < s_hi * reps; base += 8 * lpr) {
                 float4 pv[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                   const int sg = base + u * lpr + l8;
-                  pv[u] = sg < s_hi ? __ldcg(&P.rowpart[(size_t)sg * 128 + r])
-                                    : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+                  pv[u] = sg < s_hi * reps ? __ldcg(&P.rowpart[part_at(sg, r)]) : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) acc = merge_rows(acc, pv[u]);
@@ -648,13 +699,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           }
           float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
           // 12 loads per lane in flight: the 384 partials of a row at 128 CTAs come in one round trip
-          for (int base = s_lo; base < s_hi; base += 32 * 12) {
+          for (int base = s_lo * reps; base < s_hi * reps; base += 32 * 12) {
             float4 pv[12];
 #pragma unroll
             for (int u = 0; u < 12; ++u) {
               const int sg = base + u * 32 + lane;
-              pv[u] = sg < s_hi ? __ldcg(&P.rowpart[(size_t)sg * 128 + r])
-                                : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+              pv[u] = sg < s_hi * reps ? __ldcg(&P.rowpart[part_at(sg, r)]) : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int u = 0; u < 12; ++u) acc = merge_rows(acc, pv[u]);
@@ -700,9 +750,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (lane == 0) {
         ok = mbar_wait(&S.lse_free[slot], ((kb >> 1) & 1) ^ 1, P.status, P.spin_limit);
         if (ok && P.pair_done) {
-          const uint32_t want = (uint32_t)P.rows * P.epoch;
+          const uint32_t want = kDirect ? (uint32_t)(P.pair_aseg[pair + 1] - P.pair_aseg[pair]) * (uint32_t)NSTATW * P.epoch
+                                        : (uint32_t)P.rows * P.epoch;
+          const uint32_t* count = kDirect ? &P.pair_cnt[pair] : &P.pair_done[pair];
           const long long t0 = clock64();
-          while (ld_acquire(&P.pair_done[pair]) < want) {
+          while (ld_acquire(count) < want) {
             if (clock64() - t0 > P.spin_limit) { atomicCAS(P.status, 0, CAKE_ERR_TIMEOUT); ok = false; break; }
             __nanosleep(32);
           }
@@ -710,6 +762,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       }
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
+      if constexpr (kDirect) {                       // the statistics warps take it from here
+        if (lane == 0) mbar_arrive(&S.parts[slot]);
+        ++kb;
+        continue;
+      }
       float4 v;
       if (P.lse_ext) {
         // the caller's natural-log values [req][H_q][S_w]: tile row r' = i*G + h, base 2
@@ -723,22 +780,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       } else {
         v = __ldcg(reinterpret_cast<const float4*>(P.lse2 + (size_t)pair * 128) + lane);
       }
-      // -lse / scale as three bf16 terms (24 bits) in columns 0..2 of the rows' operand
       {
         const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int r = 4 * lane + e;
-          const float t = -vv[e] * P.inv_scale2;
-          const __nv_bfloat16 hi = __float2bfloat16_rn(t);
-          const float r1 = t - __bfloat162float(hi);
-          const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-          const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-          const uint32_t w0 = (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16);
-          const uint32_t w1 = (uint32_t)__bfloat16_as_ushort(lo);
-          *reinterpret_cast<uint2*>(S.ext_b + slot * kExtBytes + ext_row_offset(r)) =
-              r < P.rows ? make_uint2(w0, w1) : make_uint2(0u, 0u);
-        }
+        for (int e = 0; e < 4; ++e) put_ext_row(S.ext_b + slot * kExtBytes, 4 * lane + e, P.rows, vv[e], P.inv_scale2);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
@@ -757,11 +802,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(wg * 128);
     uint64_t* const my_full = &S.acc_full[wg];
     uint64_t* const my_empty = &S.acc_empty[wg];
-    const int b = wg;
-    (void)b;
     uint32_t tmod = 0;                              // tiles of the ops so far, modulo NWG
     uint32_t fpar = 0;                              // phase parity of my_full
     uint32_t n_a_done = 0;                          // pass-A ops this warp has delivered
+    uint32_t kbs = 0;                               // pass-B ops so far
+    // pass A: the window row of this lane, and the columns its copy of the rows sums
+    const int copy = kCopies ? (quad * P.reps) >> 2 : 0;
+    const int i_row = (kCopies ? lane_row - copy * P.rows : lane_row) / G;
+    const int c_lo = kCopies ? copy * (TILE / P.reps) : 0, c_hi = kCopies ? c_lo + TILE / P.reps : TILE;
     bool ok = true;
     for (int oi = op_lo; oi < op_hi; ++oi) {
       const ScoreOp op = get_op(oi);
@@ -771,6 +819,45 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       tmod = (tmod + (uint32_t)ntiles) % NWG;
       if (op.phase) {
         // ---------------- pass B: thread = key, columns = rows r' = i*G + h
+        if constexpr (kDirect) {
+          // One thread per row and group; every CTA adds in the same order.
+          const int slot = kbs & 1, pair = op.req * P.Hkv + op.g;
+          if (ok) ok = mbar_wait(&S.parts[slot], (kbs >> 1) & 1, P.status, P.spin_limit);
+          ++kbs;
+          float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+          const int reps = kCopies ? P.reps : 1;
+          const int s_lo = P.pair_aseg[pair], s_hi = ok ? P.pair_aseg[pair + 1] : s_lo;
+          if (lane_row < P.rows * reps) {
+            for (int sg = s_lo; sg < s_hi; sg += 8) {
+              float4 pv[8];
+#pragma unroll
+              for (int u = 0; u < 8; ++u)
+                pv[u] = sg + u < s_hi ? __ldcg(&P.rowpart[((size_t)(sg + u) * NWG + wg) * 128 + lane_row])
+                                      : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+              acc = merge_batch(acc, pv);
+            }
+          }
+          S.xrow[(slot * NWG + wg) * 128 + lane_row] = acc;
+          asm volatile("bar.sync 1, %0;" ::"n"(STAT_THREADS) : "memory");
+          if (wg == 0) {
+            acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+            if (lane_row < P.rows) {
+              for (int rp = 0; rp < reps; ++rp) {
+                float4 pv[NWG];
+#pragma unroll
+                for (int q = 0; q < NWG; ++q) pv[q] = S.xrow[(slot * NWG + q) * 128 + rp * P.rows + lane_row];
+                acc = merge_batch(acc, pv);
+              }
+            }
+            const float lz = log2f(acc.y);
+            put_ext_row(S.ext_b + slot * kExtBytes, lane_row, P.rows, acc.x + lz, P.inv_scale2);
+            if (op.key0 == 0 && lane_row < P.rows)
+              P.hrow[(size_t)pair * 128 + lane_row] = (acc.w - lz * (acc.y - acc.z)) / acc.y;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.lse_full[slot]);
+          }
+        }
         float vacc[G], hs[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) { vacc[h] = 0.f; hs[h] = 0.f; }
@@ -876,7 +963,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
       } else {
         // ---------------- pass A: thread = window row r' = i*G + h, columns = keys
-        const int i_row = lane_row / G;
         const int last = op.n + i_row;                 // last key this row may attend to
         float m = -CUDART_INF_F, z = 0.f, zwin = 0.f, w = 0.f;
         for (int it = it0; it < ntiles; it += NWG) {
@@ -886,18 +972,18 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           tc_fence_after();
           const int key0 = op.key0 + it * TILE;
           const bool interior = key0 + TILE <= op.n && it * TILE + TILE <= op.nkeys;
-          if (quad * 32 >= P.rows) {                   // these TMEM lanes hold padding rows
+          if (!kCopies && quad * 32 >= P.rows) {       // these TMEM lanes hold padding rows
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(my_empty);
             continue;
           }
 #pragma unroll 1
-          for (int c0 = 0; c0 < TILE; c0 += 32) {
+          for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
             uint32_t r[32];
             tmem_ld32_issue(taddr + c0, r);
             tmem_ld_wait(r);
-            if (c0 + 32 >= TILE) {
+            if (c0 + 32 >= c_hi) {
               tc_fence_before();
               __syncwarp();
               if (lane == 0) mbar_arrive(my_empty);
@@ -1017,22 +1103,27 @@ EncodeTiledFn encode_fn() {
 
 
 template <int G>
-cudaError_t launch_g(int device, bool entropy_b, int n_cta, cudaStream_t st, const CUtensorMap& qmap,
+cudaError_t launch_g(int device, bool entropy_b, bool copies, bool direct, int n_cta, cudaStream_t st, const CUtensorMap& qmap,
                      const CUtensorMap& kmap, const TcParams& P) {
+  typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const TcParams);
+  static const Kernel kernels[5] = {score_fused_kernel<G, false, false, false>, score_fused_kernel<G, false, false, true>,
+                                    score_fused_kernel<G, false, true, false>, score_fused_kernel<G, false, true, true>,
+                                    score_fused_kernel<G, true, false, false>};
   static PerDeviceOnce attr;
   if (attr.need(device)) {
-    cudaError_t e = cudaFuncSetAttribute(score_fused_kernel<G, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(score_fused_kernel<G, true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e != cudaSuccess) return e;
+    for (Kernel k : kernels) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+      if (e != cudaSuccess) return e;
+    }
     attr.mark(device);
   }
-  if (entropy_b) score_fused_kernel<G, true><<<n_cta, TC_THREADS, kSmemBytes, st>>>(qmap, kmap, P);
-  else           score_fused_kernel<G, false><<<n_cta, TC_THREADS, kSmemBytes, st>>>(qmap, kmap, P);
+  const Kernel k = kernels[entropy_b ? 4 : (copies ? 2 : 0) + (direct ? 1 : 0)];
+  k<<<n_cta, TC_THREADS, kSmemBytes, st>>>(qmap, kmap, P);
   return cudaGetLastError();
 }
+
+// Copies of the window rows in a pass-A tile.
+int tc_reps(int rows) { return rows == 32 ? 4 : rows == 64 ? 2 : 1; }
 
 // Cuts the `tiles` tiles of one (request, head) pair, which start at flat tile index `flat`
 // of a wave of `W` tiles shared by `n_cta` CTAs (slot c owns flat tiles
@@ -1237,7 +1328,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
   {
     int max_segs = 0;
     for (int p = 0; p < n_pairs; ++p) max_segs = std::max(max_segs, pair_aseg[p + 1] - pair_aseg[p]);
-    const int partials = max_segs * NWG;
+    const int partials = max_segs * NWG * tc_reps(ctx->rows);
     // at most 16 partials per lane (two batches of loads): 32 lanes / ways per row
     int ways = 1;
     while (ways < 32 && 2 * ways <= n_pairs && partials * 2 * ways <= 512) ways *= 2;
@@ -1258,6 +1349,14 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     };
     while (ways > 1 && !span_ok(ways)) ways >>= 1;
     ctx->tc_merge_ways = ways;
+    // With a single wave nothing runs between its pass A and its pass B, so a launch waits for the way
+    // from the partial rows to the denominators.  As long as a pair's partials are few (a thread reads
+    // one per segment, eight at a time) every CTA merges those of its own pass-B ops: the merged rows
+    // are spared a trip through global memory (store, fence, count, poll, load: 4 us of 28 at 32 pairs
+    // of 4K keys).
+    bool all_b = true;                               // every pair has a pass-B op to write its entropy rows
+    for (int p = 0; p < n_pairs; ++p) all_b = all_b && pair_bseg[p + 1] > pair_bseg[p];
+    ctx->tc_direct = n_waves == 1 && all_b && max_segs <= kDirectSegs;
   }
   return CAKE_OK;
 }
@@ -1278,6 +1377,7 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
   cake_ctx x;
   memset(&x, 0, sizeof(x));
   x.cfg = c;
+  x.rows = c.n_q_heads / c.n_kv_heads * c.window;
   x.n_sm = n_sm;
   x.n_sm_score = n_sm - reserved > 0 ? n_sm - reserved : 1;
   const int Hkv = c.n_kv_heads, n_pairs = n_req * Hkv;
@@ -1413,6 +1513,8 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.gamma = c.gamma;
   P.ind_mode = c.indicator_mode;
   P.merge_ways = ctx->tc_merge_ways;
+  P.reps = tc_reps(ctx->rows);
+  P.rep_shift = P.reps == 4 ? 2 : P.reps == 2 ? 1 : 0;
   P.spin_limit = ctx->wait_limit_cycles > 0 ? ctx->wait_limit_cycles : kSpinLimit;
   P.bessel = c.var_ddof ? (float)c.window / (float)(c.window - 1) : 1.f;
 
@@ -1433,10 +1535,10 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   cudaError_t e;
   const bool eb = lse != nullptr;
   switch (G) {
-    case 1: e = launch_g<1>(ctx->device, eb, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    case 2: e = launch_g<2>(ctx->device, eb, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    case 4: e = launch_g<4>(ctx->device, eb, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    default: e = launch_g<8>(ctx->device, eb, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 1: e = launch_g<1>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 2: e = launch_g<2>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 4: e = launch_g<4>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    default: e = launch_g<8>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
   }
   count_launch();
   prof_end(ctx, sp, st);

@@ -259,3 +259,16 @@ def test_cumulative_attention_indicator_through_the_hook():
         for g in range(w.n_kv_heads):
             assert np.array_equal(got[g], c.positions[l][g])
     cake.destroy()
+
+
+@pytest.mark.parametrize("hq,hkv,window,seq_lens", [
+    (2, 2, 32, (70001,)),              # 32 rows, two waves: copies of the rows, merger warps
+    (2, 1, 32, (100001,)),             # 64 rows, one wave, too many segments for the merge in every CTA
+    (2, 2, 32, (5121, 129)),           # 32 rows, merge in every CTA, a pair of two tiles
+    (4, 1, 32, (4097, 1000, 161)),     # 128 rows, merge in every CTA
+    (2, 2, 32, (900, 32)),             # a prompt that is all window has no column pass
+])
+def test_row_copies_and_both_ways_to_the_denominators(hq, hkv, window, seq_lens):
+    w = bf16_case(n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=seq_lens, n_layers=2 if max(seq_lens) < 9000 else 1,
+                  total_budget=(2 if max(seq_lens) < 9000 else 1) * (window + 60))
+    check_scores(w, expect_tc=True)
