@@ -60,13 +60,13 @@ void free_ctx(cake_ctx* c) {
   if (!c) return;
   cudaFree(c->d_req); cudaFree(c->d_units); cudaFree(c->d_H); cudaFree(c->d_V); cudaFree(c->d_P);
   cudaFree(c->d_budget[0]); cudaFree(c->d_budget[1]); cudaFree(c->d_status);
-  cudaFree(c->d_raw[0]); cudaFree(c->d_raw[1]);
+  for (int i = 0; i < kScoreDepth; ++i) { cudaFree(c->d_raw[i]); cudaFree(c->d_colpart[i]); cudaFree(c->d_hrow[i]); }
   cudaFree(c->d_fresh[0]); cudaFree(c->d_fresh[1]); cudaFree(c->d_lists); cudaFree(c->d_prefix); cudaFree(c->d_lstate);
   cudaFree(c->d_hist); cudaFree(c->d_fill[0]); cudaFree(c->d_fill[1]); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
-  cudaFree(c->d_rowpart); cudaFree(c->d_colpart[0]); cudaFree(c->d_colpart[1]);
+  cudaFree(c->d_rowpart);
   cudaFree(c->d_tc_ops); cudaFree(c->d_tc_index); cudaFree(c->d_tc_sync);
-  cudaFree(c->d_tc_rowpart); cudaFree(c->d_lse2_tc); cudaFree(c->d_hrow[0]); cudaFree(c->d_hrow[1]);
+  cudaFree(c->d_tc_rowpart); cudaFree(c->d_lse2_tc);
   cudaFree(c->d_dec_off); cudaFree(c->d_dec_packed_off); cudaFree(c->d_dec_score); cudaFree(c->d_dec_tmp); cudaFree(c->d_dec_pos);
   cudaFree(c->d_dec_order); cudaFree(c->d_dec_meta);
   if (c->h_budget_stage) cudaFreeHost(c->h_budget_stage);
@@ -77,7 +77,7 @@ void free_ctx(cake_ctx* c) {
   if (c->upload_done) cudaEventDestroy(c->upload_done);
   if (c->ev_main) cudaEventDestroy(c->ev_main);
   if (c->ev_side) cudaEventDestroy(c->ev_side);
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < kScoreDepth; ++i) {
     if (c->ev_score[i]) cudaEventDestroy(c->ev_score[i]);
     if (c->ev_pool[i]) cudaEventDestroy(c->ev_pool[i]);
   }
@@ -192,7 +192,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     ok = ok && cudaEventCreateWithFlags(&x->ev_evict[i], cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_main, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_side, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < kScoreDepth; ++i) {
     ok = ok && cudaEventCreateWithFlags(&x->ev_score[i], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&x->ev_pool[i], cudaEventDisableTiming) == cudaSuccess;
   }
@@ -204,8 +204,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && dev_alloc(&x->d_budget[0], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_budget[1], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_status, 1) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_raw[0], (size_t)c.n_kv_heads * T) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_raw[1], (size_t)c.n_kv_heads * T) == cudaSuccess;
+  for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_raw[i], (size_t)c.n_kv_heads * T) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_fresh[0], (size_t)c.n_kv_heads * T) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_fresh[1], (size_t)c.n_kv_heads * T) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_lists, (size_t)x->list_elems) == cudaSuccess;
@@ -214,12 +213,12 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && dev_alloc(&x->d_hist, (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_fill[0], (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_fill[1], (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_arrivals, (size_t)R * c.n_kv_heads) == cudaSuccess;
+  ok = ok && dev_alloc(&x->d_arrivals, (size_t)R * c.n_kv_heads + R) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_headsum, (size_t)R * c.n_q_heads * 2) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_pos_packed, (size_t)x->pos_packed_cap) == cudaSuccess;
   if (x->bitmap_words > 0) ok = ok && dev_alloc(&x->d_bitmap, (size_t)x->bitmap_words) == cudaSuccess;
   ok = ok && cudaMemset(x->d_hist, 0, sizeof(uint32_t) * R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && cudaMemset(x->d_arrivals, 0, sizeof(uint32_t) * R * c.n_kv_heads) == cudaSuccess;
+  ok = ok && cudaMemset(x->d_arrivals, 0, sizeof(uint32_t) * (R * c.n_kv_heads + R)) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_lse2, (size_t)R * c.n_q_heads * c.window) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_rowpart, (size_t)x->max_units * c.n_kv_heads * x->rows) == cudaSuccess;
   {
@@ -236,8 +235,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   }
   {
     const size_t a = (size_t)x->max_units * c.n_kv_heads, b = (size_t)x->max_tc_segs * kScoreWarps;
-    ok = ok && dev_alloc(&x->d_colpart[0], (a > b ? a : b) * G * 2) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_colpart[1], (a > b ? a : b) * G * 2) == cudaSuccess;
+    for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_colpart[i], (a > b ? a : b) * G * 2) == cudaSuccess;
   }
   if (x->use_tc) {
     const size_t n_index = 2 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
@@ -248,8 +246,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     ok = ok && dev_alloc(&x->d_tc_sync, 2 * (size_t)max_pairs) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_rowpart, (size_t)x->max_tc_segs * kScoreGroups * 128) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_lse2_tc, (size_t)max_pairs * 128) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_hrow[0], (size_t)max_pairs * 128) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_hrow[1], (size_t)max_pairs * 128) == cudaSuccess;
+    for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_hrow[i], (size_t)max_pairs * 128) == cudaSuccess;
   }
   // decode-time state: one slot per packed row plus one spare per (request, layer, head)
   x->dec_rows_cap = x->pos_packed_cap + x->max_lists;
@@ -334,6 +331,10 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       if (prc != CAKE_OK) return prc;
     }
     ctx->n_units = nu;
+    {
+      const int64_t partials = ctx->use_tc ? (int64_t)ctx->n_tc_bsegs * kScoreWarps : (int64_t)nu * c.n_kv_heads;
+      ctx->n_fin_parts = partials > 512 * (int64_t)n_req * c.n_kv_heads ? c.n_kv_heads : 1;
+    }
     ctx->packed_rows_bound = bound;
     memcpy(ctx->h_cu, cu, sizeof(int64_t) * (n_req + 1));
     CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_req, ctx->h_req, sizeof(ReqInfo) * n_req,
@@ -365,7 +366,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
   ctx->last_alloc = -1;
   ctx->arrived_budgets = -1;
   CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int32_t), st));
-  ctx->pool_recorded[0] = ctx->pool_recorded[1] = false;
+  for (bool& r : ctx->pool_recorded) r = false;
   ctx->evict_recorded[0] = ctx->evict_recorded[1] = false;
   CAKE_CUDA_TRY(side_after(ctx, st));
   return CAKE_OK;
@@ -379,25 +380,26 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   if (layer != ctx->n_ind || ctx->n_evicted != layer) return CAKE_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   const int par = layer & 1;
-  // the score kernel's outputs of this parity were last read by the pooling of layer - 2; the rest
-  // of that layer's cascade works on its own data and may still be running
-  if (ctx->pool_recorded[par]) CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[par], 0));
+  // the score kernel's outputs of this layer's place were last read by the pooling of layer -
+  // kScoreDepth; the rest of that layer's cascade works on its own data and may still be running
+  const int place = layer % kScoreDepth;
+  if (ctx->pool_recorded[place]) CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[place], 0));
   int32_t rc = ctx->use_tc ? launch_score_tc(ctx, layer, q_win, k, lse, st)
                            : launch_score_simt(ctx, layer, q_win, k, lse, st);
   if (rc != CAKE_OK) return rc;
   // Pooling, the preference and the stage's budgets run on their own stream beside the next layer's
   // scoring and beside the eviction of the layer before; the pooled buffer, the scatter cursors and the
   // budgets of this parity were last read by the eviction of layer - 2.
-  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_score[par], st));
-  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_score[par], 0));
+  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_score[place], st));
+  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_score[place], 0));
   if (ctx->evict_recorded[par]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_evict[par], 0));
   const int sp = prof_begin(ctx, CAKE_PROF_FINALIZE, ctx->pool_st);
   const bool budgets = ctx->last_alloc < layer;      // nobody has asked for a later stage's before
   rc = launch_arrive(ctx, layer, true, true, budgets, ctx->pool_st);
   prof_end(ctx, sp, ctx->pool_st);
   if (rc != CAKE_OK) return rc;
-  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[par], ctx->pool_st));
-  ctx->pool_recorded[par] = true;
+  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[place], ctx->pool_st));
+  ctx->pool_recorded[place] = true;
   ctx->n_ind = layer + 1;
   if (ctx->n_pref < layer + 1) ctx->n_pref = layer + 1;
   ctx->arrived_budgets = budgets ? layer : -1;
@@ -419,8 +421,8 @@ int32_t cake_allocate(cake_ctx* ctx, int32_t stage, void* stream) {
     const int32_t rc = launch_allocate(ctx, stage, ast);
     prof_end(ctx, sp, ast);
     if (rc != CAKE_OK) return rc;
-    CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[stage & 1], ast));
-    ctx->pool_recorded[stage & 1] = true;
+    CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[stage % kScoreDepth], ast));
+    ctx->pool_recorded[stage % kScoreDepth] = true;
     if (ctx->arrived_budgets >= 0 && ((ctx->arrived_budgets ^ stage) & 1) == 0) ctx->arrived_budgets = -1;   // overwritten
   }
   ctx->alloc_of_buf[stage & 1] = stage;
@@ -435,7 +437,7 @@ int32_t cake_evict(cake_ctx* ctx, int32_t stage, void* stream) {
   if (ctx->alloc_of_buf[stage & 1] != stage) return CAKE_ERR_STATE;
   if (stage > 0 && ctx->alloc_of_buf[(stage + 1) & 1] != stage - 1) return CAKE_ERR_STATE;
   (void)stream;
-  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_pool[stage & 1], 0));
+  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_pool[stage % kScoreDepth], 0));
   const int sp = prof_begin(ctx, CAKE_PROF_EVICT, ctx->side);
   int32_t rc = launch_evict(ctx, stage, ctx->side);
   prof_end(ctx, sp, ctx->side);
@@ -550,8 +552,8 @@ int32_t cake_set_indicators(cake_ctx* ctx, int32_t layer, const float* in, void*
   // parity were last used by the eviction of layer - 2, which `stream` has waited for
   const int32_t rc = launch_arrive(ctx, layer, false, false, false, ctx->pool_st);
   if (rc != CAKE_OK) return rc;
-  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[layer & 1], ctx->pool_st));
-  ctx->pool_recorded[layer & 1] = true;
+  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[layer % kScoreDepth], ctx->pool_st));
+  ctx->pool_recorded[layer % kScoreDepth] = true;
   ctx->arrived_budgets = -1;
   ctx->n_ind = layer + 1;
   return CAKE_OK;

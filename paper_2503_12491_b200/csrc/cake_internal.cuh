@@ -18,6 +18,7 @@ constexpr int kBinBits = 12;         // survivor lists are sorted by the top bit
 constexpr int kBins = 1 << kBinBits;
 constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling / scatter CTAs
 constexpr int kBitmapSmemWords = 48 * 1024;   // positions of up to 1.5 M tokens are ordered in shared memory
+constexpr int kScoreDepth = 4;        // layers whose score outputs may wait for their pooling
 constexpr int kScoreGroups = 3;      // statistics warp groups per CTA of the tensor-core score kernel
 constexpr int kScoreWarps = 4 * kScoreGroups;   // statistics warps: one column-pass partial each
 
@@ -98,9 +99,10 @@ struct cake_ctx {
   cudaEvent_t ev_pool_side;         // scratch event: pooling stream -> caller's
   cudaEvent_t ev_evict[2];          // eviction stage of that parity has finished (it reads d_fresh of that parity)
   bool evict_recorded[2];
-  cudaEvent_t ev_score[2];          // score kernel of a layer of that parity has finished
-  cudaEvent_t ev_pool[2];           // pooling (the last reader of the score outputs) and budgets of that parity have finished
-  bool pool_recorded[2];
+  cudaEvent_t ev_score[cake::kScoreDepth];   // score kernel of layer % kScoreDepth has finished
+  cudaEvent_t ev_pool[cake::kScoreDepth];    // pooling (the last reader of the score outputs) and budgets of
+                                             // layer % kScoreDepth have finished
+  bool pool_recorded[cake::kScoreDepth];
   int32_t rows;            // R = G * S_w
   int64_t sel_budget;      // B' = B_total - L * S_w
   // ---- batch state (host) ----
@@ -115,6 +117,7 @@ struct cake_ctx {
   int32_t arrived_budgets; // stage whose budgets were computed when its layer was scored (-1: none, or a
                            // preference was set since)
   int32_t max_n_tokens;    // longest prompt of the batch
+  int32_t n_fin_parts;     // CTAs that share the preference of a request
   int64_t packed_rows_bound;
   int64_t* h_cu;           // host copy of cu_seqlens [max_requests+1]
   // ---- pinned staging ----
@@ -131,7 +134,7 @@ struct cake_ctx {
   double* d_P;
   int32_t* d_budget[2];    // [max_requests][L] selectable budgets, double-buffered by stage parity
   int32_t* d_status;       // sticky device status word
-  float* d_raw[2];         // [H_kv][max_total_tokens] un-pooled indicator, by layer parity
+  float* d_raw[cake::kScoreDepth];     // [H_kv][max_total_tokens] un-pooled indicator, by layer % kScoreDepth
   float* d_fresh[2];       // [H_kv][max_total_tokens] pooled indicator of the newest layer, by layer parity
   uint2* d_lists;          // per (req, layer, head): n entries (ordered indicator key, position)
   int64_t list_elems;
@@ -140,7 +143,8 @@ struct cake_ctx {
   int64_t max_lists;
   uint32_t* d_hist;        // [max_pairs][kBins] bucket histogram of the arriving layer (zero at rest)
   int32_t* d_fill[2];      // [max_pairs][kBins] scatter cursors of the arriving layer, by layer parity
-  uint32_t* d_arrivals;    // [max_pairs] counters of a list's finished runs in the pooling (zero at rest)
+  uint32_t* d_arrivals;    // zero at rest: [max_pairs] a list's finished runs in the pooling, [max_requests] a
+                           // request's finished parts of the preference
   double* d_headsum;       // [max_requests][H_q][2] per-head entropy / variance sums of the layer
   int32_t* d_pos_packed;   // [packed rows bound] positions in packed row order
   int64_t pos_packed_cap;
@@ -148,7 +152,7 @@ struct cake_ctx {
   int64_t bitmap_words;
   float* d_lse2;           // [max_requests][H_q][S_w] base-2 log-sum-exp of window rows
   float2* d_rowpart;       // [max_units][H_kv][R] (max, sum) partials of phase A
-  float* d_colpart[2];     // partial (sum p*log2 p, sum var) of the column pass, by layer parity
+  float* d_colpart[cake::kScoreDepth]; // partial (sum p*log2 p, sum var) of the column pass, likewise
   // ---- tensor-core score path ----
   bool use_tc;
   bool hhead_from_rows;    // entropy came from pass A (d_hrow) rather than from pass B partials
@@ -186,7 +190,7 @@ struct cake_ctx {
   bool tc_direct;                 // every CTA merges the denominators of its own pass-B ops (single-wave plans)
   float4* d_tc_rowpart;           // [max_tc_segs][kScoreGroups][128]
   float* d_lse2_tc;               // [max_requests][H_kv][128], rows in tile order i*G + h
-  float* d_hrow[2];               // [max_pairs][128] sum_j p log2 p per window row, by layer parity
+  float* d_hrow[cake::kScoreDepth];   // [max_pairs][128] sum_j p log2 p per window row, by layer % kScoreDepth
 };
 
 namespace cake {

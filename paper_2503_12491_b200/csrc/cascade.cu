@@ -5,6 +5,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 
 namespace cake {
@@ -28,8 +29,8 @@ __device__ inline double warp_sum_f64(double v) {
 // Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
 __device__ inline uint32_t ordered_key(float v) {
   uint32_t b = __float_as_uint(v);
-  if (b == 0x80000000u) b = 0u;
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+  b = b == 0x80000000u ? 0u : b;
+  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
 }
 __device__ inline int bucket_of(uint32_t key) { return (kBins - 1) - (int)(key >> (32 - kBinBits)); }
 
@@ -41,8 +42,45 @@ __device__ inline int split_span(int N, int want) {
   return ns > 0 ? (chunks + ns - 1) / ns * kChunkKeys : kChunkKeys;
 }
 
-constexpr int PH_THREADS = 1024;
+// The cascade kernels' CTAs take a whole SM each, 1024 threads in four teams that work on items of their
+// own.  (As CTAs of a team each they spread over all the SMs that are free in the moment between two
+// score launches, and the next one, whose CTAs need whole SMs, waits for them: 136 against 119 us per
+// 128K layer.  As one team of 1024 an SM has a single chain of scans and barriers at a time: with 256 lists
+// of 2K tokens 97 us for the pooling and 75 us for the scatter, now 36 and 32.)
+constexpr int TEAMS = 4;
+constexpr int TEAM_THREADS = 256;
+constexpr int TEAM_WARPS = TEAM_THREADS / 32;
+__device__ __forceinline__ void team_sync() {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x / TEAM_THREADS)), "n"(TEAM_THREADS) : "memory");
+}
+// Exclusive scan of one int per thread of the team; *total gets the sum.
+__device__ inline int team_excl_scan(int v, int* warp_tot, int* total) {
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x % TEAM_THREADS) >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += n;
+  }
+  if (lane == 31) warp_tot[warp] = inc;
+  team_sync();
+  int before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < TEAM_WARPS; ++w) {
+    const int t = warp_tot[w];
+    before += w < warp ? t : 0;
+    all += t;
+  }
+  *total = all;
+  team_sync();
+  return before + inc - v;
+}
+
 constexpr int PH_PER = 4;                            // consecutive tokens per thread and pass
+constexpr int kTileTok = 4096;                       // tokens of a run on their way to shared memory at a time
+__device__ __forceinline__ void copy_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
 
 struct AllocArgs {           // budgets of one stage
   const double* dP;          // [req][L]
@@ -65,6 +103,8 @@ struct FinalizeArgs {        // preference of the layer from the score kernels' 
   int32_t* status;
   int on;                    // 0: indicators were supplied, there is nothing to finalise
   int budgets;               // compute the stage's budgets as well
+  int parts;                 // CTAs that share a request's heads (divides H_q)
+  uint32_t* arrivals;        // [req] counters of a request's finished parts (zero at rest)
   int rows, Hq;
   double inv_tau1, inv_tau2;
 };
@@ -77,55 +117,81 @@ struct AllocSmem {
   int32_t win[CAKE_MAX_LAYERS];
   double c_val[kMaxCand];
   int32_t c_lay[kMaxCand];
-  int32_t c_s[kMaxCand];
+  double red[2][TEAM_WARPS];
+  int last;
 };
 __device__ void allocate_request(const AllocArgs& A, const ReqInfo& rq, int req, int stage, const double* p_stage, AllocSmem& S);
 
-// H_h = -ln2 * sum p*log2(p), V_h = sum_j Var_i of every query head of a request, a warp per head;
-// layer values are the means over the heads and P = H^(1/tau1) * V^(1/tau2) (Eq. 4-6).  All sums run in
-// a fixed order in double precision.  Then the budgets of the stage that this layer completes.
-__device__ void finalize_request(const FinalizeArgs& F, const AllocArgs& A, const ReqInfo& rq, int req, int layer, int Hkv,
-                                 AllocSmem& S) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int G = F.Hq / Hkv;
+// H_h = -ln2 * sum p*log2(p), V_h = sum_j Var_i of the query heads h_lo .. h_hi - 1 of a request, a warp
+// or several per head; the CTA that completes a request's last heads takes the means over the heads and
+// P = H^(1/tau1) * V^(1/tau2) (Eq. 4-6), then the budgets of the stage that this layer completes.  All
+// sums run in a fixed order in double precision.
+__device__ void finalize_heads(const FinalizeArgs& F, const AllocArgs& A, const ReqInfo& rq, int req, int part, int layer,
+                               int Hkv, AllocSmem& S) {
+  constexpr int W = TEAM_WARPS;
+  const int tid = threadIdx.x % TEAM_THREADS, lane = tid & 31, warp = tid >> 5;
+  const int G = F.Hq / Hkv, n_h = F.Hq / F.parts, h_lo = part * n_h;
+  int wph = 1;                                       // warps per head
+  while (wph * 2 * n_h <= W) wph *= 2;
   double* hs = F.headsum + (size_t)req * F.Hq * 2;
-  for (int h = warp; h < F.Hq; h += PH_THREADS / 32) {
-    const int g = h / G, hl = h - g * G, pair = req * Hkv + g;
-    const float2* part = reinterpret_cast<const float2*>(F.colpart);
-    int count, stride;
-    if (F.pair_seg) {
-      const int s_lo = F.pair_seg[pair];
-      part += (size_t)s_lo * kScoreWarps * G + hl;
-      count = (F.pair_seg[pair + 1] - s_lo) * kScoreWarps;
-      stride = G;
-    } else {
-      part += ((size_t)rq.unit0 * Hkv + g) * G + hl;
-      count = rq.nunits;
-      stride = Hkv * G;
-    }
+  for (int h0 = 0; h0 < n_h; h0 += W / wph) {
+    const int h = h_lo + h0 + warp / wph, sub = warp % wph;
     double a = 0.0, b = 0.0;
-    for (int i0 = 0; i0 < count; i0 += 32 * 8) {     // eight loads per lane in flight
-      float2 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = i0 + u * 32 + lane;
-        v[u] = i < count ? __ldcg(part + (size_t)i * stride) : make_float2(0.f, 0.f);
+    if (h < h_lo + n_h) {
+      const int g = h / G, hl = h - g * G, pair = req * Hkv + g;
+      const float2* part_at = reinterpret_cast<const float2*>(F.colpart);
+      int count, stride;
+      if (F.pair_seg) {
+        const int s_lo = F.pair_seg[pair];
+        part_at += (size_t)s_lo * kScoreWarps * G + hl;
+        count = (F.pair_seg[pair + 1] - s_lo) * kScoreWarps;
+        stride = G;
+      } else {
+        part_at += ((size_t)rq.unit0 * Hkv + g) * G + hl;
+        count = rq.nunits;
+        stride = Hkv * G;
       }
+      for (int i0 = sub * 32; i0 < count; i0 += 32 * 8 * wph) {      // eight loads per lane in flight
+        float2 v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) { a += (double)v[u].x; b += (double)v[u].y; }
+        for (int u = 0; u < 8; ++u) {
+          const int i = i0 + u * 32 * wph + lane;
+          v[u] = i < count ? __ldcg(part_at + (size_t)i * stride) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { a += (double)v[u].x; b += (double)v[u].y; }
+      }
+      if (F.hrow) {
+        a = 0.0;
+        if (sub == 0)
+          for (int r = hl + lane * G; r < F.rows; r += 32 * G) a += (double)__ldcg(&F.hrow[(size_t)pair * 128 + r]);
+      }
+      a = warp_sum_f64(a);
+      b = warp_sum_f64(b);
     }
-    if (F.hrow) {
-      a = 0.0;
-      for (int r = hl + lane * G; r < F.rows; r += 32 * G) a += (double)__ldcg(&F.hrow[(size_t)pair * 128 + r]);
+    if (wph > 1) {
+      if (lane == 0) { S.red[0][warp] = a; S.red[1][warp] = b; }
+      team_sync();
+      if (sub == 0 && lane == 0)
+        for (int w = 1; w < wph; ++w) { a += S.red[0][warp + w]; b += S.red[1][warp + w]; }
+      team_sync();
     }
-    a = warp_sum_f64(a);
-    b = warp_sum_f64(b);
-    if (lane == 0) { hs[2 * h] = -0.6931471805599453 * a; hs[2 * h + 1] = b; }
+    if (h < h_lo + n_h && sub == 0 && lane == 0) { hs[2 * h] = -0.6931471805599453 * a; hs[2 * h + 1] = b; }
   }
-  __syncthreads();
+  __threadfence();
+  team_sync();
+  if (F.parts > 1) {
+    if (tid == 0) {
+      S.last = atomicAdd(&F.arrivals[req], 1u) + 1u == (uint32_t)F.parts ? 1 : 0;
+      if (S.last) F.arrivals[req] = 0;
+    }
+    team_sync();
+    if (!S.last) return;
+    __threadfence();
+  }
   if (warp != 0) return;
   double H = 0.0, V = 0.0;
-  for (int h = lane; h < F.Hq; h += 32) { H += hs[2 * h]; V += hs[2 * h + 1]; }
+  for (int h = lane; h < F.Hq; h += 32) { H += __ldcg(&hs[2 * h]); V += __ldcg(&hs[2 * h + 1]); }
   H = warp_sum_f64(H) / (double)F.Hq;
   V = warp_sum_f64(V) / (double)F.Hq;
   const double P = (F.inv_tau1 == 1.0 ? H : pow(H, F.inv_tau1)) * (F.inv_tau2 == 1.0 ? V : pow(V, F.inv_tau2));
@@ -159,127 +225,191 @@ struct ArriveArgs {
   int n_req, want, layer, L, Hkv, kp, mode, do_pool;
   int64_t T;
 };
+struct alignas(16) ArriveSmem {   // of a team
+  union { uint32_t sh[kBins]; AllocSmem alloc; };
+  float tile[2][kTileTok + 8];   // tokens jb - 4 .. jb + kTileTok + 3 of the tile at jb
+  int warp_tot[TEAM_WARPS];
+  int last;
+};
 template <int R>
-__global__ void __launch_bounds__(PH_THREADS)
+__global__ void __launch_bounds__(TEAMS * TEAM_THREADS)
 arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
-  __shared__ union { uint32_t sh[kBins]; AllocSmem alloc; } U;
-  __shared__ int warp_tot[32];
-  __shared__ int s_total, s_last;
-  uint32_t* sh = U.sh;
-  const int n_fin = F.on ? Q.n_req : 0, n_items = n_fin + Q.n_req * Q.Hkv * Q.want;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int team = (int)threadIdx.x / TEAM_THREADS, tid = threadIdx.x % TEAM_THREADS;
+  ArriveSmem& S = reinterpret_cast<ArriveSmem*>(smem_raw)[team];
+  uint32_t* sh = S.sh;
+  const int n_fin = F.on ? Q.n_req * F.parts : 0, n_items = n_fin + Q.n_req * Q.Hkv * Q.want;
   const int layer = Q.layer, L = Q.L, Hkv = Q.Hkv, kp = Q.kp, mode = Q.mode, do_pool = Q.do_pool;
   const int64_t T = Q.T;
   const float* raw = Q.raw;
   float* fresh = Q.fresh;
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-  __syncthreads();                                   // the item before is done with shared memory
-  if (item < n_fin) {
-    finalize_request(F, B, Q.reqs[item], item, layer, Hkv, U.alloc);
-    continue;
-  }
-  const int split = (item - n_fin) % Q.want, pair = (item - n_fin) / Q.want;
-  const int req = pair / Hkv, g = pair - req * Hkv;
-  const ReqInfo rq = Q.reqs[req];
-  const int span = split_span(rq.N, Q.want), nsplit = (rq.N + span - 1) / span;
-  if (split >= nsplit) continue;
-  for (int b = threadIdx.x; b < kBins; b += PH_THREADS) sh[b] = 0;
-  __syncthreads();
-  const float* src = raw + (size_t)g * T + rq.cu;
-  float* dst = fresh + (size_t)g * T + rq.cu;
-  const int t0 = split * span, t1 = min(rq.N, t0 + span);
-  for (int j0 = t0 + (int)threadIdx.x * PH_PER; j0 < t1; j0 += PH_THREADS * PH_PER) {
-    float out[PH_PER];
-    if (!do_pool) {
+  for (int item = team * gridDim.x + blockIdx.x; item < n_items; item += TEAMS * gridDim.x) {
+    team_sync();                                   // the item before is done with shared memory
+    if (item < n_fin) {
+      const int r = item / F.parts;
+      finalize_heads(F, B, Q.reqs[r], r, item - r * F.parts, layer, Hkv, S.alloc);
+      continue;
+    }
+    const int split = (item - n_fin) % Q.want, pair = (item - n_fin) / Q.want;
+    const int req = pair / Hkv, g = pair - req * Hkv;
+    const ReqInfo rq = Q.reqs[req];
+    const int span = split_span(rq.N, Q.want), nsplit = (rq.N + span - 1) / span;
+    if (split >= nsplit) continue;
+    for (int b = tid; b < kBins; b += TEAM_THREADS) sh[b] = 0;
+    team_sync();
+    const float* src = raw + (size_t)g * T + rq.cu;
+    float* dst = fresh + (size_t)g * T + rq.cu;
+    const int t0 = split * span, t1 = min(rq.N, t0 + span);
+    // Writes four tokens and counts their buckets.  Neighbours often share a bucket, so a run is counted
+    // once, at its first token; without branches (with them a warp issued some 300 instructions for its
+    // 128 tokens, and the pooling was bound by that).
+    const bool vec = (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+    auto put = [&](int j0, const float (&out)[PH_PER]) {
+      if (j0 + PH_PER <= rq.n && j0 + PH_PER <= t1) {
+        if (do_pool) {
+          if (vec) {
+            *reinterpret_cast<float4*>(dst + j0) = make_float4(out[0], out[1], out[2], out[3]);
+          } else {
 #pragma unroll
-      for (int e = 0; e < PH_PER; ++e) out[e] = j0 + e < rq.n ? dst[j0 + e] : CUDART_INF_F;
-    } else if (R >= 0) {
-      const float pad = mode == CAKE_POOL_MAX ? -CUDART_INF_F : 0.f;
-      float w[PH_PER + 2 * (R >= 0 ? R : 0)];
+            for (int e = 0; e < PH_PER; ++e) dst[j0 + e] = out[e];
+          }
+        }
+        int q[PH_PER];
 #pragma unroll
-      for (int x = 0; x < PH_PER + 2 * R; ++x) {
-        const int j = j0 - R + x;
-        w[x] = (j >= 0 && j < rq.n) ? src[j] : pad;
+        for (int e = 0; e < PH_PER; ++e) q[e] = bucket_of(ordered_key(out[e]));
+        const bool s1 = q[1] != q[0], s2 = q[2] != q[1], s3 = q[3] != q[2];
+        atomicAdd(&sh[q[0]], s1 ? 1u : s2 ? 2u : s3 ? 3u : 4u);
+        if (s1) atomicAdd(&sh[q[1]], s2 ? 1u : s3 ? 2u : 3u);
+        if (s2) atomicAdd(&sh[q[2]], s3 ? 1u : 2u);
+        if (s3) atomicAdd(&sh[q[3]], 1u);
+      } else {
+#pragma unroll
+        for (int e = 0; e < PH_PER; ++e) {
+          const int j = j0 + e;
+          if (j < t1 && j >= rq.n) {
+            dst[j] = CUDART_INF_F;
+          } else if (j < t1) {
+            if (do_pool) dst[j] = out[e];
+            atomicAdd(&sh[bucket_of(ordered_key(out[e]))], 1u);
+          }
+        }
       }
+    };
+    if constexpr (R >= 0) {
+      // A run comes in tiles, the next one on its way while one is pooled (a thread that fetched its own
+      // tokens with their neighbours waited for every four of them: 28 us for 8K tokens beside a score
+      // kernel that keeps the memory system busy).
+      const float* in = do_pool ? src : dst;
+      const float pad = mode == CAKE_POOL_MAX ? -CUDART_INF_F : 0.f;
+      auto fetch = [&](int buf, int jb) {
+        const int cnt = min(kTileTok, t1 - jb) + 8;
+        for (int i = tid; i < cnt; i += TEAM_THREADS) {
+          const int j = jb - 4 + i;
+          if (j >= 0 && j < rq.n) copy_async4(&S.tile[buf][i], in + j);
+          else S.tile[buf][i] = pad;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+      fetch(0, t0);
+      for (int jb = t0, buf = 0; jb < t1; jb += kTileTok, buf ^= 1) {
+        if (jb + kTileTok < t1) {
+          fetch(buf ^ 1, jb + kTileTok);
+          asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        team_sync();
+        for (int q = tid; q < kTileTok / PH_PER && jb + q * PH_PER < t1; q += TEAM_THREADS) {
+          float v[12];
 #pragma unroll
-      for (int e = 0; e < PH_PER; ++e) {
-        float m = w[e];
+          for (int i = 0; i < 3; ++i) {
+            const float4 f = reinterpret_cast<const float4*>(S.tile[buf])[q + i];
+            v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
+          }
+          float out[PH_PER];
 #pragma unroll
-        for (int x = 1; x <= 2 * R; ++x) m = mode == CAKE_POOL_MAX ? fmaxf(m, w[e + x]) : m + w[e + x];
-        out[e] = mode == CAKE_POOL_MAX ? m : m / (float)kp;
+          for (int e = 0; e < PH_PER; ++e) {
+            float m = v[4 + e];
+            if (do_pool) {
+              m = v[4 + e - R];
+#pragma unroll
+              for (int x = 1; x <= 2 * R; ++x) m = mode == CAKE_POOL_MAX ? fmaxf(m, v[4 + e - R + x]) : m + v[4 + e - R + x];
+              if (mode != CAKE_POOL_MAX) m /= (float)kp;
+            }
+            out[e] = m;
+          }
+          put(jb + q * PH_PER, out);
+        }
+        team_sync();
       }
     } else {
       const int r = kp >> 1;
+      for (int j0 = t0 + tid * PH_PER; j0 < t1; j0 += TEAM_THREADS * PH_PER) {
+        float out[PH_PER];
 #pragma unroll 1
-      for (int e = 0; e < PH_PER; ++e) {
-        const int j = j0 + e;
-        float m = 0.f;
-        if (j < rq.n) {
-          const int a = max(0, j - r), b = min(rq.n, j + r + 1);
-          m = src[a];
-          for (int x = a + 1; x < b; ++x) m = mode == CAKE_POOL_MAX ? fmaxf(m, src[x]) : m + src[x];
-          if (mode != CAKE_POOL_MAX) m /= (float)kp;
-        }
-        out[e] = m;
-      }
-    }
-    // write back and count buckets; neighbours often share a bucket, so runs are counted once
-    int run_bin = -1;
-    uint32_t run_len = 0;
-#pragma unroll
-    for (int e = 0; e < PH_PER; ++e) {
-      const int j = j0 + e;
-      if (j < t1) {
-        if (j >= rq.n) {
-          dst[j] = CUDART_INF_F;
-        } else {
-          if (do_pool) dst[j] = out[e];
-          const int q = bucket_of(ordered_key(out[e]));
-          if (q != run_bin) {
-            if (run_len) atomicAdd(&sh[run_bin], run_len);
-            run_bin = q;
-            run_len = 0;
+        for (int e = 0; e < PH_PER; ++e) {
+          const int j = j0 + e;
+          float m = 0.f;
+          if (j < rq.n) {
+            if (do_pool) {
+              const int a = max(0, j - r), b = min(rq.n, j + r + 1);
+              m = src[a];
+              for (int x = a + 1; x < b; ++x) m = mode == CAKE_POOL_MAX ? fmaxf(m, src[x]) : m + src[x];
+              if (mode != CAKE_POOL_MAX) m /= (float)kp;
+            } else {
+              m = dst[j];
+            }
           }
-          ++run_len;
+          out[e] = m;
         }
+        put(j0, out);
       }
     }
-    if (run_len) atomicAdd(&sh[run_bin], run_len);
-  }
-  __syncthreads();
-  uint32_t* gh = Q.hist + (size_t)pair * kBins;
-  if (nsplit > 1) {
-    for (int b = threadIdx.x; b < kBins; b += PH_THREADS)
-      if (sh[b]) atomicAdd(&gh[b], sh[b]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const uint32_t old = atomicAdd(&Q.arrivals[pair], 1u);
-      s_last = (old + 1u == (uint32_t)nsplit) ? 1 : 0;
+    team_sync();
+    uint32_t* gh = Q.hist + (size_t)pair * kBins;
+    if (nsplit > 1) {
+      for (int b = tid; b < kBins; b += TEAM_THREADS)
+        if (sh[b]) atomicAdd(&gh[b], sh[b]);
+      __threadfence();
+      team_sync();
+      if (tid == 0) {
+        const uint32_t old = atomicAdd(&Q.arrivals[pair], 1u);
+        S.last = (old + 1u == (uint32_t)nsplit) ? 1 : 0;
+      }
+      team_sync();
+      if (!S.last) continue;
+      __threadfence();
     }
-    __syncthreads();
-    if (!s_last) continue;
-    __threadfence();
-  }
-  // bucket offsets of the new list: prefix[i] = elements in buckets before i
-  int32_t* pf = Q.prefix + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
-  int32_t* fl = Q.fill + (size_t)pair * kBins;
-  constexpr int PER = kBins / PH_THREADS;
-  int cnt[PER], sum = 0;
+    // bucket offsets of the new list: prefix[i] = elements in buckets before i
+    int32_t* pf = Q.prefix + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
+    int32_t* fl = Q.fill + (size_t)pair * kBins;
+    // (a warp takes a run of the buckets, 32 at a time, so that all accesses are consecutive)
+    constexpr int PER = kBins / TEAM_THREADS;
+    const int lane = tid & 31, first = (tid >> 5) * (32 * PER) + lane;
+    int cnt[PER], sum = 0;
 #pragma unroll
-  for (int e = 0; e < PER; ++e) {
-    cnt[e] = (int)(nsplit > 1 ? __ldcg(&gh[threadIdx.x * PER + e]) : sh[threadIdx.x * PER + e]);
-    sum += cnt[e];
-  }
-  int run = block_excl_scan(sum, warp_tot, &s_total);
+    for (int e = 0; e < PER; ++e) {
+      cnt[e] = (int)(nsplit > 1 ? __ldcg(&gh[first + 32 * e]) : sh[first + 32 * e]);
+      sum += cnt[e];
+    }
+    int total;
+    int run = team_excl_scan(sum, S.warp_tot, &total);
+    run = __shfl_sync(0xffffffffu, run, 0);            // elements before the warp's run
 #pragma unroll
-  for (int e = 0; e < PER; ++e) {
-    pf[threadIdx.x * PER + e] = run;
-    fl[threadIdx.x * PER + e] = run;
-    run += cnt[e];
-    if (nsplit > 1) gh[threadIdx.x * PER + e] = 0;   // ready for the next layer
-  }
-  if (threadIdx.x == PH_THREADS - 1) pf[kBins] = run;
-  if (nsplit > 1 && threadIdx.x == 0) Q.arrivals[pair] = 0;
+    for (int e = 0; e < PER; ++e) {
+      int inc = cnt[e];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += n;
+      }
+      pf[first + 32 * e] = run + inc - cnt[e];
+      fl[first + 32 * e] = run + inc - cnt[e];
+      run += __shfl_sync(0xffffffffu, inc, 31);
+      if (nsplit > 1) gh[first + 32 * e] = 0;          // ready for the next layer
+    }
+    if (tid == 0) pf[kBins] = total;
+    if (nsplit > 1 && tid == 0) Q.arrivals[pair] = 0;
   }
 }
 
@@ -314,7 +444,7 @@ __device__ void allocate_request(const AllocArgs& A, const ReqInfo& rq, int req,
   int64_t* s_lo = S.lo;
   int32_t *s_off = S.off, *s_win = S.win;
   double* c_val = S.c_val;
-  int32_t *c_lay = S.c_lay, *c_s = S.c_s;
+  int32_t* c_lay = S.c_lay;
   const int La = stage + 1;
   int32_t* out = A.cur + (size_t)req * L;
   const int32_t* old = A.prev + (size_t)req * L;
@@ -401,18 +531,18 @@ __device__ void allocate_request(const AllocArgs& A, const ReqInfo& rq, int req,
         const int64_t s = s_lo[l] + e;
         c_val[base + e] = sP[l] / ((double)s + 0.5);
         c_lay[base + e] = l;
-        c_s[base + e] = e;
       }
     }
     __syncwarp();
+    // candidates stand in the order of the tie rule (layer, then s)
     for (int c = lane; c < ncand; c += 32) {
       const double v = c_val[c];
-      const int l = c_lay[c], e = c_s[c];
-      int64_t ahead = 0;
+      const int l = c_lay[c];
+      int ahead = 0;
+#pragma unroll 8
       for (int o = 0; o < ncand; ++o) {
         const double vo = c_val[o];
-        const int lo2 = c_lay[o], eo = c_s[o];
-        ahead += (vo > v) || (vo == v && (lo2 < l || (lo2 == l && eo < e)));
+        ahead += (vo > v || (vo == v && o < c)) ? 1 : 0;
       }
       if (ahead < need) atomicAdd(&s_win[l], 1);
     }
@@ -477,8 +607,9 @@ struct EvictArgs {
   int64_t T;
 };
 
-constexpr int SC_THREADS = 1024;
+static_assert(offsetof(ArriveSmem, tile) % 16 == 0 && sizeof(ArriveSmem) % 16 == 0, "tiles are read 16 bytes at a time");
 constexpr int SC_PER = 4;
+constexpr int SC_LOADS = 4;
 
 // Newest layer of stage `stage`: an item per (run of a request's tokens, KV head, request) scatters the
 // pooled indicators into bucket order.  Only the buckets the layer's budget can ever reach are stored
@@ -487,15 +618,19 @@ constexpr int SC_PER = 4;
 // (list_threshold): a later, smaller budget changes nothing that is stored, so the older layers need no
 // work here.  (Moving every older list's threshold at every stage was a launch of up to 31 * H_kv
 // CTAs per layer, 10 to 72 us beside the score kernel.)
-__global__ void __launch_bounds__(SC_THREADS)
+struct ScatterSmem {           // of a team
+  uint32_t cnt[kBins], base[kBins];
+  int warp_tot[TEAM_WARPS];
+};
+__global__ void __launch_bounds__(TEAMS * TEAM_THREADS)
 scatter_new(const EvictArgs A) {
-  __shared__ uint32_t s_cnt[kBins];
-  __shared__ uint32_t s_base[kBins];
-  __shared__ int warp_tot[32];
-  __shared__ int s_total;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int team = (int)threadIdx.x / TEAM_THREADS, tid = (int)threadIdx.x % TEAM_THREADS;
+  ScatterSmem& S = reinterpret_cast<ScatterSmem*>(smem_raw)[team];
+  uint32_t *s_cnt = S.cnt, *s_base = S.base;
   const int n_items = A.n_req * A.Hkv * A.want;
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    __syncthreads();
+  for (int item = team * gridDim.x + blockIdx.x; item < n_items; item += TEAMS * gridDim.x) {
+    team_sync();
     const int split = item % A.want, pair = item / A.want;
     const int req = pair / A.Hkv, g = pair - req * A.Hkv;
     const ReqInfo rq = A.reqs[req];
@@ -506,75 +641,95 @@ scatter_new(const EvictArgs A) {
     const int32_t* pf = A.prefix_all + lid * (kBins + 1);
     uint2* list = A.lists + rq.list_off + ((size_t)A.stage * A.Hkv + g) * rq.n;
     const int b = min(A.cur[(size_t)req * A.L + A.stage], rq.n);
-    if (split == 0 && threadIdx.x == 0) A.states[lid] = ListState{-1, 0xFFFFFFFFu, -1, b};
+    if (split == 0 && tid == 0) A.states[lid] = ListState{-1, 0xFFFFFFFFu, -1, b};
     // last bucket worth storing
     int less = 0;
-    for (int i = threadIdx.x; i < kBins; i += SC_THREADS) {
+    for (int i = tid; i < kBins; i += TEAM_THREADS) {
       less += __ldcg(&pf[i + 1]) < b ? 1 : 0;
       s_cnt[i] = 0;
     }
-    block_excl_scan(less, warp_tot, &s_total);
-    const int d_last = b > 0 ? min(s_total, kBins - 1) : -1;
+    int total;
+    team_excl_scan(less, S.warp_tot, &total);
+    const int d_last = b > 0 ? min(total, kBins - 1) : -1;
     const float* src = A.fresh + (size_t)g * A.T + rq.cu;
-    // pass 1: count this run's entries per bucket (runs of equal buckets at once)
-    for (int j0 = t0 + (int)threadIdx.x * SC_PER; j0 < t1; j0 += SC_THREADS * SC_PER) {
-      int run_bin = -1;
-      uint32_t run_len = 0;
+    // SC_LOADS * 4 consecutive tokens per thread at a time, all loads in flight together
+    constexpr int kStep = TEAM_THREADS * SC_PER * SC_LOADS;
+    uint32_t key[SC_LOADS][SC_PER];
+    auto fetch = [&](int jb) {
+      float v[SC_LOADS][SC_PER];
+#pragma unroll
+      for (int u = 0; u < SC_LOADS; ++u)
+#pragma unroll
+        for (int e = 0; e < SC_PER; ++e) {
+          const int j = jb + (u * TEAM_THREADS + tid) * SC_PER + e;
+          v[u][e] = j < t1 ? __ldcg(&src[j]) : 0.f;
+        }
+#pragma unroll
+      for (int u = 0; u < SC_LOADS; ++u)
+#pragma unroll
+        for (int e = 0; e < SC_PER; ++e) key[u][e] = ordered_key(v[u][e]);
+    };
+    // Buckets of four tokens; len: how many of them start here in a run of equal buckets, 0 where no run
+    // starts or the bucket is not stored.
+    struct Four { int q[SC_PER]; uint32_t len[SC_PER]; bool keep[SC_PER]; bool any; };
+    auto four = [&](int jb, int u) {
+      Four f;
+      const int j0 = jb + (u * TEAM_THREADS + tid) * SC_PER;
 #pragma unroll
       for (int e = 0; e < SC_PER; ++e) {
-        int q = -1;
-        if (j0 + e < t1) {
-          q = bucket_of(ordered_key(src[j0 + e]));
-          if (q > d_last) q = -1;
-        }
-        if (q != run_bin) {
-          if (run_len && run_bin >= 0) atomicAdd(&s_cnt[run_bin], run_len);
-          run_bin = q;
-          run_len = 0;
-        }
-        ++run_len;
+        f.q[e] = bucket_of(key[u][e]);
+        f.keep[e] = j0 + e < t1 && f.q[e] <= d_last;
       }
-      if (run_len && run_bin >= 0) atomicAdd(&s_cnt[run_bin], run_len);
+#pragma unroll
+      for (int e = 0; e < SC_PER; ++e) {
+        uint32_t n = 1;
+        bool run = true;
+#pragma unroll
+        for (int x = e + 1; x < SC_PER; ++x) {
+          run = run && f.keep[x] && f.q[x] == f.q[e];
+          n += run ? 1u : 0u;
+        }
+        const bool starts = f.keep[e] && (e == 0 || f.q[e - 1] != f.q[e]);
+        f.len[e] = starts ? n : 0u;
+      }
+      f.any = f.keep[0] || f.keep[1] || f.keep[2] || f.keep[3];
+      return f;
+    };
+    // pass 1: count this run's entries per bucket (runs of equal buckets at once)
+    for (int jb = t0; jb < t1; jb += kStep) {
+      fetch(jb);
+#pragma unroll
+      for (int u = 0; u < SC_LOADS; ++u) {
+        const Four f = four(jb, u);
+        if (!__any_sync(0xffffffffu, f.any)) continue;
+#pragma unroll
+        for (int e = 0; e < SC_PER; ++e)
+          if (f.len[e]) atomicAdd(&s_cnt[f.q[e]], f.len[e]);
+      }
     }
-    __syncthreads();
+    team_sync();
     // reserve this run's range inside every bucket of the list
     int32_t* fl = A.fill + (size_t)pair * kBins;
-    for (int q = threadIdx.x; q < kBins; q += SC_THREADS) {
+    for (int q = tid; q < kBins; q += TEAM_THREADS) {
       const uint32_t c = s_cnt[q];
       if (c) s_base[q] = (uint32_t)atomicAdd(&fl[q], (int)c);
       s_cnt[q] = 0;
     }
-    __syncthreads();
+    team_sync();
     // pass 2: place the entries
-    for (int j0 = t0 + (int)threadIdx.x * SC_PER; j0 < t1; j0 += SC_THREADS * SC_PER) {
-      uint32_t key[SC_PER];
-      int bk[SC_PER];
+    for (int jb = t0; jb < t1; jb += kStep) {
+      if (t1 - t0 > kStep) fetch(jb);                // a short run is still in registers
 #pragma unroll
-      for (int e = 0; e < SC_PER; ++e) {
-        bk[e] = -1;
-        if (j0 + e < t1) {
-          key[e] = ordered_key(src[j0 + e]);
-          const int q = bucket_of(key[e]);
-          if (q <= d_last) bk[e] = q;
+      for (int u = 0; u < SC_LOADS; ++u) {
+        const Four f = four(jb, u);
+        if (!__any_sync(0xffffffffu, f.any)) continue;
+        const uint32_t j0 = (uint32_t)(jb + (u * TEAM_THREADS + tid) * SC_PER);
+        uint32_t off = 0;
+#pragma unroll
+        for (int e = 0; e < SC_PER; ++e) {
+          if (f.len[e]) off = s_base[f.q[e]] + atomicAdd(&s_cnt[f.q[e]], f.len[e]);
+          if (f.keep[e]) list[off++] = make_uint2(key[u][e], j0 + e);
         }
-      }
-      int run_bin = -1;
-      uint32_t run_off = 0;
-#pragma unroll
-      for (int e = 0; e < SC_PER; ++e) {
-        if (bk[e] != run_bin) {
-          run_bin = bk[e];
-          if (run_bin >= 0) {
-            uint32_t len = 1;
-#pragma unroll
-            for (int f = e + 1; f < SC_PER; ++f) {
-              if (bk[f] != run_bin) break;
-              ++len;
-            }
-            run_off = s_base[run_bin] + atomicAdd(&s_cnt[run_bin], len);
-          }
-        }
-        if (run_bin >= 0) list[run_off++] = make_uint2(key[e], (uint32_t)(j0 + e));
       }
     }
   }
@@ -588,7 +743,7 @@ static void cascade_shape(const cake_ctx* ctx, int32_t layer, int extra_items, i
   const int pairs = ctx->n_req * ctx->cfg.n_kv_heads;
   int slots = ctx->n_sm;
   if (layer + 1 < ctx->cfg.n_layers) slots = ctx->use_tc ? std::max(8, ctx->n_sm - ctx->n_tc_ctas) : ctx->n_sm / 4;
-  int w = std::max(1, slots / std::max(1, pairs));
+  int w = std::max(1, slots * TEAMS / std::max(1, pairs));
   w = std::min(w, (ctx->max_n_tokens + kChunkKeys - 1) / kChunkKeys);
   *want = std::max(1, w);
   *grid = std::min(slots, pairs * *want + extra_items);
@@ -619,10 +774,13 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
   if (finalize) {
     F.on = 1;
     F.budgets = budgets ? 1 : 0;
-    F.colpart = ctx->d_colpart[layer & 1];
+    F.colpart = ctx->d_colpart[layer % kScoreDepth];
     F.pair_seg = ctx->use_tc ? ctx->d_tc_index + (ctx->n_req * c.n_kv_heads + 1) : nullptr;
-    F.hrow = ctx->use_tc && ctx->hhead_from_rows ? ctx->d_hrow[layer & 1] : nullptr;
+    F.hrow = ctx->use_tc && ctx->hhead_from_rows ? ctx->d_hrow[layer % kScoreDepth] : nullptr;
     F.headsum = ctx->d_headsum;
+    F.arrivals = ctx->d_arrivals + ctx->max_pairs;
+    // a long prompt has thousands of partial sums per head: a CTA per KV head; else one per request
+    F.parts = ctx->n_fin_parts;
     F.dH = ctx->d_H; F.dV = ctx->d_V; F.dP = ctx->d_P;
     F.status = ctx->d_status;
     F.rows = ctx->rows;
@@ -630,7 +788,7 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
     F.inv_tau2 = 1.0 / (double)c.tau2;
   }
   ArriveArgs Q;
-  Q.raw = ctx->d_raw[layer & 1];
+  Q.raw = ctx->d_raw[layer % kScoreDepth];
   Q.fresh = ctx->d_fresh[layer & 1];
   Q.reqs = ctx->d_req;
   Q.hist = ctx->d_hist;
@@ -641,14 +799,24 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
   Q.kp = c.pool_kernel; Q.mode = c.pool_mode; Q.do_pool = do_pool ? 1 : 0;
   Q.T = ctx->total_tokens;
   int grid;
-  cascade_shape(ctx, layer, finalize ? ctx->n_req : 0, &Q.want, &grid);
+  cascade_shape(ctx, layer, finalize ? ctx->n_req * F.parts : 0, &Q.want, &grid);
   const AllocArgs B = alloc_args(ctx, layer);
+  static PerDeviceOnce attr;
+  if (attr.need(ctx->device)) {
+    const int bytes = (int)(TEAMS * sizeof(ArriveSmem));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(arrive_layer<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(arrive_layer<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(arrive_layer<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(arrive_layer<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(arrive_layer<-1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    attr.mark(ctx->device);
+  }
   switch (c.pool_kernel / 2) {
-    case 0: arrive_layer<0><<<grid, PH_THREADS, 0, st>>>(Q, F, B); break;
-    case 1: arrive_layer<1><<<grid, PH_THREADS, 0, st>>>(Q, F, B); break;
-    case 2: arrive_layer<2><<<grid, PH_THREADS, 0, st>>>(Q, F, B); break;
-    case 3: arrive_layer<3><<<grid, PH_THREADS, 0, st>>>(Q, F, B); break;
-    default: arrive_layer<-1><<<grid, PH_THREADS, 0, st>>>(Q, F, B); break;
+    case 0: arrive_layer<0><<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ArriveSmem), st>>>(Q, F, B); break;
+    case 1: arrive_layer<1><<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ArriveSmem), st>>>(Q, F, B); break;
+    case 2: arrive_layer<2><<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ArriveSmem), st>>>(Q, F, B); break;
+    case 3: arrive_layer<3><<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ArriveSmem), st>>>(Q, F, B); break;
+    default: arrive_layer<-1><<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ArriveSmem), st>>>(Q, F, B); break;
   }
   count_launch();
   return cuda_status(cudaGetLastError());
@@ -676,7 +844,12 @@ int32_t launch_evict(cake_ctx* ctx, int32_t stage, cudaStream_t st) {
   A.T = ctx->total_tokens;
   int grid;
   cascade_shape(ctx, stage, 0, &A.want, &grid);
-  scatter_new<<<grid, SC_THREADS, 0, st>>>(A);
+  static PerDeviceOnce attr;
+  if (attr.need(ctx->device)) {
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(scatter_new, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TEAMS * sizeof(ScatterSmem))));
+    attr.mark(ctx->device);
+  }
+  scatter_new<<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ScatterSmem), st>>>(A);
   count_launch();
   return cuda_status(cudaGetLastError());
 }

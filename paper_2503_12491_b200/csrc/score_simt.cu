@@ -351,8 +351,8 @@ int32_t run(cake_ctx* ctx, int32_t layer, const void* q_win, const void* k, cons
   prof_end(ctx, sp, st);
   sp = prof_begin(ctx, CAKE_PROF_SCORE, st);
   score_colstats_simt<T><<<grid, NT, smem, st>>>(
-      (const T*)q_win, (const T*)k, ctx->d_req, ctx->d_units, ctx->d_lse2, ctx->d_raw[layer & 1],
-      ctx->d_colpart[layer & 1], c.n_q_heads, c.n_kv_heads, c.window, c.head_dim, ctx->total_tokens, scale2,
+      (const T*)q_win, (const T*)k, ctx->d_req, ctx->d_units, ctx->d_lse2, ctx->d_raw[layer % kScoreDepth],
+      ctx->d_colpart[layer % kScoreDepth], c.n_q_heads, c.n_kv_heads, c.window, c.head_dim, ctx->total_tokens, scale2,
       c.gamma, c.var_ddof, c.indicator_mode);
   count_launch();
   prof_end(ctx, sp, st);

@@ -86,7 +86,7 @@ struct TcParams {
   float scale2, inv_scale2, gamma, bessel;
   int ind_mode;                 // CAKE_IND_*
   int merge_ways;               // rows the merger warp merges side by side: 1, or 2 to 32 when pairs are short
-  int reps, rep_shift;          // copies of the window rows in a pass-A tile: 128 / rows for 32 and 64 rows, else 1
+  int reps;                     // copies of the window rows in a pass-A tile: 128 / rows for 32 and 64 rows, else 1
 };
 
 // ------------------------------------------------------------------ PTX
@@ -321,7 +321,8 @@ struct Smem {
   uint32_t* a_done;    // [NSTATW] pass-A ops whose partial rows each statistics warp has written
   uint8_t* ext_a;      // the constant key-side operand of the extra K step of pass B
   uint8_t* ext_b;      // [2] its row-side operand: -lse/scale of the current / next pass-B op
-  float4* xrow;        // [2][NWG][128] direct merge: a group's merged rows of the current / next pass-B op
+  float4* xrow;        // [2][NWG][128] partial rows of a group: copies of a row in pass A, then (direct merge) the
+                       //   group's share of a pair's partials for the current / next pass-B op
   ScoreOp* ops;        // [kSmemOps] the first ops of this CTA's program
 };
 
@@ -611,12 +612,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         return true;
       };
-      // partial `pi` of row r: (segment, group) pi / reps, copy pi % reps of the row
-      const int reps = kCopies ? P.reps : 1;
-      auto part_at = [&](int pi, int r) -> size_t {
-        if constexpr (kCopies) return (size_t)(pi >> P.rep_shift) * 128 + (pi & (P.reps - 1)) * P.rows + r;
-        else return (size_t)pi * 128 + r;
-      };
       if constexpr (kDirect) {
         // nothing to merge here: the statistics warps do it
       } else if (P.merge_ways > 1) {
@@ -650,12 +645,13 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
             float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
             if (active) {
-              for (int base = s_lo * reps; base < s_hi * reps; base += 8 * lpr) {
+              for (int base = s_lo; base < s_hi; base += 8 * lpr) {
                 float4 pv[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                   const int sg = base + u * lpr + l8;
-                  pv[u] = sg < s_hi * reps ? __ldcg(&P.rowpart[part_at(sg, r)]) : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+                  pv[u] = sg < s_hi ? __ldcg(&P.rowpart[(size_t)sg * 128 + r])
+                                    : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) acc = merge_rows(acc, pv[u]);
@@ -699,12 +695,13 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           }
           float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
           // 12 loads per lane in flight: the 384 partials of a row at 128 CTAs come in one round trip
-          for (int base = s_lo * reps; base < s_hi * reps; base += 32 * 12) {
+          for (int base = s_lo; base < s_hi; base += 32 * 12) {
             float4 pv[12];
 #pragma unroll
             for (int u = 0; u < 12; ++u) {
               const int sg = base + u * 32 + lane;
-              pv[u] = sg < s_hi * reps ? __ldcg(&P.rowpart[part_at(sg, r)]) : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+              pv[u] = sg < s_hi ? __ldcg(&P.rowpart[(size_t)sg * 128 + r])
+                                : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int u = 0; u < 12; ++u) acc = merge_rows(acc, pv[u]);
@@ -825,9 +822,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           if (ok) ok = mbar_wait(&S.parts[slot], (kbs >> 1) & 1, P.status, P.spin_limit);
           ++kbs;
           float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-          const int reps = kCopies ? P.reps : 1;
           const int s_lo = P.pair_aseg[pair], s_hi = ok ? P.pair_aseg[pair + 1] : s_lo;
-          if (lane_row < P.rows * reps) {
+          if (lane_row < P.rows) {
             for (int sg = s_lo; sg < s_hi; sg += 8) {
               float4 pv[8];
 #pragma unroll
@@ -842,12 +838,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           if (wg == 0) {
             acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
             if (lane_row < P.rows) {
-              for (int rp = 0; rp < reps; ++rp) {
-                float4 pv[NWG];
+              float4 pv[NWG];
 #pragma unroll
-                for (int q = 0; q < NWG; ++q) pv[q] = S.xrow[(slot * NWG + q) * 128 + rp * P.rows + lane_row];
-                acc = merge_batch(acc, pv);
-              }
+              for (int q = 0; q < NWG; ++q) pv[q] = S.xrow[(slot * NWG + q) * 128 + lane_row];
+              acc = merge_batch(acc, pv);
             }
             const float lz = log2f(acc.y);
             put_ext_row(S.ext_b + slot * kExtBytes, lane_row, P.rows, acc.x + lz, P.inv_scale2);
@@ -1065,7 +1059,17 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // Deliver this warp's 32 partial rows of the segment.  Making them visible to the other
         // CTAs takes a fence of a few thousand cycles; the merger warp pays it once per op for all
         // twelve warps, which only tell it, inside the CTA, that their rows are written.
-        __stcg(&P.rowpart[((size_t)op.seg * NWG + wg) * 128 + lane_row], make_float4(m, z, zwin, w));
+        float4 part = make_float4(m, z, zwin, w);
+        if constexpr (kCopies) {
+          // the group's copies of a row become one partial (two slots: a reader of this op's is done
+          // before it reaches the next op's barrier)
+          float4* x = S.xrow + ((n_a_done & 1) * NWG + wg) * 128;
+          x[lane_row] = part;
+          asm volatile("bar.sync %0, 128;" ::"r"(2 + wg) : "memory");
+          if (copy == 0)
+            for (int c = 1; c < P.reps; ++c) part = merge_rows(part, x[c * P.rows + lane_row]);
+        }
+        if (!kCopies || copy == 0) __stcg(&P.rowpart[((size_t)op.seg * NWG + wg) * 128 + lane_row], part);
         __syncwarp();
         ++n_a_done;
         if (lane == 0) smem_store_release(&S.a_done[warp], n_a_done);
@@ -1328,7 +1332,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
   {
     int max_segs = 0;
     for (int p = 0; p < n_pairs; ++p) max_segs = std::max(max_segs, pair_aseg[p + 1] - pair_aseg[p]);
-    const int partials = max_segs * NWG * tc_reps(ctx->rows);
+    const int partials = max_segs * NWG;
     // at most 16 partials per lane (two batches of loads): 32 lanes / ways per row
     int ways = 1;
     while (ways < 32 && 2 * ways <= n_pairs && partials * 2 * ways <= 512) ways *= 2;
@@ -1501,9 +1505,9 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.lse2 = ctx->d_lse2_tc;
   P.lse_ext = lse;
   P.rowpart = ctx->d_tc_rowpart;
-  P.raw = ctx->d_raw[layer & 1];
-  P.colpart = ctx->d_colpart[layer & 1];
-  P.hrow = ctx->d_hrow[layer & 1];
+  P.raw = ctx->d_raw[layer % kScoreDepth];
+  P.colpart = ctx->d_colpart[layer % kScoreDepth];
+  P.hrow = ctx->d_hrow[layer % kScoreDepth];
   P.n_pairs = n_pairs;
   P.status = ctx->d_status;
   P.T = ctx->total_tokens;
@@ -1514,7 +1518,6 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.ind_mode = c.indicator_mode;
   P.merge_ways = ctx->tc_merge_ways;
   P.reps = tc_reps(ctx->rows);
-  P.rep_shift = P.reps == 4 ? 2 : P.reps == 2 ? 1 : 0;
   P.spin_limit = ctx->wait_limit_cycles > 0 ? ctx->wait_limit_cycles : kSpinLimit;
   P.bessel = c.var_ddof ? (float)c.window / (float)(c.window - 1) : 1.f;
 

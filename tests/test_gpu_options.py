@@ -272,3 +272,34 @@ def test_row_copies_and_both_ways_to_the_denominators(hq, hkv, window, seq_lens)
     w = bf16_case(n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=seq_lens, n_layers=2 if max(seq_lens) < 9000 else 1,
                   total_budget=(2 if max(seq_lens) < 9000 else 1) * (window + 60))
     check_scores(w, expect_tc=True)
+
+
+@pytest.mark.parametrize("seq_lens,budget,pool", [
+    ((4096 + 31, 4096 + 33, 77), 300, 7),            # runs that end a token before and after a tile, odd offsets
+    ((8192 + 32, 40), 1000, 5),                      # a whole number of tiles, a prompt of eight tokens
+    ((20481, 3, 5000), 2500, 1),                     # several runs per list; a prompt shorter than a quad
+    ((9001, 4500), 200, 11),                         # the generic pooling
+])
+def test_lists_at_the_edges_of_tiles_and_runs(seq_lens, budget, pool):
+    """One fp32 layer with a window of 2: the retained positions are the exact top-k of the device's own
+    indicators (value descending, position ascending), at every place a list may be cut into runs."""
+    w = fp32_case(n_layers=1, window=2, seq_lens=seq_lens, pool_kernel=pool, total_budget=budget)
+    qs, ks, vs = harness.device_inputs(w)
+    cake = harness.cake_for(w)
+    cake.begin(w.cu_seqlens)
+    cake.score_layer(0, qs[0], ks[0])
+    ind = cake.get_indicators(0).cpu().numpy().astype(np.float64)
+    cake.allocate(0)
+    cake.evict(0)
+    budgets = cake.get_budgets().cpu().numpy()
+    for r, N in enumerate(seq_lens):
+        n = N - w.window
+        ref = O.score_layer(to_np(qs[0][r]), to_np(ks[0][:, w.cu_seqlens[r]:w.cu_seqlens[r + 1]]), gamma=w.gamma, pool_kernel=pool)
+        got = cake.get_positions(r, 0, int(budgets[r, 0])).cpu().numpy()
+        for g in range(w.n_kv_heads):
+            mine = ind[g, w.cu_seqlens[r]:w.cu_seqlens[r] + n]
+            assert_close(mine, ref["indicator"][g], f"indicator r{r} g{g}")
+            want = np.concatenate([O.topk_keep(mine, int(budgets[r, 0]) - w.window), np.arange(n, N)])
+            assert np.array_equal(got[g], want), (r, g)
+    assert cake.status() == 0
+    cake.destroy()
