@@ -3,6 +3,7 @@
 // translation units; this file only validates arguments and enqueues work.
 #include "cake_internal.cuh"
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdlib>
@@ -39,12 +40,12 @@ cudaError_t dev_alloc(T** p, size_t count) {
   return cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T));
 }
 
-int32_t choose_unit_keys(int64_t total_tokens, int n_kv_heads, int n_sm) {
-  // Aim for about four CTAs per SM across the (unit, KV head) grid, units of 64..1024 keys.
+int32_t choose_unit_keys(int64_t total_tokens, int n_kv_heads, int n_sm, int tile) {
+  // Aim for about four CTAs per SM across the (unit, KV head) grid, units of whole tiles up to 1024 keys.
   int64_t per = total_tokens * n_kv_heads / ((int64_t)4 * n_sm);
-  per = per / kSimtTileKeys * kSimtTileKeys;
-  if (per < kSimtTileKeys) per = kSimtTileKeys;
-  if (per > 1024) per = 1024;
+  per = per / tile * tile;
+  if (per < tile) per = tile;
+  if (per > kSimtMaxUnit) per = kSimtMaxUnit;
   return (int32_t)per;
 }
 
@@ -64,6 +65,7 @@ void free_ctx(cake_ctx* c) {
   cudaFree(c->d_fresh[0]); cudaFree(c->d_fresh[1]); cudaFree(c->d_lists); cudaFree(c->d_prefix); cudaFree(c->d_lstate);
   cudaFree(c->d_hist); cudaFree(c->d_fill[0]); cudaFree(c->d_fill[1]); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
+  cudaFree(c->d_scores); cudaFree(c->d_simt_arrivals);
   cudaFree(c->d_rowpart);
   cudaFree(c->d_tc_ops); cudaFree(c->d_tc_index); cudaFree(c->d_tc_sync);
   cudaFree(c->d_tc_rowpart); cudaFree(c->d_lse2_tc);
@@ -167,8 +169,8 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
 
   const int64_t T = c.max_total_tokens;
   const int64_t R = c.max_requests;
-  // a unit never spans requests: at most T/64 + R units
-  x->max_units = (int32_t)(T / kSimtTileKeys + R + 1);
+  // a unit never spans requests: at most T / kSimtMinUnit + R units
+  x->max_units = (int32_t)(T / kSimtMinUnit + R + 1);
   x->list_elems = T * c.n_layers * c.n_kv_heads;
   x->max_lists = R * c.n_layers * c.n_kv_heads;
   {
@@ -224,6 +226,16 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   {
     const char* force = getenv("CAKE_SCORE_PATH");       // "simt" forces the SIMT kernels
     x->use_tc = tc_path_supported(c) && !(force && strcmp(force, "simt") == 0);
+  }
+  if (!x->use_tc) {
+    // all logits of a batch if they fit CAKE_SIMT_SCORES_MB (environment, default 256), at least one unit's
+    const char* mb = getenv("CAKE_SIMT_SCORES_MB");
+    const int64_t most = mb ? (int64_t)std::max(0, atoi(mb)) << 18 : kMaxScoreElems;
+    const int64_t per_key = (int64_t)c.n_kv_heads * x->rows;
+    x->scores_elems = std::max<int64_t>(kSimtMaxUnit * per_key, std::min<int64_t>(most, (T + R * kSimtMaxUnit) * per_key));
+    ok = ok && dev_alloc(&x->d_scores, (size_t)x->scores_elems) == cudaSuccess;
+    ok = ok && dev_alloc(&x->d_simt_arrivals, (size_t)R * c.n_kv_heads) == cudaSuccess;
+    ok = ok && cudaMemset(x->d_simt_arrivals, 0, sizeof(uint32_t) * R * c.n_kv_heads) == cudaSuccess;
   }
   const int64_t max_pairs = R * c.n_kv_heads;
   x->max_pairs = (int32_t)max_pairs;
@@ -303,7 +315,8 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       CAKE_CUDA_TRY(cudaEventSynchronize(ctx->upload_done));
       ctx->upload_pending = false;
     }
-    const int32_t unit_keys = choose_unit_keys(T, c.n_kv_heads, ctx->n_sm);
+    const int32_t unit_keys = choose_unit_keys(T, c.n_kv_heads, ctx->n_sm, simt_tile_keys(ctx->rows));
+    ctx->unit_keys = unit_keys;
     int32_t nu = 0;
     ctx->max_n_tokens = 0;
     int64_t list_off = 0, bound = 0;
@@ -319,9 +332,11 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       q.unit0 = nu;
       for (int32_t k0 = 0; k0 < q.N; k0 += unit_keys) {
         ScoreUnit& u = ctx->h_units[nu++];
-        u.req = r; u.key0 = k0; u.nkeys = q.N - k0 < unit_keys ? q.N - k0 : unit_keys; u.pad = 0;
+        u.req = r; u.key0 = k0; u.nkeys = q.N - k0 < unit_keys ? q.N - k0 : unit_keys;
+        u.cu = q.cu; u.n = q.n; u.unit0 = q.unit0;
       }
       q.nunits = nu - q.unit0;
+      for (int32_t i = q.unit0; i < nu; ++i) ctx->h_units[i].nunits = q.nunits;
       const int64_t full = (int64_t)c.n_layers * q.N;
       bound += (int64_t)c.n_kv_heads * (c.total_budget < full ? c.total_budget : full);
     }

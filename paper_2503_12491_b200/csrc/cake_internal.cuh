@@ -12,7 +12,9 @@
 namespace cake {
 
 constexpr int kMaxRows = 128;        // G * S_w rows handled per KV head
-constexpr int kSimtTileKeys = 64;    // keys per tile of the SIMT score kernels
+constexpr int kSimtMinUnit = 64;      // fewest keys of a score unit of the SIMT score kernels
+constexpr int kSimtMaxUnit = 1024;
+constexpr int64_t kMaxScoreElems = 64ll << 20;   // logits the SIMT kernels keep between their two steps (256 MB)
 constexpr int kSimtThreads = 256;
 constexpr int kBinBits = 12;         // survivor lists are sorted by the top bits of the indicator
 constexpr int kBins = 1 << kBinBits;
@@ -36,10 +38,13 @@ struct ReqInfo {
 
 // A run of consecutive keys of one request handled by one CTA of a score kernel.
 struct ScoreUnit {
+  int64_t cu;        // first token row of the request inside the packed K
   int32_t req;
   int32_t key0;
   int32_t nkeys;
-  int32_t pad;
+  int32_t n;         // non-window keys of the request
+  int32_t unit0;     // first unit of the request
+  int32_t nunits;    // units of the request
 };
 
 // One step of a CTA's program in the tensor-core score kernel: a run of consecutive
@@ -152,6 +157,10 @@ struct cake_ctx {
   int64_t bitmap_words;
   float* d_lse2;           // [max_requests][H_q][S_w] base-2 log-sum-exp of window rows
   float2* d_rowpart;       // [max_units][H_kv][R] (max, sum) partials of phase A
+  float* d_scores;         // SIMT path: logits between its two kernels
+  int64_t scores_elems;
+  uint32_t* d_simt_arrivals;   // [max_pairs] finished units of a (request, head) (zero at rest)
+  int32_t unit_keys;       // keys of a full score unit of the batch
   float* d_colpart[cake::kScoreDepth]; // partial (sum p*log2 p, sum var) of the column pass, likewise
   // ---- tensor-core score path ----
   bool use_tc;
@@ -198,6 +207,7 @@ namespace cake {
 void count_launch(int64_t n = 1);
 
 // score_simt.cu
+int32_t simt_tile_keys(int rows);     // keys per tile: score units are multiples of it
 int32_t launch_score_simt(cake_ctx* ctx, int32_t layer, const void* q_win, const void* k,
                           const float* lse, cudaStream_t st);
 // score_tc.cu

@@ -303,3 +303,20 @@ def test_lists_at_the_edges_of_tiles_and_runs(seq_lens, budget, pool):
             assert np.array_equal(got[g], want), (r, g)
     assert cake.status() == 0
     cake.destroy()
+
+
+@pytest.mark.parametrize("scores_mb", ["256", "0"])
+@pytest.mark.parametrize("dtype,hq,hkv,window,d,seq_lens", [
+    ("fp32", 4, 4, 16, 64, (1100, 129, 17)),         # 16 rows
+    ("fp32", 6, 2, 11, 128, (900, 64)),              # 33 rows, G = 3
+    ("bf16", 6, 2, 8, 128, (1025, 40)),              # 24 rows, which the tensor-core kernel does not take
+    ("fp32", 4, 1, 32, 128, (3000, 333)),            # 128 rows
+    ("fp32", 8, 1, 8, 64, (700,)),                   # 64 rows, G = 8
+])
+@pytest.mark.parametrize("lse", [False, True])
+def test_simt_scores_at_every_row_count(monkeypatch, scores_mb, dtype, hq, hkv, window, d, seq_lens, lse):
+    """Every tile shape of the SIMT kernels, units with ragged ends, and the logits in one piece or (no
+    more than one unit of 1024 keys at a time) slice by slice."""
+    monkeypatch.setenv("CAKE_SIMT_SCORES_MB", scores_mb)
+    kw = dict(n_q_heads=hq, n_kv_heads=hkv, window=window, head_dim=d, seq_lens=seq_lens, n_layers=1, total_budget=window + 60)
+    check_scores((fp32_case if dtype == "fp32" else bf16_case)(**kw), expect_tc=False, lse=lse)
