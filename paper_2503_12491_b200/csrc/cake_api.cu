@@ -395,10 +395,12 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   if (layer != ctx->n_ind || ctx->n_evicted != layer) return CAKE_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   const int par = layer & 1;
-  // the score kernel's outputs of this layer's place were last read by the pooling of layer -
-  // kScoreDepth; the rest of that layer's cascade works on its own data and may still be running
-  const int place = layer % kScoreDepth;
-  if (ctx->pool_recorded[place]) CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[place], 0));
+  // The score kernel's outputs of a layer's place were last read by the pooling of layer - kScoreDepth
+  // (the rest of that layer's cascade works on its own data and may still be running).  One wait serves
+  // this layer and the next kScoreWait - 1: the pooling stream runs in order.
+  const int place = layer % kScoreDepth, newest = layer + kScoreWait - 1 - kScoreDepth;
+  if (layer % kScoreWait == 0 && newest >= 0 && ctx->pool_recorded[newest % kScoreDepth])
+    CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[newest % kScoreDepth], 0));
   int32_t rc = ctx->use_tc ? launch_score_tc(ctx, layer, q_win, k, lse, st)
                            : launch_score_simt(ctx, layer, q_win, k, lse, st);
   if (rc != CAKE_OK) return rc;

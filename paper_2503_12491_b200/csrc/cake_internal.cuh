@@ -20,7 +20,9 @@ constexpr int kBinBits = 12;         // survivor lists are sorted by the top bit
 constexpr int kBins = 1 << kBinBits;
 constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling / scatter CTAs
 constexpr int kBitmapSmemWords = 48 * 1024;   // positions of up to 1.5 M tokens are ordered in shared memory
-constexpr int kScoreDepth = 4;        // layers whose score outputs may wait for their pooling
+constexpr int kScoreDepth = 8;        // layers whose score outputs may wait for their pooling
+constexpr int kScoreWait = 4;         // every so many layers the caller's stream waits for earlier pooling: an event
+                                      // wait between two score launches keeps the second from starting early
 constexpr int kScoreGroups = 3;      // statistics warp groups per CTA of the tensor-core score kernel
 constexpr int kScoreWarps = 4 * kScoreGroups;   // statistics warps: one column-pass partial each
 
