@@ -497,9 +497,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           tma_load_3d_hint(dst, &k_map, &S.full[s], 0, (int)(row0 + it * TILE), 0, pol);
         }
       }
-      // The next kernel of the stream may start once every CTA has issued its last loads; in launches
-      // too short for the cascade kernels beside them (one wave, column pass alone) once it is done with its
-      // statistics.  Earlier the next kernel's CTAs take the SMs that are left to those kernels: when they
+      // The next kernel of the stream may start once every CTA has issued its last loads; in shorter
+      // launches (one wave, column pass alone) once it is done with its statistics.  Earlier the next kernel's CTAs take the SMs that are left to those kernels: when they
       // could start with this kernel, layers of the 4K MHA and 32K GQA prompts took 10 % longer, and with the
       // last op 8 %; as it is, 1 to 7 % less than without an early start (1465 -> 1385 us at 32K GQA).
       if constexpr (!kDirect && !kEntropyB) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -828,10 +827,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         if constexpr (kDirect) {
           // One thread per row and group; every CTA adds in the same order.
           const int slot = kbs & 1, pair = op.req * P.Hkv + op.g;
+          const int s_lo = P.pair_aseg[pair];        // read before the wait
+          int s_hi = P.pair_aseg[pair + 1];
           if (ok) ok = mbar_wait(&S.parts[slot], (kbs >> 1) & 1, P.status, P.spin_limit);
+          if (!ok) s_hi = s_lo;
           ++kbs;
           float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-          const int s_lo = P.pair_aseg[pair], s_hi = ok ? P.pair_aseg[pair + 1] : s_lo;
           if (lane_row < P.rows) {
             for (int sg = s_lo; sg < s_hi; sg += 8) {
               float4 pv[8];
@@ -1117,7 +1118,7 @@ EncodeTiledFn encode_fn() {
 
 
 template <int G>
-cudaError_t launch_g(int device, bool entropy_b, bool copies, bool direct, int n_cta, cudaStream_t st, const CUtensorMap& qmap,
+cudaError_t launch_g(int device, bool entropy_b, bool copies, bool direct, bool early, int n_cta, cudaStream_t st, const CUtensorMap& qmap,
                      const CUtensorMap& kmap, const TcParams& P) {
   typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const TcParams);
   static const Kernel kernels[5] = {score_fused_kernel<G, false, false, false>, score_fused_kernel<G, false, false, true>,
@@ -1141,7 +1142,7 @@ cudaError_t launch_g(int device, bool entropy_b, bool copies, bool direct, int n
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, qmap, kmap, P);
 }
 
@@ -1556,11 +1557,15 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   }
   cudaError_t e;
   const bool eb = lse != nullptr;
+  // An early start takes SMs from the cascade kernels.  The column pass of a single wave is so short that
+  // these set the pace: it starts when the launch before it is done (32 layers of 16 heads and 12.7K keys:
+  // 730 us with an early start, 690 without).
+  const bool early = !(eb && ctx->n_tc_waves == 1);
   switch (G) {
-    case 1: e = launch_g<1>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    case 2: e = launch_g<2>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    case 4: e = launch_g<4>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    default: e = launch_g<8>(ctx->device, eb, P.reps > 1, ctx->tc_direct, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 1: e = launch_g<1>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 2: e = launch_g<2>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 4: e = launch_g<4>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    default: e = launch_g<8>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
   }
   count_launch();
   prof_end(ctx, sp, st);
