@@ -67,12 +67,13 @@ void free_ctx(cake_ctx* c) {
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
   cudaFree(c->d_scores); cudaFree(c->d_simt_arrivals);
   cudaFree(c->d_rowpart);
-  cudaFree(c->d_tc_tables); cudaFree(c->d_tc_sync);
+  cudaFree(c->d_tc_ops); cudaFree(c->d_tc_index); cudaFree(c->d_tc_sync);
   cudaFree(c->d_tc_rowpart); cudaFree(c->d_lse2_tc);
   cudaFree(c->d_dec_off); cudaFree(c->d_dec_packed_off); cudaFree(c->d_dec_score); cudaFree(c->d_dec_tmp); cudaFree(c->d_dec_pos);
   cudaFree(c->d_dec_order); cudaFree(c->d_dec_meta);
   if (c->h_budget_stage) cudaFreeHost(c->h_budget_stage);
-  if (c->h_tc_tables) cudaFreeHost(c->h_tc_tables);
+  if (c->h_tc_ops) cudaFreeHost(c->h_tc_ops);
+  if (c->h_tc_index) cudaFreeHost(c->h_tc_index);
   if (c->h_req) cudaFreeHost(c->h_req);
   if (c->h_units) cudaFreeHost(c->h_units);
   if (c->upload_done) cudaEventDestroy(c->upload_done);
@@ -242,17 +243,18 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     const int64_t segs = tc_max_segments(c, x->n_sm);
     if (x->use_tc && segs > ((int64_t)1 << 24)) { free_ctx(x); return CAKE_ERR_ARG; }
     x->max_tc_segs = (int32_t)segs;
-    x->max_tc_ops = (int32_t)(2 * segs);
-    x->max_tc_runs = tc_max_runs(c, x->max_tc_ops, x->n_sm);
+    x->max_tc_ops = (int32_t)(3 * segs + 8);
   }
   {
     const size_t a = (size_t)x->max_units * c.n_kv_heads, b = (size_t)x->max_tc_segs * kScoreWarps;
     for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_colpart[i], (a > b ? a : b) * G * 2) == cudaSuccess;
   }
   if (x->use_tc) {
-    const size_t tables = tc_tables_bytes((int)max_pairs, x->n_sm, x->max_tc_ops, x->max_tc_runs);
-    ok = ok && cudaMallocHost((void**)&x->h_tc_tables, tables) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_tc_tables, tables) == cudaSuccess;
+    const size_t n_index = 2 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
+    ok = ok && cudaMallocHost((void**)&x->h_tc_ops, sizeof(ScoreOp) * x->max_tc_ops) == cudaSuccess;
+    ok = ok && cudaMallocHost((void**)&x->h_tc_index, sizeof(int32_t) * n_index) == cudaSuccess;
+    ok = ok && dev_alloc(&x->d_tc_ops, x->max_tc_ops) == cudaSuccess;
+    ok = ok && dev_alloc(&x->d_tc_index, n_index) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_sync, 2 * (size_t)max_pairs) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_rowpart, (size_t)x->max_tc_segs * kScoreGroups * 128) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_lse2_tc, (size_t)max_pairs * 128) == cudaSuccess;
@@ -355,7 +357,12 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
     CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_units, ctx->h_units, sizeof(ScoreUnit) * nu,
                                   cudaMemcpyHostToDevice, st));
     if (ctx->use_tc && ctx->n_tc_ctas > 0) {
-      CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_tc_tables, ctx->h_tc_tables, ctx->tc_tables_used, cudaMemcpyHostToDevice, st));
+      const size_t n_index = 2 * (size_t)(n_req * c.n_kv_heads + 1) + 2 * (size_t)(ctx->n_sm + 1);
+      CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_tc_ops, ctx->h_tc_ops,
+                                    sizeof(ScoreOp) * (ctx->n_tc_ops_full + ctx->n_tc_ops_b),
+                                    cudaMemcpyHostToDevice, st));
+      CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_tc_index, ctx->h_tc_index, sizeof(int32_t) * n_index,
+                                    cudaMemcpyHostToDevice, st));
     }
     CAKE_CUDA_TRY(cudaEventRecord(ctx->upload_done, st));
     ctx->upload_pending = true;
@@ -756,7 +763,7 @@ int32_t cake_plan_info(const cake_ctx* ctx, int32_t* out8) {
   out8[3] = tc && ctx->n_tc_ctas > 0 ? ctx->tc_merge_ways : 0;
   out8[4] = tc ? ctx->n_tc_asegs : 0;
   out8[5] = tc ? ctx->n_tc_bsegs : 0;
-  out8[6] = tc ? ctx->n_tc_ops : 0;
+  out8[6] = tc ? ctx->n_tc_ops_full : 0;
   out8[7] = ctx->n_sm - ctx->n_sm_score;
   return CAKE_OK;
 }

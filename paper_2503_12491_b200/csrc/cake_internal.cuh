@@ -65,13 +65,6 @@ struct ScoreOp {
   int32_t pad;
 };
 
-// A run of consecutive tiles of one op: what a CTA takes next.
-struct ScoreRun {
-  int32_t tile0;     // first tile, counted inside the op
-  uint16_t op;       // the op, counted inside the CTA's program
-  uint16_t count;    // tiles
-};
-
 // Retained set of one (request, layer, head) list, whose entries (ordered key, position) are stored by
 // bucket.  The first three fields are derived from the list and the budgets of the moment when the
 // retained set is read out (sorted_positions).
@@ -81,8 +74,6 @@ struct ListState {
   int32_t pos_cut;       //   or key == thr_key and position <= pos_cut
   int32_t kept;          // budget the list arrived with: entries beyond it are not stored
 };
-
-constexpr int kIndexPairs = 3, kIndexCtas = 2;       // parts of the index block of either length
 
 struct LayerPtrs {
   const void* k[CAKE_MAX_LAYERS];
@@ -196,17 +187,15 @@ struct cake_ctx {
   int64_t wait_limit_cycles;      // bound of every device-side wait (0 = the default, about 2 s)
   int32_t debug_epoch_skew;       // test hook: added to the launch count the cross-CTA waits expect
   int32_t n_tc_asegs, n_tc_bsegs;          // pass-A / pass-B segments per layer
-  int32_t n_tc_ops, max_tc_ops;
+  int32_t n_tc_ops_full, n_tc_ops_b, max_tc_ops;
   uint32_t tc_epoch;              // both-pass launches since cake_begin
-  // Tables of the current batch, one block (pinned / device): index | ops | runs.  index, P = n_req * H_kv:
-  //   pair_aseg [P+1] | pair_bseg [P+1] | group_begin [P+1]
-  //   | cta_op [n_sm+1] | cta_run [n_sm+1].  No runs: every op is taken whole, in the order of the ops.
-  uint8_t *h_tc_tables, *d_tc_tables;
-  size_t tc_tables_used;
-  int32_t n_tc_runs, max_tc_runs, n_tc_groups;
-  cake::ScoreOp *h_tc_ops, *d_tc_ops;       // inside the block
-  cake::ScoreRun *h_tc_runs, *d_tc_runs;
-  int32_t *h_tc_index, *d_tc_index;
+  cake::ScoreOp* h_tc_ops;        // pinned: [both-pass programs][pass-B-only programs]
+  cake::ScoreOp* d_tc_ops;
+  // pinned / device index block of the current batch, P = n_req * H_kv pairs:
+  //   pair_aseg [P+1] | pair_bseg [P+1] | cta_op of the both-pass programs [n_sm+1]
+  //   | cta_op of the pass-B-only programs [n_sm+1]
+  int32_t* h_tc_index;
+  int32_t* d_tc_index;
   uint32_t* d_tc_sync;            // [max_pairs] delivered partial rows, then [max_pairs] merged rows
   int tc_merge_ways;              // rows the merger warp handles side by side (a power of two up to 32), chosen with the plan
   bool tc_direct;                 // every CTA merges the denominators of its own pass-B ops (single-wave plans)
@@ -226,8 +215,6 @@ int32_t launch_score_simt(cake_ctx* ctx, int32_t layer, const void* q_win, const
 // score_tc.cu
 bool tc_path_supported(const cake_config& c);
 int64_t tc_max_segments(const cake_config& c, int n_sm);
-int32_t tc_max_runs(const cake_config& c, int32_t max_ops, int n_sm);
-size_t tc_tables_bytes(int max_pairs, int n_sm, int32_t max_ops, int32_t max_runs);
 int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req);
 int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_req, const int64_t* cu,
                       int32_t* info8);

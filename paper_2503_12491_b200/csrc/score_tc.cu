@@ -14,15 +14,15 @@
 // never reaches HBM.
 //
 // Schedule.  The (request, KV head) pairs of a layer are grouped into waves of at
-// most kWaveBytes of K.  Every CTA owns the same slice of a wave in both passes.  Its pass A runs
-// kLagTiles ahead of the end of the wave that its pass B is in, and the two take turns of kStepTiles,
+// most kWaveBytes of K.  Every CTA owns the same slice of a wave in both passes and runs
+//     A(wave 0), A(wave 1), B(wave 0), A(wave 2), B(wave 1), ... , B(last wave)
 // so pass B re-reads a wave's K from L2 shortly after pass A brought it in, and DRAM
 // sees K once.  Pass B of a pair needs the pair's softmax denominators, i.e. every
 // CTA's pass-A partial rows.  The merge is spread over the grid by rows: the merger warp
 // of CTA (pair * rows + r) % grid waits until all partials of the pair are delivered, loads
-// row r's partials in a single round trip, merges them and counts the row as done.  The lag
-// puts kLagTiles of pass A between a wave's pass A and its pass B, so pass B's wait on that count is
-// normally already satisfied.
+// row r's partials in a single round trip, merges them and counts the row as done.  The pass A
+// of the next wave sits between a pair's pass A and its pass B, so pass B's wait on
+// that count is normally already satisfied.
 //
 // Warp roles in a CTA of 512 threads: warps 0..11 are "statistics" warps in three groups of
 // four (a group takes every third accumulator tile, a warp owns 32 of its TMEM lanes, works
@@ -62,17 +62,11 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kChunkSumMax = 65536.f;   // a pass-A chunk sum beyond this moves the row's reference
 constexpr int64_t kWaveBytes = 32ll << 20;
 constexpr int kDirectSegs = 40;       // segments of a pair up to which every CTA merges its rows for itself
-constexpr int kLagTiles = 24;         // pass-A tiles of later waves that go before a wave's first pass-B tile
-constexpr int kStepTiles = 16;        // tiles of either pass between changes to the other
-constexpr int kRunsPerCta = 300;      // ... or as many as make this many runs, if that is more
+constexpr int kWaveDepth = 1;         // pass B of a wave follows pass A of the wave this far ahead
 
 struct TcParams {
   const ScoreOp* ops;
   const int32_t* cta_op;        // [n_cta + 1]
-  const ScoreRun* runs;
-  const int32_t* cta_run;       // [n_cta + 1]
-  const int32_t* group_begin;   // [n_groups + 1] first pair of every merge group
-  int n_groups;
   const ReqInfo* reqs;
   const int32_t* pair_aseg;     // [pairs + 1] pass-A segment ranges per pair
   uint32_t* pair_cnt;           // [pairs] delivered pass-A partials (monotonic over layers)
@@ -330,15 +324,12 @@ struct Smem {
   float4* xrow;        // [2][NWG][128] partial rows of a group: copies of a row in pass A, then (direct merge) the
                        //   group's share of a pair's partials for the current / next pass-B op
   ScoreOp* ops;        // [kSmemOps] the first ops of this CTA's program
-  ScoreRun* runs;      // [kSmemRuns] its first runs
 };
 
 constexpr size_t kQBytes = 2 * SLAB_BYTES;
-constexpr int kSmemOps = 128;        // ops and runs of a CTA's program kept in shared memory
-constexpr int kSmemRuns = 384;
+constexpr int kSmemOps = 128;        // ops of a CTA's program kept in shared memory
 constexpr size_t kSmemBytes = 1024 /*align*/ + 2 * kQBytes + (size_t)STAGES * 2 * SLAB_BYTES + 320 +
-                              128 + 3 * kExtBytes + 2 * NWG * 128 * sizeof(float4) + kSmemOps * sizeof(ScoreOp) +
-                              kSmemRuns * sizeof(ScoreRun) + 64;
+                              128 + 3 * kExtBytes + 2 * NWG * 128 * sizeof(float4) + kSmemOps * sizeof(ScoreOp) + 64;
 static_assert(kSmemBytes <= 227 * 1024, "a CTA has 227 KB of shared memory");
 
 __device__ __forceinline__ Smem carve(uint8_t* base) {
@@ -362,8 +353,7 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   s.ext_a = p;                p += kExtBytes;
   s.ext_b = p;                p += 2 * kExtBytes;
   s.xrow = (float4*)p;        p += 2 * NWG * 128 * sizeof(float4);
-  s.ops = (ScoreOp*)p;        p += kSmemOps * sizeof(ScoreOp);
-  s.runs = (ScoreRun*)p;
+  s.ops = (ScoreOp*)p;
   return s;
 }
 
@@ -414,32 +404,11 @@ __device__ __forceinline__ void put_ext_row(uint8_t* ext, int r, int rows, float
   *reinterpret_cast<uint2*>(ext + ext_row_offset(r)) = r < rows ? make_uint2(w0, w1) : make_uint2(0u, 0u);
 }
 
-// Which of the two query buffers an op uses; the TMA and the MMA warp walk the same runs and agree.  A
-// column-pass op holds its buffer to its end.  A row-pass op needs one only until its queries are in tensor
-// memory: beside a column-pass op it takes the other buffer, and the next column-pass op has that one
-// after it, so that its queries are there before its predecessor has ended.
-struct QBuffers {
-  uint32_t uses[2] = {0, 0};
-  int last = 1, b_buf = 0, a_buf = 0;
-  bool had_b = false;
-  __device__ __forceinline__ int of_run(int phase, bool first) {
-    if (first) {
-      if (phase) { b_buf = had_b ? b_buf ^ 1 : last ^ 1; had_b = true; last = b_buf; }
-      else { a_buf = had_b ? b_buf ^ 1 : last ^ 1; last = a_buf; }
-    }
-    return phase ? b_buf : a_buf;
-  }
-};
-
 // ------------------------------------------------------------------ kernel
 // kCopies: the window has 32 or 64 rows and a pass-A tile holds them 4 or 2 times, so that every
 // statistics warp has rows to work on: copy c sums the c-th part of a key tile's columns.
-// kPlan, how a CTA's program is ordered (see tc_build_plan): kRuns by the runs of tiles in its table; kWhole
-// by whole ops, in the order of the op table, so that nothing is carried from one run of an op to its next
-// (with run tables and carried sums the whole-op plans were 2 to 6 % slower); kDirect as kWhole, with one
-// wave, and every CTA merges the partial rows of its own pass-B ops.
-enum { kRuns, kWhole, kDirectMerge };
-template <int G, bool kEntropyB, bool kCopies, int kPlan>
+// kDirect: one wave; every CTA merges the partial rows of its own pass-B ops (see tc_build_plan).
+template <int G, bool kEntropyB, bool kCopies, bool kDirect>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                    const TcParams P) {
@@ -449,9 +418,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   const int n_slab = P.d / 64;
   const uint32_t stage_bytes = (uint32_t)(TILE * P.d * 2);
   const int rows_pad = (P.rows + 15) & ~15;
-  constexpr bool kDirect = kPlan == kDirectMerge, kOps = kPlan != kRuns;
   const int op_lo = P.cta_op[blockIdx.x], op_hi = P.cta_op[blockIdx.x + 1];
-  const int run_lo = kOps ? op_lo : P.cta_run[blockIdx.x], run_hi = kOps ? op_hi : P.cta_run[blockIdx.x + 1];
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) { mbar_init(&S.full[i], 1); mbar_init(&S.empty[i], 1); }
@@ -461,38 +428,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     for (int i = 0; i < NSTATW; ++i) S.a_done[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // The program of this CTA: a global read per op would put an L2 round trip on every op.  It is a list of
-  // ops (a pass over consecutive keys of a pair) and the order in which their tiles are taken: runs of
-  // consecutive tiles, the ops of either pass in order, the two passes in turn.  Loads first, so that the
-  // two tables come in one round trip.
-  static_assert(kSmemRuns <= TC_THREADS && kSmemOps <= TC_THREADS, "a thread loads an op and a run");
-  ScoreOp my_op;
-  ScoreRun my_run;
-  const bool has_op = (int)threadIdx.x < min(op_hi - op_lo, kSmemOps);
-  const bool has_run = !kOps && (int)threadIdx.x < min(run_hi - run_lo, kSmemRuns);
-  if (has_run) my_run = P.runs[run_lo + threadIdx.x];
-  if (has_op) my_op = P.ops[op_lo + threadIdx.x];
-  if (has_run) S.runs[threadIdx.x] = my_run;
-  if (has_op) S.ops[threadIdx.x] = my_op;
+  // the program of this CTA: a global read per op would put an L2 round trip on every op
+  for (int i = threadIdx.x; i < min(op_hi - op_lo, kSmemOps); i += TC_THREADS) S.ops[i] = P.ops[op_lo + i];
   auto get_op = [&](int oi) -> ScoreOp {
     return oi - op_lo < kSmemOps ? S.ops[oi - op_lo] : P.ops[oi];
-  };
-  auto tiles_of = [](const ScoreOp& op) { return (op.nkeys + TILE - 1) / TILE; };
-  // The i-th step of the program: tiles [tile0, tile1) of an op.
-  struct Step { ScoreOp op; int tile0, tile1; bool first, last; };
-  auto get_step = [&](int i) -> Step {
-    Step u;
-    if constexpr (kOps) {
-      u.op = get_op(i);
-      u.tile0 = 0; u.tile1 = tiles_of(u.op); u.first = u.last = true;
-      if (kEntropyB && !u.op.phase) u.tile1 = 0;             // the column pass alone
-    } else {
-      const ScoreRun run = i - run_lo < kSmemRuns ? S.runs[i - run_lo] : P.runs[i];
-      u.op = get_op(op_lo + run.op);
-      u.tile0 = run.tile0; u.tile1 = run.tile0 + run.count;
-      u.first = u.tile0 == 0; u.last = u.tile1 == tiles_of(u.op);
-    }
-    return u;
   };
   // rows of the query tiles that TMA never writes must read as zero
   for (int i = threadIdx.x; i < (int)(2 * kQBytes / 16); i += TC_THREADS)
@@ -529,29 +468,26 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       __syncwarp();
       // pass A's tiles are read again by pass B: keep them in L2; pass B's read is the last
       const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
-      uint32_t t = 0;
-      QBuffers qbuf;
+      uint32_t t = 0, qn = 0;
       bool ok = true;
-      for (int ri = run_lo; ri < run_hi && ok; ++ri) {
-        const Step u = get_step(ri);
-        const ScoreOp& op = u.op;
-        if (u.tile1 <= u.tile0) continue;
+      for (int oi = op_lo; oi < op_hi && ok; ++oi) {
+        const ScoreOp op = get_op(oi);
+        if (op.nkeys <= 0) continue;
         const uint64_t pol = (op.phase || !P.pair_done) ? drop : keep;
-        const int qb = qbuf.of_run(op.phase, u.first);
-        if (u.first) {
-          // the buffer's previous queries must have been used
-          ok = mbar_wait(&S.q_empty[qb], (qbuf.uses[qb] & 1) ^ 1, P.status, P.spin_limit);
-          ++qbuf.uses[qb];
-          if (!ok) break;
-          const int reps = kCopies && !op.phase ? P.reps : 1;
-          mbar_expect_tx(&S.q_full[qb], (uint32_t)(reps * P.rows * P.d * 2));
-          for (int rp = 0; rp < reps; ++rp)
-            for (int sl = 0; sl < n_slab; ++sl)
-              tma_load_4d(S.q + qb * kQBytes + sl * SLAB_BYTES + rp * P.rows * 128, &q_map, &S.q_full[qb], sl * 64, op.g * G,
-                          0, op.req);
-        }
+        const int qb = qn & 1;
+        // the MMAs of the op that used this query buffer two ops ago must be done
+        ok = mbar_wait(&S.q_empty[qb], ((qn >> 1) & 1) ^ 1, P.status, P.spin_limit);
+        ++qn;
+        if (!ok) break;
+        const int reps = kCopies && !op.phase ? P.reps : 1;
+        mbar_expect_tx(&S.q_full[qb], (uint32_t)(reps * P.rows * P.d * 2));
+        for (int rp = 0; rp < reps; ++rp)
+          for (int sl = 0; sl < n_slab; ++sl)
+            tma_load_4d(S.q + qb * kQBytes + sl * SLAB_BYTES + rp * P.rows * 128, &q_map, &S.q_full[qb], sl * 64, op.g * G,
+                        0, op.req);
         const int64_t row0 = op.base + op.key0;
-        for (int it = u.tile0; it < u.tile1; ++it, ++t) {
+        const int ntiles = (op.nkeys + TILE - 1) / TILE;
+        for (int it = 0; it < ntiles; ++it, ++t) {
           const int s = t % STAGES;
           ok = mbar_wait(&S.empty[s], ((t / STAGES) & 1) ^ 1, P.status, P.spin_limit);
           if (!ok) break;
@@ -570,51 +506,47 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const uint32_t issued = t;
       for (uint32_t u = issued > STAGES ? issued - STAGES : 0; u < issued; ++u)
         mbar_wait(&S.full[u % STAGES], (u / STAGES) & 1, P.status, P.spin_limit);
-      for (int u = 0; u < 2; ++u)
-        if (qbuf.uses[u] > 0) mbar_wait(&S.q_full[u], (qbuf.uses[u] - 1) & 1, P.status, P.spin_limit);
+      for (uint32_t u = qn > 2 ? qn - 2 : 0; u < qn; ++u)
+        mbar_wait(&S.q_full[u & 1], (u >> 1) & 1, P.status, P.spin_limit);
     }
   } else if (warp == WARP_MMA) {
     // ------------------------------------------------ MMA issuer (converged warp, elected lane issues)
     {
-      uint32_t t = 0, kbm = 0;
-      QBuffers qbuf;
+      uint32_t t = 0, qn = 0, kbm = 0;
       const uint32_t k_lo0 = (smem_u32(S.k) & 0x3FFFFu) >> 4;
       const uint32_t ext_a_lo = ((smem_u32(S.ext_a) & 0x3FFFFu) >> 4) | kExtDescLoLbo;
       bool ok = true;
-      for (int ri = run_lo; ri < run_hi && ok; ++ri) {
-        const Step u = get_step(ri);
-        const ScoreOp& op = u.op;
-        if (u.tile1 <= u.tile0) continue;
+      for (int oi = op_lo; oi < op_hi && ok; ++oi) {
+        const ScoreOp op = get_op(oi);
+        if (op.nkeys <= 0) continue;
         const uint32_t idesc = op.phase ? instr_desc(128, rows_pad) : instr_desc(128, TILE);
         const int eslot = kbm & 1;
         const uint32_t ext_b_lo = ((smem_u32(S.ext_b + eslot * kExtBytes) & 0x3FFFFu) >> 4) | kExtDescLoLbo;
-        const int qb = qbuf.of_run(op.phase, u.first);
+        const int qb = qn & 1;
+        ok = mbar_wait(&S.q_full[qb], (qn >> 1) & 1, P.status, P.spin_limit);
+        ++qn;
+        if (!ok) break;
         const uint32_t qaddr = smem_u32(S.q + qb * kQBytes);
         const uint32_t q_lo = (qaddr & 0x3FFFFu) >> 4;      // address field of the descriptors
         const uint32_t tmem_q = tmem_base + (uint32_t)TMEM_Q_COL;
-        if (u.first) {
-          ok = mbar_wait(&S.q_full[qb], qbuf.uses[qb] & 1, P.status, P.spin_limit);
-          ++qbuf.uses[qb];
-          if (!ok) break;
-          if (!op.phase) {
-            // pass A multiplies every key tile by the same queries: hold them in tensor memory, so
-            // that an MMA reads only the key tile from shared memory.  The copies run in issue
-            // order behind the previous op's MMAs and ahead of this op's; the buffer is free again
-            // once they have run.
-            tc_fence_after();
-            for (int sl = 0; sl < n_slab; ++sl)
+        if (!op.phase) {
+          // pass A multiplies every key tile by the same queries: hold them in tensor memory, so
+          // that an MMA reads only the key tile from shared memory.  The copies run in issue
+          // order behind the previous op's MMAs and ahead of this op's.
+          tc_fence_after();
+          for (int sl = 0; sl < n_slab; ++sl)
 #pragma unroll
-              for (int ks = 0; ks < 4; ++ks)
-                tmem_cp_128x256b(tmem_q + (uint32_t)((sl * 4 + ks) * 8),
-                                 smem_desc(qaddr + sl * SLAB_BYTES + ks * 32));
-            umma_commit(&S.q_empty[qb]);
-          } else {
-            // the rows' -lse/scale operand of this op (written by the denominator warp)
-            ok = mbar_wait(&S.lse_full[eslot], (kbm >> 1) & 1, P.status, P.spin_limit);
-            if (!ok) break;
-          }
+            for (int ks = 0; ks < 4; ++ks)
+              tmem_cp_128x256b(tmem_q + (uint32_t)((sl * 4 + ks) * 8),
+                               smem_desc(qaddr + sl * SLAB_BYTES + ks * 32));
         }
-        for (int it = u.tile0; it < u.tile1; ++it, ++t) {
+        if (op.phase) {
+          // the rows' -lse/scale operand of this op (written by the denominator warp)
+          ok = mbar_wait(&S.lse_full[eslot], (kbm >> 1) & 1, P.status, P.spin_limit);
+          if (!ok) break;
+        }
+        const int ntiles = (op.nkeys + TILE - 1) / TILE;
+        for (int it = 0; it < ntiles; ++it, ++t) {
           const int s = t % STAGES, b = t % NBUF;
           ok = mbar_wait(&S.acc_empty[b], ((t / NBUF) & 1) ^ 1, P.status, P.spin_limit);
           if (!ok) break;
@@ -654,8 +586,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           umma_commit(&S.empty[s]);
           umma_commit(&S.acc_full[b]);
         }
-        if (op.phase && u.last) {
-          umma_commit(&S.q_empty[qb]);       // query buffer free once every MMA of the op has run
+        umma_commit(&S.q_empty[qb]);     // query buffer free once every MMA of the op has run
+        if (op.phase) {
           umma_commit(&S.lse_free[eslot]);   // and so is the op's -lse/scale operand
           ++kbm;
         }
@@ -692,13 +624,13 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // nothing to merge here: the statistics warps do it
       } else if (P.merge_ways > 1) {
         // Short pairs (a ragged batch, MHA): a wave holds several pairs whose rows have few
-        // partials each, so the rows of up to `ways` (2 to 32) consecutive pairs of a wave are merged side
-        // by side, by 32 / ways lanes each, and the wave's denominators are ready that much sooner.
+        // partials each, so the rows of `ways` (2 to 32) consecutive pairs are merged side by side,
+        // by 32 / ways lanes each, and the wave's denominators are ready that much sooner.
         const int ways = P.merge_ways, lpr = 32 / ways;         // lanes per row
         const int sub = lane / lpr, l8 = lane % lpr;
-        for (int gi = 0; gi < P.n_groups && ok; ++gi) {
-          const int pair = P.group_begin[gi] + sub;
-          const bool have = pair < P.group_begin[gi + 1];
+        for (int p0 = 0; p0 < P.n_pairs && ok; p0 += ways) {
+          const int pair = p0 + sub;
+          const bool have = pair < P.n_pairs;
           const int s_lo = have ? P.pair_aseg[pair] * NWG : 0, s_hi = have ? P.pair_aseg[pair + 1] * NWG : 0;
           const int r0 = have ? (int)((blockIdx.x + gridDim.x - (unsigned)(((long long)pair * P.rows) % gridDim.x)) % gridDim.x)
                               : P.rows;
@@ -884,19 +816,15 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const int i_row = (kCopies ? lane_row - copy * P.rows : lane_row) / G;
     const int c_lo = kCopies ? copy * (TILE / P.reps) : 0, c_hi = kCopies ? c_lo + TILE / P.reps : TILE;
     bool ok = true;
-    // statistics of the op of either pass that is under way
-    float m = -CUDART_INF_F, z = 0.f, zwin = 0.f, w = 0.f;     // pass A: of this lane's row
-    float col_v = 0.f, col_h = 0.f;                            // pass B: of head `lane`, over the warp's keys so far
-    for (int ri = run_lo; ri < run_hi; ++ri) {
-      const Step u = get_step(ri);
-      const ScoreOp& op = u.op;
-      if (u.tile1 <= u.tile0) continue;
-      const int tile1 = u.tile1;
-      const int it0 = u.tile0 + (int)((wg + NWG - tmod) % NWG);     // the group's first tile of the run
-      tmod = (tmod + (uint32_t)(u.tile1 - u.tile0)) % NWG;
+    for (int oi = op_lo; oi < op_hi; ++oi) {
+      const ScoreOp op = get_op(oi);
+      if (op.nkeys <= 0) continue;
+      const int ntiles = (op.nkeys + TILE - 1) / TILE;
+      const int it0 = (int)((wg + NWG - tmod) % NWG);            // the group's first tile of the op
+      tmod = (tmod + (uint32_t)ntiles) % NWG;
       if (op.phase) {
         // ---------------- pass B: thread = key, columns = rows r' = i*G + h
-        if (kDirect) {
+        if constexpr (kDirect) {
           // One thread per row and group; every CTA adds in the same order.
           const int slot = kbs & 1, pair = op.req * P.Hkv + op.g;
           const int s_lo = P.pair_aseg[pair];        // read before the wait
@@ -934,11 +862,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             if (lane == 0) mbar_arrive(&S.lse_full[slot]);
           }
         }
-        float vacc[G], hs[G];                        // of this lane's keys in the run
+        float vacc[G], hs[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) { vacc[h] = 0.f; hs[h] = 0.f; }
         const float inv_sw = 1.f / (float)P.Sw, inv_g = 1.f / (float)G;
-        for (int it = it0; it < tile1; it += NWG) {
+        for (int it = it0; it < ntiles; it += NWG) {
           if (ok) ok = mbar_wait(my_full, fpar, P.status, P.spin_limit);
           fpar ^= 1u;
           if (!ok) continue;
@@ -1022,9 +950,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             P.raw[op.base + j] = combine_indicator(P.ind_mode, P.gamma, mean, var, (float)P.Sw);
           }
         }
-        // Fixed-order reduction over the warp's keys, at the end of every run: what is carried to the op's
-        // next run is one sum per lane, not G of them (16 registers less beside pass A's).
-        float run_v = 0.f, run_h = 0.f;
+        // fixed-order reduction over the warp's keys
 #pragma unroll
         for (int h = 0; h < G; ++h) {
           float x = vacc[h], y = hs[h];
@@ -1033,20 +959,17 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             x += __shfl_xor_sync(0xffffffffu, x, o);
             if (kEntropyB) y += __shfl_xor_sync(0xffffffffu, y, o);
           }
-          if (lane == h) { run_v = x; run_h = y; }
-        }
-        col_v = kOps || u.first ? run_v : col_v + run_v;
-        if (kEntropyB) col_h = kOps || u.first ? run_h : col_h + run_h;
-        if ((kOps || u.last) && lane < G) {
-          float* dst = P.colpart + (((size_t)op.seg * NSTATW + warp) * G + lane) * 2;
-          dst[0] = col_h;
-          dst[1] = col_v;
+          if (lane == h) {
+            float* dst = P.colpart + (((size_t)op.seg * NSTATW + warp) * G + h) * 2;
+            dst[0] = y;
+            dst[1] = x;
+          }
         }
       } else {
         // ---------------- pass A: thread = window row r' = i*G + h, columns = keys
-        const int last_key = op.n + i_row;             // last key this row may attend to
-        if (kOps || u.first) { m = -CUDART_INF_F; z = 0.f; zwin = 0.f; w = 0.f; }
-        for (int it = it0; it < tile1; it += NWG) {
+        const int last = op.n + i_row;                 // last key this row may attend to
+        float m = -CUDART_INF_F, z = 0.f, zwin = 0.f, w = 0.f;
+        for (int it = it0; it < ntiles; it += NWG) {
           if (ok) ok = mbar_wait(my_full, fpar, P.status, P.spin_limit);
           fpar ^= 1u;
           if (!ok) continue;
@@ -1115,7 +1038,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 #pragma unroll
               for (int e = 0; e < 32; ++e) {
                 const int j = key0 + c0 + e;
-                const bool vis = (it * TILE + c0 + e < op.nkeys) && j <= last_key;
+                const bool vis = (it * TILE + c0 + e < op.nkeys) && j <= last;
                 cm = vis ? fmaxf(cm, __uint_as_float(r[e])) : cm;
               }
               if (cm != -CUDART_INF_F) {
@@ -1131,7 +1054,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
                   const int j = key0 + c0 + e;
-                  const bool vis = (it * TILE + c0 + e < op.nkeys) && j <= last_key;
+                  const bool vis = (it * TILE + c0 + e < op.nkeys) && j <= last;
                   const bool obs = j < op.n;
                   const float tt = fmaf(__uint_as_float(r[e]), P.scale2, -m);
                   const float ee = vis ? ex2(tt) : 0.f;
@@ -1143,7 +1066,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
           }
         }
-        if (!kOps && !u.last) continue;
         // Deliver this warp's 32 partial rows of the segment.  Making them visible to the other
         // CTAs takes a fence of a few thousand cycles; the merger warp pays it once per op for all
         // twelve warps, which only tell it, inside the CTA, that their rows are written.
@@ -1196,13 +1118,12 @@ EncodeTiledFn encode_fn() {
 
 
 template <int G>
-cudaError_t launch_g(int device, bool entropy_b, bool copies, int plan, bool early, int n_cta, cudaStream_t st, const CUtensorMap& qmap,
+cudaError_t launch_g(int device, bool entropy_b, bool copies, bool direct, bool early, int n_cta, cudaStream_t st, const CUtensorMap& qmap,
                      const CUtensorMap& kmap, const TcParams& P) {
   typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const TcParams);
-  static const Kernel kernels[7] = {score_fused_kernel<G, false, false, kRuns>, score_fused_kernel<G, false, false, kWhole>,
-                                    score_fused_kernel<G, false, false, kDirectMerge>, score_fused_kernel<G, false, true, kRuns>,
-                                    score_fused_kernel<G, false, true, kWhole>, score_fused_kernel<G, false, true, kDirectMerge>,
-                                    score_fused_kernel<G, true, false, kWhole>};
+  static const Kernel kernels[5] = {score_fused_kernel<G, false, false, false>, score_fused_kernel<G, false, false, true>,
+                                    score_fused_kernel<G, false, true, false>, score_fused_kernel<G, false, true, true>,
+                                    score_fused_kernel<G, true, false, false>};
   static PerDeviceOnce attr;
   if (attr.need(device)) {
     for (Kernel k : kernels) {
@@ -1211,7 +1132,7 @@ cudaError_t launch_g(int device, bool entropy_b, bool copies, int plan, bool ear
     }
     attr.mark(device);
   }
-  const Kernel k = kernels[entropy_b ? 6 : (copies ? 3 : 0) + plan];
+  const Kernel k = kernels[entropy_b ? 4 : (copies ? 2 : 0) + (direct ? 1 : 0)];
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_cta, 1, 1);
   cfg.blockDim = dim3(TC_THREADS, 1, 1);
@@ -1231,10 +1152,11 @@ int tc_reps(int rows) { return rows == 32 ? 4 : rows == 64 ? 2 : 1; }
 // Cuts the `tiles` tiles of one (request, head) pair, which start at flat tile index `flat`
 // of a wave of `W` tiles shared by `n_cta` CTAs (slot c owns flat tiles
 // [c*W/n_cta, (c+1)*W/n_cta)), into per-slot segments; slot c belongs to CTA (c+rot)%n_cta.
-struct CutOp { ScoreOp op; int32_t cta, wave; };
-void cut_pair(std::vector<CutOp>& ops, int wave, int rot, int n_cta, int64_t W, int64_t flat,
+// With `split`, a slot's segment of two or more tiles becomes two ops (pad = 1: first half,
+// pad = 2: second half) that the program builder may place apart.
+void cut_pair(std::vector<std::vector<ScoreOp>>& per_cta, int rot, int n_cta, int64_t W, int64_t flat,
               int tiles, int keys, int req, int g, int phase, int32_t& seg_counter, int64_t base,
-              int n_obs) {
+              int n_obs, bool split = false) {
   int t0 = 0;
   while (t0 < tiles) {
     const int64_t f = flat + t0;
@@ -1243,14 +1165,20 @@ void cut_pair(std::vector<CutOp>& ops, int wave, int rot, int n_cta, int64_t W, 
     while (c > 0 && (int64_t)c * W / n_cta > f) --c;
     const int64_t share_end = (int64_t)(c + 1) * W / n_cta;
     const int t1 = (int)((share_end - flat) < tiles ? (share_end - flat) : tiles);
-    ScoreOp op;
-    op.base = base; op.n = n_obs; op.pad = 0;
-    op.req = req; op.g = g; op.key0 = t0 * TILE;
-    const int kend = t1 * TILE < keys ? t1 * TILE : keys;
-    op.nkeys = kend - t0 * TILE;
-    op.phase = phase;
-    op.seg = seg_counter++;
-    ops.push_back(CutOp{op, (c + rot) % n_cta, wave});
+    const int parts = (split && t1 - t0 >= 2) ? 2 : 1;
+    const int tm = t0 + (t1 - t0 + 1) / 2;
+    for (int part = 0; part < parts; ++part) {
+      const int a = part == 0 ? t0 : tm, b = (parts == 2 && part == 0) ? tm : t1;
+      ScoreOp op;
+      op.base = base; op.n = n_obs;
+      op.pad = parts == 2 ? part + 1 : 0;
+      op.req = req; op.g = g; op.key0 = a * TILE;
+      const int kend = b * TILE < keys ? b * TILE : keys;
+      op.nkeys = kend - a * TILE;
+      op.phase = phase;
+      op.seg = seg_counter++;
+      per_cta[(c + rot) % n_cta].push_back(op);
+    }
     t0 = t1;
   }
 }
@@ -1291,20 +1219,7 @@ int64_t tc_max_segments(const cake_config& c, int n_sm) {
   const int64_t bytes = (int64_t)c.n_kv_heads * c.max_total_tokens * c.head_dim * 2;
   int64_t waves = 2 * (bytes / kWaveBytes) + 2;
   if (waves > pairs) waves = pairs;
-  return pairs + waves * n_sm;
-}
-
-// Upper bound on the runs of a batch: every op ends a run and may cut one of the other pass,
-// a program changes between the passes at most 2 * kRunsPerCta times, and a run has at most kMaxRun tiles.
-constexpr int kMaxRun = 0x7FFF;
-int32_t tc_max_runs(const cake_config& c, int32_t max_ops, int n_sm) {
-  return 2 * max_ops + n_sm * (2 * kRunsPerCta + 64) + (int32_t)(4 * (c.max_total_tokens * c.n_kv_heads / TILE / kMaxRun + 1));
-}
-
-// The tables of a batch are one block: index | ops | runs.
-size_t tc_tables_bytes(int max_pairs, int n_sm, int32_t max_ops, int32_t max_runs) {
-  return ((kIndexPairs * (size_t)(max_pairs + 1) + kIndexCtas * (size_t)(n_sm + 1) + 3) / 4 * 4) * sizeof(int32_t) +
-         (size_t)max_ops * sizeof(ScoreOp) + (size_t)max_runs * sizeof(ScoreRun);
+  return pairs + (waves + 2) * n_sm;          // + the two waves whose ops are halved
 }
 
 // Builds the per-CTA programs of the batch in ctx->h_req[0..n_req): `full` = both passes
@@ -1318,8 +1233,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
   for (int r = 0; r < n_req; ++r) tilesA_total += (int64_t)Hkv * ((ctx->h_req[r].N + TILE - 1) / TILE);
   int n_cta = (int)(tilesA_total < ctx->n_sm_score ? tilesA_total : ctx->n_sm_score);
   ctx->n_tc_ctas = n_cta;
-  ctx->n_tc_ops = ctx->n_tc_runs = 0;
-  ctx->tc_tables_used = 0;
+  ctx->n_tc_ops_full = ctx->n_tc_ops_b = 0;
   ctx->n_tc_asegs = ctx->n_tc_bsegs = 0;
   ctx->n_tc_waves = 0;
   if (n_cta == 0) return CAKE_OK;
@@ -1346,24 +1260,27 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     n_cta = best_n;
     ctx->n_tc_ctas = n_cta;
   }
-  // Order of a CTA's tiles: pass A runs kLagTiles ahead of the wave that pass B is in, and from there the
-  // passes take kStepTiles in turn.  The lag covers the way from a wave's last pass-A tile to its merged
-  // denominators (7 us, plus what the slowest CTA is late), which otherwise stands in every wave.
-  // Measured per 8 layers of the 8 x (8K..64K) batch: whole waves in turn (A0 A1 B0 A2 B1 ...) 10.56 ms, a lag
-  // of 8 / 12 / 16 / 20 tiles with 12-tile steps 9.11 / 9.02 / 9.00 / 8.98, 24 with 16-tile steps as 20; steps of 1 / 3 / 6 tiles at a lag
-  // of 8: 10.6 / 9.38 / 9.20 (each change of pass drains the statistics warps' load pipeline).  At one 128K
-  // request: 3.97 ms against 4.06 / 4.02 / 3.99 / 3.92.  A key tile is used again a wave and the lag later.
-  std::vector<CutOp> cuts;
-  cuts.reserve(4 * n_cta + 4 * n_pairs);
+  // Program of a CTA, by waves:  A0 A1 B0 A2 B1 ... A(n-1) B(n-2) B(n-1).  Pass B of a wave waits
+  // for the wave's merged denominators, which trail the slowest CTA's pass A by some 7 us; in
+  // the steady state the pass A in between covers that.  At the two ends it does not, so there
+  // (when the waves are single pairs, and there are at least four) one op is halved and its halves
+  // placed apart: A2's first half goes before B0, and B(n-3)'s second half goes after A(n-1).
+  std::vector<std::vector<std::vector<ScoreOp>>> was(n_waves), wbs(n_waves);   // [wave][CTA]
+  std::vector<std::vector<ScoreOp>> full(n_cta), bonly(n_cta);
   int32_t aseg = 0, bseg = 0;
-  ctx->h_tc_index = (int32_t*)ctx->h_tc_tables;
   int32_t* pair_aseg = ctx->h_tc_index;                    // [pairs+1]
   int32_t* pair_bseg = ctx->h_tc_index + (n_pairs + 1);    // [pairs+1]
+  const bool ends = kWaveDepth == 1 && n_waves >= 4;
+  auto single = [&](int wv) { return wave_begin[wv + 1] - wave_begin[wv] == 1; };
+  const int split_a = ends && single(2) ? 2 : -1;
+  const int split_b = ends && single(n_waves - 3) ? n_waves - 3 : -1;
   int rot = 0;
   for (int wv = 0; wv < n_waves; ++wv) {
     int64_t WA = 0;
     for (int p = wave_begin[wv]; p < wave_begin[wv + 1]; ++p)
       WA += (ctx->h_req[p / Hkv].N + TILE - 1) / TILE;
+    was[wv].assign(n_cta, {});
+    wbs[wv].assign(n_cta, {});
     int64_t fa = 0;
     for (int p = wave_begin[wv]; p < wave_begin[wv + 1]; ++p) {
       const int r = p / Hkv, g = p % Hkv;
@@ -1372,102 +1289,63 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
       pair_aseg[p] = aseg;
       pair_bseg[p] = bseg;
       const int64_t base = (int64_t)g * T + rq.cu;
-      cut_pair(cuts, wv, rot, n_cta, WA, fa, ta, rq.N, r, g, 0, aseg, base, rq.n);
+      cut_pair(was[wv], rot, n_cta, WA, fa, ta, rq.N, r, g, 0, aseg, base, rq.n, wv == split_a);
       // pass B walks the same flat tile positions, so a CTA re-reads the tiles it brought in
-      if (tb > 0) cut_pair(cuts, wv, rot, n_cta, WA, fa, tb, rq.n, r, g, 1, bseg, base, rq.n);
+      if (tb > 0) cut_pair(wbs[wv], rot, n_cta, WA, fa, tb, rq.n, r, g, 1, bseg, base, rq.n, wv == split_b);
       fa += ta;
     }
     // a wave's remainder tiles land on different CTAs each time (golden-ratio stride)
     rot = (rot + (int)(n_cta * 0.381966) + 1) % n_cta;
   }
+  // which = 0: every op, 1: first halves and unsplit ops, 2: second halves
+  auto put = [&](std::vector<ScoreOp>& dst, const std::vector<ScoreOp>& src, int which) {
+    for (const ScoreOp& op : src)
+      if (which == 0 || (which == 1 && op.pad != 2) || (which == 2 && op.pad == 2)) dst.push_back(op);
+  };
+  for (int cta = 0; cta < n_cta; ++cta) {
+    for (int wv = 0; wv < n_waves; ++wv) {
+      // pass A of this wave
+      if (wv == split_a) {
+        put(full[cta], was[wv][cta], 1);                       // A2 first half
+        put(full[cta], wbs[wv - 2][cta], 0);                   // B0 (held back one slot)
+        put(full[cta], was[wv][cta], 2);                       // A2 second half
+      } else {
+        put(full[cta], was[wv][cta], 0);
+      }
+      // pass B of the wave kWaveDepth behind
+      if (split_b >= 0 && wv == split_b + 2) put(full[cta], wbs[split_b][cta], 2);   // B(n-3) second half, after A(n-1)
+      const int bw = wv - kWaveDepth;
+      if (bw >= 0 && !(split_a >= 0 && bw == split_a - 2 && wv == split_a - 1)) {
+        if (bw == split_b) put(full[cta], wbs[bw][cta], 1);    // B(n-3) first half in its usual place
+        else put(full[cta], wbs[bw][cta], 0);
+      }
+      put(bonly[cta], wbs[wv][cta], 0);
+    }
+    for (int wv = n_waves > kWaveDepth ? n_waves - kWaveDepth : 0; wv < n_waves; ++wv)
+      put(full[cta], wbs[wv][cta], 0);
+  }
   pair_aseg[n_pairs] = aseg;
   pair_bseg[n_pairs] = bseg;
   if (aseg > ctx->max_tc_segs || bseg > ctx->max_tc_segs) return CAKE_ERR_CAPACITY;
 
-  int32_t* group_begin = ctx->h_tc_index + 2 * (n_pairs + 1);                   // [pairs+1]
-  int32_t* cta_ops = ctx->h_tc_index + kIndexPairs * (n_pairs + 1);             // [n_sm+1] each
-  int32_t *run_full = cta_ops + (ctx->n_sm + 1);
-  const int32_t n_ops = (int32_t)cuts.size();
-  if (n_ops > ctx->max_tc_ops) return CAKE_ERR_CAPACITY;
-  const size_t ops_at = ((kIndexPairs * (size_t)(n_pairs + 1) + kIndexCtas * (size_t)(ctx->n_sm + 1) + 3) / 4 * 4) * sizeof(int32_t);
-  const size_t runs_at = ops_at + (size_t)n_ops * sizeof(ScoreOp);
-  ScoreOp* h_ops = ctx->h_tc_ops = (ScoreOp*)(ctx->h_tc_tables + ops_at);
-  ScoreRun* h_runs = ctx->h_tc_runs = (ScoreRun*)(ctx->h_tc_tables + runs_at);
-  ctx->n_tc_ops = n_ops;
-  // The ops by CTA, in the order they were cut: by wave, and in a wave by pair.
-  std::vector<int32_t> wave_of(n_ops), tiles_of(n_ops), place(n_cta + 1, 0);
-  for (const CutOp& u : cuts) ++place[u.cta + 1];
+  int32_t* cta_full = ctx->h_tc_index + 2 * (n_pairs + 1);   // [n_sm+1]
+  int32_t* cta_b = cta_full + (ctx->n_sm + 1);               // [n_sm+1]
+  int64_t total = 0;
+  for (int cta = 0; cta < n_cta; ++cta) total += (int64_t)(full[cta].size() + bonly[cta].size());
+  if (total > ctx->max_tc_ops) return CAKE_ERR_CAPACITY;
+  int32_t o = 0;
   for (int cta = 0; cta < n_cta; ++cta) {
-    place[cta + 1] += place[cta];
-    if (place[cta + 1] - place[cta] > 0xFFFF) return CAKE_ERR_CAPACITY;
+    cta_full[cta] = o;
+    for (const ScoreOp& op : full[cta]) ctx->h_tc_ops[o++] = op;
   }
-  for (int cta = 0; cta <= n_cta; ++cta) cta_ops[cta] = place[cta];
-  for (const CutOp& u : cuts) {
-    const int32_t o = place[u.cta]++;
-    h_ops[o] = u.op;
-    wave_of[o] = u.wave;
-    tiles_of[o] = (u.op.nkeys + TILE - 1) / TILE;
-  }
-  int32_t n_runs = 0;
-  bool fits = true;
-  // A cursor over the ops of one pass of a CTA: takes the next n tiles as runs.
-  struct Cursor { int32_t at, done; };
-  auto take = [&](Cursor& c, int phase, int lo, int hi, int64_t n) {
-    while (n > 0) {
-      while (c.at < hi && h_ops[c.at].phase != phase) ++c.at;
-      if (c.at >= hi) return;
-      const int32_t k = (int32_t)std::min<int64_t>(std::min<int64_t>(n, kMaxRun), tiles_of[c.at] - c.done);
-      if (n_runs >= ctx->max_tc_runs) { fits = false; return; }
-      h_runs[n_runs++] = ScoreRun{c.done, (uint16_t)(c.at - lo), (uint16_t)k};
-      n -= k;
-      c.done += k;
-      if (c.done == tiles_of[c.at]) { ++c.at; c.done = 0; }
-    }
-  };
-  std::vector<int64_t> end_a(n_waves), end_b(n_waves);          // tiles of the CTA up to the end of a wave
-  std::vector<uint8_t> after_a(n_waves, 1);                     // pass B of the wave follows all of pass A, in every CTA
+  cta_full[n_cta] = o;
+  ctx->n_tc_ops_full = o;
   for (int cta = 0; cta < n_cta; ++cta) {
-    const int lo = cta_ops[cta], hi = cta_ops[cta + 1];
-    run_full[cta] = n_runs;
-    int64_t ta = 0, tb = 0;
-    for (int wv = 0, o = lo; wv < n_waves; ++wv) {
-      for (; o < hi && wave_of[o] == wv; ++o) (h_ops[o].phase ? tb : ta) += tiles_of[o];
-      end_a[wv] = ta;
-      end_b[wv] = tb;
-    }
-    const int64_t step = std::max<int64_t>(kStepTiles, (ta + tb + kRunsPerCta - 1) / kRunsPerCta);
-    Cursor ca{lo, 0}, cb{lo, 0};
-    int64_t a = 0, b = 0;
-    for (int wv = 0; wv < n_waves; ++wv) {
-      const int64_t from = std::min(ta, end_a[wv] + kLagTiles);
-      if (from < ta) after_a[wv] = 0;
-      if (a < from) { take(ca, 0, lo, hi, from - a); a = from; }
-      while (b < end_b[wv]) {
-        const int64_t left = end_b[wv] - b, nb = a < ta ? std::min(step, left) : left, na = std::min(step, ta - a);
-        take(cb, 1, lo, hi, nb);
-        b += nb;
-        take(ca, 0, lo, hi, na);
-        a += na;
-      }
-    }
-    take(ca, 0, lo, hi, ta - a);
+    cta_b[cta] = o;
+    for (const ScoreOp& op : bonly[cta]) ctx->h_tc_ops[o++] = op;
   }
-  run_full[n_cta] = n_runs;
-  if (!fits) return CAKE_ERR_CAPACITY;
-  // No op is cut (few waves, or the lag reaches to the end): put the ops in the order of their runs instead.
-  // (The column pass alone takes the ops of pass B in the table's order either way.)
-  if (n_runs == n_ops) {
-    std::vector<ScoreOp> in_order(n_ops);
-    for (int cta = 0; cta < n_cta; ++cta)
-      for (int i = run_full[cta]; i < run_full[cta + 1]; ++i) in_order[i] = h_ops[cta_ops[cta] + h_runs[i].op];
-    memcpy(h_ops, in_order.data(), sizeof(ScoreOp) * n_ops);
-    n_runs = 0;
-  }
-  ctx->tc_tables_used = runs_at + (size_t)n_runs * sizeof(ScoreRun);
-  ctx->n_tc_runs = n_runs;
-  ctx->d_tc_index = (int32_t*)ctx->d_tc_tables;
-  ctx->d_tc_ops = (ScoreOp*)(ctx->d_tc_tables + ops_at);
-  ctx->d_tc_runs = (ScoreRun*)(ctx->d_tc_tables + runs_at);
+  cta_b[n_cta] = o;
+  ctx->n_tc_ops_b = o - ctx->n_tc_ops_full;
   ctx->n_tc_asegs = aseg;
   ctx->n_tc_bsegs = bseg;
   // several rows at a time when there are pairs to take them from and a row has few partials
@@ -1475,25 +1353,26 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     int max_segs = 0;
     for (int p = 0; p < n_pairs; ++p) max_segs = std::max(max_segs, pair_aseg[p + 1] - pair_aseg[p]);
     const int partials = max_segs * NWG;
-    int max_pairs = 0;
-    for (int wv = 0; wv < n_waves; ++wv) max_pairs = std::max(max_pairs, wave_begin[wv + 1] - wave_begin[wv]);
     // at most 16 partials per lane (two batches of loads): 32 lanes / ways per row
     int ways = 1;
-    while (ways < 32 && ways < max_pairs && partials * 2 * ways <= 512) ways *= 2;
+    while (ways < 32 && 2 * ways <= n_pairs && partials * 2 * ways <= 512) ways *= 2;
     if (n_pairs < 4) ways = 1;
+    // The merger handles `ways` consecutive pairs at once and waits for the pass A of all of them.
+    // A CTA's program only guarantees A(w+1) before B(w): a group that reached from wave w into
+    // wave w+2 would make B(w) wait for an A(w+2) that comes after it.  So every group must lie
+    // in at most two adjacent waves.
+    std::vector<int> wave_of(n_pairs, 0);
+    for (int wv = 0; wv < n_waves; ++wv)
+      for (int p = wave_begin[wv]; p < wave_begin[wv + 1]; ++p) wave_of[p] = wv;
+    auto span_ok = [&](int wy) {
+      for (int p0 = 0; p0 < n_pairs; p0 += wy) {
+        const int p1 = std::min(n_pairs, p0 + wy) - 1;
+        if (wave_of[p1] - wave_of[p0] > kWaveDepth) return false;
+      }
+      return true;
+    };
+    while (ways > 1 && !span_ok(ways)) ways >>= 1;
     ctx->tc_merge_ways = ways;
-    // The merger handles a group of up to `ways` consecutive pairs at once and waits for the pass A of all
-    // of them.  B(w) must not wait for an A that comes after it in some CTA's order, so a group lies inside
-    // a wave; from the first wave whose pass B follows all of pass A, groups may cross the waves' borders
-    // (a group more is 2 us more between the last A and the last B: 47.8 against 50.4 us for 8 pairs in two
-    // waves).
-    int ng = 0;
-    for (int wv = 0, p0 = 0; wv < n_waves; ++wv) {
-      const int p1 = after_a[wv] ? n_pairs : wave_begin[wv + 1];
-      for (; p0 < p1; p0 += std::min(ways, p1 - p0)) group_begin[ng++] = p0;
-    }
-    group_begin[ng] = n_pairs;
-    ctx->n_tc_groups = ng;
     // With a single wave nothing runs between its pass A and its pass B, so a launch waits for the way
     // from the partial rows to the denominators.  As long as a pair's partials are few (a thread reads
     // one per segment, eight at a time) every CTA merges those of its own pass-B ops: the merged rows
@@ -1501,7 +1380,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     // of 4K keys).
     bool all_b = true;                               // every pair has a pass-B op to write its entropy rows
     for (int p = 0; p < n_pairs; ++p) all_b = all_b && pair_bseg[p + 1] > pair_bseg[p];
-    ctx->tc_direct = n_waves == 1 && all_b && max_segs <= kDirectSegs && n_runs == 0;
+    ctx->tc_direct = n_waves == 1 && all_b && max_segs <= kDirectSegs;
   }
   return CAKE_OK;
 }
@@ -1511,12 +1390,11 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
 // info8[7] = the number of the violated property:
 //   1  every key tile of every pair is covered exactly once by the pass-A ops, and every non-window
 //      tile exactly once by the pass-B ops
-//   2  inside every CTA's program the tiles of an op, and the ops of a pass, come in order, and every
-//      pass-A tile of a wave w' <= w precedes the first pass-B tile of wave w (so a wave's pass B can only
-//      ever wait for pass-A tiles that wait for nothing but the pass B of earlier waves)
-//   3  the pass A of the pairs that the merger warps handle side by side comes before the first pass B of any
-//      of them in every CTA's program, and the groups cover all pairs
-//   4  op counts, run counts and segment numbers stay inside the tables the context would allocate
+//   2  inside every CTA's program the pass-B ops come in non-decreasing wave order and every
+//      pass-A op of a wave w' <= w precedes the first pass-B op of wave w (so a wave's pass B can
+//      only ever wait for pass-A ops that wait for nothing themselves)
+//   3  the pairs the merger warps handle side by side lie in at most two adjacent waves
+//   4  op counts and segment numbers stay inside the tables the context would allocate
 int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_req, const int64_t* cu,
                       int32_t* info8) {
   if (!tc_path_supported(c)) return CAKE_ERR_ARG;
@@ -1536,20 +1414,17 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
   }
   x.h_req = reqs.data();
   x.max_tc_segs = (int32_t)tc_max_segments(c, n_sm);
-  x.max_tc_ops = 2 * x.max_tc_segs;
-  x.max_tc_runs = tc_max_runs(c, x.max_tc_ops, n_sm);
-  std::vector<int64_t> tables((tc_tables_bytes(n_pairs, n_sm, x.max_tc_ops, x.max_tc_runs) + 7) / 8), tables_d(1);
-  x.h_tc_tables = (uint8_t*)tables.data();
-  x.d_tc_tables = (uint8_t*)tables_d.data();           // offsets from it are never read here
+  x.max_tc_ops = 3 * x.max_tc_segs + 8;
+  std::vector<ScoreOp> ops((size_t)x.max_tc_ops);
+  std::vector<int32_t> index(2 * (size_t)(n_pairs + 1) + 2 * (size_t)(n_sm + 1));
+  x.h_tc_ops = ops.data();
+  x.h_tc_index = index.data();
   const int32_t rc = tc_build_plan(&x, n_req);
   info8[0] = x.n_tc_ctas; info8[1] = x.n_tc_waves; info8[2] = x.tc_merge_ways; info8[3] = x.n_tc_asegs;
-  info8[4] = x.n_tc_bsegs; info8[5] = x.n_tc_ops; info8[6] = x.n_tc_bsegs; info8[7] = 0;
+  info8[4] = x.n_tc_bsegs; info8[5] = x.n_tc_ops_full; info8[6] = x.n_tc_ops_b; info8[7] = 0;
   if (rc != CAKE_OK || x.n_tc_ctas == 0) return rc;
   auto fail = [&](int what) { info8[7] = what; return (int32_t)CAKE_ERR_STATE; };
-  const int32_t* index = x.h_tc_index;
-  const ScoreOp* ops = x.h_tc_ops;
-  const ScoreRun* runs = x.h_tc_runs;
-  if (x.n_tc_ops > x.max_tc_ops || x.n_tc_runs > x.max_tc_runs || x.tc_tables_used > tables.size() * 8 || x.n_tc_asegs > x.max_tc_segs ||
+  if (x.n_tc_ops_full + x.n_tc_ops_b > x.max_tc_ops || x.n_tc_asegs > x.max_tc_segs ||
       x.n_tc_bsegs > x.max_tc_segs) return fail(4);
   // waves as the builder forms them
   std::vector<int> wave_of(n_pairs, 0);
@@ -1558,8 +1433,7 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
     for (int wv = 0; wv + 1 < (int)wb.size(); ++wv)
       for (int p = wb[wv]; p < wb[wv + 1]; ++p) wave_of[p] = wv;
   }
-  const int32_t* cta_full = index + kIndexPairs * (n_pairs + 1);
-  const int32_t* run_full = cta_full + (n_sm + 1);
+  const int32_t* cta_full = index.data() + 2 * (n_pairs + 1);
   // 1: coverage, per pair and pass, in tiles
   std::vector<std::vector<int>> cover[2];
   for (int ph = 0; ph < 2; ++ph) {
@@ -1569,36 +1443,22 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
       cover[ph][p].assign(((ph ? rq.n : rq.N) + TILE - 1) / TILE, 0);
     }
   }
-  std::vector<int> reach(x.n_tc_waves, x.n_tc_waves - 1);      // last wave whose pass A precedes a wave's pass B
   for (int cta = 0; cta < x.n_tc_ctas; ++cta) {
+    int last_b_wave = -1;
     std::vector<int> first_b_pos(x.n_tc_waves + 1, -1);
     std::vector<int> last_a_pos(x.n_tc_waves + 1, -1);
-    std::vector<int> done(cta_full[cta + 1] - cta_full[cta], 0);
-    int last_op[2] = {-1, -1};
-    const bool whole = x.n_tc_runs == 0;
-    const int steps = whole ? (int)done.size() : run_full[cta + 1] - run_full[cta];
-    for (int pos = 0; pos < steps; ++pos) {
-      struct { int op, tile0, count; } run = {pos, 0, 0};
-      if (whole) {
-        run.count = (ops[cta_full[cta] + pos].nkeys + TILE - 1) / TILE;
-      } else {
-        const ScoreRun& u = runs[run_full[cta] + pos];
-        run.op = u.op; run.tile0 = u.tile0; run.count = u.count;
-      }
-      if (run.op >= (int)done.size() || run.count < 1) return fail(1);
-      const ScoreOp& op = ops[cta_full[cta] + run.op];
+    for (int o = cta_full[cta]; o < cta_full[cta + 1]; ++o) {
+      const ScoreOp& op = ops[o];
       const int p = op.req * Hkv + op.g;
       if (p < 0 || p >= n_pairs || op.key0 % TILE != 0 || op.nkeys <= 0) return fail(1);
       if (op.seg < 0 || op.seg >= (op.phase ? x.n_tc_bsegs : x.n_tc_asegs)) return fail(4);
-      if (run.op < last_op[op.phase] || run.tile0 != done[run.op]) return fail(2);
-      last_op[op.phase] = run.op;
-      done[run.op] += run.count;
-      if (done[run.op] > (op.nkeys + TILE - 1) / TILE) return fail(1);
-      const int t0 = op.key0 / TILE + run.tile0, t1 = t0 + run.count;
+      const int t0 = op.key0 / TILE, t1 = (op.key0 + op.nkeys + TILE - 1) / TILE;
       if (t1 > (int)cover[op.phase][p].size()) return fail(1);
       for (int t = t0; t < t1; ++t) cover[op.phase][p][t] += 1;
-      const int wv = wave_of[p];
+      const int wv = wave_of[p], pos = o - cta_full[cta];
       if (op.phase) {
+        if (wv < last_b_wave) return fail(2);
+        last_b_wave = wv;
         if (first_b_pos[wv] < 0) first_b_pos[wv] = pos;
       } else {
         last_a_pos[wv] = pos;
@@ -1608,20 +1468,16 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
       if (first_b_pos[w] >= 0)
         for (int w2 = 0; w2 <= w; ++w2)
           if (last_a_pos[w2] > first_b_pos[w]) return fail(2);
-    for (int w = 0; w < x.n_tc_waves; ++w)
-      for (int w2 = w + 1; first_b_pos[w] >= 0 && w2 <= reach[w]; ++w2)
-        if (last_a_pos[w2] > first_b_pos[w]) reach[w] = w2 - 1;
   }
   for (int ph = 0; ph < 2; ++ph)
     for (int p = 0; p < n_pairs; ++p)
       for (int v : cover[ph][p])
         if (v != 1) return fail(1);
   // 3: merge groups
-  const int32_t* group_begin = index + 2 * (n_pairs + 1);
-  if (group_begin[0] != 0 || group_begin[x.n_tc_groups] != n_pairs) return fail(3);
-  for (int gi = 0; gi < x.n_tc_groups; ++gi) {
-    const int p0 = group_begin[gi], p1 = group_begin[gi + 1] - 1;
-    if (p1 < p0 || p1 - p0 >= x.tc_merge_ways || wave_of[p1] > reach[wave_of[p0]]) return fail(3);
+  const int ways = x.tc_merge_ways;
+  for (int p0 = 0; p0 < n_pairs; p0 += ways) {
+    const int p1 = std::min(n_pairs, p0 + ways) - 1;
+    if (wave_of[p1] - wave_of[p0] > kWaveDepth) return fail(3);
   }
   return CAKE_OK;
 }
@@ -1664,9 +1520,6 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   TcParams P;
   P.ops = ctx->d_tc_ops;
   P.reqs = ctx->d_req;
-  P.runs = ctx->d_tc_runs;
-  P.group_begin = ctx->d_tc_index + 2 * (n_pairs + 1);
-  P.n_groups = ctx->n_tc_groups;
   P.pair_aseg = ctx->d_tc_index;
   P.pair_cnt = ctx->d_tc_sync;
   P.lse2 = ctx->d_lse2_tc;
@@ -1689,31 +1542,30 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.bessel = c.var_ddof ? (float)c.window / (float)(c.window - 1) : 1.f;
 
   const int sp = prof_begin(ctx, CAKE_PROF_SCORE, st);
-  const int32_t* cta_full = ctx->d_tc_index + kIndexPairs * (n_pairs + 1);
-  P.cta_op = cta_full;
-  P.cta_run = cta_full + (ctx->n_sm + 1);
+  const int32_t* cta_full = ctx->d_tc_index + 2 * (n_pairs + 1);
   if (lse) {
     // denominators supplied: pass B alone, entropy from its columns
     ctx->hhead_from_rows = false;
+    P.cta_op = cta_full + (ctx->n_sm + 1);
     P.pair_done = nullptr;
     P.epoch = 0;
   } else {
     ctx->hhead_from_rows = true;
+    P.cta_op = cta_full;
     P.pair_done = ctx->d_tc_sync + ctx->max_pairs;
     P.epoch = ++ctx->tc_epoch + (uint32_t)ctx->debug_epoch_skew;
   }
   cudaError_t e;
   const bool eb = lse != nullptr;
-  const int plan = ctx->tc_direct ? kDirectMerge : ctx->n_tc_runs == 0 ? kWhole : kRuns;
   // An early start takes SMs from the cascade kernels.  The column pass of a single wave is so short that
   // these set the pace: it starts when the launch before it is done (32 layers of 16 heads and 12.7K keys:
   // 730 us with an early start, 690 without).
   const bool early = !(eb && ctx->n_tc_waves == 1);
   switch (G) {
-    case 1: e = launch_g<1>(ctx->device, eb, P.reps > 1, plan, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    case 2: e = launch_g<2>(ctx->device, eb, P.reps > 1, plan, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    case 4: e = launch_g<4>(ctx->device, eb, P.reps > 1, plan, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
-    default: e = launch_g<8>(ctx->device, eb, P.reps > 1, plan, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 1: e = launch_g<1>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 2: e = launch_g<2>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    case 4: e = launch_g<4>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
+    default: e = launch_g<8>(ctx->device, eb, P.reps > 1, ctx->tc_direct, early, ctx->n_tc_ctas, st, qmap, kmap, P); break;
   }
   count_launch();
   prof_end(ctx, sp, st);

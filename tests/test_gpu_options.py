@@ -274,18 +274,6 @@ def test_row_copies_and_both_ways_to_the_denominators(hq, hkv, window, seq_lens)
     check_scores(w, expect_tc=True)
 
 
-@pytest.mark.parametrize("hq,hkv,window,seq_lens", [
-    (4, 4, 32, (100001,)),             # four waves of one pair, copies of the rows
-    (16, 4, 32, (60001, 40001)),       # 128 rows, waves of several pairs
-    (8, 1, 16, (140003,)),             # one wave: pass A whole, then pass B
-])
-def test_passes_that_alternate_inside_a_program(monkeypatch, hq, hkv, window, seq_lens):
-    # half the SMs, so that pass A is longer than pass B's lag behind it
-    monkeypatch.setenv("CAKE_RESERVED_SMS", "74")
-    w = bf16_case(n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=seq_lens, n_layers=1, total_budget=window + 60)
-    check_scores(w, expect_tc=True)
-
-
 @pytest.mark.parametrize("seq_lens,budget,pool", [
     ((4096 + 31, 4096 + 33, 77), 300, 7),            # runs that end a token before and after a tile, odd offsets
     ((8192 + 32, 40), 1000, 5),                      # a whole number of tiles, a prompt of eight tokens
