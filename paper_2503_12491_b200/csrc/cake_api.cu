@@ -250,7 +250,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_colpart[i], (a > b ? a : b) * G * 2) == cudaSuccess;
   }
   if (x->use_tc) {
-    const size_t n_index = 2 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
+    const size_t n_index = 3 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
     ok = ok && cudaMallocHost((void**)&x->h_tc_ops, sizeof(ScoreOp) * x->max_tc_ops) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&x->h_tc_index, sizeof(int32_t) * n_index) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_ops, x->max_tc_ops) == cudaSuccess;
@@ -357,7 +357,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
     CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_units, ctx->h_units, sizeof(ScoreUnit) * nu,
                                   cudaMemcpyHostToDevice, st));
     if (ctx->use_tc && ctx->n_tc_ctas > 0) {
-      const size_t n_index = 2 * (size_t)(n_req * c.n_kv_heads + 1) + 2 * (size_t)(ctx->n_sm + 1);
+      const size_t n_index = 3 * (size_t)(n_req * c.n_kv_heads + 1) + 2 * (size_t)(ctx->n_sm + 1);
       CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_tc_ops, ctx->h_tc_ops,
                                     sizeof(ScoreOp) * (ctx->n_tc_ops_full + ctx->n_tc_ops_b),
                                     cudaMemcpyHostToDevice, st));

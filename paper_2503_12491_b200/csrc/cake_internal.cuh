@@ -192,8 +192,9 @@ struct cake_ctx {
   cake::ScoreOp* h_tc_ops;        // pinned: [both-pass programs][pass-B-only programs]
   cake::ScoreOp* d_tc_ops;
   // pinned / device index block of the current batch, P = n_req * H_kv pairs:
-  //   pair_aseg [P+1] | pair_bseg [P+1] | cta_op of the both-pass programs [n_sm+1]
+  //   pair_aseg [P+1] | pair_bseg [P+1] | group_begin [P+1] | cta_op of the both-pass programs [n_sm+1]
   //   | cta_op of the pass-B-only programs [n_sm+1]
+  int32_t n_tc_groups;            // groups of pairs the merger warps take at once
   int32_t* h_tc_index;
   int32_t* d_tc_index;
   uint32_t* d_tc_sync;            // [max_pairs] delivered partial rows, then [max_pairs] merged rows

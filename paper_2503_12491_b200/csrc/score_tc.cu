@@ -67,6 +67,8 @@ constexpr int kWaveDepth = 1;         // pass B of a wave follows pass A of the 
 struct TcParams {
   const ScoreOp* ops;
   const int32_t* cta_op;        // [n_cta + 1]
+  const int32_t* group_begin;   // [n_groups + 1] first pair of every merge group; null: every merge_ways pairs
+  int n_groups;
   const ReqInfo* reqs;
   const int32_t* pair_aseg;     // [pairs + 1] pass-A segment ranges per pair
   uint32_t* pair_cnt;           // [pairs] delivered pass-A partials (monotonic over layers)
@@ -628,9 +630,9 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // by 32 / ways lanes each, and the wave's denominators are ready that much sooner.
         const int ways = P.merge_ways, lpr = 32 / ways;         // lanes per row
         const int sub = lane / lpr, l8 = lane % lpr;
-        for (int p0 = 0; p0 < P.n_pairs && ok; p0 += ways) {
-          const int pair = p0 + sub;
-          const bool have = pair < P.n_pairs;
+        for (int gi = 0; gi < P.n_groups && ok; ++gi) {
+          const int pair = (P.group_begin ? P.group_begin[gi] : gi * ways) + sub;
+          const bool have = pair < (P.group_begin ? P.group_begin[gi + 1] : P.n_pairs);
           const int s_lo = have ? P.pair_aseg[pair] * NWG : 0, s_hi = have ? P.pair_aseg[pair + 1] * NWG : 0;
           const int r0 = have ? (int)((blockIdx.x + gridDim.x - (unsigned)(((long long)pair * P.rows) % gridDim.x)) % gridDim.x)
                               : P.rows;
@@ -1328,7 +1330,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
   pair_bseg[n_pairs] = bseg;
   if (aseg > ctx->max_tc_segs || bseg > ctx->max_tc_segs) return CAKE_ERR_CAPACITY;
 
-  int32_t* cta_full = ctx->h_tc_index + 2 * (n_pairs + 1);   // [n_sm+1]
+  int32_t* cta_full = ctx->h_tc_index + 3 * (n_pairs + 1);   // [n_sm+1]
   int32_t* cta_b = cta_full + (ctx->n_sm + 1);               // [n_sm+1]
   int64_t total = 0;
   for (int cta = 0; cta < n_cta; ++cta) total += (int64_t)(full[cta].size() + bonly[cta].size());
@@ -1357,22 +1359,22 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     int ways = 1;
     while (ways < 32 && 2 * ways <= n_pairs && partials * 2 * ways <= 512) ways *= 2;
     if (n_pairs < 4) ways = 1;
-    // The merger handles `ways` consecutive pairs at once and waits for the pass A of all of them.
-    // A CTA's program only guarantees A(w+1) before B(w): a group that reached from wave w into
-    // wave w+2 would make B(w) wait for an A(w+2) that comes after it.  So every group must lie
-    // in at most two adjacent waves.
-    std::vector<int> wave_of(n_pairs, 0);
-    for (int wv = 0; wv < n_waves; ++wv)
-      for (int p = wave_begin[wv]; p < wave_begin[wv + 1]; ++p) wave_of[p] = wv;
-    auto span_ok = [&](int wy) {
-      for (int p0 = 0; p0 < n_pairs; p0 += wy) {
-        const int p1 = std::min(n_pairs, p0 + wy) - 1;
-        if (wave_of[p1] - wave_of[p0] > kWaveDepth) return false;
-      }
-      return true;
-    };
-    while (ways > 1 && !span_ok(ways)) ways >>= 1;
     ctx->tc_merge_ways = ways;
+    // The merger handles up to `ways` consecutive pairs at once and waits for the pass A of all of them.  A
+    // group that reaches from wave w into w+1 makes B(w) wait for the end of A(w+1), which comes right
+    // before it, and for the way from there to the denominators; one that reaches into w+2 would make it
+    // wait for an A that comes after it.  So a group lies inside a wave (8 requests of 8K to 64K, groups of
+    // 2 pairs: 10.28 ms against 10.87 with groups across two waves), except in the last two: their pass B
+    // follows all of pass A, and every group less is 2 us less between the two (47.8 against 50.4 us for 8
+    // pairs in two waves).
+    int32_t* group_begin = ctx->h_tc_index + 2 * (n_pairs + 1);
+    int ng = 0;
+    for (int wv = 0, p0 = 0; wv < n_waves; ++wv) {
+      const int p1 = wv + 2 >= n_waves ? n_pairs : wave_begin[wv + 1];
+      for (; p0 < p1; p0 += std::min(ways, p1 - p0)) group_begin[ng++] = p0;
+    }
+    group_begin[ng] = n_pairs;
+    ctx->n_tc_groups = ng;
     // With a single wave nothing runs between its pass A and its pass B, so a launch waits for the way
     // from the partial rows to the denominators.  As long as a pair's partials are few (a thread reads
     // one per segment, eight at a time) every CTA merges those of its own pass-B ops: the merged rows
@@ -1393,7 +1395,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
 //   2  inside every CTA's program the pass-B ops come in non-decreasing wave order and every
 //      pass-A op of a wave w' <= w precedes the first pass-B op of wave w (so a wave's pass B can
 //      only ever wait for pass-A ops that wait for nothing themselves)
-//   3  the pairs the merger warps handle side by side lie in at most two adjacent waves
+//   3  the pairs the merger warps handle side by side lie in one wave or in the last two
 //   4  op counts and segment numbers stay inside the tables the context would allocate
 int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_req, const int64_t* cu,
                       int32_t* info8) {
@@ -1416,7 +1418,7 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
   x.max_tc_segs = (int32_t)tc_max_segments(c, n_sm);
   x.max_tc_ops = 3 * x.max_tc_segs + 8;
   std::vector<ScoreOp> ops((size_t)x.max_tc_ops);
-  std::vector<int32_t> index(2 * (size_t)(n_pairs + 1) + 2 * (size_t)(n_sm + 1));
+  std::vector<int32_t> index(3 * (size_t)(n_pairs + 1) + 2 * (size_t)(n_sm + 1));
   x.h_tc_ops = ops.data();
   x.h_tc_index = index.data();
   const int32_t rc = tc_build_plan(&x, n_req);
@@ -1433,7 +1435,7 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
     for (int wv = 0; wv + 1 < (int)wb.size(); ++wv)
       for (int p = wb[wv]; p < wb[wv + 1]; ++p) wave_of[p] = wv;
   }
-  const int32_t* cta_full = index.data() + 2 * (n_pairs + 1);
+  const int32_t* cta_full = index.data() + 3 * (n_pairs + 1);
   // 1: coverage, per pair and pass, in tiles
   std::vector<std::vector<int>> cover[2];
   for (int ph = 0; ph < 2; ++ph) {
@@ -1474,10 +1476,12 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
       for (int v : cover[ph][p])
         if (v != 1) return fail(1);
   // 3: merge groups
-  const int ways = x.tc_merge_ways;
-  for (int p0 = 0; p0 < n_pairs; p0 += ways) {
-    const int p1 = std::min(n_pairs, p0 + ways) - 1;
-    if (wave_of[p1] - wave_of[p0] > kWaveDepth) return fail(3);
+  const int32_t* group_begin = index.data() + 2 * (n_pairs + 1);
+  if (group_begin[0] != 0 || group_begin[x.n_tc_groups] != n_pairs) return fail(3);
+  for (int gi = 0; gi < x.n_tc_groups; ++gi) {
+    const int p0 = group_begin[gi], p1 = group_begin[gi + 1] - 1;
+    if (p1 < p0 || p1 - p0 >= x.tc_merge_ways || (wave_of[p1] != wave_of[p0] && wave_of[p0] + 2 < x.n_tc_waves)) return fail(3);
+    if (x.n_tc_waves <= 2 && p0 != gi * x.tc_merge_ways) return fail(3);
   }
   return CAKE_OK;
 }
@@ -1520,6 +1524,9 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   TcParams P;
   P.ops = ctx->d_tc_ops;
   P.reqs = ctx->d_req;
+  // with one or two waves the groups are those of the plain rule, which spares the merger a read per group
+  P.group_begin = ctx->n_tc_waves > 2 ? ctx->d_tc_index + 2 * (n_pairs + 1) : nullptr;
+  P.n_groups = ctx->n_tc_groups;
   P.pair_aseg = ctx->d_tc_index;
   P.pair_cnt = ctx->d_tc_sync;
   P.lse2 = ctx->d_lse2_tc;
@@ -1542,7 +1549,7 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.bessel = c.var_ddof ? (float)c.window / (float)(c.window - 1) : 1.f;
 
   const int sp = prof_begin(ctx, CAKE_PROF_SCORE, st);
-  const int32_t* cta_full = ctx->d_tc_index + 2 * (n_pairs + 1);
+  const int32_t* cta_full = ctx->d_tc_index + 3 * (n_pairs + 1);
   if (lse) {
     // denominators supplied: pass B alone, entropy from its columns
     ctx->hhead_from_rows = false;

@@ -267,6 +267,7 @@ def test_cumulative_attention_indicator_through_the_hook():
     (2, 2, 32, (5121, 129)),           # 32 rows, merge in every CTA, a pair of two tiles
     (4, 1, 32, (4097, 1000, 161)),     # 128 rows, merge in every CTA
     (2, 2, 32, (900, 32)),             # a prompt that is all window has no column pass
+    (16, 4, 32, (60001, 40001)),       # 128 rows, four waves of several pairs: merge groups that end with their wave
 ])
 def test_row_copies_and_both_ways_to_the_denominators(hq, hkv, window, seq_lens):
     w = bf16_case(n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=seq_lens, n_layers=2 if max(seq_lens) < 9000 else 1,
