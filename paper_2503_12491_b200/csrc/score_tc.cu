@@ -25,8 +25,8 @@
 // that count is normally already satisfied.
 //
 // Warp roles in a CTA of 512 threads: warps 0..11 are "statistics" warps in three groups of
-// four (a group takes every third accumulator tile, a warp owns 32 of its TMEM lanes, works
-// alone and writes its own partial results), warp 12 issues TMA loads, warp 13 owns the
+// four (a group takes every third accumulator tile, a warp owns 32 of its TMEM lanes and writes
+// its own partial results; warps meet only where partial rows are exchanged, see xrow_slot), warp 12 issues TMA loads, warp 13 owns the
 // tensor-memory allocation and issues the MMAs (both as converged warps with an elected lane),
 // warp 14 publishes this CTA's finished pass-A ops to the grid and merges rows, warp 15 stages
 // the denominators of the next pass-B op in shared memory.  Every wait
@@ -324,7 +324,7 @@ struct Smem {
   uint8_t* ext_a;      // the constant key-side operand of the extra K step of pass B
   uint8_t* ext_b;      // [2] its row-side operand: -lse/scale of the current / next pass-B op
   float4* xrow;        // [2][NWG][128] partial rows of a group: copies of a row in pass A, then (direct merge) the
-                       //   group's share of a pair's partials for the current / next pass-B op
+                       //   group's share of a pair's partials of a pass-B op; slots by xrow_slot
   ScoreOp* ops;        // [kSmemOps] the first ops of this CTA's program
 };
 
@@ -405,6 +405,15 @@ __device__ __forceinline__ void put_ext_row(uint8_t* ext, int r, int rows, float
   const uint32_t w1 = (uint32_t)__bfloat16_as_ushort(lo);
   *reinterpret_cast<uint2*>(ext + ext_row_offset(r)) = r < rows ? make_uint2(w0, w1) : make_uint2(0u, 0u);
 }
+
+// Slot of the exchange rows (Smem::xrow) that a statistics warp uses after n_a pass-A ops and n_b pass-B
+// ops.  A use writes its slot, meets a barrier and reads: the group's barrier in pass A (the warps of the
+// first copy read their group's rows), the barrier of all statistics warps in a direct merge (group 0 reads
+// every group's).  The next use may therefore not write the same slot, since slower warps still read it, but
+// the one after that may: its writers have met the readers at the barrier between.  So the slots
+// alternate over the whole program, from the last pass-A op into the first pass-B op too, and pass A may
+// not follow a direct merge, whose readers a group's barrier does not meet (one wave: it never does).
+__host__ __device__ constexpr int xrow_slot(uint32_t n_a, uint32_t n_b) { return (int)((n_a + n_b) & 1u); }
 
 // ------------------------------------------------------------------ kernel
 // kCopies: the window has 32 or 64 rows and a pass-A tile holds them 4 or 2 times, so that every
@@ -799,8 +808,9 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
   } else {
     // ------------------------------------------------ statistics warps
-    // Every warp works alone: it owns TMEM lanes 32*quad.. of the tiles its group takes, writes
-    // its own partial results and never waits for another statistics warp.
+    // Every warp owns TMEM lanes 32*quad.. of the tiles its group takes and writes its own partial
+    // results.  It waits for other statistics warps only where rows are exchanged: with kCopies for its
+    // group at the end of a pass-A op, with kDirect for all of them at the start of a pass-B op.
     // Group wg takes the tiles t with t % NWG == wg; with as many buffers as groups that is
     // always buffer wg, whose "ready" barrier the group then meets in consecutive phases.
     const int wg = warp >> 2;
@@ -828,7 +838,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // ---------------- pass B: thread = key, columns = rows r' = i*G + h
         if constexpr (kDirect) {
           // One thread per row and group; every CTA adds in the same order.
-          const int slot = kbs & 1, pair = op.req * P.Hkv + op.g;
+          const int slot = kbs & 1, xslot = xrow_slot(n_a_done, kbs), pair = op.req * P.Hkv + op.g;
           const int s_lo = P.pair_aseg[pair];        // read before the wait
           int s_hi = P.pair_aseg[pair + 1];
           if (ok) ok = mbar_wait(&S.parts[slot], (kbs >> 1) & 1, P.status, P.spin_limit);
@@ -845,14 +855,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               acc = merge_batch(acc, pv);
             }
           }
-          S.xrow[(slot * NWG + wg) * 128 + lane_row] = acc;
+          S.xrow[(xslot * NWG + wg) * 128 + lane_row] = acc;
           asm volatile("bar.sync 1, %0;" ::"n"(STAT_THREADS) : "memory");
           if (wg == 0) {
             acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
             if (lane_row < P.rows) {
               float4 pv[NWG];
 #pragma unroll
-              for (int q = 0; q < NWG; ++q) pv[q] = S.xrow[(slot * NWG + q) * 128 + lane_row];
+              for (int q = 0; q < NWG; ++q) pv[q] = S.xrow[(xslot * NWG + q) * 128 + lane_row];
               acc = merge_batch(acc, pv);
             }
             const float lz = log2f(acc.y);
@@ -1073,9 +1083,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // twelve warps, which only tell it, inside the CTA, that their rows are written.
         float4 part = make_float4(m, z, zwin, w);
         if constexpr (kCopies) {
-          // the group's copies of a row become one partial (two slots: a reader of this op's is done
-          // before it reaches the next op's barrier)
-          float4* x = S.xrow + ((n_a_done & 1) * NWG + wg) * 128;
+          // the group's copies of a row become one partial
+          float4* x = S.xrow + (xrow_slot(n_a_done, kbs) * NWG + wg) * 128;
           x[lane_row] = part;
           asm volatile("bar.sync %0, 128;" ::"r"(2 + wg) : "memory");
           if (copy == 0)
@@ -1397,6 +1406,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
 //      only ever wait for pass-A ops that wait for nothing themselves)
 //   3  the pairs the merger warps handle side by side lie in one wave or in the last two
 //   4  op counts and segment numbers stay inside the tables the context would allocate
+//   5  no statistics warp writes a slot of the exchange rows that another may still read (xrow_slot)
 int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_req, const int64_t* cu,
                       int32_t* info8) {
   if (!tc_path_supported(c)) return CAKE_ERR_ARG;
@@ -1470,6 +1480,27 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
       if (first_b_pos[w] >= 0)
         for (int w2 = 0; w2 <= w; ++w2)
           if (last_a_pos[w2] > first_b_pos[w]) return fail(2);
+    // 5: between two uses of a slot lies a use whose barrier the first one's readers and the second one's
+    // writers both meet: any use after a pass-A op (its readers and writers are of one group), a pass-B op
+    // after a direct merge
+    if (tc_reps(x.rows) > 1 || x.tc_direct) {
+      uint32_t n_a = 0, n_b = 0;
+      int last[2] = {-1, -1}, last_phase[2] = {0, 0}, uses = 0, last_merge = -1;
+      for (int o = cta_full[cta]; o < cta_full[cta + 1]; ++o) {
+        const int phase = ops[o].phase;
+        if (phase ? x.tc_direct : tc_reps(x.rows) > 1) {
+          const int slot = xrow_slot(n_a, n_b);
+          if (last[slot] >= 0 && (last_phase[slot] ? last_merge : uses - 1) <= last[slot]) return fail(5);
+          last[slot] = uses;
+          last_phase[slot] = phase;
+          if (phase) last_merge = uses;
+          ++uses;
+        }
+        // kbs counts the pass-B ops of the direct merge only
+        if (!phase) ++n_a;
+        else if (x.tc_direct) ++n_b;
+      }
+    }
   }
   for (int ph = 0; ph < 2; ++ph)
     for (int p = 0; p < n_pairs; ++p)

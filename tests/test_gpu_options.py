@@ -81,7 +81,9 @@ def check_scores(w, *, cake_kw=None, oracle_kw=None, expect_tc=None, lse=False):
             assert_close(V[r, l], refs[l][r]["V"], f"V l{l} r{r}")
             assert_close(P[r, l], refs[l][r]["P"], f"P l{l} r{r}")
     assert cake.status() == 0
+    plan = cake.plan_info()
     cake.destroy()
+    return plan
 
 
 @pytest.mark.parametrize("kernel", [1, 3, 5, 7, 9, 13])
@@ -273,6 +275,17 @@ def test_row_copies_and_both_ways_to_the_denominators(hq, hkv, window, seq_lens)
     w = bf16_case(n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=seq_lens, n_layers=2 if max(seq_lens) < 9000 else 1,
                   total_budget=(2 if max(seq_lens) < 9000 else 1) * (window + 60))
     check_scores(w, expect_tc=True)
+
+
+@pytest.mark.parametrize("n_req,tokens,ops", [(12, 250, 3), (20, 130, 5), (16, 250, 4)])
+@pytest.mark.parametrize("kv_heads,per", [(32, 1), (16, 2)])
+def test_many_row_pass_ops_before_a_merge_in_every_cta(n_req, tokens, ops, kv_heads, per):
+    """Batches of short prompts, 32 and 64 window rows: several copies of the rows are summed by every CTA,
+    op after op, before the first merge of a pair uses the same exchange rows."""
+    w = bf16_case(n_q_heads=32, n_kv_heads=kv_heads, head_dim=128, window=32, seq_lens=(tokens,) * (n_req * per), n_layers=2,
+                  total_budget=2 * 60)
+    plan = check_scores(w, expect_tc=True)
+    assert plan["waves"] == 1 and plan["a_segments"] == ops * plan["ctas"]
 
 
 @pytest.mark.parametrize("seq_lens,budget,pool", [

@@ -57,6 +57,18 @@ def test_random_ragged_batches_and_sm_counts():
     assert seen_ways >= {1, 4}                            # both merger modes were exercised
 
 
+def test_exchange_rows_with_many_row_pass_ops_per_cta():
+    """One-wave plans of short prompts with 32 and 64 window rows: a CTA has 1 to 7 row-pass ops before its
+    first column-pass op, and the rows of the last one may still be read when that starts."""
+    for heads, kv_heads, per in [(32, 32, 1), (32, 16, 2)]:
+        seen = set()
+        for n_req, tokens in [(4, 250), (8, 250), (12, 250), (16, 250), (20, 130), (24, 130), (28, 130), (7, 500)]:
+            rc, info = check(heads, kv_heads, 32, 128, [tokens] * (n_req * per), 148, 16)
+            assert rc == 0 and info[7] == 0 and info[1] == 1, (heads, kv_heads, n_req, tokens, info)
+            seen.add(info[3] // info[0])
+        assert {1, 3, 5} <= seen
+
+
 def test_shapes_of_the_simt_path_are_refused():
     rc, info = check(4, 4, 16, 64, [512], 148, 16)       # 16 rows: not a multiple of 32
     assert rc == binding.CAKE_ERR_ARG
