@@ -291,7 +291,9 @@ int32_t cake_uses_tensor_cores(const cake_ctx* ctx);
  *                       other readings); then the entry that comes last in the order (score
  *                       descending, position ascending) among those tokens is evicted and its
  *                       slot becomes the free one, so the head is back at its frozen budget.
- *                       Rows never move; layers may be stepped in any order, each once per token.
+ *                       Rows never move; layers may be stepped in any order, each once per token, on
+ *                       any streams on which a layer's own steps follow one another; a stream capture
+ *                       may record them.
  *   cake_decode_get_state  entries of one (request, layer) in ascending token position:
  *                       positions_out int32 [H_kv][len], scores_out fp32 [H_kv][len] (0 for the
  *                       window entries), slots_out int32 [H_kv][len] (slot of each entry inside

@@ -710,6 +710,9 @@ int32_t cake_decode_begin(cake_ctx* ctx, const void* const* k_layers, const void
   if (rc != CAKE_OK) return rc;
   ctx->dec_update_mode = update_mode;
   ctx->dec_last_layer = -1;
+  ctx->dec_captured = false;
+  const StepPlace here = step_place(st);
+  for (int l = 0; l < c.n_layers; ++l) ctx->dec_place[l] = here;
   ctx->dec_ready = true;
   return CAKE_OK;
 }

@@ -75,6 +75,12 @@ struct ListState {
   int32_t kept;          // budget the list arrived with: entries beyond it are not stored
 };
 
+// Where a decode step was enqueued: the stream, by its unique id or in a capture by its handle (0:
+// unknown), and the stream capture that recorded it (0: none, the step ran).
+struct StepPlace {
+  unsigned long long stream, capture;
+};
+
 struct LayerPtrs {
   const void* k[CAKE_MAX_LAYERS];
   const void* v[CAKE_MAX_LAYERS];
@@ -182,7 +188,10 @@ struct cake_ctx {
   int32_t* d_dec_order;           // per head: rank in ascending position -> slot
   int4* d_dec_meta;               // [max_lists] (len, free slot, next position, frozen budget)
   int32_t* h_budget_stage;        // pinned [max_requests*L] read-back of the final budgets
-  int32_t dec_last_layer;         // layer of the latest decode step on the cluster form, -1 = none yet
+  int32_t dec_last_layer;         // layer of the latest decode step if it was on the cluster form, else -1
+  cake::StepPlace dec_last;       // where that step was enqueued
+  cake::StepPlace dec_place[CAKE_MAX_LAYERS];   // the same of every layer's latest step (or of the set-up of the cache)
+  bool dec_captured;              // a step of this cache was recorded by a stream capture
   int32_t h_dec_cap[CAKE_MAX_LAYERS];   // slots of the largest head of every layer
   int64_t wait_limit_cycles;      // bound of every device-side wait (0 = the default, about 2 s)
   int32_t debug_epoch_skew;       // test hook: added to the launch count the cross-CTA waits expect
@@ -228,6 +237,7 @@ int32_t launch_evict(cake_ctx* ctx, int32_t stage, cudaStream_t st);
 // decode.cu
 int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache, void* v_cache,
                             int64_t* row_offsets, cudaStream_t st);
+StepPlace step_place(cudaStream_t st);
 int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, const void* k_new,
                            const void* v_new, void* k_cache, void* v_cache, cudaStream_t st);
 int32_t launch_decode_read(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* positions, float* scores,

@@ -779,6 +779,22 @@ int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache,
   return run_gather(ctx, ptrs, ctx->d_dec_packed_off, ctx->d_dec_off, ctx->d_pos_packed, k_cache, v_cache, st);
 }
 
+StepPlace step_place(cudaStream_t st) {
+  StepPlace p = {0, 0};
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaError_t e = cudaStreamGetCaptureInfo(st, &capturing, &id);
+  if (e == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
+    e = cudaStreamGetId(st, &p.stream);
+  } else if (e == cudaSuccess) {
+    // a capture does not permit asking for the id: the handle, unless every thread has its own stream of it
+    p.capture = id;
+    p.stream = st == cudaStreamPerThread ? 0 : (unsigned long long)(uintptr_t)st;
+  }
+  if (e != cudaSuccess) { cudaGetLastError(); p.stream = 0; }
+  return p;
+}
+
 int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, const void* k_new,
                            const void* v_new, void* k_cache, void* v_cache, cudaStream_t st) {
   const cake_config& c = ctx->cfg;
@@ -817,11 +833,18 @@ int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, cons
   const bool use_cluster = aligned && (size_t)(G + 3) * words * sizeof(float) <= kDecSmemMax && !(env && env[0] == '0');
   // A step may start while the kernel before it in the stream still runs, read its layer's state and
   // bring the layer's keys towards the SMs, and then wait.  That state was last written by the same
-  // layer's previous step.  A step lets its successor start only after its own predecessor has
-  // finished, so everything but that one predecessor is complete by then; hence not when the
-  // predecessor may be this layer's own previous step, or the set-up of the cache.
-  const bool early = ctx->dec_last_layer >= 0 && ctx->dec_last_layer != layer;
-  ctx->dec_last_layer = use_cluster ? layer : -1;
+  // layer's previous step (or by the set-up of the cache).  A step lets its successor start only after its
+  // own predecessor in the stream has finished, so what was enqueued on this stream before the step before
+  // this one is complete by then.  Hence only when the step before this one is another layer's on this
+  // stream, and this layer's own one was on this stream too (a step on another stream may have been
+  // ordered before this one by an event that the launch waits for, or may not: no early start).  A captured
+  // graph runs as a whole behind everything before it, so steps that ran earlier are complete when it
+  // starts; steps beside a replayed graph cannot tell what it has stepped.
+  const StepPlace here = step_place(st);
+  auto same = [](const StepPlace& a, const StepPlace& b) { return a.stream != 0 && a.stream == b.stream && a.capture == b.capture; };
+  const StepPlace& own = ctx->dec_place[layer];
+  const bool early = ctx->dec_last_layer >= 0 && ctx->dec_last_layer != layer && same(ctx->dec_last, here) &&
+                     (here.capture ? own.capture != here.capture || same(own, here) : !ctx->dec_captured && same(own, here));
   cudaError_t e;
   if (use_cluster)
     e = c.dtype == CAKE_DTYPE_FP32 ? launch_step_cluster<float>(ctx->device, G, grid, csize, (int)words, early, st, A)
@@ -830,6 +853,9 @@ int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, cons
     e = c.dtype == CAKE_DTYPE_FP32 ? launch_step<float>(ctx->device, G, grid, smem, st, A)
                                    : launch_step<__nv_bfloat16>(ctx->device, G, grid, smem, st, A);
   count_launch();
+  ctx->dec_last_layer = use_cluster && e == cudaSuccess ? layer : -1;
+  ctx->dec_last = ctx->dec_place[layer] = here;
+  ctx->dec_captured = ctx->dec_captured || here.capture != 0;
   return cuda_status(e);
 }
 

@@ -4,6 +4,8 @@ is read back, the oracle takes the same step from that state, and the two result
 positions bit for bit, scores within 1e-3 relative, cache rows bit for bit.  Where the oracle's
 two lowest scores lie within 1e-3 of each other the device may evict either (fp32 against
 float64)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -181,3 +183,114 @@ def test_decode_tensors_off_a_32_byte_boundary_give_the_same_state():
     assert torch.equal(states[0][0], states[1][0]) and torch.equal(states[0][2], states[1][2])
     assert torch.allclose(states[0][1], states[1][1], rtol=1e-4, atol=1e-9)
     assert torch.equal(states[0][3], states[1][3]) and torch.equal(states[0][4], states[1][4])
+
+
+def decode_pair(w, tokens):
+    """Two contexts with the same finished prefill and decode cache, and the new rows of every step."""
+    qs, ks, vs = harness.device_inputs(w)
+    gen = torch.Generator().manual_seed(w.seed + 29)
+    shapes = [(w.n_q_heads, 1.5), (w.n_kv_heads, 1.0), (w.n_kv_heads, 1.0)]
+    new = [[[(torch.randn(len(w.seq_lens), h, w.head_dim, generator=gen) * s).to(w.torch_dtype).cuda() for h, s in shapes]
+            for _ in range(w.n_layers)] for _ in range(tokens)]
+    out = []
+    for _ in range(2):
+        cake = harness.cake_for(w)
+        cake.run(qs, ks, vs, w.cu_seqlens)
+        out.append((cake, *cake.decode_begin(ks, vs)[:2]))
+    torch.cuda.synchronize()
+    return out, new
+
+
+def assert_same_decode_state(w, one, two):
+    torch.cuda.synchronize()
+    budgets = one[0].get_budgets().cpu().numpy()
+    for r in range(len(w.seq_lens)):
+        for l in range(w.n_layers):
+            a, b = (c[0].decode_get_state(r, l, int(budgets[r, l])) for c in (one, two))
+            assert all(torch.equal(x, y) for x, y in zip(a, b)), (r, l)
+    assert torch.equal(one[1], two[1]) and torch.equal(one[2], two[2])
+    assert one[0].status() == 0 and two[0].status() == 0
+    one[0].destroy()
+    two[0].destroy()
+
+
+@pytest.mark.parametrize("layers,budget,streams", [(2, 900, (0, 1)), (3, 300, (0, 1, 0)), (4, 1200, (0, 0, 1, 1))])
+def test_decode_layers_on_streams_of_their_own(layers, budget, streams):
+    """Every layer is stepped on a fixed stream, the layers of a token interleaved over two of them: the
+    same states as with all steps on one stream."""
+    w = synth.scaled(synth.workload(3), n_layers=layers, n_q_heads=8, n_kv_heads=2, seq_lens=(budget * 2 + 77,),
+                     total_budget=layers * budget)
+    (one, two), new = decode_pair(w, tokens=12)
+    side = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for token in new:
+        for l, x in enumerate(token):
+            one[0].decode_step(l, *x, *one[1:])
+    for token in new:
+        for l, x in enumerate(token):
+            with torch.cuda.stream(side[streams[l]]):
+                two[0].decode_step(l, *x, *two[1:])
+    assert_same_decode_state(w, one, two)
+
+
+def capture(rt, streams, body):
+    """The graph of what `body` enqueues, captured on streams[0] with the others forked from it and joined."""
+    def ok(res):
+        assert int(res[0]) == 0, res[0]
+        return res[1:]
+    main = streams[0]
+    ok(rt.cudaStreamBeginCapture(main.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal))
+    body()
+    for s in streams[1:]:
+        main.wait_stream(s)
+    graph, = ok(rt.cudaStreamEndCapture(main.cuda_stream))
+    lib, count = ctypes.CDLL("libcudart.so.12"), ctypes.c_size_t(0)
+    handle = ctypes.c_void_p(int(graph))
+    assert lib.cudaGraphGetEdges_v2(handle, None, None, None, ctypes.byref(count)) == 0
+    nodes, data = [(ctypes.c_void_p * count.value)() for _ in range(2)], (ctypes.c_uint8 * (8 * count.value))()
+    assert lib.cudaGraphGetEdges_v2(handle, *nodes, data, ctypes.byref(count)) == 0
+    return graph, [data[8 * i + 2] for i in range(count.value)], ok          # (from_port, to_port, type, ...)
+
+
+def test_captured_decode_steps_start_early_only_behind_another_layers_step():
+    """In a capture the early start shows as the type of the edge between two launches (1: the second may
+    start before the first has finished).  Steps of two layers in turn on one stream have such edges, and the
+    replayed graph gives the states of plain steps; a layer's step right behind its own previous one, with
+    the other layer on another stream, has none."""
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    w = synth.scaled(synth.workload(3), n_layers=2, n_q_heads=8, n_kv_heads=2, seq_lens=(1900,), total_budget=2 * 900)
+    (one, two), new = decode_pair(w, tokens=4)
+    for token in new:
+        for l, x in enumerate(token):
+            one[0].decode_step(l, *x, *one[1:])
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(a):                        # outside a capture first: kernel attributes are set then
+        for l in range(2):
+            two[0].decode_step(l, *new[0][l], *two[1:])
+        torch.cuda.synchronize()
+
+    def in_turn():
+        with torch.cuda.stream(a):
+            for token in new[1:]:
+                for l, x in enumerate(token):
+                    two[0].decode_step(l, *x, *two[1:])
+
+    def own_predecessor():
+        with torch.cuda.stream(a):
+            two[0].decode_step(0, *new[1][0], *two[1:])
+        b.wait_stream(a)
+        with torch.cuda.stream(b):
+            two[0].decode_step(1, *new[1][1], *two[1:])
+        with torch.cuda.stream(a):
+            two[0].decode_step(0, *new[2][0], *two[1:])
+
+    graph, types, ok = capture(rt, [a, b], own_predecessor)          # never launched
+    assert types and all(t == 0 for t in types)
+    ok(rt.cudaGraphDestroy(graph))
+    graph, types, ok = capture(rt, [a], in_turn)
+    assert len(types) == 5 and all(t == 1 for t in types)
+    run, = ok(rt.cudaGraphInstantiate(graph, 0))
+    ok(rt.cudaGraphLaunch(run, a.cuda_stream))
+    torch.cuda.synchronize()
+    assert_same_decode_state(w, one, two)
+    ok(rt.cudaGraphExecDestroy(run))
+    ok(rt.cudaGraphDestroy(graph))
