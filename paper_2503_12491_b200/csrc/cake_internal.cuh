@@ -307,6 +307,37 @@ struct PerDeviceOnce {
   void mark(int device) { if (device >= 0 && device < kOnceDevices) done[device] = true; }
 };
 
+// The widest cluster a kernel may be launched with: `wide`, beyond the portable 8, only where the current
+// device can hold one such cluster of its largest CTAs (a partition of a device, or a share of its SMs, may
+// not, and the launch would fail), and never above CAKE_MAX_CLUSTER (environment).  `wide_fits` is what
+// cluster_fits said.
+template <typename Kernel>
+cudaError_t cluster_fits(Kernel kernel, int size, int threads, size_t smem, bool* fits) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)size, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)size;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+  *fits = e == cudaSuccess && n >= 1;
+  if (e == cudaErrorInvalidClusterSize) { cudaGetLastError(); return cudaSuccess; }
+  return e;
+}
+constexpr int kPortableCluster = 8;
+inline int widest_cluster(bool wide_fits, int wide) {
+  const char* env = getenv("CAKE_MAX_CLUSTER");
+  const int most = env && env[0] ? atoi(env) : wide;
+  const int w = wide_fits ? wide : kPortableCluster;
+  return most < 1 ? 1 : most < w ? most : w;
+}
+
 // Tracing spans (no-ops unless cake_profile_enable was called).
 int prof_begin(cake_ctx* ctx, int kind, cudaStream_t st);
 void prof_end(cake_ctx* ctx, int span, cudaStream_t st);

@@ -23,8 +23,8 @@ namespace cake {
 namespace {
 
 constexpr int DEC_THREADS = 512;
-constexpr int DEC_CLUSTER = 8;    // most CTAs that share a head in the cluster form of the step kernel,
-constexpr int DEC_CLUSTER_WIDE = 16;   //   and the most (beyond the portable 8) where the grid is small
+constexpr int DEC_CLUSTER = kPortableCluster;   // most CTAs that share a head in the cluster form of the step kernel,
+constexpr int DEC_CLUSTER_WIDE = 16;   //   and the most where the grid is small and the device holds such a cluster
 constexpr int DEC_CTA_ENTRIES = 256;       // entries per CTA up to which a head is spread no further
 constexpr size_t kDecSmemMax = 200 * 1024;
 constexpr int DEC_ROWS = 4;       // cache rows a half-warp has in flight in the logit loop
@@ -708,20 +708,30 @@ cudaError_t launch_step_cluster_g(dim3 grid, int csize, int cap_words, bool earl
   return cudaLaunchKernelEx(&cfg, decode_step_cluster_kernel<T, G>, A, csize, cap_words);
 }
 
+// Once per device: the kernels' attributes, and whether it holds a cluster of DEC_CLUSTER_WIDE of them all.
 template <typename T>
-cudaError_t launch_step_cluster(int device, int G, dim3 grid, int csize, int cap_words, bool early, cudaStream_t st,
-                                const DecodeArgs& A) {
+cudaError_t prepare_step_cluster(int device, bool* wide) {
   static PerDeviceOnce attr;
-  if (attr.need(device)) {
-    cudaError_t e = cudaSuccess;
+  static bool fits[kOnceDevices];
+  if (!attr.need(device)) { *wide = fits[device]; return cudaSuccess; }
+  cudaError_t e = cudaSuccess;
+  bool all = true, one;
 #define CAKE_DEC_ATTR(GG) \
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemMax); \
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
-    CAKE_DEC_ATTR(1); CAKE_DEC_ATTR(2); CAKE_DEC_ATTR(4); CAKE_DEC_ATTR(8);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemMax); \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); \
+  if (e == cudaSuccess) e = cluster_fits(decode_step_cluster_kernel<T, GG>, DEC_CLUSTER_WIDE, DEC_THREADS, kDecSmemMax, &one); \
+  all = all && e == cudaSuccess && one
+  CAKE_DEC_ATTR(1); CAKE_DEC_ATTR(2); CAKE_DEC_ATTR(4); CAKE_DEC_ATTR(8);
 #undef CAKE_DEC_ATTR
-    if (e != cudaSuccess) return e;
-    attr.mark(device);
-  }
+  if (e != cudaSuccess) return e;
+  if (device >= 0 && device < kOnceDevices) fits[device] = all;
+  attr.mark(device);
+  *wide = all;
+  return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t launch_step_cluster(int G, dim3 grid, int csize, int cap_words, bool early, cudaStream_t st, const DecodeArgs& A) {
   const size_t smem = (size_t)(G + 3) * cap_words * sizeof(float);
   switch (G) {
     case 1: return launch_step_cluster_g<T, 1>(grid, csize, cap_words, early, smem, st, A);
@@ -818,13 +828,17 @@ int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, cons
   // A head is spread over the fewest CTAs that leave each at most DEC_CTA_ENTRIES entries (one
   // pass of its sixteen warps over 16 key rows each), up to DEC_CLUSTER, or up to DEC_CLUSTER_WIDE
   // while the grid still fits the SMs (at one request of eight heads 64 CTAs would leave half of
-  // them idle).  Heads whose share does not fit a CTA's shared memory even then, tensors that do
+  // them idle) and the device holds such a cluster.  Heads whose share does not fit a CTA's shared memory even then, tensors that do
   // not start on a 32-byte boundary, and all heads with CAKE_DECODE_CLUSTER=0, stay on one CTA of
   // the form that reads 8 bytes at a time and can work in global memory.
   const int64_t max_cap = ctx->h_dec_cap[layer];
   const int64_t heads = (int64_t)c.n_kv_heads * ctx->n_req;
+  bool wide = false;
+  CAKE_CUDA_TRY(c.dtype == CAKE_DTYPE_FP32 ? prepare_step_cluster<float>(ctx->device, &wide)
+                                           : prepare_step_cluster<__nv_bfloat16>(ctx->device, &wide));
+  const int widest = widest_cluster(wide, DEC_CLUSTER_WIDE);
   int csize = 1;
-  while (max_cap > (int64_t)csize * DEC_CTA_ENTRIES &&
+  while (max_cap > (int64_t)csize * DEC_CTA_ENTRIES && csize * 2 <= widest &&
          (csize < DEC_CLUSTER || (csize < DEC_CLUSTER_WIDE && heads * csize * 2 <= ctx->n_sm)))
     csize *= 2;
   const int64_t words = (max_cap + csize - 1) / csize + 2 * (c.pool_kernel / 2) + 2;
@@ -847,8 +861,8 @@ int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, cons
                      (here.capture ? own.capture != here.capture || same(own, here) : !ctx->dec_captured && same(own, here));
   cudaError_t e;
   if (use_cluster)
-    e = c.dtype == CAKE_DTYPE_FP32 ? launch_step_cluster<float>(ctx->device, G, grid, csize, (int)words, early, st, A)
-                                   : launch_step_cluster<__nv_bfloat16>(ctx->device, G, grid, csize, (int)words, early, st, A);
+    e = c.dtype == CAKE_DTYPE_FP32 ? launch_step_cluster<float>(G, grid, csize, (int)words, early, st, A)
+                                   : launch_step_cluster<__nv_bfloat16>(G, grid, csize, (int)words, early, st, A);
   else
     e = c.dtype == CAKE_DTYPE_FP32 ? launch_step<float>(ctx->device, G, grid, smem, st, A)
                                    : launch_step<__nv_bfloat16>(ctx->device, G, grid, smem, st, A);

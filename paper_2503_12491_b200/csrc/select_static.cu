@@ -12,8 +12,9 @@ constexpr int SEL_THREADS = 512;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
 constexpr int kSelMaxWords = 32768;            // limit of the entry point: heads * ceil(n/32)
 constexpr int SEL_BINS = 2048;                 // digits of 11, 11 and 10 bits
-constexpr int SEL_CLUSTER = 8;                 // most CTAs per head; SEL_CLUSTER_WIDE where few heads leave SMs idle
-constexpr int SEL_CLUSTER_WIDE = 16;
+constexpr int SEL_CLUSTER = kPortableCluster;  // most CTAs per head; SEL_CLUSTER_WIDE where few heads leave SMs idle
+constexpr int SEL_CLUSTER_WIDE = 16;           //   and the device holds such a cluster
+constexpr int SEL_WIDE_CTAS = 128;             // CTAs (one per SM) up to which clusters of SEL_CLUSTER_WIDE are taken
 constexpr int kSelShare = 2048;                // values per CTA below which a head is spread no further
 constexpr int kSelSmemKeys = 40 * 1024;        // keys a CTA holds in shared memory; a larger share is read again
 
@@ -226,15 +227,21 @@ extern "C" int32_t cake_select_positions_static(const float* values, int32_t n_h
   int dev = -1;
   CAKE_CUDA_TRY(cudaGetDevice(&dev));
   static PerDeviceOnce attr;
+  static bool fits[kOnceDevices];
+  bool wide = dev >= 0 && dev < kOnceDevices && fits[dev];
   if (attr.need(dev)) {
     CAKE_CUDA_TRY(cudaFuncSetAttribute(select_positions_static, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemKeys * 4));
     CAKE_CUDA_TRY(cudaFuncSetAttribute(select_positions_static, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    CAKE_CUDA_TRY(cluster_fits(select_positions_static, SEL_CLUSTER_WIDE, SEL_THREADS, (size_t)kSelSmemKeys * 4, &wide));
+    if (dev >= 0 && dev < kOnceDevices) fits[dev] = wide;
     attr.mark(dev);
   }
   // as many CTAs per head as leave each kSelShare values, up to 8, or 16 where that still fits the
-  // device side by side (one 1024-thread CTA per SM)
+  // device side by side (one 512-thread CTA per SM)
+  const int widest = widest_cluster(wide, SEL_CLUSTER_WIDE);
   int csize = 1;
-  while ((int64_t)csize * kSelShare < n && (csize < SEL_CLUSTER || (csize < SEL_CLUSTER_WIDE && n_heads * csize * 2 <= 128))) csize *= 2;
+  while ((int64_t)csize * kSelShare < n && csize * 2 <= widest &&
+         (csize < SEL_CLUSTER || (csize < SEL_CLUSTER_WIDE && n_heads * csize * 2 <= SEL_WIDE_CTAS))) csize *= 2;
   const int share = ((n + csize - 1) / csize + 31) / 32 * 32;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n_heads * csize), 1, 1);

@@ -11,7 +11,7 @@ import pytest
 import torch
 
 from oracle import cake_oracle as O
-from paper_2503_12491_b200 import synth, harness
+from paper_2503_12491_b200 import binding, synth, harness
 from paper_2503_12491_b200.binding import CAKE_POOL_AVG, CAKE_POOL_MAX, CakeError, CAKE_ERR_STATE
 
 pytestmark = pytest.mark.gpu
@@ -292,5 +292,59 @@ def test_captured_decode_steps_start_early_only_behind_another_layers_step():
     ok(rt.cudaGraphLaunch(run, a.cuda_stream))
     torch.cuda.synchronize()
     assert_same_decode_state(w, one, two)
+    ok(rt.cudaGraphExecDestroy(run))
+    ok(rt.cudaGraphDestroy(graph))
+
+
+def cluster_widths(graph):
+    """The cluster dimension of every kernel of a captured graph."""
+    lib, n = ctypes.CDLL("libcudart.so.12"), ctypes.c_size_t(0)
+    handle = ctypes.c_void_p(int(graph))
+    assert lib.cudaGraphGetNodes(handle, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert lib.cudaGraphGetNodes(handle, nodes, ctypes.byref(n)) == 0
+    out = []
+    for node in nodes:
+        val = (ctypes.c_uint32 * 16)()
+        assert lib.cudaGraphKernelNodeGetAttribute(ctypes.c_void_p(node), 4, val) == 0      # cluster dimension
+        out.append(val[0])
+    return out
+
+
+@pytest.mark.parametrize("bound", [None, 16, 8, 4, 1])
+def test_cluster_width_follows_its_bound(monkeypatch, bound):
+    """Heads that the decode step spreads over 16 CTAs, and a selection that does: with a lower bound, as on a
+    device that holds no cluster of 16, the launches stay within it and the results are the same."""
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    w = synth.scaled(synth.workload(3), n_layers=1, n_q_heads=4, n_kv_heads=2, seq_lens=(8000,), total_budget=4500)
+    (one, two), new = decode_pair(w, tokens=2)
+    vals = torch.randn(2, 70001, generator=torch.Generator().manual_seed(3)).cuda()
+    want = binding.select_positions_static(vals, 900)
+    for token in new:
+        one[0].decode_step(0, *token[0], *one[1:])
+    if bound is not None:
+        monkeypatch.setenv("CAKE_MAX_CLUSTER", str(bound))
+    out = torch.empty_like(want)
+    two[0].decode_step(0, *new[0][0], *two[1:])
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+
+    def body():
+        with torch.cuda.stream(st):
+            two[0].decode_step(0, *new[1][0], *two[1:])
+            binding.select_positions_static(vals, 900, out=out)
+
+    graph, _, ok = capture(rt, [st], body)
+    assert sorted(cluster_widths(graph)) == [bound or 16, bound or 16]
+    run, = ok(rt.cudaGraphInstantiate(graph, 0))
+    ok(rt.cudaGraphLaunch(run, st.cuda_stream))
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    got, ref = ([x.clone() for x in c[0].decode_get_state(0, 0, 4500)] for c in (two, one))
+    assert torch.equal(got[0], ref[0]) and torch.equal(got[2], ref[2])
+    assert torch.allclose(got[1], ref[1], rtol=RTOL, atol=1e-12)
+    for c in (one, two):
+        assert c[0].status() == 0
+        c[0].destroy()
     ok(rt.cudaGraphExecDestroy(run))
     ok(rt.cudaGraphDestroy(graph))
