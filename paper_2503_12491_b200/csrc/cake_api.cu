@@ -15,6 +15,22 @@ namespace cake {
 static std::atomic<int64_t> g_launches{0};
 void count_launch(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+StepPlace step_place(cudaStream_t st) {
+  StepPlace p = {0, 0};
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaError_t e = cudaStreamGetCaptureInfo(st, &capturing, &id);
+  if (e == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
+    e = cudaStreamGetId(st, &p.stream);
+  } else if (e == cudaSuccess) {
+    // a capture does not permit asking for the id: the handle, unless every thread has its own stream of it
+    p.capture = id;
+    p.stream = st == cudaStreamPerThread ? 0 : (unsigned long long)(uintptr_t)st;
+  }
+  if (e != cudaSuccess) { cudaGetLastError(); p.stream = 0; }
+  return p;
+}
+
 int prof_begin(cake_ctx* ctx, int kind, cudaStream_t st) {
   Profiler& p = ctx->prof;
   if (!p.on || p.used >= p.cap) return -1;
@@ -380,6 +396,8 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
   ctx->alloc_of_buf[0] = ctx->alloc_of_buf[1] = -1;
   ctx->last_alloc = -1;
   ctx->arrived_budgets = -1;
+  ctx->pool_waited = -1;
+  ctx->score_stream = 0;
   CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int32_t), st));
   for (bool& r : ctx->pool_recorded) r = false;
   ctx->evict_recorded[0] = ctx->evict_recorded[1] = false;
@@ -397,10 +415,16 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   const int par = layer & 1;
   // The score kernel's outputs of a layer's place were last read by the pooling of layer - kScoreDepth
   // (the rest of that layer's cascade works on its own data and may still be running).  One wait serves
-  // this layer and the next kScoreWait - 1: the pooling stream runs in order.
-  const int place = layer % kScoreDepth, newest = layer + kScoreWait - 1 - kScoreDepth;
-  if (layer % kScoreWait == 0 && newest >= 0 && ctx->pool_recorded[newest % kScoreDepth])
-    CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[newest % kScoreDepth], 0));
+  // this layer and the next kScoreWait - 1 on this stream: the pooling stream runs in order.
+  const int place = layer % kScoreDepth, need = layer - kScoreDepth;
+  const unsigned long long sid = step_place(st).stream;
+  if (sid == 0 || sid != ctx->score_stream) ctx->pool_waited = -1;
+  ctx->score_stream = sid;
+  if (need >= 0 && ctx->pool_waited < need) {
+    const int newest = need + kScoreWait - 1;
+    if (ctx->pool_recorded[newest % kScoreDepth]) CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[newest % kScoreDepth], 0));
+    ctx->pool_waited = newest;
+  }
   int32_t rc = ctx->use_tc ? launch_score_tc(ctx, layer, q_win, k, lse, st)
                            : launch_score_simt(ctx, layer, q_win, k, lse, st);
   if (rc != CAKE_OK) return rc;

@@ -21,8 +21,9 @@ constexpr int kBins = 1 << kBinBits;
 constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling / scatter CTAs
 constexpr int kBitmapSmemWords = 48 * 1024;   // positions of up to 1.5 M tokens are ordered in shared memory
 constexpr int kScoreDepth = 8;        // layers whose score outputs may wait for their pooling
-constexpr int kScoreWait = 4;         // every so many layers the caller's stream waits for earlier pooling: an event
-                                      // wait between two score launches keeps the second from starting early
+constexpr int kScoreWait = 4;         // layers that one wait of the caller's stream for earlier pooling serves: an
+                                      // event wait between two score launches keeps the second from starting early
+static_assert(kScoreWait < kScoreDepth, "the pooling that is waited for is enqueued already");
 constexpr int kScoreGroups = 3;      // statistics warp groups per CTA of the tensor-core score kernel
 constexpr int kScoreWarps = 4 * kScoreGroups;   // statistics warps: one column-pass partial each
 
@@ -116,6 +117,8 @@ struct cake_ctx {
   cudaEvent_t ev_pool[cake::kScoreDepth];    // pooling (the last reader of the score outputs) and budgets of
                                              // layer % kScoreDepth have finished
   bool pool_recorded[cake::kScoreDepth];
+  int32_t pool_waited;              // newest layer whose pooling the stream of the latest score launch has waited for
+  unsigned long long score_stream;  // that stream (0: unknown)
   int32_t rows;            // R = G * S_w
   int64_t sel_budget;      // B' = B_total - L * S_w
   // ---- batch state (host) ----
@@ -217,6 +220,7 @@ struct cake_ctx {
 namespace cake {
 
 void count_launch(int64_t n = 1);
+StepPlace step_place(cudaStream_t st);
 
 // score_simt.cu
 int32_t simt_tile_keys(int rows);     // keys per tile: score units are multiples of it
@@ -237,7 +241,6 @@ int32_t launch_evict(cake_ctx* ctx, int32_t stage, cudaStream_t st);
 // decode.cu
 int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache, void* v_cache,
                             int64_t* row_offsets, cudaStream_t st);
-StepPlace step_place(cudaStream_t st);
 int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, const void* k_new,
                            const void* v_new, void* k_cache, void* v_cache, cudaStream_t st);
 int32_t launch_decode_read(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* positions, float* scores,

@@ -789,22 +789,6 @@ int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache,
   return run_gather(ctx, ptrs, ctx->d_dec_packed_off, ctx->d_dec_off, ctx->d_pos_packed, k_cache, v_cache, st);
 }
 
-StepPlace step_place(cudaStream_t st) {
-  StepPlace p = {0, 0};
-  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  unsigned long long id = 0;
-  cudaError_t e = cudaStreamGetCaptureInfo(st, &capturing, &id);
-  if (e == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
-    e = cudaStreamGetId(st, &p.stream);
-  } else if (e == cudaSuccess) {
-    // a capture does not permit asking for the id: the handle, unless every thread has its own stream of it
-    p.capture = id;
-    p.stream = st == cudaStreamPerThread ? 0 : (unsigned long long)(uintptr_t)st;
-  }
-  if (e != cudaSuccess) { cudaGetLastError(); p.stream = 0; }
-  return p;
-}
-
 int32_t launch_decode_step(cake_ctx* ctx, int32_t layer, const void* q_new, const void* k_new,
                            const void* v_new, void* k_cache, void* v_cache, cudaStream_t st) {
   const cake_config& c = ctx->cfg;

@@ -557,6 +557,46 @@ def test_runs_are_bitwise_reproducible():
     assert torch.equal(outs[0][3], outs[1][3])
 
 
+def test_scores_wait_for_the_pooling_whose_outputs_they_replace():
+    """Score outputs live in a ring of eight layers.  The pooling of every layer is held back behind a slow
+    stream that supplies layers 0 and 8; layer 9 takes the place of layer 1 on a stream that has waited for
+    nothing so far."""
+    w = synth.scaled(synth.workload(3), n_layers=12, n_q_heads=8, n_kv_heads=2, seq_lens=(700,), total_budget=12 * 90)
+    qs, ks, vs = harness.device_inputs(w)
+    given = torch.rand(w.n_kv_heads, w.total_tokens, device="cuda")
+    pref = torch.linspace(1.0, 2.0, 12, dtype=torch.float64, device="cuda").view(1, 12)
+
+    def run(slow, fast, hold):
+        cake = harness.cake_for(w)
+        cake.begin(w.cu_seqlens)
+        cake.set_preferences(pref)
+        torch.cuda.synchronize()
+        for l in range(12):
+            if l in (0, 8):
+                with torch.cuda.stream(slow):
+                    if l == 0 and hold:
+                        torch.cuda._sleep(100_000_000)           # 50 ms or more
+                    cake.set_indicators(l, given)
+            else:
+                with torch.cuda.stream(fast):
+                    cake.score_layer(l, qs[l], ks[l])
+            cake.allocate(l)
+            cake.evict(l)
+        out = cake.compact(ks, vs)
+        torch.cuda.synchronize()
+        assert cake.status() == 0
+        got = [x.clone() for x in out[2:]] + [x.clone() for x in cake.get_preferences()[:2]]
+        n = int(out[2][-1])
+        cake.destroy()
+        return n, got
+
+    main = torch.cuda.current_stream()
+    n, want = run(main, main, False)
+    m, got = run(torch.cuda.Stream(), torch.cuda.Stream(), True)
+    assert n == m and torch.equal(got[0], want[0]) and torch.equal(got[1][:n], want[1][:n])
+    assert torch.equal(got[2][:, 1:8], want[2][:, 1:8]) and torch.equal(got[3][:, 9:], want[3][:, 9:])
+
+
 def test_compaction_reads_values_from_pinned_host_memory():
     """V (and K) handed to the gather as page-locked host tensors give the same packed cache as
     device tensors: only the retained rows cross the bus."""
