@@ -111,7 +111,11 @@ typedef struct cake_config {
 } cake_config;
 
 /* Allocates a context (device state and scratch sized from the capacities) on
- * the current device.  The only entry point that allocates device memory. */
+ * the current device.  The only entry point that allocates device memory.
+ * Two parts only make the path faster and shrink where memory is short: the
+ * score outputs of up to 8 layers in flight (H_kv * max_total_tokens * 4 bytes a
+ * layer; 2 at least) and, for shapes and types without a tensor-core kernel, the
+ * logits kept between two kernels (CAKE_SIMT_SCORES_MB, default 256 MB). */
 int32_t cake_create(const cake_config* cfg, cake_ctx** out);
 /* Synchronises the device and frees everything the context owns. */
 int32_t cake_destroy(cake_ctx* ctx);

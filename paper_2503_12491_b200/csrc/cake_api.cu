@@ -222,7 +222,6 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && dev_alloc(&x->d_budget[0], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_budget[1], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_status, 1) == cudaSuccess;
-  for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_raw[i], (size_t)c.n_kv_heads * T) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_fresh[0], (size_t)c.n_kv_heads * T) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_fresh[1], (size_t)c.n_kv_heads * T) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_lists, (size_t)x->list_elems) == cudaSuccess;
@@ -244,12 +243,6 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     x->use_tc = tc_path_supported(c) && !(force && strcmp(force, "simt") == 0);
   }
   if (!x->use_tc) {
-    // all logits of a batch if they fit CAKE_SIMT_SCORES_MB (environment, default 256), at least one unit's
-    const char* mb = getenv("CAKE_SIMT_SCORES_MB");
-    const int64_t most = mb ? (int64_t)std::max(0, atoi(mb)) << 18 : kMaxScoreElems;
-    const int64_t per_key = (int64_t)c.n_kv_heads * x->rows;
-    x->scores_elems = std::max<int64_t>(kSimtMaxUnit * per_key, std::min<int64_t>(most, (T + R * kSimtMaxUnit) * per_key));
-    ok = ok && dev_alloc(&x->d_scores, (size_t)x->scores_elems) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_simt_arrivals, (size_t)R * c.n_kv_heads) == cudaSuccess;
     ok = ok && cudaMemset(x->d_simt_arrivals, 0, sizeof(uint32_t) * R * c.n_kv_heads) == cudaSuccess;
   }
@@ -261,10 +254,15 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     x->max_tc_segs = (int32_t)segs;
     x->max_tc_ops = (int32_t)(3 * segs + 8);
   }
-  {
+  // score outputs of one layer; two layers' at least, so that one is scored while the other is pooled
+  auto alloc_place = [&](int i) {
     const size_t a = (size_t)x->max_units * c.n_kv_heads, b = (size_t)x->max_tc_segs * kScoreWarps;
-    for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_colpart[i], (a > b ? a : b) * G * 2) == cudaSuccess;
-  }
+    return dev_alloc(&x->d_raw[i], (size_t)c.n_kv_heads * T) == cudaSuccess &&
+           dev_alloc(&x->d_colpart[i], (a > b ? a : b) * G * 2) == cudaSuccess &&
+           (!x->use_tc || dev_alloc(&x->d_hrow[i], (size_t)max_pairs * 128) == cudaSuccess);
+  };
+  const int places = std::min(kScoreDepth, c.n_layers);      // more than the layers have no use
+  while (ok && x->score_depth < std::min(2, places)) ok = alloc_place(x->score_depth++);
   if (x->use_tc) {
     const size_t n_index = 3 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
     ok = ok && cudaMallocHost((void**)&x->h_tc_ops, sizeof(ScoreOp) * x->max_tc_ops) == cudaSuccess;
@@ -274,7 +272,6 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     ok = ok && dev_alloc(&x->d_tc_sync, 2 * (size_t)max_pairs) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_rowpart, (size_t)x->max_tc_segs * kScoreGroups * 128) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_lse2_tc, (size_t)max_pairs * 128) == cudaSuccess;
-    for (int i = 0; i < kScoreDepth; ++i) ok = ok && dev_alloc(&x->d_hrow[i], (size_t)max_pairs * 128) == cudaSuccess;
   }
   // decode-time state: one slot per packed row plus one spare per (request, layer, head)
   x->dec_rows_cap = x->pos_packed_cap + x->max_lists;
@@ -293,7 +290,27 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && cudaMemset(x->d_P, 0, sizeof(double) * R * c.n_layers) == cudaSuccess;
   ok = ok && cudaMemset(x->d_H, 0, sizeof(double) * R * c.n_layers) == cudaSuccess;
   ok = ok && cudaMemset(x->d_V, 0, sizeof(double) * R * c.n_layers) == cudaSuccess;
-  if (!ok) { cudaGetLastError(); free_ctx(x); return CAKE_ERR_CUDA; }
+  // What only makes the path faster takes what is left: a smaller work area or fewer places are no error.
+  if (ok && !x->use_tc) {
+    // all logits of a batch if they fit CAKE_SIMT_SCORES_MB (environment, default 256), at least one unit's
+    const char* mb = getenv("CAKE_SIMT_SCORES_MB");
+    const int64_t most = mb ? (int64_t)std::max(0, atoi(mb)) << 18 : kMaxScoreElems;
+    const int64_t per_key = (int64_t)c.n_kv_heads * x->rows, least = kSimtMaxUnit * per_key;
+    x->scores_elems = std::max<int64_t>(least, std::min<int64_t>(most, (T + R * kSimtMaxUnit) * per_key));
+    while (!(ok = dev_alloc(&x->d_scores, (size_t)x->scores_elems) == cudaSuccess) && x->scores_elems > least)
+      x->scores_elems = std::max<int64_t>(least, x->scores_elems / 2);
+  }
+  while (ok && x->score_depth < places) {
+    const int i = x->score_depth;
+    if (!alloc_place(i)) {
+      cudaFree(x->d_raw[i]); cudaFree(x->d_colpart[i]); cudaFree(x->d_hrow[i]);
+      x->d_raw[i] = x->d_colpart[i] = x->d_hrow[i] = nullptr;
+      break;
+    }
+    ++x->score_depth;
+  }
+  cudaGetLastError();                             // an allocation above may have failed
+  if (!ok) { free_ctx(x); return CAKE_ERR_CUDA; }
   x->n_req = -1;                                  // no batch yet
   *out = x;
   return CAKE_OK;
@@ -413,15 +430,16 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   if (layer != ctx->n_ind || ctx->n_evicted != layer) return CAKE_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   const int par = layer & 1;
-  // The score kernel's outputs of a layer's place were last read by the pooling of layer - kScoreDepth
+  // The score kernel's outputs of a layer's place were last read by the pooling of layer - score_depth
   // (the rest of that layer's cascade works on its own data and may still be running).  One wait serves
-  // this layer and the next kScoreWait - 1 on this stream: the pooling stream runs in order.
-  const int place = layer % kScoreDepth, need = layer - kScoreDepth;
+  // the layers of half the ring on this stream, since the pooling stream runs in order: an event wait
+  // between two score launches keeps the second from starting early.
+  const int place = layer % kScoreDepth, need = layer - ctx->score_depth;
   const unsigned long long sid = step_place(st).stream;
   if (sid == 0 || sid != ctx->score_stream) ctx->pool_waited = -1;
   ctx->score_stream = sid;
   if (need >= 0 && ctx->pool_waited < need) {
-    const int newest = need + kScoreWait - 1;
+    const int newest = need + std::max(1, ctx->score_depth / 2) - 1;
     if (ctx->pool_recorded[newest % kScoreDepth]) CAKE_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev_pool[newest % kScoreDepth], 0));
     ctx->pool_waited = newest;
   }

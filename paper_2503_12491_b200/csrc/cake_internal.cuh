@@ -20,10 +20,7 @@ constexpr int kBinBits = 12;         // survivor lists are sorted by the top bit
 constexpr int kBins = 1 << kBinBits;
 constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling / scatter CTAs
 constexpr int kBitmapSmemWords = 48 * 1024;   // positions of up to 1.5 M tokens are ordered in shared memory
-constexpr int kScoreDepth = 8;        // layers whose score outputs may wait for their pooling
-constexpr int kScoreWait = 4;         // layers that one wait of the caller's stream for earlier pooling serves: an
-                                      // event wait between two score launches keeps the second from starting early
-static_assert(kScoreWait < kScoreDepth, "the pooling that is waited for is enqueued already");
+constexpr int kScoreDepth = 8;        // layers whose score outputs may wait for their pooling, where memory allows
 constexpr int kScoreGroups = 3;      // statistics warp groups per CTA of the tensor-core score kernel
 constexpr int kScoreWarps = 4 * kScoreGroups;   // statistics warps: one column-pass partial each
 
@@ -113,6 +110,8 @@ struct cake_ctx {
   cudaEvent_t ev_pool_side;         // scratch event: pooling stream -> caller's
   cudaEvent_t ev_evict[2];          // eviction stage of that parity has finished (it reads d_fresh of that parity)
   bool evict_recorded[2];
+  int32_t score_depth;              // places for score outputs: kScoreDepth, or fewer (see cake_create); layer l uses
+                                    // place l % score_depth
   cudaEvent_t ev_score[cake::kScoreDepth];   // score kernel of layer % kScoreDepth has finished
   cudaEvent_t ev_pool[cake::kScoreDepth];    // pooling (the last reader of the score outputs) and budgets of
                                              // layer % kScoreDepth have finished
@@ -150,7 +149,7 @@ struct cake_ctx {
   double* d_P;
   int32_t* d_budget[2];    // [max_requests][L] selectable budgets, double-buffered by stage parity
   int32_t* d_status;       // sticky device status word
-  float* d_raw[cake::kScoreDepth];     // [H_kv][max_total_tokens] un-pooled indicator, by layer % kScoreDepth
+  float* d_raw[cake::kScoreDepth];     // [H_kv][max_total_tokens] un-pooled indicator, by layer % score_depth
   float* d_fresh[2];       // [H_kv][max_total_tokens] pooled indicator of the newest layer, by layer parity
   uint2* d_lists;          // per (req, layer, head): n entries (ordered indicator key, position)
   int64_t list_elems;
@@ -214,7 +213,7 @@ struct cake_ctx {
   bool tc_direct;                 // every CTA merges the denominators of its own pass-B ops (single-wave plans)
   float4* d_tc_rowpart;           // [max_tc_segs][kScoreGroups][128]
   float* d_lse2_tc;               // [max_requests][H_kv][128], rows in tile order i*G + h
-  float* d_hrow[cake::kScoreDepth];   // [max_pairs][128] sum_j p log2 p per window row, by layer % kScoreDepth
+  float* d_hrow[cake::kScoreDepth];   // [max_pairs][128] sum_j p log2 p per window row, by layer % score_depth
 };
 
 namespace cake {

@@ -774,9 +774,9 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
   if (finalize) {
     F.on = 1;
     F.budgets = budgets ? 1 : 0;
-    F.colpart = ctx->d_colpart[layer % kScoreDepth];
+    F.colpart = ctx->d_colpart[layer % ctx->score_depth];
     F.pair_seg = ctx->use_tc ? ctx->d_tc_index + (ctx->n_req * c.n_kv_heads + 1) : nullptr;
-    F.hrow = ctx->use_tc && ctx->hhead_from_rows ? ctx->d_hrow[layer % kScoreDepth] : nullptr;
+    F.hrow = ctx->use_tc && ctx->hhead_from_rows ? ctx->d_hrow[layer % ctx->score_depth] : nullptr;
     F.headsum = ctx->d_headsum;
     F.arrivals = ctx->d_arrivals + ctx->max_pairs;
     // a long prompt has thousands of partial sums per head: a CTA per KV head; else one per request
@@ -788,7 +788,7 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
     F.inv_tau2 = 1.0 / (double)c.tau2;
   }
   ArriveArgs Q;
-  Q.raw = ctx->d_raw[layer % kScoreDepth];
+  Q.raw = ctx->d_raw[layer % ctx->score_depth];
   Q.fresh = ctx->d_fresh[layer & 1];
   Q.reqs = ctx->d_req;
   Q.hist = ctx->d_hist;

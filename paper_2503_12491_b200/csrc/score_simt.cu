@@ -400,7 +400,7 @@ int32_t run(cake_ctx* ctx, int32_t layer, const void* q_win, const void* k, cons
   sp = prof_begin(ctx, CAKE_PROF_SCORE, st);
   ColArgs B;
   B.units = ctx->d_units; B.lse2 = ctx->d_lse2; B.scores = ctx->d_scores;
-  B.raw = ctx->d_raw[layer % kScoreDepth]; B.colpart = ctx->d_colpart[layer % kScoreDepth];
+  B.raw = ctx->d_raw[layer % ctx->score_depth]; B.colpart = ctx->d_colpart[layer % ctx->score_depth];
   B.unit_keys = ctx->unit_keys; B.Hq = c.n_q_heads; B.Hkv = c.n_kv_heads; B.Sw = c.window;
   B.T_tokens = ctx->total_tokens; B.gamma = c.gamma; B.ddof = c.var_ddof; B.ind_mode = c.indicator_mode;
   for (int u0 = 0; u0 < ctx->n_units; u0 += slice) {

@@ -1563,9 +1563,9 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.lse2 = ctx->d_lse2_tc;
   P.lse_ext = lse;
   P.rowpart = ctx->d_tc_rowpart;
-  P.raw = ctx->d_raw[layer % kScoreDepth];
-  P.colpart = ctx->d_colpart[layer % kScoreDepth];
-  P.hrow = ctx->d_hrow[layer % kScoreDepth];
+  P.raw = ctx->d_raw[layer % ctx->score_depth];
+  P.colpart = ctx->d_colpart[layer % ctx->score_depth];
+  P.hrow = ctx->d_hrow[layer % ctx->score_depth];
   P.n_pairs = n_pairs;
   P.status = ctx->d_status;
   P.T = ctx->total_tokens;

@@ -319,6 +319,35 @@ def test_lists_at_the_edges_of_tiles_and_runs(seq_lens, budget, pool):
     cake.destroy()
 
 
+@pytest.mark.parametrize("make,tokens,short", [(bf16_case, 1 << 24, 600 << 20), (bf16_case, 1 << 24, 1400 << 20), (fp32_case, 1 << 22, 550 << 20)])
+def test_a_context_that_only_fits_with_less_scratch(make, tokens, short):
+    """With less free memory than a context takes when it can have all (the ring of score outputs, 268 MB a
+    layer for 2^24 tokens of 4 heads; 67 MB for 2^22, and 256 MB of logits), creation succeeds and results are the same."""
+    w = make(n_layers=9, n_q_heads=4, n_kv_heads=4, window=32, seq_lens=(900, 333), total_budget=9 * 90)
+    qs, ks, vs = harness.device_inputs(w)
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    before = free()
+    roomy = harness.cake_for(w, max_total_tokens=tokens)
+    size = before - free()
+    want = roomy.run(qs, ks, vs, w.cu_seqlens)
+    n = int(want[2][-1])
+    roomy.destroy()
+    assert size > 2 * short
+    hog = torch.empty(free() - (size - short), dtype=torch.uint8, device="cuda")
+    tight = harness.cake_for(w, max_total_tokens=tokens)
+    del hog
+    torch.cuda.empty_cache()
+    got = tight.run(qs, ks, vs, w.cu_seqlens)
+    assert all(torch.equal(x[:n], y[:n]) for x, y in zip(got, want))
+    assert tight.status() == 0
+    tight.destroy()
+
+
 @pytest.mark.parametrize("scores_mb", ["256", "0"])
 @pytest.mark.parametrize("dtype,hq,hkv,window,d,seq_lens", [
     ("fp32", 4, 4, 16, 64, (1100, 129, 17)),         # 16 rows
