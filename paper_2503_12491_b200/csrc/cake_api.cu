@@ -77,7 +77,7 @@ void free_ctx(cake_ctx* c) {
   if (!c) return;
   cudaFree(c->d_req); cudaFree(c->d_units); cudaFree(c->d_H); cudaFree(c->d_V); cudaFree(c->d_P);
   cudaFree(c->d_budget[0]); cudaFree(c->d_budget[1]); cudaFree(c->d_status);
-  for (int i = 0; i < kScoreDepth; ++i) { cudaFree(c->d_raw[i]); cudaFree(c->d_colpart[i]); cudaFree(c->d_hrow[i]); }
+  cudaFree(c->d_ring);
   cudaFree(c->d_fresh[0]); cudaFree(c->d_fresh[1]); cudaFree(c->d_lists); cudaFree(c->d_prefix); cudaFree(c->d_lstate);
   cudaFree(c->d_hist); cudaFree(c->d_fill[0]); cudaFree(c->d_fill[1]); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
@@ -254,15 +254,6 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     x->max_tc_segs = (int32_t)segs;
     x->max_tc_ops = (int32_t)(3 * segs + 8);
   }
-  // score outputs of one layer; two layers' at least, so that one is scored while the other is pooled
-  auto alloc_place = [&](int i) {
-    const size_t a = (size_t)x->max_units * c.n_kv_heads, b = (size_t)x->max_tc_segs * kScoreWarps;
-    return dev_alloc(&x->d_raw[i], (size_t)c.n_kv_heads * T) == cudaSuccess &&
-           dev_alloc(&x->d_colpart[i], (a > b ? a : b) * G * 2) == cudaSuccess &&
-           (!x->use_tc || dev_alloc(&x->d_hrow[i], (size_t)max_pairs * 128) == cudaSuccess);
-  };
-  const int places = std::min(kScoreDepth, c.n_layers);      // more than the layers have no use
-  while (ok && x->score_depth < std::min(2, places)) ok = alloc_place(x->score_depth++);
   if (x->use_tc) {
     const size_t n_index = 3 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
     ok = ok && cudaMallocHost((void**)&x->h_tc_ops, sizeof(ScoreOp) * x->max_tc_ops) == cudaSuccess;
@@ -290,24 +281,42 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && cudaMemset(x->d_P, 0, sizeof(double) * R * c.n_layers) == cudaSuccess;
   ok = ok && cudaMemset(x->d_H, 0, sizeof(double) * R * c.n_layers) == cudaSuccess;
   ok = ok && cudaMemset(x->d_V, 0, sizeof(double) * R * c.n_layers) == cudaSuccess;
-  // What only makes the path faster takes what is left: a smaller work area or fewer places are no error.
-  if (ok && !x->use_tc) {
-    // all logits of a batch if they fit CAKE_SIMT_SCORES_MB (environment, default 256), at least one unit's
+  // What only makes the path faster takes what is left, and may be smaller: the ring of score outputs (no
+  // more places than layers, two at least so that one layer is scored while another is pooled), then the
+  // SIMT path's logits.
+  auto round_up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+  const size_t n_part = std::max((size_t)x->max_units * c.n_kv_heads, (size_t)x->max_tc_segs * kScoreWarps) * G * 2;
+  const size_t raw_bytes = round_up((size_t)c.n_kv_heads * T * sizeof(float)), part_bytes = round_up(n_part * sizeof(float));
+  const size_t place_bytes = raw_bytes + part_bytes + (x->use_tc ? (size_t)max_pairs * 128 * sizeof(float) : 0);
+  // all logits of a batch if they fit CAKE_SIMT_SCORES_MB (environment, default 256), at least one unit's
+  auto alloc_scores = [&]() {
+    if (x->use_tc) return true;
     const char* mb = getenv("CAKE_SIMT_SCORES_MB");
     const int64_t most = mb ? (int64_t)std::max(0, atoi(mb)) << 18 : kMaxScoreElems;
     const int64_t per_key = (int64_t)c.n_kv_heads * x->rows, least = kSimtMaxUnit * per_key;
     x->scores_elems = std::max<int64_t>(least, std::min<int64_t>(most, (T + R * kSimtMaxUnit) * per_key));
-    while (!(ok = dev_alloc(&x->d_scores, (size_t)x->scores_elems) == cudaSuccess) && x->scores_elems > least)
+    for (;;) {
+      if (dev_alloc(&x->d_scores, (size_t)x->scores_elems) == cudaSuccess) return true;
+      if (x->scores_elems == least) return false;
       x->scores_elems = std::max<int64_t>(least, x->scores_elems / 2);
-  }
-  while (ok && x->score_depth < places) {
-    const int i = x->score_depth;
-    if (!alloc_place(i)) {
-      cudaFree(x->d_raw[i]); cudaFree(x->d_colpart[i]); cudaFree(x->d_hrow[i]);
-      x->d_raw[i] = x->d_colpart[i] = x->d_hrow[i] = nullptr;
-      break;
     }
-    ++x->score_depth;
+  };
+  const int places = std::min(kScoreDepth, c.n_layers), least_places = std::min(2, places);
+  for (int d = places; ok && x->score_depth == 0; d = std::max(least_places, d / 2)) {
+    const bool fits = dev_alloc(&x->d_ring, d * place_bytes) == cudaSuccess;
+    if (fits && alloc_scores()) {
+      x->score_depth = d;
+    } else {
+      if (fits) cudaFree(x->d_ring);
+      x->d_ring = nullptr;
+      ok = d > least_places;
+    }
+  }
+  for (int i = 0; i < x->score_depth; ++i) {
+    uint8_t* p = x->d_ring + i * place_bytes;
+    x->d_raw[i] = (float*)p;
+    x->d_colpart[i] = (float*)(p + raw_bytes);
+    if (x->use_tc) x->d_hrow[i] = (float*)(p + raw_bytes + part_bytes);
   }
   cudaGetLastError();                             // an allocation above may have failed
   if (!ok) { free_ctx(x); return CAKE_ERR_CUDA; }

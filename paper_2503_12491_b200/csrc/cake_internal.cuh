@@ -149,6 +149,7 @@ struct cake_ctx {
   double* d_P;
   int32_t* d_budget[2];    // [max_requests][L] selectable budgets, double-buffered by stage parity
   int32_t* d_status;       // sticky device status word
+  uint8_t* d_ring;         // one allocation for the places of d_raw, d_colpart and d_hrow
   float* d_raw[cake::kScoreDepth];     // [H_kv][max_total_tokens] un-pooled indicator, by layer % score_depth
   float* d_fresh[2];       // [H_kv][max_total_tokens] pooled indicator of the newest layer, by layer parity
   uint2* d_lists;          // per (req, layer, head): n entries (ordered indicator key, position)
