@@ -102,13 +102,18 @@ bool ptrs(PyObject* seq, at::ScalarType want, bool pinned_ok, std::vector<const 
 }
 
 // One pointer per layer in both arrays; missing ones are null.
-bool per_layer(std::vector<const void*>& k, std::vector<const void*>& v, size_t layers) {
-  if (k.size() > layers || v.size() > layers) {
+bool per_layer(std::vector<const void*>& k, std::vector<const void*>& v, long layers) {
+  if (PyErr_Occurred()) return false;               // `layers` was not a number
+  if (layers < 0 || layers > CAKE_MAX_LAYERS) {
+    PyErr_SetString(PyExc_ValueError, "no such number of layers");
+    return false;
+  }
+  if (k.size() > (size_t)layers || v.size() > (size_t)layers) {
     PyErr_SetString(PyExc_IndexError, "more tensors than layers");
     return false;
   }
-  k.resize(layers, nullptr);
-  v.resize(layers, nullptr);
+  k.resize((size_t)layers, nullptr);
+  v.resize((size_t)layers, nullptr);
   return true;
 }
 
@@ -237,7 +242,7 @@ PyObject* compact(PyObject*, PyObject* const* a, Py_ssize_t n) {
   // rows over the bus
   if (!ptrs(a[5], e, true, k) || !ptrs(a[6], e, true, v) || !ptr(a[7], kAny, &ko) || !ptr(a[8], kAny, &vo) ||
       !ptr(a[9], at::ScalarType::Long, &off) || !ptr(a[10], at::ScalarType::Int, &pos)) return nullptr;
-  if (!per_layer(k, v, (size_t)INT(1))) return nullptr;
+  if (!per_layer(k, v, PyLong_AsLong(a[1]))) return nullptr;
   cake_ctx* c = ctx_of(a[0]);
   const int32_t lo = INT(3), hi = INT(4);
   DONE(lib.compact(c, lo, hi, k.data(), v.data(), ko, vo, (int64_t*)off, (int32_t*)pos, st));
@@ -253,9 +258,9 @@ PyObject* compact_int4(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!ptrs(a[4], e, false, k) || !ptrs(a[5], e, false, v)) return nullptr;
   for (int i = 0; i < 9; ++i)
     if (!ptr(a[6 + i], kAny, &o[i])) return nullptr;
+  if (!per_layer(k, v, PyLong_AsLong(a[1]))) return nullptr;
   cake_ctx* c = ctx_of(a[0]);
   const int32_t layers = INT(1), group = INT(3);
-  if (!per_layer(k, v, (size_t)layers)) return nullptr;
   DONE(lib.compact_int4(c, 0, layers, k.data(), v.data(), group, (uint8_t*)o[0], (float*)o[1], (float*)o[2], (uint8_t*)o[3],
                         (float*)o[4], (float*)o[5], (int64_t*)o[6], (int64_t*)o[7], (int32_t*)o[8], st));
 }
@@ -263,24 +268,41 @@ PyObject* compact_int4(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // clear_unused(tensors, offsets): zeroes the rows of every tensor beyond the last entry of its offsets
 PyObject* clear_unused(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!arity(n, 2)) return nullptr;
-  std::vector<const void*> t, off;
-  if (!ptrs(a[0], kAny, false, t) || !ptrs(a[1], at::ScalarType::Long, false, off)) return nullptr;
-  const int32_t m = (int32_t)t.size();
   void* bufs[CAKE_CLEAR_MAX];
   const int64_t* used[CAKE_CLEAR_MAX];
   int64_t bytes[CAKE_CLEAR_MAX], rows[CAKE_CLEAR_MAX];
-  if (m > CAKE_CLEAR_MAX || off.size() != t.size()) {
-    PyErr_SetString(PyExc_ValueError, "clear_unused: too many tensors");
-    return nullptr;
-  }
-  for (int32_t i = 0; i < m; ++i) {
-    const at::Tensor& x = THPVariable_Unpack(PySequence_Fast_GET_ITEM(a[0], i));
-    const at::Tensor& o = THPVariable_Unpack(PySequence_Fast_GET_ITEM(a[1], i));
-    bufs[i] = const_cast<void*>(t[i]);
-    rows[i] = x.size(0);
-    bytes[i] = rows[i] > 0 ? (int64_t)x.nbytes() / rows[i] : 0;
-    used[i] = (const int64_t*)off[i] + (o.numel() - 1);
-  }
+  int32_t m = 0;
+  auto fill = [&](PyObject* tensors, PyObject* offsets) {
+    const Py_ssize_t count = PySequence_Fast_GET_SIZE(tensors);
+    if (count > CAKE_CLEAR_MAX || PySequence_Fast_GET_SIZE(offsets) != count) {
+      PyErr_SetString(PyExc_ValueError, "clear_unused: too many tensors, or not an offsets tensor for each");
+      return false;
+    }
+    for (; m < (int32_t)count; ++m) {
+      PyObject *x = PySequence_Fast_GET_ITEM(tensors, m), *o = PySequence_Fast_GET_ITEM(offsets, m);
+      void* off;
+      if (!THPVariable_Check(x) || !THPVariable_Check(o)) {
+        PyErr_SetString(PyExc_TypeError, "expected a torch.Tensor");
+        return false;
+      }
+      if (!ptr(x, kAny, &bufs[m]) || !ptr(o, at::ScalarType::Long, &off)) return false;
+      const at::Tensor &t = THPVariable_Unpack(x), &u = THPVariable_Unpack(o);
+      if (t.dim() < 1 || u.numel() < 1) {
+        PyErr_SetString(PyExc_ValueError, "clear_unused: a tensor without rows, or empty offsets");
+        return false;
+      }
+      rows[m] = t.size(0);
+      bytes[m] = rows[m] > 0 ? (int64_t)t.nbytes() / rows[m] : 0;
+      used[m] = (const int64_t*)off + (u.numel() - 1);
+    }
+    return true;
+  };
+  PyObject* tensors = PySequence_Fast(a[0], "expected a sequence of tensors");
+  PyObject* offsets = tensors ? PySequence_Fast(a[1], "expected a sequence of tensors") : nullptr;
+  const bool ok = offsets && fill(tensors, offsets);
+  Py_XDECREF(tensors);
+  Py_XDECREF(offsets);
+  if (!ok) return nullptr;
   DONE(lib.clear_unused(m, bufs, bytes, rows, used, st));
 }
 

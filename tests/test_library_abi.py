@@ -3,6 +3,10 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
+
+import pytest
 
 from paper_2503_12491_b200 import binding, build
 
@@ -40,6 +44,18 @@ def test_config_struct_matches_header_layout():
     assert binding.CakeConfig.indicator_mode.offset == 72
     assert binding.CakeConfig.alloc_mode.offset == 76
     assert binding.CakeConfig.pyramid_slope.offset == 80
+
+
+@pytest.mark.parametrize("call", ["clear_unused((None,), (None,))", "clear_unused(iter([None]), iter([None]))",
+                                  "clear_unused((torch.zeros(2),), ())", "clear_unused(1, 2)",
+                                  "compact(0, -1, True, 0, 0, [], [], None, None, None, None)",
+                                  "compact(0, 'x', True, 0, 0, [], [], None, None, None, None)",
+                                  "compact_int4(0, -1, True, 32, [], [], *[None] * 9)"])
+def test_arguments_the_native_marshalling_cannot_take_raise(call):
+    """In a process of their own: a Python error, not the end of the process."""
+    code = f"import torch; from paper_2503_12491_b200 import binding; binding.load_library(); binding._fast.{call}"
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 1 and re.search(r"^(TypeError|ValueError): ", r.stderr, flags=re.M), (r.returncode, r.stderr[-300:])
 
 
 def test_argument_errors_need_no_gpu():
