@@ -9,6 +9,7 @@ library is missing or a tensor is not on a CUDA device the call fails.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import List, Optional, Sequence, Tuple
@@ -114,10 +115,22 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         if name not in ("cake_packed_rows_bound", "cake_strerror", "cake_launch_count",
                         "cake_decode_rows_bound"):
             fn.restype = i32
-    from . import _cake_py
-    _cake_py.init(path)
-    _lib, _fast = lib, _cake_py
+    fast = _load_native()
+    fast.init(path)
+    _lib, _fast = lib, fast
     return lib
+
+
+def _load_native():
+    """The extension module built for this interpreter and this torch.  Raises if there is none."""
+    from .build import binding_path
+    path = binding_path()
+    if not os.path.exists(path):
+        raise ImportError(f"{path} not found: build it with `python -m paper_2503_12491_b200.build`")
+    spec = importlib.util.spec_from_file_location(__package__ + "._cake_py", path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
 
 
 def strerror(code: int) -> str:

@@ -1,4 +1,4 @@
-"""Builds libcake.so (sm_100a only, nvcc) and _cake_py.so (the binding's native half, g++) in-tree.
+"""Builds libcake.so (sm_100a only, nvcc) and the binding's native half (_cake_py.*.so, g++) in-tree.
 
     python -m paper_2503_12491_b200.build [--force] [--verbose]
 """
@@ -17,10 +17,16 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libcake.so")
 PY_SOURCE = os.path.join(CSRC, "py_args.cpp")
-PY_LIB = os.path.join(PKG, "_cake_py.so")
 
 SOURCES = ["cake_api.cu", "score_simt.cu", "score_tc.cu", "cascade.cu", "compact.cu",
            "decode.cu", "quant.cu", "select_static.cu"]
+
+
+def binding_path() -> str:
+    """The binding's native half for this interpreter and this torch: its file name has both, since it is
+    built against either's ABI and another one's must not be loaded."""
+    import torch
+    return os.path.join(PKG, f"_cake_py.torch-{torch.__version__}.{sysconfig.get_config_var('SOABI')}.so")
 
 
 def _nvcc() -> str:
@@ -54,8 +60,8 @@ def _run(cmd: List[str], what: str, verbose: bool) -> None:
 
 def build_binding(force: bool = False, verbose: bool = False) -> None:
     """Compiles the native half of binding.py against this interpreter and its torch."""
-    deps = [PY_SOURCE, os.path.join(INCLUDE, "cake.h")]
-    if not force and os.path.exists(PY_LIB) and all(os.path.getmtime(f) <= os.path.getmtime(PY_LIB) for f in deps):
+    deps, out = [PY_SOURCE, os.path.join(INCLUDE, "cake.h")], binding_path()
+    if not force and os.path.exists(out) and all(os.path.getmtime(f) <= os.path.getmtime(out) for f in deps):
         return
     import torch
     home = os.path.dirname(torch.__file__)
@@ -64,8 +70,8 @@ def build_binding(force: bool = False, verbose: bool = False) -> None:
     _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", INCLUDE,
           "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(home, "include"), "-isystem", cuda,
-          PY_SOURCE, "-o", PY_LIB, "-L", libs, f"-Wl,-rpath,{libs}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
-          "-lc10_cuda", "-ldl"], "_cake_py.so", verbose)
+          PY_SOURCE, "-o", out, "-L", libs, f"-Wl,-rpath,{libs}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
+          "-lc10_cuda", "-ldl"], os.path.basename(out), verbose)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -5,8 +5,10 @@ import os
 import re
 import subprocess
 import sys
+import sysconfig
 
 import pytest
+import torch
 
 from paper_2503_12491_b200 import binding, build
 
@@ -56,6 +58,18 @@ def test_arguments_the_native_marshalling_cannot_take_raise(call):
     code = f"import torch; from paper_2503_12491_b200 import binding; binding.load_library(); binding._fast.{call}"
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 1 and re.search(r"^(TypeError|ValueError): ", r.stderr, flags=re.M), (r.returncode, r.stderr[-300:])
+
+
+def test_native_half_belongs_to_this_interpreter_and_torch(monkeypatch):
+    """The file name has both; what was built for another torch is neither loaded nor taken as up to date."""
+    build.build()
+    path = build.binding_path()
+    assert os.path.exists(path) and torch.__version__ in path and sysconfig.get_config_var("SOABI") in path
+    assert binding._load_native().__file__ == path
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".other")
+    assert build.binding_path() != path
+    with pytest.raises(ImportError, match="build it with"):
+        binding._load_native()
 
 
 def test_argument_errors_need_no_gpu():
