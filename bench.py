@@ -26,7 +26,7 @@ if ROOT not in sys.path:
 METRIC = "CAKE score+evict+compact prompt tokens/s"
 # DRAM bytes of one score-kernel launch at workload 4 from the ncu capture under profiles/;
 # set to None whenever the kernel changes until the counters are taken again.
-SCORE_KERNEL_DRAM_BYTES = None
+SCORE_KERNEL_DRAM_BYTES = 285221376 + 11139584
 UNIT = "tokens/s"
 
 
@@ -350,9 +350,8 @@ def main():
                 "unit": "GB/s", "frac": (achieved / hbm_peak) if achieved else None,
                 "peak_kind": f"{peak_kind} copy bandwidth",
                 "traffic": SCORE_KERNEL_DRAM_BYTES if args.workload == 4 else None,
-                "traffic_source": "profiles/score_fused_kernel_llama31-8b-gqa-128k_2layers.md "
-                                  "(dram__bytes_read.sum + dram__bytes_write.sum of one launch; a "
-                                  "launch of the reduced case is a full-size launch)",
+                "traffic_source": "ncu: dram__bytes_read.sum + dram__bytes_write.sum of one launch of "
+                                  "the two-layer profiling case, whose launches are full-size",
                 "bytes_per_launch": per_launch_bytes, "ms_per_launch": dom_ms,
                 "launches_timed": prof[dom]["spans"],
                 "blocks": block_stats(block_ms, block_mhz, args.steps),

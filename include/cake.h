@@ -250,8 +250,9 @@ int32_t cake_status(cake_ctx* ctx, int32_t* device_status_out, void* stream);
 
 /* ---- tracing ------------------------------------------------------------ */
 #define CAKE_PROF_SCORE       0  /* window scores: softmax denominators and column statistics   */
-#define CAKE_PROF_FINALIZE    1  /* preference + pooling                                         */
-#define CAKE_PROF_ALLOCATE    2
+#define CAKE_PROF_FINALIZE    1  /* preference, pooling and the budgets of the layer's own stage */
+#define CAKE_PROF_ALLOCATE    2  /* budgets computed by a launch of their own: stages whose
+                                    preferences were set by the caller; else no spans            */
 #define CAKE_PROF_EVICT       3
 #define CAKE_PROF_COMPACT     4
 #define CAKE_PROF_KINDS       5
@@ -302,9 +303,11 @@ int32_t cake_uses_tensor_cores(const cake_ctx* ctx);
  *                       positions_out int32 [H_kv][len], scores_out fp32 [H_kv][len] (0 for the
  *                       window entries), slots_out int32 [H_kv][len] (slot of each entry inside
  *                       its head's cap slots); any may be NULL.
- * A head with more than 200 KB / (4 * (G + 1)) slots (10239 at G = 4) does not fit the step
- * kernel's shared memory and works in a global-memory area of the context instead (same
- * results, a slower step for that head). */
+ * Heads of more than 256 slots are spread over a thread-block cluster of up to 16 CTAs.  One CTA
+ * works on a head by itself where the tensors do not start on a 32-byte boundary or the cluster form is
+ * switched off (CAKE_DECODE_CLUSTER=0), and where a CTA's share of the head does not fit its shared
+ * memory; a head of more than 200 KB / (4 * (G + 1)) slots (10239 at G = 4) then works in a
+ * global-memory area of the context (same results, a slower step). */
 int64_t cake_decode_rows_bound(const cake_ctx* ctx);
 int32_t cake_decode_begin(cake_ctx* ctx, const void* const* k_layers, const void* const* v_layers,
                           void* k_cache, void* v_cache, int64_t* row_offsets_out, int32_t update_mode,

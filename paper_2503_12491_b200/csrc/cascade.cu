@@ -46,7 +46,8 @@ __device__ inline int split_span(int N, int want) {
 // own.  (As CTAs of a team each they spread over all the SMs that are free in the moment between two
 // score launches, and the next one, whose CTAs need whole SMs, waits for them: 136 against 119 us per
 // 128K layer.  As one team of 1024 an SM has a single chain of scans and barriers at a time: with 256 lists
-// of 2K tokens 97 us for the pooling and 75 us for the scatter, now 36 and 32.)
+// of 2K tokens 97 us for the pooling and 75 us for the scatter beside the scoring, 43 and 28 as it is; 36
+// and 29 by themselves.)
 constexpr int TEAMS = 4;
 constexpr int TEAM_THREADS = 256;
 constexpr int TEAM_WARPS = TEAM_THREADS / 32;

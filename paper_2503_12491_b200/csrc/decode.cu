@@ -121,7 +121,8 @@ __device__ __forceinline__ void worse_of(float& v, int& i, float ov, int oi) {
   if (ov < v || (ov == v && oi > i)) { v = ov; i = oi; }
 }
 
-// One CTA per (KV head, request).  Dynamic shared memory: p[G][cap] (logits, then unnormalised
+// One CTA per (KV head, request): heads that the cluster form below does not take (see
+// launch_decode_step).  Dynamic shared memory: p[G][cap] (logits, then unnormalised
 // probabilities by slot) and abar[cap] (group-mean attention by rank).
 template <typename T, int G>
 __global__ void __launch_bounds__(DEC_THREADS)
@@ -484,10 +485,11 @@ constexpr unsigned long long kNoKey = ~0ull;
 // memory from the first read on, so its shift needs no further meeting.
 //
 // Bound: the latency of one chain per layer and token (state -> slots -> key rows -> two cluster
-// barriers -> stores), about 8 us of it with heads of up to 256 entries per CTA; the keys of a layer
-// (8 MB at budgets of 4096) take 1.3 us at the copy rate.  Cut by slot with a third meeting for the
-// pooled window, a fourth for the list shift, and shuffles for the dot products it was 22 us per
-// launch at budgets of 4096 and 37 us for four requests at 768; now 12 and 10.
+// barriers -> stores); the keys of a layer (8 MB at budgets of 4096) take 1.3 us at the copy rate, 30 %
+// of the issue slots and 10 % of the DRAM rate are used.  A launch by itself takes 11 to 14 us at
+// budgets of 4096 and 10 to 11 us for four requests at 768; launches that start early follow one another every
+// 8.3 us (128K prompt) to 9.4 us.  Cut by slot with a third meeting for the pooled window, a fourth for
+// the list shift, and shuffles for the dot products they followed every 26 us.
 // Dynamic shared memory: (G + 3) words per entry of the largest window (logits, mean, slot, score).
 template <typename T, int G>
 __global__ void __launch_bounds__(DEC_THREADS, 2)

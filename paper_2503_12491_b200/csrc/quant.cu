@@ -206,9 +206,11 @@ constexpr int QU_WARPS = 4;
 // so that each lane computes one scale (an IEEE division) for one row and group instead of all
 // of them for every row.
 //
-// Bound: instruction issue, closely followed by memory (rows in, codes and scales out).  One warp per
+// Bound: the latency of a warp's chain (positions, rows, ranges, rows again, codes) at the 20 warps that
+// 80 registers leave an SM; neither issue slots (54 % busy; ALU and FMA pipes 36 % each) nor DRAM (34 %) are
+// full: 60 us for 262 K rows, 190 us for 1.05 M (GQA 32/8, d = 128, group 32).  One warp per
 // row with its own search for the row's block and a division near every half-integer, and a CTA per
-// key group, took 562 + 445 us for 1.05 M rows (GQA 32/8, d = 128, group 32).  Keeping the 32 key rows in
+// key group, took 562 + 445 us for 1.05 M rows.  Keeping the 32 key rows in
 // registers instead of reading them twice halved the warps in flight and took 1.2 times as long.
 template <typename T, int D, int GW, bool kVec>
 __global__ void __launch_bounds__(QU_WARPS * 32, sizeof(T) == 2 ? 6 : 5)

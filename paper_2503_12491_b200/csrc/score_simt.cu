@@ -59,8 +59,9 @@ template <typename T, int TY> struct Shape {
   static constexpr size_t kSmem = 2 * (size_t)STAGE * sizeof(T) + 8 * NT * sizeof(float2);
 };
 
-// One CTA per (unit, KV head).  Bound: the FMA pipe (393 M FMAs per layer at 128 rows, d = 128 and 4 heads of
-// 6K keys: 11 us).  The next piece of the rows is copied to shared memory while a piece is multiplied, and
+// One CTA per (unit, KV head).  Bound: issue slots (61 % busy) and the last wave: 393 M FMAs per layer at
+// 128 rows, d = 128 and 4 heads of 6K keys are 11 us of the FMA pipe, which is 45 % busy in the 38 us that it
+// takes; 376 CTAs for 444 places leave an SM with two or three.  The next piece of the rows is copied to shared memory while a piece is multiplied, and
 // three CTAs share an SM.  (One CTA per SM that staged whole rows of 134 KB before it multiplied took
 // 56 us there, and its second pass over the keys another 45.)
 template <typename T, int TY>
@@ -265,7 +266,8 @@ struct ColArgs {
 };
 
 // One CTA per (unit, KV head): 64 keys at a time, a lane per key, and four quarters of the window rows
-// on two warps each.  Bound: exponentials and the latency of the loads.
+// on two warps each.  Bound: the latency of the loads: 14 us for 4 heads of 6K keys and 128 rows at 30 % of the
+// issue slots and 7 % of the special-function unit.
 constexpr int COL_KEYS = 64;
 template <int GM>          // query heads per KV head, at most
 __global__ void __launch_bounds__(NT)

@@ -126,7 +126,7 @@ def test_decode_other_update_readings(mode):
 
 @pytest.mark.parametrize("cluster", ["1", "0"])
 def test_decode_large_heads(monkeypatch, cluster):
-    """Heads of 512 slots or more are spread over a thread-block cluster; with that form switched
+    """Heads of more than 256 slots are spread over a thread-block cluster; with that form switched
     off a head beyond the 5688 slots that G = 8 leaves in shared memory works in the context's
     global work area.  Both must match the oracle like the one-CTA form does."""
     monkeypatch.setenv("CAKE_DECODE_CLUSTER", cluster)

@@ -2,11 +2,11 @@
 
 `cake_select_positions_static` serves callers that may not allocate device memory at call
 time (code inside another framework's memory plan, latency-critical serving loops): its
-scratch is a fixed array inside the library.  Here its output is compared, bit for bit as for
+working memory is the shared memory of its kernel.  Here its output is compared, bit for bit as for
 every index result in this suite, with what the ordinary entry points (cake_set_indicators ->
 cake_allocate -> cake_evict -> cake_get_positions on a one-layer context) select from the
-same values, on two calls in a row so that the second one meets the first one's leftovers in
-the shared scratch.  This file sorts last on purpose: a run that stops at the first failure
+same values, on two calls in a row so that the second one meets what the first one left in
+shared memory.  This file sorts last on purpose: a run that stops at the first failure
 has then already run every other test.
 """
 import numpy as np
@@ -66,7 +66,7 @@ def test_static_selection_rejects_what_does_not_fit():
     lib = binding.load_library()
     vals = torch.zeros(1, 64, dtype=torch.float32, device="cuda")
     out = torch.zeros(1, 64, dtype=torch.int32, device="cuda")
-    # 33 heads of 32768 values need 33792 bitmap words: one more than the built-in scratch holds
+    # 33 heads of 32768 values: 33792 words of 32 values, beyond the limit of 32768
     rc = lib.cake_select_positions_static(vals.data_ptr(), 33, 32768, 8, out.data_ptr(), None)
     assert rc == CAKE_ERR_CAPACITY
     assert lib.cake_select_positions_static(vals.data_ptr(), 1, 64, 65, out.data_ptr(), None) == CAKE_ERR_ARG
