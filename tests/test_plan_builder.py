@@ -1,6 +1,7 @@
 """The score kernel's launch plan, built and checked on the host alone (no GPU): random ragged
 batches, head counts and SM counts through cake_plan_check, which verifies tile coverage, the
-order of every CTA's program, the wave span of merge groups and the table bounds."""
+order of every CTA's program, the wave span of merge groups, the table bounds and the slots of the
+rows that statistics warps exchange."""
 import ctypes
 
 import numpy as np
