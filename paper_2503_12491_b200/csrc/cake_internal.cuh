@@ -313,9 +313,9 @@ struct PerDeviceOnce {
 // The widest cluster a kernel may be launched with: `wide`, beyond the portable 8, only where the current
 // device can hold one such cluster of its largest CTAs (a partition of a device, or a share of its SMs, may
 // not, and the launch would fail), and never above CAKE_MAX_CLUSTER (environment).  `wide_fits` is what
-// cluster_fits said.
+// cluster_fits said; it allows the kernel such clusters, and answers no where the device cannot say.
 template <typename Kernel>
-cudaError_t cluster_fits(Kernel kernel, int size, int threads, size_t smem, bool* fits) {
+bool cluster_fits(Kernel kernel, int size, int threads, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)size, 1, 1);
   cfg.blockDim = dim3((unsigned)threads, 1, 1);
@@ -328,10 +328,10 @@ cudaError_t cluster_fits(Kernel kernel, int size, int threads, size_t smem, bool
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
-  *fits = e == cudaSuccess && n >= 1;
-  if (e == cudaErrorInvalidClusterSize) { cudaGetLastError(); return cudaSuccess; }
-  return e;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess && n >= 1;
 }
 constexpr int kPortableCluster = 8;
 inline int widest_cluster(bool wide_fits, int wide) {

@@ -717,12 +717,10 @@ cudaError_t prepare_step_cluster(int device, bool* wide) {
   static bool fits[kOnceDevices];
   if (!attr.need(device)) { *wide = fits[device]; return cudaSuccess; }
   cudaError_t e = cudaSuccess;
-  bool all = true, one;
+  bool all = true;
 #define CAKE_DEC_ATTR(GG) \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemMax); \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_step_cluster_kernel<T, GG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); \
-  if (e == cudaSuccess) e = cluster_fits(decode_step_cluster_kernel<T, GG>, DEC_CLUSTER_WIDE, DEC_THREADS, kDecSmemMax, &one); \
-  all = all && e == cudaSuccess && one
+  all = e == cudaSuccess && cluster_fits(decode_step_cluster_kernel<T, GG>, DEC_CLUSTER_WIDE, DEC_THREADS, kDecSmemMax) && all
   CAKE_DEC_ATTR(1); CAKE_DEC_ATTR(2); CAKE_DEC_ATTR(4); CAKE_DEC_ATTR(8);
 #undef CAKE_DEC_ATTR
   if (e != cudaSuccess) return e;

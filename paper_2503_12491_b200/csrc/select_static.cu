@@ -231,8 +231,7 @@ extern "C" int32_t cake_select_positions_static(const float* values, int32_t n_h
   bool wide = dev >= 0 && dev < kOnceDevices && fits[dev];
   if (attr.need(dev)) {
     CAKE_CUDA_TRY(cudaFuncSetAttribute(select_positions_static, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemKeys * 4));
-    CAKE_CUDA_TRY(cudaFuncSetAttribute(select_positions_static, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    CAKE_CUDA_TRY(cluster_fits(select_positions_static, SEL_CLUSTER_WIDE, SEL_THREADS, (size_t)kSelSmemKeys * 4, &wide));
+    wide = cluster_fits(select_positions_static, SEL_CLUSTER_WIDE, SEL_THREADS, (size_t)kSelSmemKeys * 4);
     if (dev >= 0 && dev < kOnceDevices) fits[dev] = wide;
     attr.mark(dev);
   }
