@@ -19,8 +19,8 @@
  *     none synchronises the host with the device except cake_status,
  *     cake_profile_read and cake_destroy, which say so.
  *   - Stream order.  cake_score_layer runs on the caller's stream.  Everything
- *     that follows a layer's scoring (pooling, preference, cake_allocate,
- *     cake_evict) is enqueued on streams the context owns, ordered after that
+ *     that follows a layer's scoring (pooling, preference, cake_allocate) is
+ *     enqueued on a stream the context owns, ordered after that
  *     layer's score kernel by events, so that it runs beside the scoring of the
  *     following layers.  cake_compact, every cake_get_* / cake_set_* call, cake_begin
  *     and cake_status first make the stream they are given wait for that
@@ -161,10 +161,10 @@ int32_t cake_allocate(cake_ctx* ctx, int32_t stage, void* stream);
  * among the stored (indicator, position) pairs; survivors keep their stored
  * indicator.  The window tokens are always kept.  Needs cake_allocate(stage)
  * and stages in order.
- * The stored pairs of a layer are kept sorted by the leading bits of the
- * indicator (written once, when the layer arrives); a later, smaller budget
- * only moves the list's threshold, which selects the same set as a TopK on the
- * surviving pairs would. */
+ * Budgets only shrink, so the set that a TopK on the surviving pairs would leave
+ * is the first entries of all of the layer's stored pairs, as many as the budget
+ * says: it is found where it is read (cake_compact, the getters), and this call
+ * enqueues no work of its own. */
 int32_t cake_evict(cake_ctx* ctx, int32_t stage, void* stream);
 
 /* Gathers the retained rows of layers [layer_lo, layer_hi) (Eq. 12: K^ = K[D,:],
@@ -253,13 +253,13 @@ int32_t cake_status(cake_ctx* ctx, int32_t* device_status_out, void* stream);
 #define CAKE_PROF_FINALIZE    1  /* preference, pooling and the budgets of the layer's own stage */
 #define CAKE_PROF_ALLOCATE    2  /* budgets computed by a launch of their own: stages whose
                                     preferences were set by the caller; else no spans            */
-#define CAKE_PROF_EVICT       3
+#define CAKE_PROF_EVICT       3  /* no spans: an eviction enqueues nothing of its own             */
 #define CAKE_PROF_COMPACT     4
 #define CAKE_PROF_KINDS       5
 /* While enabled, every stage of the path brackets its kernels with CUDA events
  * on the stream the stage runs on: the caller's stream for the score kernel and
- * the compaction, the context's own streams for pooling/preference, budgets and
- * eviction (this perturbs back-to-back launches slightly). */
+ * the compaction, the context's own stream for pooling/preference and budgets
+ * (this perturbs back-to-back launches slightly). */
 int32_t cake_profile_enable(cake_ctx* ctx, int32_t on);
 /* Synchronises `stream`; returns, per CAKE_PROF_* kind, the milliseconds and
  * the number of bracketed spans accumulated since the last read (HOST arrays

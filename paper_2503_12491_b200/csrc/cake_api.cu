@@ -78,8 +78,7 @@ void free_ctx(cake_ctx* c) {
   cudaFree(c->d_req); cudaFree(c->d_units); cudaFree(c->d_H); cudaFree(c->d_V); cudaFree(c->d_P);
   cudaFree(c->d_budget[0]); cudaFree(c->d_budget[1]); cudaFree(c->d_status);
   cudaFree(c->d_ring);
-  cudaFree(c->d_fresh[0]); cudaFree(c->d_fresh[1]); cudaFree(c->d_lists); cudaFree(c->d_prefix); cudaFree(c->d_lstate);
-  cudaFree(c->d_hist); cudaFree(c->d_fill[0]); cudaFree(c->d_fill[1]); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
+  cudaFree(c->d_store); cudaFree(c->d_prefix); cudaFree(c->d_hist); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
   cudaFree(c->d_scores); cudaFree(c->d_simt_arrivals);
   cudaFree(c->d_rowpart);
@@ -94,15 +93,12 @@ void free_ctx(cake_ctx* c) {
   if (c->h_units) cudaFreeHost(c->h_units);
   if (c->upload_done) cudaEventDestroy(c->upload_done);
   if (c->ev_main) cudaEventDestroy(c->ev_main);
-  if (c->ev_side) cudaEventDestroy(c->ev_side);
   for (int i = 0; i < kScoreDepth; ++i) {
     if (c->ev_score[i]) cudaEventDestroy(c->ev_score[i]);
     if (c->ev_pool[i]) cudaEventDestroy(c->ev_pool[i]);
   }
   if (c->ev_pool_side) cudaEventDestroy(c->ev_pool_side);
-  for (int i = 0; i < 2; ++i) if (c->ev_evict[i]) cudaEventDestroy(c->ev_evict[i]);
   if (c->pool_st) cudaStreamDestroy(c->pool_st);
-  if (c->side) cudaStreamDestroy(c->side);
   if (c->prof.spans) {
     for (int i = 0; i < c->prof.cap; ++i) {
       if (c->prof.spans[i].a) cudaEventDestroy(c->prof.spans[i].a);
@@ -114,18 +110,15 @@ void free_ctx(cake_ctx* c) {
   delete c;
 }
 
-// Orders the internal streams after everything enqueued so far on the caller's stream.
+// Orders the internal stream after everything enqueued so far on the caller's stream.
 cudaError_t side_after(cake_ctx* c, cudaStream_t st) {
   cudaError_t e = cudaEventRecord(c->ev_main, st);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_main, 0);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->pool_st, c->ev_main, 0);
   return e;
 }
-// Orders the caller's stream after everything enqueued so far on the internal streams.
+// Orders the caller's stream after everything enqueued so far on the internal stream.
 cudaError_t main_after_side(cake_ctx* c, cudaStream_t st) {
-  cudaError_t e = cudaEventRecord(c->ev_side, c->side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_side, 0);
-  if (e == cudaSuccess) e = cudaEventRecord(c->ev_pool_side, c->pool_st);
+  cudaError_t e = cudaEventRecord(c->ev_pool_side, c->pool_st);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_pool_side, 0);
   return e;
 }
@@ -187,29 +180,24 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   const int64_t R = c.max_requests;
   // a unit never spans requests: at most T / kSimtMinUnit + R units
   x->max_units = (int32_t)(T / kSimtMinUnit + R + 1);
-  x->list_elems = T * c.n_layers * c.n_kv_heads;
   x->max_lists = R * c.n_layers * c.n_kv_heads;
   {
     // packed rows: H_kv * sum_r min(B_total, L * N_r) <= H_kv * min(R * B_total, L * T)
     const int64_t a = R * c.total_budget, b = (int64_t)c.n_layers * T;
     x->pos_packed_cap = (int64_t)c.n_kv_heads * (a < b ? a : b);
     // a request longer than the shared-memory bitmap orders its positions in global scratch:
-    // one bitmap of ceil(n/32) words per (request, layer, head) list
-    x->bitmap_words = T > (int64_t)kBitmapSmemWords * 32
-                          ? (int64_t)c.n_layers * c.n_kv_heads * (T / 32 + R + 1) : 0;
+    // one bitmap of ceil((n + 3)/32) words per (request, layer, head)
+    x->bitmap_words = T + 3 > (int64_t)kBitmapSmemWords * 32
+                          ? (int64_t)c.n_layers * c.n_kv_heads * (T / 32 + 2 * R + 1) : 0;
   }
   x->h_cu = (int64_t*)calloc((size_t)R + 1, sizeof(int64_t));
   bool ok = x->h_cu != nullptr;
   ok = ok && cudaMallocHost((void**)&x->h_req, sizeof(ReqInfo) * R) == cudaSuccess;
   ok = ok && cudaMallocHost((void**)&x->h_units, sizeof(ScoreUnit) * x->max_units) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->upload_done, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && cudaStreamCreateWithFlags(&x->side, cudaStreamNonBlocking) == cudaSuccess;
   ok = ok && cudaStreamCreateWithFlags(&x->pool_st, cudaStreamNonBlocking) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_pool_side, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 2; ++i)
-    ok = ok && cudaEventCreateWithFlags(&x->ev_evict[i], cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_main, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && cudaEventCreateWithFlags(&x->ev_side, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < kScoreDepth; ++i) {
     ok = ok && cudaEventCreateWithFlags(&x->ev_score[i], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&x->ev_pool[i], cudaEventDisableTiming) == cudaSuccess;
@@ -222,14 +210,10 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && dev_alloc(&x->d_budget[0], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_budget[1], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_status, 1) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_fresh[0], (size_t)c.n_kv_heads * T) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_fresh[1], (size_t)c.n_kv_heads * T) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_lists, (size_t)x->list_elems) == cudaSuccess;
+  // (vector loads of a row's end may reach seven values beyond the last row)
+  ok = ok && dev_alloc(&x->d_store, (size_t)c.n_layers * c.n_kv_heads * T + 8) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_prefix, (size_t)x->max_lists * (kBins + 1)) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_lstate, (size_t)x->max_lists) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_hist, (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_fill[0], (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
-  ok = ok && dev_alloc(&x->d_fill[1], (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_arrivals, (size_t)R * c.n_kv_heads + R) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_headsum, (size_t)R * c.n_q_heads * 2) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_pos_packed, (size_t)x->pos_packed_cap) == cudaSuccess;
@@ -361,15 +345,13 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
     ctx->unit_keys = unit_keys;
     int32_t nu = 0;
     ctx->max_n_tokens = 0;
-    int64_t list_off = 0, bound = 0;
+    int64_t bound = 0;
     for (int r = 0; r < n_req; ++r) {
       ReqInfo& q = ctx->h_req[r];
       q.cu = cu[r];
       q.N = (int32_t)(cu[r + 1] - cu[r]);
       q.n = q.N - c.window;
       q.keep_all = q.N <= c.total_budget / c.n_layers ? 1 : 0;
-      q.list_off = list_off;
-      list_off += (int64_t)q.n * c.n_layers * c.n_kv_heads;
       if (q.N > ctx->max_n_tokens) ctx->max_n_tokens = q.N;
       q.unit0 = nu;
       for (int32_t k0 = 0; k0 < q.N; k0 += unit_keys) {
@@ -382,7 +364,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       const int64_t full = (int64_t)c.n_layers * q.N;
       bound += (int64_t)c.n_kv_heads * (c.total_budget < full ? c.total_budget : full);
     }
-    if (list_off > ctx->list_elems || nu > ctx->max_units) return CAKE_ERR_CAPACITY;
+    if (nu > ctx->max_units) return CAKE_ERR_CAPACITY;
     if (ctx->use_tc) {
       const int32_t prc = tc_build_plan(ctx, n_req);
       if (prc != CAKE_OK) return prc;
@@ -426,7 +408,6 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
   ctx->score_stream = 0;
   CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(int32_t), st));
   for (bool& r : ctx->pool_recorded) r = false;
-  ctx->evict_recorded[0] = ctx->evict_recorded[1] = false;
   CAKE_CUDA_TRY(side_after(ctx, st));
   return CAKE_OK;
 }
@@ -438,9 +419,8 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   if (ctx->n_req > 0 && (!q_win || !k)) return CAKE_ERR_ARG;
   if (layer != ctx->n_ind || ctx->n_evicted != layer) return CAKE_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
-  const int par = layer & 1;
   // The score kernel's outputs of a layer's place were last read by the pooling of layer - score_depth
-  // (the rest of that layer's cascade works on its own data and may still be running).  One wait serves
+  // (nothing later reads them).  One wait serves
   // the layers of half the ring on this stream, since the pooling stream runs in order: an event wait
   // between two score launches keeps the second from starting early.
   const int place = layer % kScoreDepth, need = layer - ctx->score_depth;
@@ -455,12 +435,9 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   int32_t rc = ctx->use_tc ? launch_score_tc(ctx, layer, q_win, k, lse, st)
                            : launch_score_simt(ctx, layer, q_win, k, lse, st);
   if (rc != CAKE_OK) return rc;
-  // Pooling, the preference and the stage's budgets run on their own stream beside the next layer's
-  // scoring and beside the eviction of the layer before; the pooled buffer, the scatter cursors and the
-  // budgets of this parity were last read by the eviction of layer - 2.
+  // Pooling, the preference and the stage's budgets run on their own stream beside the next layer's scoring.
   CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_score[place], st));
   CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_score[place], 0));
-  if (ctx->evict_recorded[par]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_evict[par], 0));
   const int sp = prof_begin(ctx, CAKE_PROF_FINALIZE, ctx->pool_st);
   const bool budgets = ctx->last_alloc < layer;      // nobody has asked for a later stage's before
   rc = launch_arrive(ctx, layer, true, true, budgets, ctx->pool_st);
@@ -480,11 +457,9 @@ int32_t cake_allocate(cake_ctx* ctx, int32_t stage, void* stream) {
   if (stage >= ctx->n_pref) return CAKE_ERR_STATE;
   (void)stream;                      // ordered by the internal streams
   // The scores' launch has already computed the budgets of its own stage, unless preferences were set
-  // since; any other stage is computed here.  Its buffer was last read by the eviction of stage - 2,
-  // and the budgets of stage - 1, which it falls back to, were written on this stream.
+  // since; any other stage is computed here, behind the budgets of stage - 1, which it falls back to.
   if (ctx->arrived_budgets != stage) {
     cudaStream_t ast = ctx->pool_st;
-    if (ctx->evict_recorded[stage & 1]) CAKE_CUDA_TRY(cudaStreamWaitEvent(ast, ctx->ev_evict[stage & 1], 0));
     const int sp = prof_begin(ctx, CAKE_PROF_ALLOCATE, ast);
     const int32_t rc = launch_allocate(ctx, stage, ast);
     prof_end(ctx, sp, ast);
@@ -505,13 +480,9 @@ int32_t cake_evict(cake_ctx* ctx, int32_t stage, void* stream) {
   if (ctx->alloc_of_buf[stage & 1] != stage) return CAKE_ERR_STATE;
   if (stage > 0 && ctx->alloc_of_buf[(stage + 1) & 1] != stage - 1) return CAKE_ERR_STATE;
   (void)stream;
-  CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_pool[stage % kScoreDepth], 0));
-  const int sp = prof_begin(ctx, CAKE_PROF_EVICT, ctx->side);
-  int32_t rc = launch_evict(ctx, stage, ctx->side);
-  prof_end(ctx, sp, ctx->side);
-  if (rc != CAKE_OK) return rc;
-  CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_evict[stage & 1], ctx->side));
-  ctx->evict_recorded[stage & 1] = true;
+  // The eviction of a stage is its budgets: every layer keeps the first entries of its stored indicators in the
+  // order of EVICT, as many as its budget says, and budgets only shrink (Proposition 1), so that set is the same
+  // whether it is cut down stage by stage or found where it is read (sorted_positions).
   ctx->n_evicted = stage + 1;
   return CAKE_OK;
 }
@@ -585,7 +556,7 @@ int32_t cake_get_indicators(cake_ctx* ctx, int32_t layer, float* out, void* stre
   if (ctx->n_req < 0 || layer != ctx->n_ind - 1) return CAKE_ERR_STATE;
   if (ctx->total_tokens == 0) return CAKE_OK;
   CAKE_CUDA_TRY(main_after_side(ctx, (cudaStream_t)stream));
-  CAKE_CUDA_TRY(cudaMemcpyAsync(out, ctx->d_fresh[layer & 1],
+  CAKE_CUDA_TRY(cudaMemcpyAsync(out, layer_store(ctx, layer),
                                 sizeof(float) * ctx->cfg.n_kv_heads * ctx->total_tokens,
                                 cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
   return CAKE_OK;
@@ -612,12 +583,11 @@ int32_t cake_set_indicators(cake_ctx* ctx, int32_t layer, const float* in, void*
   // earlier stages may still be working on the internal streams
   CAKE_CUDA_TRY(main_after_side(ctx, (cudaStream_t)stream));
   if (ctx->total_tokens > 0)
-    CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_fresh[layer & 1], in,
+    CAKE_CUDA_TRY(cudaMemcpyAsync(layer_store(ctx, layer), in,
                                   sizeof(float) * ctx->cfg.n_kv_heads * ctx->total_tokens,
                                   cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
   CAKE_CUDA_TRY(side_after(ctx, (cudaStream_t)stream));
-  // bucket histogram of the supplied values (they are taken as already pooled); the cursors of this
-  // parity were last used by the eviction of layer - 2, which `stream` has waited for
+  // bucket histogram of the supplied values (they are taken as already pooled)
   const int32_t rc = launch_arrive(ctx, layer, false, false, false, ctx->pool_st);
   if (rc != CAKE_OK) return rc;
   CAKE_CUDA_TRY(cudaEventRecord(ctx->ev_pool[layer % kScoreDepth], ctx->pool_st));
@@ -631,8 +601,8 @@ int32_t cake_set_preferences(cake_ctx* ctx, int32_t n_set, const double* P, void
   if (!ctx || !P) return CAKE_ERR_ARG;
   if (ctx->n_req < 0) return CAKE_ERR_STATE;
   if (n_set < 1 || n_set > ctx->cfg.n_layers) return CAKE_ERR_ARG;
-  // A layer that has been evicted stored only the entries its budget could still reach; a new
-  // preference could make that budget grow again (Proposition 1 would no longer hold).
+  // A new preference could make the budget of a layer that has been evicted grow again (Proposition 1 would
+  // no longer hold).
   if (ctx->n_evicted > 0) return CAKE_ERR_STATE;
   if (ctx->n_req > 0) {
     CAKE_CUDA_TRY(main_after_side(ctx, (cudaStream_t)stream));
@@ -694,7 +664,6 @@ int32_t cake_profile_enable(cake_ctx* ctx, int32_t on) {
 
 int32_t cake_profile_read(cake_ctx* ctx, double* ms_out, int64_t* spans_out, void* stream) {
   if (!ctx || !ms_out || !spans_out) return CAKE_ERR_ARG;
-  CAKE_CUDA_TRY(cudaStreamSynchronize(ctx->side));
   CAKE_CUDA_TRY(cudaStreamSynchronize(ctx->pool_st));
   CAKE_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
   for (int k = 0; k < CAKE_PROF_KINDS; ++k) { ms_out[k] = 0.0; spans_out[k] = 0; }

@@ -16,10 +16,12 @@ constexpr int kSimtMinUnit = 64;      // fewest keys of a score unit of the SIMT
 constexpr int kSimtMaxUnit = 1024;
 constexpr int64_t kMaxScoreElems = 64ll << 20;   // logits the SIMT kernels keep between their two steps (256 MB)
 constexpr int kSimtThreads = 256;
-constexpr int kBinBits = 12;         // survivor lists are sorted by the top bits of the indicator
+constexpr int kBinBits = 12;         // buckets of the indicators: their top bits
 constexpr int kBins = 1 << kBinBits;
-constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling / scatter CTAs
+constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling
 constexpr int kBitmapSmemWords = 48 * 1024;   // positions of up to 1.5 M tokens are ordered in shared memory
+
+constexpr int kSelectSmemWords = 50 * 1024;   // dynamic shared memory of the selection: bitmap and list of candidates
 constexpr int kScoreDepth = 8;        // layers whose score outputs may wait for their pooling, where memory allows
 constexpr int kScoreGroups = 3;      // statistics warp groups per CTA of the tensor-core score kernel
 constexpr int kScoreWarps = 4 * kScoreGroups;   // statistics warps: one column-pass partial each
@@ -31,7 +33,6 @@ struct ReqInfo {
   int32_t n;         // N - S_w non-window tokens
   int32_t keep_all;  // 1: N <= floor(B_total/L), nothing is evicted
   int32_t pad;
-  int64_t list_off;  // first entry of this request's lists; list (layer, head) holds n entries
   int32_t unit0;     // first score unit of the request
   int32_t nunits;    // number of score units of the request
 };
@@ -63,16 +64,6 @@ struct ScoreOp {
   int32_t pad;
 };
 
-// Retained set of one (request, layer, head) list, whose entries (ordered key, position) are stored by
-// bucket.  The first three fields are derived from the list and the budgets of the moment when the
-// retained set is read out (sorted_positions).
-struct ListState {
-  int32_t bucket;        // threshold bucket d; all buckets before it are kept; -1: nothing kept
-  uint32_t thr_key;      // inside bucket d an entry is kept if key > thr_key,
-  int32_t pos_cut;       //   or key == thr_key and position <= pos_cut
-  int32_t kept;          // budget the list arrived with: entries beyond it are not stored
-};
-
 // Where a decode step was enqueued: the stream, by its unique id or in a capture by its handle (0:
 // unknown), and the stream capture that recorded it (0: none, the step ran).
 struct StepPlace {
@@ -102,14 +93,10 @@ struct cake_ctx {
   int n_sm;
   int n_sm_score;          // SMs the persistent score kernel occupies; the rest stay free for the
                            // cascade kernels of the previous layer, which run beside it
-  // The cascade of layer l (pooling, preference, budgets, eviction) runs on an internal side
-  // stream while the caller's stream already scores layer l+1; events order the two.
-  cudaStream_t side;
-  cudaStream_t pool_st;             // pooling, preference and budgets of layer l+1, beside the eviction of layer l
-  cudaEvent_t ev_main, ev_side;     // scratch events: caller's stream -> side, side -> caller's
-  cudaEvent_t ev_pool_side;         // scratch event: pooling stream -> caller's
-  cudaEvent_t ev_evict[2];          // eviction stage of that parity has finished (it reads d_fresh of that parity)
-  bool evict_recorded[2];
+  // What follows the scores of layer l (pooling, preference, budgets) runs on an internal stream
+  // while the caller's stream already scores layer l+1; events order the two.
+  cudaStream_t pool_st;             // pooling, preference and budgets
+  cudaEvent_t ev_main, ev_pool_side;   // scratch events: caller's stream -> pool_st, and back
   int32_t score_depth;              // places for score outputs: kScoreDepth, or fewer (see cake_create); layer l uses
                                     // place l % score_depth
   cudaEvent_t ev_score[cake::kScoreDepth];   // score kernel of layer % kScoreDepth has finished
@@ -151,14 +138,10 @@ struct cake_ctx {
   int32_t* d_status;       // sticky device status word
   uint8_t* d_ring;         // one allocation for the places of d_raw, d_colpart and d_hrow
   float* d_raw[cake::kScoreDepth];     // [H_kv][max_total_tokens] un-pooled indicator, by layer % score_depth
-  float* d_fresh[2];       // [H_kv][max_total_tokens] pooled indicator of the newest layer, by layer parity
-  uint2* d_lists;          // per (req, layer, head): n entries (ordered indicator key, position)
-  int64_t list_elems;
-  int32_t* d_prefix;       // [max_lists][kBins+1] bucket offsets of every list
-  cake::ListState* d_lstate;   // [max_lists]
-  int64_t max_lists;
+  float* d_store;          // [L][H_kv][tokens of the batch] pooled indicators of every layer, +inf on the windows
+  int64_t max_lists;       // (request, layer, head) triples
+  int32_t* d_prefix;       // [max_lists][kBins+1] bucket offsets of every (request, layer, head)
   uint32_t* d_hist;        // [max_pairs][kBins] bucket histogram of the arriving layer (zero at rest)
-  int32_t* d_fill[2];      // [max_pairs][kBins] scatter cursors of the arriving layer, by layer parity
   uint32_t* d_arrivals;    // zero at rest: [max_pairs] a list's finished runs in the pooling, [max_requests] a
                            // request's finished parts of the preference
   double* d_headsum;       // [max_requests][H_q][2] per-head entropy / variance sums of the layer
@@ -237,7 +220,6 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
 // cascade.cu
 int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize, bool budgets, cudaStream_t st);
 int32_t launch_allocate(cake_ctx* ctx, int32_t stage, cudaStream_t st);
-int32_t launch_evict(cake_ctx* ctx, int32_t stage, cudaStream_t st);
 // decode.cu
 int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache, void* v_cache,
                             int64_t* row_offsets, cudaStream_t st);
@@ -261,6 +243,18 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
                              int32_t* out, int64_t capacity, cudaStream_t st);
 int32_t launch_get_positions(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* out,
                              int64_t capacity, cudaStream_t st);
+
+// Pooled indicators of a layer of the current batch: [H_kv][T].
+inline float* layer_store(const cake_ctx* ctx, int32_t layer) {
+  return ctx->d_store + (size_t)layer * ctx->cfg.n_kv_heads * ctx->total_tokens;
+}
+
+// Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
+__device__ __forceinline__ uint32_t ordered_key(float v) {
+  uint32_t b = __float_as_uint(v);
+  b = b == 0x80000000u ? 0u : b;
+  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
 
 // The eviction indicator of one key from the mean and variance of its window attention
 // (Section 4.3, Eq. 11, and the combinations of the paper's indicator ablation).

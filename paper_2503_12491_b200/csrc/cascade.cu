@@ -1,5 +1,6 @@
-// Layer finalisation (preference, pooling), the device-side budget allocator and the bucket-sorted
-// survivor lists that the per-head top-k eviction of the cascade works on.
+// What follows a layer's scores: its preference, the budgets of its stage (device side), and its pooled
+// indicators with their distribution, from which the per-head top-k of the eviction is found where a retained
+// set is read.
 #include "cake_internal.cuh"
 
 #include <math_constants.h>
@@ -20,21 +21,12 @@ __device__ inline double warp_sum_f64(double v) {
 }
 
 // --------------------------------------------------------------- pool + bins
-// Survivor lists are kept sorted by bucket, not by position.  A key's bucket is the top
-// kBinBits bits of its order-preserving integer image, counted from the top (bucket 0 holds
-// the largest values).  When a layer arrives, its pooled indicators are histogrammed here and
-// scattered into bucket order by the eviction kernel; from then on "keep the top b" means
-// "all buckets before the one that contains the b-th element, plus the best part of that
-// bucket", so a later, smaller budget only moves a threshold and rewrites nothing.
-// Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
-__device__ inline uint32_t ordered_key(float v) {
-  uint32_t b = __float_as_uint(v);
-  b = b == 0x80000000u ? 0u : b;
-  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
-}
+// A key's (ordered_key's) bucket is its top kBinBits bits, counted from the top (bucket 0 holds the largest values).
+// When a layer arrives, its pooled indicators are histogrammed: "the top b" are then all values of the buckets
+// before the one that contains the b-th, and the best part of that bucket.
 __device__ inline int bucket_of(uint32_t key) { return (kBins - 1) - (int)(key >> (32 - kBinBits)); }
 
-// Token ranges of the pooling and scatter items: a request's tokens in at most `want` equal runs, a
+// Token ranges of the pooling items: a request's tokens in at most `want` equal runs, a
 // multiple of kChunkKeys long.
 __device__ inline int split_span(int N, int want) {
   const int chunks = (N + kChunkKeys - 1) / kChunkKeys;
@@ -42,12 +34,11 @@ __device__ inline int split_span(int N, int want) {
   return ns > 0 ? (chunks + ns - 1) / ns * kChunkKeys : kChunkKeys;
 }
 
-// The cascade kernels' CTAs take a whole SM each, 1024 threads in four teams that work on items of their
-// own.  (As CTAs of a team each they spread over all the SMs that are free in the moment between two
-// score launches, and the next one, whose CTAs need whole SMs, waits for them: 136 against 119 us per
-// 128K layer.  As one team of 1024 an SM has a single chain of scans and barriers at a time: with 256 lists
-// of 2K tokens 97 us for the pooling and 75 us for the scatter beside the scoring, 43 and 28 as it is; 36
-// and 29 by themselves.)
+// The CTAs of arrive_layer take a whole SM each, 1024 threads in four teams that work on items of their own.
+// (As CTAs of a team each they spread over all the SMs that are free in the moment between two score
+// launches, and the next one, whose CTAs need whole SMs, waits for them: 136 against 119 us per 128K layer.
+// As one team of 1024 an SM has a single chain of scans and barriers at a time: with 256 lists of 2K tokens 97 us
+// beside the scoring, 43 as it is; 36 by themselves.)
 constexpr int TEAMS = 4;
 constexpr int TEAM_THREADS = 256;
 constexpr int TEAM_WARPS = TEAM_THREADS / 32;
@@ -209,20 +200,22 @@ __device__ void finalize_heads(const FinalizeArgs& F, const AllocArgs& A, const 
 // SMs the next layer's score kernel leaves free (a grid beyond those would sit on SMs that kernel
 // needs whole, and hold up all of its CTAs); its CTAs take items in turn:
 //   - the preference and the stage's budgets of a request (first, their chain of steps is the longest);
-//   - a run of a request's tokens of one KV head: fresh[g][t] = pool(raw[g][.]) over the request's
+//   - a run of a request's tokens of one KV head: store[g][t] = pool(raw[g][.]) over the request's
 //     non-window tokens, +inf on the window (Section 4.3); with do_pool = 0 the pooled values are
-//     already in `fresh`.  A thread owns PH_PER consecutive tokens per pass.  The bucket histogram of
+//     already there.  A thread owns PH_PER consecutive tokens per pass.  The bucket histogram of
 //     the (request, head) is accumulated in `hist`; the CTA that adds the last run turns it into
-//     the list's bucket offsets, once in `prefix` and once as the scatter's cursors in `fill`.
+//     bucket offsets, `prefix`.
+// Nothing here depends on the budgets, and nothing else is done for an eviction: which tokens a budget keeps is
+// found where a retained set is read (sorted_positions).  Placing every layer's values in bucket order was a launch
+// of its own per layer, 6 to 60 us on the few SMs that the score kernel leaves free.
 // R = pool_kernel / 2 when that is at most 3, else -1 (any kernel size, one global read per tap).
 struct ArriveArgs {
   const float* raw;
-  float* fresh;
+  float* store;
   const ReqInfo* reqs;
   uint32_t* hist;
   uint32_t* arrivals;
   int32_t* prefix;
-  int32_t* fill;
   int n_req, want, layer, L, Hkv, kp, mode, do_pool;
   int64_t T;
 };
@@ -243,7 +236,6 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
   const int layer = Q.layer, L = Q.L, Hkv = Q.Hkv, kp = Q.kp, mode = Q.mode, do_pool = Q.do_pool;
   const int64_t T = Q.T;
   const float* raw = Q.raw;
-  float* fresh = Q.fresh;
   for (int item = team * gridDim.x + blockIdx.x; item < n_items; item += TEAMS * gridDim.x) {
     team_sync();                                   // the item before is done with shared memory
     if (item < n_fin) {
@@ -259,7 +251,7 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
     for (int b = tid; b < kBins; b += TEAM_THREADS) sh[b] = 0;
     team_sync();
     const float* src = raw + (size_t)g * T + rq.cu;
-    float* dst = fresh + (size_t)g * T + rq.cu;
+    float* dst = Q.store + (size_t)g * T + rq.cu;
     const int t0 = split * span, t1 = min(rq.N, t0 + span);
     // Writes four tokens and counts their buckets.  Neighbours often share a bucket, so a run is counted
     // once, at its first token; without branches (with them a warp issued some 300 instructions for its
@@ -381,9 +373,8 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
       if (!S.last) continue;
       __threadfence();
     }
-    // bucket offsets of the new list: prefix[i] = elements in buckets before i
+    // bucket offsets: prefix[i] = values in buckets before i
     int32_t* pf = Q.prefix + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
-    int32_t* fl = Q.fill + (size_t)pair * kBins;
     // (a warp takes a run of the buckets, 32 at a time, so that all accesses are consecutive)
     constexpr int PER = kBins / TEAM_THREADS;
     const int lane = tid & 31, first = (tid >> 5) * (32 * PER) + lane;
@@ -405,7 +396,6 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
         if (lane >= o) inc += n;
       }
       pf[first + 32 * e] = run + inc - cnt[e];
-      fl[first + 32 * e] = run + inc - cnt[e];
       run += __shfl_sync(0xffffffffu, inc, 31);
       if (nsplit > 1) gh[first + 32 * e] = 0;          // ready for the next layer
     }
@@ -595,150 +585,11 @@ __global__ void allocate_budgets(const AllocArgs A, const ReqInfo* __restrict__ 
   allocate_request(A, reqs[blockIdx.x], blockIdx.x, stage, nullptr, S);
 }
 
-// -------------------------------------------------------------------- evict
-struct EvictArgs {
-  const float* fresh;
-  uint2* lists;
-  const int32_t* prefix_all;
-  ListState* states;
-  int32_t* fill;           // [pairs][kBins] cursors, set to the bucket offsets when the layer arrived
-  const ReqInfo* reqs;
-  const int32_t* cur;      // budgets of this stage
-  int n_req, want, stage, L, Hkv;
-  int64_t T;
-};
-
 static_assert(offsetof(ArriveSmem, tile) % 16 == 0 && sizeof(ArriveSmem) % 16 == 0, "tiles are read 16 bytes at a time");
-constexpr int SC_PER = 4;
-constexpr int SC_LOADS = 4;
-
-// Newest layer of stage `stage`: an item per (run of a request's tokens, KV head, request) scatters the
-// pooled indicators into bucket order.  Only the buckets the layer's budget can ever reach are stored
-// (the budget never grows again, Proposition 1).  Where exactly the budget cuts a list is
-// derived from the list and the budget of the moment by whoever reads the retained set
-// (list_threshold): a later, smaller budget changes nothing that is stored, so the older layers need no
-// work here.  (Moving every older list's threshold at every stage was a launch of up to 31 * H_kv
-// CTAs per layer, 10 to 72 us beside the score kernel.)
-struct ScatterSmem {           // of a team
-  uint32_t cnt[kBins], base[kBins];
-  int warp_tot[TEAM_WARPS];
-};
-__global__ void __launch_bounds__(TEAMS * TEAM_THREADS)
-scatter_new(const EvictArgs A) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
-  const int team = (int)threadIdx.x / TEAM_THREADS, tid = (int)threadIdx.x % TEAM_THREADS;
-  ScatterSmem& S = reinterpret_cast<ScatterSmem*>(smem_raw)[team];
-  uint32_t *s_cnt = S.cnt, *s_base = S.base;
-  const int n_items = A.n_req * A.Hkv * A.want;
-  for (int item = team * gridDim.x + blockIdx.x; item < n_items; item += TEAMS * gridDim.x) {
-    team_sync();
-    const int split = item % A.want, pair = item / A.want;
-    const int req = pair / A.Hkv, g = pair - req * A.Hkv;
-    const ReqInfo rq = A.reqs[req];
-    const int span = split_span(rq.N, A.want);
-    const int t0 = split * span, t1 = min(rq.n, t0 + span);
-    if (t0 >= rq.N) continue;
-    const size_t lid = ((size_t)req * A.L + A.stage) * A.Hkv + g;
-    const int32_t* pf = A.prefix_all + lid * (kBins + 1);
-    uint2* list = A.lists + rq.list_off + ((size_t)A.stage * A.Hkv + g) * rq.n;
-    const int b = min(A.cur[(size_t)req * A.L + A.stage], rq.n);
-    if (split == 0 && tid == 0) A.states[lid] = ListState{-1, 0xFFFFFFFFu, -1, b};
-    // last bucket worth storing
-    int less = 0;
-    for (int i = tid; i < kBins; i += TEAM_THREADS) {
-      less += __ldcg(&pf[i + 1]) < b ? 1 : 0;
-      s_cnt[i] = 0;
-    }
-    int total;
-    team_excl_scan(less, S.warp_tot, &total);
-    const int d_last = b > 0 ? min(total, kBins - 1) : -1;
-    const float* src = A.fresh + (size_t)g * A.T + rq.cu;
-    // SC_LOADS * 4 consecutive tokens per thread at a time, all loads in flight together
-    constexpr int kStep = TEAM_THREADS * SC_PER * SC_LOADS;
-    uint32_t key[SC_LOADS][SC_PER];
-    auto fetch = [&](int jb) {
-      float v[SC_LOADS][SC_PER];
-#pragma unroll
-      for (int u = 0; u < SC_LOADS; ++u)
-#pragma unroll
-        for (int e = 0; e < SC_PER; ++e) {
-          const int j = jb + (u * TEAM_THREADS + tid) * SC_PER + e;
-          v[u][e] = j < t1 ? __ldcg(&src[j]) : 0.f;
-        }
-#pragma unroll
-      for (int u = 0; u < SC_LOADS; ++u)
-#pragma unroll
-        for (int e = 0; e < SC_PER; ++e) key[u][e] = ordered_key(v[u][e]);
-    };
-    // Buckets of four tokens; len: how many of them start here in a run of equal buckets, 0 where no run
-    // starts or the bucket is not stored.
-    struct Four { int q[SC_PER]; uint32_t len[SC_PER]; bool keep[SC_PER]; bool any; };
-    auto four = [&](int jb, int u) {
-      Four f;
-      const int j0 = jb + (u * TEAM_THREADS + tid) * SC_PER;
-#pragma unroll
-      for (int e = 0; e < SC_PER; ++e) {
-        f.q[e] = bucket_of(key[u][e]);
-        f.keep[e] = j0 + e < t1 && f.q[e] <= d_last;
-      }
-#pragma unroll
-      for (int e = 0; e < SC_PER; ++e) {
-        uint32_t n = 1;
-        bool run = true;
-#pragma unroll
-        for (int x = e + 1; x < SC_PER; ++x) {
-          run = run && f.keep[x] && f.q[x] == f.q[e];
-          n += run ? 1u : 0u;
-        }
-        const bool starts = f.keep[e] && (e == 0 || f.q[e - 1] != f.q[e]);
-        f.len[e] = starts ? n : 0u;
-      }
-      f.any = f.keep[0] || f.keep[1] || f.keep[2] || f.keep[3];
-      return f;
-    };
-    // pass 1: count this run's entries per bucket (runs of equal buckets at once)
-    for (int jb = t0; jb < t1; jb += kStep) {
-      fetch(jb);
-#pragma unroll
-      for (int u = 0; u < SC_LOADS; ++u) {
-        const Four f = four(jb, u);
-        if (!__any_sync(0xffffffffu, f.any)) continue;
-#pragma unroll
-        for (int e = 0; e < SC_PER; ++e)
-          if (f.len[e]) atomicAdd(&s_cnt[f.q[e]], f.len[e]);
-      }
-    }
-    team_sync();
-    // reserve this run's range inside every bucket of the list
-    int32_t* fl = A.fill + (size_t)pair * kBins;
-    for (int q = tid; q < kBins; q += TEAM_THREADS) {
-      const uint32_t c = s_cnt[q];
-      if (c) s_base[q] = (uint32_t)atomicAdd(&fl[q], (int)c);
-      s_cnt[q] = 0;
-    }
-    team_sync();
-    // pass 2: place the entries
-    for (int jb = t0; jb < t1; jb += kStep) {
-      if (t1 - t0 > kStep) fetch(jb);                // a short run is still in registers
-#pragma unroll
-      for (int u = 0; u < SC_LOADS; ++u) {
-        const Four f = four(jb, u);
-        if (!__any_sync(0xffffffffu, f.any)) continue;
-        const uint32_t j0 = (uint32_t)(jb + (u * TEAM_THREADS + tid) * SC_PER);
-        uint32_t off = 0;
-#pragma unroll
-        for (int e = 0; e < SC_PER; ++e) {
-          if (f.len[e]) off = s_base[f.q[e]] + atomicAdd(&s_cnt[f.q[e]], f.len[e]);
-          if (f.keep[e]) list[off++] = make_uint2(key[u][e], j0 + e);
-        }
-      }
-    }
-  }
-}
 
 }  // namespace
 
-// CTAs of the cascade kernels, and runs per (request, head).  While the next layer is scored they run on the
+// CTAs of arrive_layer, and runs per (request, head).  While the next layer is scored they run on the
 // SMs its kernel leaves free; behind the last layer the whole device is theirs.
 static void cascade_shape(const cake_ctx* ctx, int32_t layer, int extra_items, int* want, int* grid) {
   const int pairs = ctx->n_req * ctx->cfg.n_kv_heads;
@@ -790,12 +641,11 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
   }
   ArriveArgs Q;
   Q.raw = ctx->d_raw[layer % ctx->score_depth];
-  Q.fresh = ctx->d_fresh[layer & 1];
+  Q.store = layer_store(ctx, layer);
   Q.reqs = ctx->d_req;
   Q.hist = ctx->d_hist;
   Q.arrivals = ctx->d_arrivals;
   Q.prefix = ctx->d_prefix;
-  Q.fill = ctx->d_fill[layer & 1];
   Q.n_req = ctx->n_req; Q.layer = layer; Q.L = c.n_layers; Q.Hkv = c.n_kv_heads;
   Q.kp = c.pool_kernel; Q.mode = c.pool_mode; Q.do_pool = do_pool ? 1 : 0;
   Q.T = ctx->total_tokens;
@@ -826,31 +676,6 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
 int32_t launch_allocate(cake_ctx* ctx, int32_t stage, cudaStream_t st) {
   if (ctx->n_req == 0) return CAKE_OK;
   allocate_budgets<<<ctx->n_req, 32, 0, st>>>(alloc_args(ctx, stage), ctx->d_req, stage);
-  count_launch();
-  return cuda_status(cudaGetLastError());
-}
-
-int32_t launch_evict(cake_ctx* ctx, int32_t stage, cudaStream_t st) {
-  const cake_config& c = ctx->cfg;
-  if (ctx->n_req == 0) return CAKE_OK;
-  EvictArgs A;
-  A.fresh = ctx->d_fresh[stage & 1];
-  A.lists = ctx->d_lists;
-  A.prefix_all = ctx->d_prefix;
-  A.states = ctx->d_lstate;
-  A.fill = ctx->d_fill[stage & 1];
-  A.reqs = ctx->d_req;
-  A.cur = ctx->d_budget[stage & 1];
-  A.n_req = ctx->n_req; A.stage = stage; A.L = c.n_layers; A.Hkv = c.n_kv_heads;
-  A.T = ctx->total_tokens;
-  int grid;
-  cascade_shape(ctx, stage, 0, &A.want, &grid);
-  static PerDeviceOnce attr;
-  if (attr.need(ctx->device)) {
-    CAKE_CUDA_TRY(cudaFuncSetAttribute(scatter_new, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TEAMS * sizeof(ScatterSmem))));
-    attr.mark(ctx->device);
-  }
-  scatter_new<<<grid, TEAMS * TEAM_THREADS, TEAMS * sizeof(ScatterSmem), st>>>(A);
   count_launch();
   return cuda_status(cudaGetLastError());
 }

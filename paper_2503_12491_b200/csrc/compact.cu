@@ -1,10 +1,13 @@
 // Gather-compaction of the retained K/V rows into the packed varlen cache
 // (Eq. 12: K^ = K[D,:], V^ = V[D,:]) and the position getter.
 //
-// The survivor lists are in bucket order; the packed cache is in ascending token position.
-// Positions are distinct integers below n, so the ordering is a bitmap: every retained
-// position sets its bit, and the rank of a bit is the number of bits before it.
+// The retained set of a (request, layer, KV head) at a budget b is the first b of its stored indicators in the
+// order (indicator descending, position ascending)  (Section 4.2 EVICT, Eq. 12).  It is found here, where it is
+// read out, from the indicators and their bucket offsets.  The packed cache is in ascending token position: every retained position sets its bit in a bitmap,
+// and the rank of a bit is the number of bits before it.
 #include "cake_internal.cuh"
+
+#include <algorithm>
 
 namespace cake {
 namespace {
@@ -18,6 +21,8 @@ __global__ void __launch_bounds__(OFF_THREADS)
 block_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ row_off, int64_t* __restrict__ key_off,
               int64_t* __restrict__ dec_off, int nblk, int L, int lo, int hi, int Hkv, int Sw, int group) {
   __shared__ int64_t tot[2][32];
+  // sorted_positions starts beside this kernel: it waits for it only before it writes
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = (int)blockDim.x >> 5;
   int64_t base0 = 0, base1 = 0;                       // rows and key groups (or heads) so far
   for (int i0 = 0; i0 < nblk; i0 += (int)blockDim.x) {
@@ -58,38 +63,31 @@ block_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ row_off,
   }
 }
 
-constexpr int kTieCap = 2048;
+constexpr int kTieCap = 512;                         // entries of equal rank but for their position that are ranked one by one
+constexpr int kFewEntries = 64;                      // entries that are ranked without another histogram
+constexpr int SP_BINS = 1024;                        // (22 - clz in the code is 32 - clz - log2 of this)
+constexpr int SP_BATCH = 4;                          // groups of 32 entries a warp has in flight
 
-struct EvictSmem {
-  uint32_t hist[1024];
-  int32_t ties[kTieCap];
+struct SelectSmem {
+  uint32_t hist[SP_BINS];
+  uint2 ties[kTieCap];                               // (key, position)
   int warp_tot[32];
-  int total;
-  uint32_t sel_digit, sel_rem, sel_cnt;
-  int32_t tie_count, pos_cut;
+  int total, count, tie_count;
+  int bucket, start, n_in;
+  uint32_t sel_bin, sel_rem, sel_cnt;
 };
 
-// Among `cnt` entries (all in one bucket), finds the digit (10 bits at `shift`) that holds the
-// krem-th largest key among the entries whose bits above shift+10 equal `prefix_bits`.
-__device__ inline void radix_digit(const uint2* __restrict__ e, int cnt, uint32_t mask,
-                                   uint32_t prefix_bits, int shift, uint32_t krem, EvictSmem& S) {
-  for (int b = threadIdx.x; b < 1024; b += blockDim.x) S.hist[b] = 0;
-  __syncthreads();
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-    const uint32_t key = __ldcg(&e[i]).x;
-    if ((key & mask) == prefix_bits) atomicAdd(&S.hist[(key >> shift) & 1023u], 1u);
-  }
-  __syncthreads();
-  // digits from the top: thread t owns digits 1023-4t .. 1020-4t
-  const int per = 1024 / blockDim.x;
+// Bins of the histogram from the top: the one that holds the krem-th entry, how many of its entries are wanted,
+// and its size.
+__device__ inline void find_bin(uint32_t krem, SelectSmem& S) {
+  const int per = max(1, SP_BINS / (int)blockDim.x);
   int mine = 0;
-  for (int q = 0; q < per; ++q) mine += (int)S.hist[1023 - (threadIdx.x * per + q)];
+  for (int q = 0; q < per; ++q) mine += (int)S.hist[SP_BINS - 1 - (threadIdx.x * per + q)];
   int above = block_excl_scan(mine, S.warp_tot, &S.total);
   for (int q = 0; q < per; ++q) {
-    const int dg = 1023 - (threadIdx.x * per + q);
-    const int h = (int)S.hist[dg];
+    const int bin = SP_BINS - 1 - (threadIdx.x * per + q), h = (int)S.hist[bin];
     if ((uint32_t)above < krem && (uint32_t)(above + h) >= krem) {
-      S.sel_digit = (uint32_t)dg;
+      S.sel_bin = (uint32_t)bin;
       S.sel_rem = krem - (uint32_t)above;
       S.sel_cnt = (uint32_t)h;
     }
@@ -97,170 +95,252 @@ __device__ inline void radix_digit(const uint2* __restrict__ e, int cnt, uint32_
   }
   __syncthreads();
 }
-
-// Where the budget b cuts one list: the retained set is its first b entries in the order (indicator
-// descending, position ascending)  (Section 4.2 EVICT, Eq. 12).
-__device__ void list_threshold(const int32_t* __restrict__ pf, const uint2* __restrict__ list, int b, ListState* out,
-                               EvictSmem& S) {
-  if (b <= 0) {
-    if (threadIdx.x == 0) *out = ListState{-1, 0xFFFFFFFFu, -1, 0};
-    return;
-  }
-  // threshold bucket d: first bucket with prefix[d+1] >= b
-  int less = 0;
-  for (int i = threadIdx.x; i < kBins; i += blockDim.x) less += __ldcg(&pf[i + 1]) < b ? 1 : 0;
-  block_excl_scan(less, S.warp_tot, &S.total);
-  const int d = S.total;
+__device__ inline void clear_hist(SelectSmem& S) {
+  for (int i = threadIdx.x; i < SP_BINS; i += blockDim.x) S.hist[i] = 0;
   __syncthreads();
-  if (d >= kBins) {                                  // b exceeds the stored entries: keep all
-    if (threadIdx.x == 0) *out = ListState{kBins - 1, 0u, 0x7FFFFFFF, __ldcg(&pf[kBins])};
-    return;
+}
+// Counts a bin for every lane that has one (>= 0).  Pooled values repeat: a run of equal bins in
+// neighbouring lanes is counted once.  Called by whole warps.
+__device__ __forceinline__ void count_bin(int bin, SelectSmem& S) {
+  if (!__any_sync(0xffffffffu, bin >= 0)) return;
+  const int lane = threadIdx.x & 31, before = __shfl_up_sync(0xffffffffu, bin, 1);
+  const bool first = lane == 0 || bin != before;
+  const uint32_t firsts = __ballot_sync(0xffffffffu, first);
+  if (first && bin >= 0) {
+    const uint32_t later = lane < 31 ? firsts >> (lane + 1) : 0u;
+    atomicAdd(&S.hist[bin], later ? (uint32_t)__ffs(later) : 32u - lane);
   }
-  const int start = __ldcg(&pf[d]), cnt = __ldcg(&pf[d + 1]) - start;
-  const uint32_t rem = (uint32_t)(b - start);
-  if ((int)rem >= cnt) {
-    if (threadIdx.x == 0) *out = ListState{d, 0u, 0x7FFFFFFF, b};
-    return;
-  }
-  const uint2* e = list + start;
-  constexpr int low = 32 - kBinBits;                 // key bits below the bucket bits (20)
-  radix_digit(e, cnt, 0u, 0u, low - 10, rem, S);
-  uint32_t pre = S.sel_digit << (low - 10);
-  uint32_t krem = S.sel_rem;
-  __syncthreads();
-  radix_digit(e, cnt, 1023u << (low - 10), pre, 0, krem, S);
-  pre |= S.sel_digit;
-  const uint32_t need_eq = S.sel_rem, n_eq = S.sel_cnt;
-  __syncthreads();
-  // full key of the threshold: bucket bits + the 20 selected bits
-  const uint32_t thr = ((uint32_t)(kBins - 1 - d) << low) | pre;
-  int32_t pos_cut = 0x7FFFFFFF;
-  if (need_eq < n_eq) {
-    // ties at the threshold: the need_eq lowest positions win
-    if (threadIdx.x == 0) { S.tie_count = 0; S.pos_cut = 0x7FFFFFFF; }
-    __syncthreads();
-    if (n_eq <= (uint32_t)kTieCap) {
-      for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-        const uint2 v = __ldcg(&e[i]);
-        if (v.x == thr) S.ties[atomicAdd(&S.tie_count, 1)] = (int32_t)v.y;
-      }
-      __syncthreads();
-      for (int i = threadIdx.x; i < (int)n_eq; i += blockDim.x) {
-        const int32_t p = S.ties[i];
-        uint32_t r = 0;
-        for (int o = 0; o < (int)n_eq; ++o) r += S.ties[o] < p ? 1u : 0u;
-        if (r == need_eq - 1) S.pos_cut = p;
-      }
-      __syncthreads();
-    } else {
-      // many ties: bisect the position (positions are distinct)
-      int lo = 0, hi = 0x7FFFFFFF;                   // smallest cut with count(pos <= cut) >= need_eq
-      while (lo < hi) {
-        const int mid = lo + ((hi - lo) >> 1);
-        int c = 0;
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-          const uint2 v = __ldcg(&e[i]);
-          c += (v.x == thr && (int32_t)v.y <= mid) ? 1 : 0;
-        }
-        block_excl_scan(c, S.warp_tot, &S.total);
-        const int tot = S.total;
-        __syncthreads();
-        if ((uint32_t)tot >= need_eq) hi = mid; else lo = mid + 1;
-      }
-      if (threadIdx.x == 0) S.pos_cut = lo;
-      __syncthreads();
-    }
-    pos_cut = S.pos_cut;
-  }
-  if (threadIdx.x == 0) *out = ListState{d, thr, pos_cut, b};
 }
 
-
-// One CTA per (head, layer in [lo, hi), request): where the current budget cuts the list (kept in
-// its state for whoever needs the stored indicators too), then the retained positions in ascending order, then the window, written at out[base + g*len ...].  `bitmap` is dynamic
-// shared memory when the request's n bits fit, else a slice of global scratch.
+// One CTA per (head, layer in [lo, hi), request): which positions the current budget b keeps, then these in ascending
+// order, then the window, written at out[base + g*len ...].
+//   1. The bucket offsets say which bucket holds the b-th largest value, and how many of its entries are wanted.
+//   2. One pass over the values, eight to a lane: the bits of those in the buckets before are set, those inside go
+//      to a list in shared memory, as (key, position).  If there are too many for it, the steps below go over all values.
+//   3. Histograms of SP_BINS equal parts of the bucket's keys narrow it to the bin that holds the b-th value, until that
+//      has few entries (usually at once); these are ranked by (key, position).
+//   4. Ranks of the bits, positions.
+// Bound: the pass over the values, and between the steps the latency of the chain, which other lists' CTAs on the SM
+// hide: 46 us for 256 lists of 131 040 values (134 MB), 29 for 512 of 26 000, 20 for 1024 of 4064.  Placing every layer's
+// values in bucket order when it arrived made this step 31, 27 and 22 us, for a launch of 7 to 76 us per layer.
+// Without the bucket offsets three digit histograms of all values took 300 us in the first case and 137 in the
+// second (run lengths, and atomics on few hot bins), and a sample in their place 129 and 133, since the candidates
+// on either side of the cut are many where a layer keeps much.  `bits` is shared memory when the request's n
+// bits fit, else a slice of global scratch.
 template <int POS_THREADS>
-__global__ void __launch_bounds__(POS_THREADS)
-sorted_positions(const uint2* __restrict__ lists, const int32_t* __restrict__ prefix_all,
-                 ListState* __restrict__ states, const ReqInfo* __restrict__ reqs,
-                 const int32_t* __restrict__ budget, const int64_t* __restrict__ offsets,
-                 int32_t* __restrict__ out, uint32_t* __restrict__ scratch, int64_t scratch_words,
-                 int req0, int lo, int L, int Hkv, int Sw, int smem_words, int64_t capacity) {
-  extern __shared__ uint32_t sh_bits[];
-  __shared__ int warp_tot[32];
-  __shared__ EvictSmem S;
-  __shared__ ListState st;
+__global__ void __launch_bounds__(POS_THREADS, 1024 / POS_THREADS)
+sorted_positions(const float* __restrict__ store, const int32_t* __restrict__ prefix_all, const ReqInfo* __restrict__ reqs, const int32_t* __restrict__ budget,
+                 const int64_t* __restrict__ offsets, int32_t* __restrict__ out, uint32_t* __restrict__ scratch,
+                 int64_t scratch_words, int req0, int lo, int L, int Hkv, int Sw, int smem_words, int cap, int64_t T,
+                 int64_t capacity) {
+  extern __shared__ __align__(16) uint32_t sh_dyn[];
+  __shared__ SelectSmem S;
   const int g = blockIdx.x, layer = lo + blockIdx.y, req = req0 + blockIdx.z;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int WARPS = POS_THREADS / 32;
   const ReqInfo rq = reqs[req];
-  const size_t lid = ((size_t)req * L + layer) * Hkv + g;
+  const int n = rq.n;
   const int b = budget[(size_t)req * L + layer];
   const int len = b + Sw;
-  int32_t* dst = out + (offsets ? offsets[(size_t)req * L + layer] : 0) + (int64_t)g * len;
   // without row offsets the caller gave a capacity: never write past it
   const int64_t room = offsets ? (int64_t)len : capacity - (int64_t)g * len;
-  const int words = (rq.n + 31) >> 5;
-  uint32_t* bits = sh_bits;
-  const bool in_smem = words <= smem_words;
-  if (!in_smem) {
+  // The offsets are written by the kernel before this one, which may still run; nothing else that is read here is.
+  auto row_start = [&]() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return out + (offsets ? __ldcg(&offsets[(size_t)req * L + layer]) : 0) + (int64_t)g * len;
+  };
+  if (b <= 0 || b >= n) {
+    int32_t* dst = row_start();
+    for (int t = threadIdx.x; t < (b <= 0 ? 0 : n); t += POS_THREADS)
+      if (t < room) dst[t] = t;
+    for (int t = threadIdx.x; t < Sw; t += POS_THREADS)
+      if (b + t < room) dst[b + t] = n + t;
+    return;
+  }
+  // Element q = a + i of the row, counted from the 16-byte boundary at or before its start, is value i: lanes load
+  // whole groups of four, and bits and positions count in elements until they are written out.
+  const float* const v = store + ((size_t)layer * Hkv + g) * T + rq.cu;
+  const int a = (int)((reinterpret_cast<uintptr_t>(v) >> 2) & 3), end = a + n;
+  const int words = (end + 31) >> 5;
+  uint2* const list = reinterpret_cast<uint2*>(sh_dyn + smem_words);
+  uint32_t* bits = sh_dyn;
+  if (words > smem_words) {
     const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     bits = scratch + cta * (size_t)scratch_words;
   }
-  for (int wi = threadIdx.x; wi < words; wi += POS_THREADS) bits[wi] = 0;
-  if (in_smem) __syncthreads(); else { __threadfence_block(); __syncthreads(); }
-  const int32_t* pf = prefix_all + lid * (kBins + 1);
-  const uint2* list = lists + rq.list_off + ((size_t)layer * Hkv + g) * rq.n;
-  // a list never grows again (Proposition 1): entries beyond the budget it arrived with were not stored
-  const int arrived = states[lid].kept;
-  list_threshold(pf, list, min(min(b, rq.n), arrived), &st, S);
-  __syncthreads();
-  if (threadIdx.x == 0) states[lid] = ListState{st.bucket, st.thr_key, st.pos_cut, arrived};
-  if (st.bucket >= 0 && b > 0) {
-    const int start = pf[st.bucket], end = pf[st.bucket + 1];
-    for (int i = threadIdx.x; i < end; i += POS_THREADS) {
-      const uint2 e = list[i];
-      const bool keep = i < start || e.x > st.thr_key || (e.x == st.thr_key && (int32_t)e.y <= st.pos_cut);
-      if (keep && e.y < (uint32_t)rq.n) atomicOr(&bits[e.y >> 5], 1u << (e.y & 31));
+  // the bucket with prefix[d] < b <= prefix[d + 1]
+  const int32_t* pf = prefix_all + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
+  {
+    constexpr int PER = kBins / POS_THREADS;
+    int at[PER + 1];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) at[q] = __ldg(&pf[q * POS_THREADS + threadIdx.x]);
+    at[PER] = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int next = __ldg(&pf[q * POS_THREADS + threadIdx.x + 1]);
+      if (at[q] < b && next >= b) { S.bucket = q * POS_THREADS + threadIdx.x; S.start = at[q]; S.n_in = next - at[q]; }
     }
   }
+  if (threadIdx.x == 0) { S.count = 0; S.tie_count = 0; }
   __syncthreads();
-  // rank of every word, then expand
-  const int per = (words + POS_THREADS - 1) / POS_THREADS;
-  const int w0 = threadIdx.x * per, w1 = min(words, w0 + per);
-  int cnt = 0;
-  for (int wi = w0; wi < w1; ++wi) cnt += __popc(bits[wi]);
-  // exclusive scan over the block
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int inc = cnt;
+  const int d = S.bucket, n_in = S.n_in;
+  uint32_t krem = (uint32_t)(b - S.start);           // entries of the bucket that are kept
+  uint32_t klo = (uint32_t)(kBins - 1 - d) << (32 - kBinBits), khi = klo | ((1u << (32 - kBinBits)) - 1u);
+  const bool listed = n_in <= cap;
+  if (listed) {
+    // In buckets above zero the bits of a float are compared as they are: as signed integers they have the order of
+    // the keys there, and everything else lies below.
+    const bool plain = klo > 0x80000000u;
+    const int ilo = (int)(klo ^ 0x80000000u), ihi = (int)(khi ^ 0x80000000u);
+    const uint4* const v4 = reinterpret_cast<const uint4*>(v - a);
+    const int n_oct = (end + 7) >> 3;                // (up to seven elements beyond the row are loaded, and not looked at)
+    uint4 next[2];
+    auto fetch = [&](int o) {
+      next[0] = next[1] = make_uint4(0, 0, 0, 0);
+      if (o < n_oct) { next[0] = __ldcg(v4 + 2 * o); next[1] = __ldcg(v4 + 2 * o + 1); }
+    };
+    fetch(warp * 32 + lane);
+    for (int o0 = warp * 32; o0 < n_oct; o0 += POS_THREADS) {
+      const int o = o0 + lane;
+      uint32_t x[8] = {next[0].x, next[0].y, next[0].z, next[0].w, next[1].x, next[1].y, next[1].z, next[1].w};
+      fetch(o + POS_THREADS);
+      if (!plain) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  if (lane == 31) warp_tot[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    const int w = lane < POS_THREADS / 32 ? warp_tot[lane] : 0;
-    int winc = w;
+        for (int e = 0; e < 8; ++e) x[e] = ordered_key(__uint_as_float(x[e])) ^ 0x80000000u;
+      }
+      uint32_t above = 0, in = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int n = __shfl_up_sync(0xffffffffu, winc, o);
-      if (lane >= o) winc += n;
+      for (int e = 0; e < 8; ++e) {
+        above |= (int)x[e] > ihi ? 1u << e : 0u;
+        in |= (int)x[e] >= ilo ? 1u << e : 0u;
+      }
+      // elements of the row among the eight
+      const int lo_e = max(0, a - 8 * o), hi_e = min(8, max(0, end - 8 * o));
+      const uint32_t row = (0xFFu << lo_e) & (0xFFu >> (8 - hi_e));
+      above &= row;
+      in &= row & ~above;
+      if (o < n_oct) reinterpret_cast<uint8_t*>(bits)[o] = (uint8_t)above;
+      if (!__any_sync(0xffffffffu, in != 0)) continue;
+      const int mine = __popc(in);
+      int inc = mine;
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, s);
+        if (lane >= s) inc += t;
+      }
+      int at = 0;
+      if (lane == 31) at = atomicAdd(&S.count, inc);
+      at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (in >> e & 1u) list[at++] = make_uint2(x[e] ^ 0x80000000u, (uint32_t)(8 * o + e));
     }
-    warp_tot[lane] = winc - w;
+    if (threadIdx.x < 4 && n_oct + (int)threadIdx.x < 4 * words) reinterpret_cast<uint8_t*>(bits)[n_oct + threadIdx.x] = 0;
   }
+  __threadfence_block();
   __syncthreads();
-  int rank = warp_tot[warp] + inc - cnt;
-  for (int wi = w0; wi < w1; ++wi) {
-    uint32_t m = bits[wi];
+  const int cnt = listed ? n_in : n;
+  // f(key, element, whether there is such an entry), whole warps
+  auto for_entries = [&](auto f) {
+    for (int i0 = warp * 32 * SP_BATCH; i0 < cnt; i0 += WARPS * 32 * SP_BATCH) {
+      uint2 x[SP_BATCH];
+#pragma unroll
+      for (int u = 0; u < SP_BATCH; ++u) {
+        const int i = i0 + 32 * u + lane;
+        x[u] = make_uint2(0u, 0u);
+        if (i < cnt) x[u] = listed ? list[i] : make_uint2(ordered_key(__ldcg(v + i)), (uint32_t)(a + i));
+      }
+#pragma unroll
+      for (int u = 0; u < SP_BATCH; ++u)
+        if (i0 + 32 * u < cnt) f(x[u].x, (int)x[u].y, i0 + 32 * u + lane < cnt);
+    }
+  };
+  uint32_t n_bin = (uint32_t)n_in;
+  while (n_bin > (uint32_t)kFewEntries && klo < khi) {
+    const uint32_t width = khi - klo;
+    const int shift = width < SP_BINS ? 0 : 22 - __clz(width);
+    clear_hist(S);
+    for_entries([&](uint32_t key, int, bool have) {
+      count_bin(have && key >= klo && key <= khi ? (int)((key - klo) >> shift) : -1, S);
+    });
+    __syncthreads();
+    find_bin(krem, S);
+    klo += S.sel_bin << shift;
+    if (khi - klo >= 1u << shift) khi = klo + ((1u << shift) - 1u);
+    krem = S.sel_rem;
+    n_bin = S.sel_cnt;
+    __syncthreads();
+  }
+  // every entry above the bin, and krem of its n_bin entries
+  int pos_cut = -1;                                  // more than kTieCap are equal: up to this position
+  const bool few = n_bin <= (uint32_t)kTieCap;
+  if (!few) {
+    int plo = a, phi = end - 1;                      // smallest cut with count(pos <= cut) >= krem
+    while (plo < phi) {
+      const int mid = plo + ((phi - plo) >> 1);
+      int c = 0;
+      for_entries([&](uint32_t key, int pos, bool have) { c += have && key == klo && pos <= mid ? 1 : 0; });
+      block_excl_scan(c, S.warp_tot, &S.total);
+      const int tot = S.total;
+      __syncthreads();
+      if ((uint32_t)tot >= krem) phi = mid; else plo = mid + 1;
+    }
+    pos_cut = plo;
+  }
+  if (!listed) {
+    for (int wi = threadIdx.x; wi < words; wi += POS_THREADS) bits[wi] = 0;
+    __threadfence_block();
+    __syncthreads();
+  }
+  for_entries([&](uint32_t key, int pos, bool have) {
+    if (have && (key > khi || (key == klo && pos <= pos_cut))) atomicOr(&bits[pos >> 5], 1u << (pos & 31));
+    if (few && have && key >= klo && key <= khi) S.ties[atomicAdd(&S.tie_count, 1)] = make_uint2(key, (uint32_t)pos);
+  });
+  __threadfence_block();
+  __syncthreads();
+  if (few) {
+    for (int i = threadIdx.x; i < (int)n_bin; i += POS_THREADS) {
+      const uint2 e = S.ties[i];
+      uint32_t ahead = 0;
+      for (int o = 0; o < (int)n_bin; ++o) {
+        const uint2 x = S.ties[o];
+        ahead += x.x > e.x || (x.x == e.x && x.y < e.y) ? 1u : 0u;
+      }
+      if (ahead < krem) atomicOr(&bits[e.y >> 5], 1u << (e.y & 31));
+    }
+    __threadfence_block();
+    __syncthreads();
+  }
+  int32_t* const dst = row_start();
+  for (int t = threadIdx.x; t < Sw; t += POS_THREADS)
+    if (b + t < room) dst[b + t] = n + t;
+  // Ranks of the bits: a warp takes a run of the words, 32 at a time, so that its lanes write close together.
+  const int run = (words + 32 * WARPS - 1) / (32 * WARPS) * 32, w0 = min(words, warp * run), w1 = min(words, w0 + run);
+  int ones = 0;
+  for (int wi = w0 + lane; wi < w1; wi += 32) ones += __popc(bits[wi]);
+  ones = __reduce_add_sync(0xffffffffu, ones);
+  if (lane == 0) S.warp_tot[warp] = ones;
+  __syncthreads();
+  int rank = __reduce_add_sync(0xffffffffu, lane < warp ? S.warp_tot[lane] : 0);
+  for (int wb = w0; wb < w1; wb += 32) {
+    uint32_t m = wb + lane < w1 ? bits[wb + lane] : 0u;
+    const int mine = __popc(m);
+    int inc = mine;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, s);
+      if (lane >= s) inc += t;
+    }
+    int at = rank + inc - mine;
     while (m) {
       const int bit = __ffs(m) - 1;
       m &= m - 1;
-      if (rank < b && rank < room) dst[rank] = (wi << 5) + bit;
-      ++rank;
+      if (at < b && at < room) dst[at] = ((wb + lane) << 5) + bit - a;
+      ++at;
     }
+    rank += __shfl_sync(0xffffffffu, inc, 31);
   }
-  for (int t = threadIdx.x; t < Sw; t += POS_THREADS)
-    if (b + t < room) dst[b + t] = rq.n + t;
 }
 
 constexpr int GA_THREADS = 128;
@@ -347,13 +427,15 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
   const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
   int max_n = 0;
   for (int r = req0; r < req0 + n_req; ++r) max_n = ctx->h_req[r].n > max_n ? ctx->h_req[r].n : max_n;
-  int need_words = (max_n + 31) / 32;
-  int smem_words = need_words < kBitmapSmemWords ? need_words : kBitmapSmemWords;
+  const int need_words = (max_n + 3 + 31) / 32;
+  const int smem_words = need_words <= kBitmapSmemWords ? (need_words + 1) / 2 * 2 : 0;
+  // list of a bucket's entries, 8 bytes each: a sixteenth of the values, or all of a short prompt's
+  const int cap = std::min(std::max(2048, max_n / 16), (kSelectSmemWords - smem_words) / 2);
   static PerDeviceOnce attr;
   if (attr.need(ctx->device)) {
-    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitmapSmemWords * 4));
-    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitmapSmemWords * 4));
-    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitmapSmemWords * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelectSmemWords * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelectSmemWords * 4));
+    CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelectSmemWords * 4));
     attr.mark(ctx->device);
   }
   const int64_t ctas = (int64_t)c.n_kv_heads * (hi - lo) * n_req;
@@ -362,16 +444,27 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
   const dim3 grid(c.n_kv_heads, hi - lo, n_req);
   // A list is a chain of scans and short passes: with more lists than the device holds CTAs of 1024
   // threads, smaller ones keep more chains in flight (1024 lists of 4K tokens: 42 us with 1024 threads).
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.dynamicSmemBytes = (size_t)(smem_words + 2 * cap) * 4;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = offsets ? 1 : 0;                    // behind run_offsets, which wrote them
+  cudaError_t e;
 #define CAKE_POSITIONS(NT)                                                                                                \
-  sorted_positions<NT><<<grid, NT, (size_t)smem_words * 4, st>>>(                                                         \
-      ctx->d_lists, ctx->d_prefix, ctx->d_lstate, ctx->d_req, budget, offsets, out, ctx->d_bitmap, need_words, req0, lo,  \
-      c.n_layers, c.n_kv_heads, c.window, smem_words, capacity)
-  if (ctas <= 2 * ctx->n_sm) CAKE_POSITIONS(1024);
-  else if (ctas <= 4 * ctx->n_sm) CAKE_POSITIONS(512);
-  else CAKE_POSITIONS(256);
+  cfg.blockDim = dim3(NT);                                                                                                \
+  e = cudaLaunchKernelEx(&cfg, sorted_positions<NT>, (const float*)ctx->d_store, (const int32_t*)ctx->d_prefix,           \
+                         (const ReqInfo*)ctx->d_req, budget, offsets, out, ctx->d_bitmap, (int64_t)need_words, req0, lo,  \
+                         c.n_layers, c.n_kv_heads, c.window, smem_words, cap, ctx->total_tokens, capacity)
+  if (ctas <= ctx->n_sm) { CAKE_POSITIONS(1024); }
+  else if (ctas <= 2 * ctx->n_sm) { CAKE_POSITIONS(512); }
+  else { CAKE_POSITIONS(256); }
 #undef CAKE_POSITIONS
   count_launch();
-  return cuda_status(cudaGetLastError());
+  return cuda_status(e);
 }
 
 // Rows of the packed order into k_out / v_out (dec_off: into the decode layout).

@@ -29,51 +29,30 @@ constexpr int DEC_CTA_ENTRIES = 256;       // entries per CTA up to which a head
 constexpr size_t kDecSmemMax = 200 * 1024;
 constexpr int DEC_ROWS = 4;       // cache rows a half-warp has in flight in the logit loop
 
-__device__ __forceinline__ float key_to_float(uint32_t key) {
-  const uint32_t b = (key & 0x80000000u) ? (key & 0x7FFFFFFFu) : ~key;
-  return __uint_as_float(b);
-}
-
 // One CTA per (head, layer, request): positions (ascending, from the packed order), identity
-// slot order, and the stored indicator of every survivor, found by binary search of its position.
+// slot order, and the stored indicator of every survivor (0 for the window).
 __global__ void __launch_bounds__(DEC_THREADS)
-decode_build(const uint2* __restrict__ lists, const int32_t* __restrict__ prefix_all,
-             const ListState* __restrict__ states, const ReqInfo* __restrict__ reqs,
+decode_build(const float* __restrict__ store, const ReqInfo* __restrict__ reqs,
              const int32_t* __restrict__ budget, const int64_t* __restrict__ packed_off,
              const int32_t* __restrict__ pos_packed, const int64_t* __restrict__ dec_off,
              float* __restrict__ score, int32_t* __restrict__ pos, int32_t* __restrict__ order,
-             int4* __restrict__ meta, int L, int Hkv, int Sw) {
+             int4* __restrict__ meta, int L, int Hkv, int Sw, int64_t T) {
   const int g = blockIdx.x, layer = blockIdx.y, req = blockIdx.z;
   const ReqInfo rq = reqs[req];
   const int blk = req * L + layer;
-  const size_t lid = (size_t)blk * Hkv + g;
   const int b = budget[blk];
   const int len = b + Sw, cap = len + 1;
   const int32_t* src = pos_packed + packed_off[blk] + (int64_t)g * len;
+  const float* values = store + ((size_t)layer * Hkv + g) * T + rq.cu;
   const int64_t base = dec_off[blk] + (int64_t)g * cap;
   for (int i = threadIdx.x; i < cap; i += DEC_THREADS) {
-    pos[base + i] = i < len ? src[i] : -1;
+    const int p = i < len ? src[i] : -1;
+    const float v = i < b ? values[p] : 0.f;
+    pos[base + i] = p;
     order[base + i] = i;
-    score[base + i] = 0.f;
+    score[base + i] = v == 0.f ? 0.f : v;              // (-0 is stored as +0)
   }
-  if (threadIdx.x == 0) meta[lid] = make_int4(len, len, rq.N, b);
-  __syncthreads();
-  const ListState st = states[lid];
-  if (st.bucket < 0 || b <= 0) return;
-  const int32_t* pf = prefix_all + lid * (kBins + 1);
-  const uint2* list = lists + rq.list_off + ((size_t)layer * Hkv + g) * rq.n;
-  const int start = pf[st.bucket], end = pf[st.bucket + 1];
-  for (int i = threadIdx.x; i < end; i += DEC_THREADS) {
-    const uint2 e = list[i];
-    const bool keep = i < start || e.x > st.thr_key || (e.x == st.thr_key && (int32_t)e.y <= st.pos_cut);
-    if (!keep) continue;
-    int lo = 0, hi = b - 1;                          // positions of the non-window survivors are sorted
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (src[mid] < (int32_t)e.y) lo = mid + 1; else hi = mid;
-    }
-    if (src[lo] == (int32_t)e.y) score[base + lo] = key_to_float(e.x);
-  }
+  if (threadIdx.x == 0) meta[(size_t)blk * Hkv + g] = make_int4(len, len, rq.N, b);
 }
 
 struct DecodeArgs {
@@ -772,18 +751,18 @@ int32_t launch_decode_begin(cake_ctx* ctx, const LayerPtrs& ptrs, void* k_cache,
   const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
   int32_t rc = run_offsets(ctx, 0, c.n_layers, ctx->d_dec_packed_off, nullptr, 1, ctx->d_dec_off, st);
   if (rc != CAKE_OK) return rc;
+  // positions in packed order (context scratch), then the decode state and the rows
+  rc = run_sorted_positions(ctx, 0, ctx->n_req, 0, c.n_layers, ctx->d_dec_packed_off, ctx->d_pos_packed, 0, st);
+  if (rc != CAKE_OK) return rc;
   if (row_offsets)
     CAKE_CUDA_TRY(cudaMemcpyAsync(row_offsets, ctx->d_dec_off, sizeof(int64_t) * (ctx->n_req * c.n_layers + 1),
                                   cudaMemcpyDeviceToDevice, st));
   if (ctx->n_req == 0) return CAKE_OK;
-  // positions in packed order (context scratch), then the decode state and the rows
-  rc = run_sorted_positions(ctx, 0, ctx->n_req, 0, c.n_layers, ctx->d_dec_packed_off, ctx->d_pos_packed, 0, st);
-  if (rc != CAKE_OK) return rc;
   const dim3 grid(c.n_kv_heads, c.n_layers, ctx->n_req);
-  decode_build<<<grid, DEC_THREADS, 0, st>>>(ctx->d_lists, ctx->d_prefix, ctx->d_lstate, ctx->d_req, budget,
-                                             ctx->d_dec_packed_off, ctx->d_pos_packed, ctx->d_dec_off,
-                                             ctx->d_dec_score, ctx->d_dec_pos, ctx->d_dec_order,
-                                             ctx->d_dec_meta, c.n_layers, c.n_kv_heads, c.window);
+  decode_build<<<grid, DEC_THREADS, 0, st>>>(ctx->d_store, ctx->d_req, budget, ctx->d_dec_packed_off,
+                                             ctx->d_pos_packed, ctx->d_dec_off, ctx->d_dec_score, ctx->d_dec_pos,
+                                             ctx->d_dec_order, ctx->d_dec_meta, c.n_layers, c.n_kv_heads, c.window,
+                                             ctx->total_tokens);
   count_launch();
   CAKE_CUDA_TRY(cudaGetLastError());
   return run_gather(ctx, ptrs, ctx->d_dec_packed_off, ctx->d_dec_off, ctx->d_pos_packed, k_cache, v_cache, st);

@@ -18,12 +18,6 @@ constexpr int SEL_WIDE_CTAS = 128;             // CTAs (one per SM) up to which 
 constexpr int kSelShare = 2048;                // values per CTA below which a head is spread no further
 constexpr int kSelSmemKeys = 40 * 1024;        // keys a CTA holds in shared memory; a larger share is read again
 
-// Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
-__device__ __forceinline__ uint32_t sel_key(float v) {
-  uint32_t b = __float_as_uint(v);
-  if (b == 0x80000000u) b = 0u;
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
 __device__ __forceinline__ uint32_t sel_cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -85,7 +79,7 @@ select_positions_static(const float* __restrict__ values, int n, int keep, int32
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int i = i0 + u * SEL_THREADS + (int)threadIdx.x;
-        k[u] = i < cnt ? (round > 0 && held ? keys[i] : sel_key(__ldg(&v[i]))) : 0u;
+        k[u] = i < cnt ? (round > 0 && held ? keys[i] : ordered_key(__ldg(&v[i]))) : 0u;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -162,7 +156,7 @@ select_positions_static(const float* __restrict__ values, int n, int keep, int32
   const int per = (cnt + SEL_THREADS - 1) / SEL_THREADS * 32;        // values per warp, whole ballots
   const int w_lo = min(cnt, warp * per), w_hi = min(cnt, w_lo + per);
   uint2 mine = make_uint2(0, 0);
-  auto key_at = [&](int i) { return i < w_hi ? (held ? keys[i] : sel_key(__ldg(&v[i]))) : 0u; };
+  auto key_at = [&](int i) { return i < w_hi ? (held ? keys[i] : ordered_key(__ldg(&v[i]))) : 0u; };
   for (int i0 = w_lo; i0 < w_hi; i0 += 128) {
     uint32_t k[4];
 #pragma unroll

@@ -1,0 +1,59 @@
+"""Which positions a budget keeps, where the selection can go wrong: rows that start at every 16-byte offset
+and end around the groups of 8 and 32 values, threshold buckets with more values than the list in shared
+memory holds, many equal values at the cut, thresholds below zero, infinite and lowest values.
+Positions are whole numbers and are compared exactly with the oracle's TopK on the same values."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cake_oracle as O
+from paper_2503_12491_b200 import harness, synth
+
+pytestmark = pytest.mark.gpu
+
+WINDOW = 2
+
+
+def values(kind, n, rng):
+    x = rng.normal(size=n).astype(np.float32)
+    if kind == "spread":
+        return np.exp(x)
+    if kind == "one bucket":                         # distinct values with the same leading bits
+        return (1.0 + rng.permutation(n) / (16.0 * n)).astype(np.float32)
+    if kind == "all equal":
+        return np.full(n, 0.25, dtype=np.float32)
+    if kind == "ties":                               # a third of the values equal, around the cut
+        return np.where(rng.random(n) < 0.33, np.float32(1.0), np.exp(x))
+    if kind == "negative":
+        return -np.exp(x)
+    x[rng.random(n) < 0.1] = np.inf                  # "extremes"
+    x[rng.random(n) < 0.3] = np.finfo(np.float32).min
+    return x
+
+
+@pytest.mark.parametrize("lens", [(901, 902, 903, 904, 31, 33), (3, 34, 35, 4090, 4103), (40007,), (131072,)])
+@pytest.mark.parametrize("kind", ["spread", "one bucket", "all equal", "ties", "negative", "extremes"])
+def test_positions_of_a_budget(kind, lens):
+    w = synth.scaled(synth.workload(1), n_layers=1, n_q_heads=3, n_kv_heads=3, window=WINDOW, seq_lens=lens,
+                     total_budget=WINDOW + max(lens) // 7 + 1)
+    rng = np.random.default_rng(len(kind) + max(lens))
+    ind = np.zeros((w.n_kv_heads, w.total_tokens), dtype=np.float32)
+    cu = w.cu_seqlens
+    for g in range(w.n_kv_heads):
+        for r, N in enumerate(lens):
+            ind[g, cu[r]:cu[r] + N - WINDOW] = values(kind, N - WINDOW, rng)
+    cake = harness.cake_for(w)
+    cake.begin(cu)
+    cake.set_preferences(torch.ones(len(lens), 1, dtype=torch.float64, device="cuda"))
+    cake.set_indicators(0, torch.from_numpy(ind).cuda())
+    cake.allocate(0)
+    cake.evict(0)
+    budgets = cake.get_budgets().cpu().numpy()
+    for r, N in enumerate(lens):
+        n, b = N - WINDOW, int(budgets[r, 0])
+        got = cake.get_positions(r, 0, b).cpu().numpy()
+        for g in range(w.n_kv_heads):
+            want = np.concatenate([O.topk_keep(ind[g, cu[r]:cu[r] + n].astype(np.float64), b - WINDOW), np.arange(n, N)])
+            assert np.array_equal(got[g], want), (r, g)
+    assert cake.status() == 0
+    cake.destroy()
