@@ -345,7 +345,7 @@ int32_t cake_plan_info(const cake_ctx* ctx, int32_t* out8);
 /* Builds the score kernel's launch plan for a batch on the HOST alone (no device, no context: it
  * runs without a GPU) and checks what the kernel relies on: every key tile covered exactly once
  * per pass, every CTA's program ordered so that a wave's column pass can only wait for row-pass
- * ops that wait for nothing, merge groups within one wave or the last two, table sizes, and that no warp
+ * ops that wait for nothing, merge groups within one wave, table sizes, and that no warp
  * overwrites exchanged rows which another may still read.  n_sm = SMs of
  * the device to plan for, reserved_sms as CAKE_RESERVED_SMS.  info8 (HOST, 8 int32): CTAs,
  * waves, merge ways, pass-A segments, pass-B segments, ops of the two-pass programs, ops of the

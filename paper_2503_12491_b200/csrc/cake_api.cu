@@ -82,8 +82,7 @@ void free_ctx(cake_ctx* c) {
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
   cudaFree(c->d_scores); cudaFree(c->d_simt_arrivals);
   cudaFree(c->d_rowpart);
-  cudaFree(c->d_tc_ops); cudaFree(c->d_tc_index); cudaFree(c->d_tc_sync);
-  cudaFree(c->d_tc_rowpart); cudaFree(c->d_lse2_tc);
+  cudaFree(c->d_tc_ops); cudaFree(c->d_tc_index); cudaFree(c->d_tc_exch);
   cudaFree(c->d_dec_off); cudaFree(c->d_dec_packed_off); cudaFree(c->d_dec_score); cudaFree(c->d_dec_tmp); cudaFree(c->d_dec_pos);
   cudaFree(c->d_dec_order); cudaFree(c->d_dec_meta);
   if (c->h_budget_stage) cudaFreeHost(c->h_budget_stage);
@@ -239,14 +238,12 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     x->max_tc_ops = (int32_t)(3 * segs + 8);
   }
   if (x->use_tc) {
-    const size_t n_index = 3 * (size_t)(max_pairs + 1) + 2 * (size_t)(x->n_sm + 1);
+    const size_t n_index = tc_index_size(max_pairs, x->n_sm);
     ok = ok && cudaMallocHost((void**)&x->h_tc_ops, sizeof(ScoreOp) * x->max_tc_ops) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&x->h_tc_index, sizeof(int32_t) * n_index) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_ops, x->max_tc_ops) == cudaSuccess;
     ok = ok && dev_alloc(&x->d_tc_index, n_index) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_tc_sync, 2 * (size_t)max_pairs) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_tc_rowpart, (size_t)x->max_tc_segs * kScoreGroups * 128) == cudaSuccess;
-    ok = ok && dev_alloc(&x->d_lse2_tc, (size_t)max_pairs * 128) == cudaSuccess;
+    ok = ok && dev_alloc(&x->d_tc_exch, tc_exchange_bytes(max_pairs, x->max_tc_segs)) == cudaSuccess;
   }
   // decode-time state: one slot per packed row plus one spare per (request, layer, head)
   x->dec_rows_cap = x->pos_packed_cap + x->max_lists;
@@ -381,7 +378,7 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
     CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_units, ctx->h_units, sizeof(ScoreUnit) * nu,
                                   cudaMemcpyHostToDevice, st));
     if (ctx->use_tc && ctx->n_tc_ctas > 0) {
-      const size_t n_index = 3 * (size_t)(n_req * c.n_kv_heads + 1) + 2 * (size_t)(ctx->n_sm + 1);
+      const size_t n_index = tc_index_size((int64_t)n_req * c.n_kv_heads, ctx->n_sm);
       CAKE_CUDA_TRY(cudaMemcpyAsync(ctx->d_tc_ops, ctx->h_tc_ops,
                                     sizeof(ScoreOp) * (ctx->n_tc_ops_full + ctx->n_tc_ops_b),
                                     cudaMemcpyHostToDevice, st));
@@ -393,8 +390,9 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
   }
   if (n_req == 0) { ctx->n_units = 0; ctx->packed_rows_bound = 0; ctx->n_tc_ctas = 0; }
   if (ctx->use_tc) {
-    ctx->tc_epoch = 0;
-    CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_tc_sync, 0, sizeof(uint32_t) * 2 * ctx->max_pairs, st));
+    ctx->tc_tag = 0;
+    if (ctx->n_tc_ctas > 0)
+      CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_tc_exch, 0, tc_exchange_bytes((int64_t)n_req * c.n_kv_heads, ctx->n_tc_asegs), st));
   }
   ctx->n_req = n_req;
   ctx->total_tokens = T;

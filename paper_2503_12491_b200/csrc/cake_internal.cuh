@@ -183,7 +183,7 @@ struct cake_ctx {
   int32_t debug_epoch_skew;       // test hook: added to the launch count the cross-CTA waits expect
   int32_t n_tc_asegs, n_tc_bsegs;          // pass-A / pass-B segments per layer
   int32_t n_tc_ops_full, n_tc_ops_b, max_tc_ops;
-  uint32_t tc_epoch;              // both-pass launches since cake_begin
+  uint32_t tc_tag;                // both-pass launches since cake_begin: mark of the rows they exchange
   cake::ScoreOp* h_tc_ops;        // pinned: [both-pass programs][pass-B-only programs]
   cake::ScoreOp* d_tc_ops;
   // pinned / device index block of the current batch, P = n_req * H_kv pairs:
@@ -192,11 +192,9 @@ struct cake_ctx {
   int32_t n_tc_groups;            // groups of pairs the merger warps take at once
   int32_t* h_tc_index;
   int32_t* d_tc_index;
-  uint32_t* d_tc_sync;            // [max_pairs] delivered partial rows, then [max_pairs] merged rows
   int tc_merge_ways;              // rows the merger warp handles side by side (a power of two up to 32), chosen with the plan
   bool tc_direct;                 // every CTA merges the denominators of its own pass-B ops (single-wave plans)
-  float4* d_tc_rowpart;           // [max_tc_segs][kScoreGroups][128]
-  float* d_lse2_tc;               // [max_requests][H_kv][128], rows in tile order i*G + h
+  uint8_t* d_tc_exch;             // rows that the CTAs of a score launch exchange (tc_exchange_bytes); cleared in cake_begin
   float* d_hrow[cake::kScoreDepth];   // [max_pairs][128] sum_j p log2 p per window row, by layer % score_depth
 };
 
@@ -211,6 +209,8 @@ int32_t launch_score_simt(cake_ctx* ctx, int32_t layer, const void* q_win, const
                           const float* lse, cudaStream_t st);
 // score_tc.cu
 bool tc_path_supported(const cake_config& c);
+size_t tc_index_size(int64_t pairs, int n_sm);
+size_t tc_exchange_bytes(int64_t pairs, int64_t segs);
 int64_t tc_max_segments(const cake_config& c, int n_sm);
 int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req);
 int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_req, const int64_t* cu,

@@ -19,18 +19,27 @@
 // so pass B re-reads a wave's K from L2 shortly after pass A brought it in, and DRAM
 // sees K once.  Pass B of a pair needs the pair's softmax denominators, i.e. every
 // CTA's pass-A partial rows.  The merge is spread over the grid by rows: the merger warp
-// of CTA (pair * rows + r) % grid waits until all partials of the pair are delivered, loads
-// row r's partials in a single round trip, merges them and counts the row as done.  The pass A
-// of the next wave sits between a pair's pass A and its pass B, so pass B's wait on
-// that count is normally already satisfied.
+// of CTA (pair * rows + r) % grid waits for row r's partials, merges them and hands the row to all
+// CTAs.  The pass A of the next wave sits between a pair's pass A and its pass B, so the
+// denominators are normally there in time.
+//
+// Exchange.  Rows that go from CTA to CTA carry the mark of their launch beside the data, in one 16- or 8-byte
+// access: the reader polls the data itself.  With counters (fence, count, poll, load, and the same again for
+// the merged rows) the denominators came 7 to 12 us after the last CTA's pass A; they come after 4.
+//
+// Bound.  A key tile of 128 keys and 128 rows is 16 384 exponentials per pass: 1024 cycles of the special-function
+// unit.  A statistics warp takes 3400 to 3700 cycles for its share of three tiles (3072 at the unit's rate) with the
+// next TMEM columns on their way during the arithmetic; with a load, a wait and a check per 32 columns it
+// took 3800 (pass B) and 4600 (pass A).  128K layer, 128 CTAs: 120 us per launch before, 111 now: long
+// prompts run into the device's power limit, of which the MMAs take the largest part (610 W above idle
+// at this kernel's rate, whatever the operands' source or the tile's width; the statistics 235 W).
 //
 // Warp roles in a CTA of 512 threads: warps 0..11 are "statistics" warps in three groups of
 // four (a group takes every third accumulator tile, a warp owns 32 of its TMEM lanes and writes
 // its own partial results; warps meet only where partial rows are exchanged, see xrow_slot), warp 12 issues TMA loads, warp 13 owns the
 // tensor-memory allocation and issues the MMAs (both as converged warps with an elected lane),
-// warp 14 publishes this CTA's finished pass-A ops to the grid and merges rows, warp 15 stages
-// the denominators of the next pass-B op in shared memory.  Every wait
-// (mbarrier or flag) is bounded; a timed-out wait raises CAKE_ERR_TIMEOUT and the CTA
+// warp 14 merges rows, warp 15 stages the denominators of the next pass-B op in shared memory.  Every wait
+// (mbarrier or exchanged row) is bounded; a timed-out wait raises CAKE_ERR_TIMEOUT and the CTA
 // drains and exits.
 #include "cake_internal.cuh"
 
@@ -46,11 +55,10 @@ namespace {
 
 constexpr int TILE = 128;            // keys per tile
 constexpr int STAGES = 4;            // K tiles in flight
-constexpr int NBUF = 3;              // accumulator buffers: 3 x 128 of the 512 TMEM columns
-constexpr int TMEM_Q_COL = NBUF * 128;   // + 64 columns: the window queries as pass A's A operand
+constexpr int NBUF = 4;              // accumulator buffers of 128 columns, all of tensor memory: one more than there are
+                                     // groups, so that a group's next tile is multiplied while it holds this one
 constexpr int NWG = kScoreGroups;    // statistics warp groups
-static_assert(NWG == NBUF, "one accumulator buffer per statistics group");
-static_assert(NWG * 4 <= 16, "a_done holds one counter per statistics warp");
+static_assert((NBUF & (NBUF - 1)) == 0, "a tile's buffer and phase are bit fields of its number");
 constexpr int STAT_THREADS = NWG * 128;
 constexpr int TC_THREADS = STAT_THREADS + 128;  // + TMA, MMA, row-merger and denominator warps
 constexpr int WARP_TMA = NWG * 4, WARP_MMA = NWG * 4 + 1, WARP_MERGE = NWG * 4 + 2,
@@ -59,10 +67,11 @@ constexpr int NSTATW = NWG * 4;      // statistics warps
 constexpr int SLAB_BYTES = TILE * 128;   // one 64-element slab of a 128-row tile
 constexpr long long kSpinLimit = 4000000000ll;   // default cycles (~2 s) before a wait gives up
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kChunkSumMax = 65536.f;   // a pass-A chunk sum beyond this moves the row's reference
+constexpr float kTileSumMax = 1.2676506e30f;    // pass A: a tile whose sum is beyond 2^100 is taken again from its maxima,
+constexpr float kShiftSum = 256.f;              // one beyond this moves the row's reference up afterwards
 constexpr int64_t kWaveBytes = 32ll << 20;
+constexpr int kLseStride = 16;        // merged rows lie a line of L2 (128 bytes) apart, see lse2
 constexpr int kDirectSegs = 40;       // segments of a pair up to which every CTA merges its rows for itself
-constexpr int kWaveDepth = 1;         // pass B of a wave follows pass A of the wave this far ahead
 
 struct TcParams {
   const ScoreOp* ops;
@@ -71,17 +80,17 @@ struct TcParams {
   int n_groups;
   const ReqInfo* reqs;
   const int32_t* pair_aseg;     // [pairs + 1] pass-A segment ranges per pair
-  uint32_t* pair_cnt;           // [pairs] delivered pass-A partials (monotonic over layers)
-  uint32_t* pair_done;          // [pairs] merged rows (monotonic over layers); null = pass B only
-  float* lse2;                  // [pair][128] in tile row order r' = i*G + h
+  int both;                     // 0: pass B alone
+  uint32_t tag, want;           // mark of this launch's exchanged rows, and the one that readers wait for
+  uint2* lse2;                  // [pair][128] in tile row order r' = i*G + h, kLseStride apart: base-2 log-sum-exp, tag.  A
+                                // line that several CTAs write while others poll it costs a round trip per write
   const float* lse_ext;         // caller's natural-log LSE [req][H_q][S_w], or null
-  float4* rowpart;              // pass A out: [A-segment][group][128] (m, z_all, z_win, w)
+  float4* rowpart;              // pass A out: [A-segment][group][128], see pack_part
   float* raw;                   // pass B out: [H_kv][T]
   float* colpart;               // pass B out: [B-segment][statistics warp][G][2]
   float* hrow;                  // [pair][128] sum_j p log2 p of every window row
   int32_t* status;
   int64_t T;
-  uint32_t epoch;
   long long spin_limit;         // cycles after which a wait gives up and raises CAKE_ERR_TIMEOUT
   int n_pairs;
   int Hkv, Hq, Sw, rows, d;
@@ -142,6 +151,13 @@ __device__ __forceinline__ void tma_load_3d_hint(void* dst, const CUtensorMap* m
       ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
       : "memory");
 }
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int c0, int c1, int c2) {
+  asm volatile(
+      "{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
+      "@e cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];\n}"
+      ::"l"(map), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
@@ -183,15 +199,6 @@ __device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint32_t a_lo, uint32_t
       ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kAcc), "r"(kDescHi)
       : "memory");
 }
-template <int kAcc>
-__device__ __forceinline__ void umma_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_lo, uint32_t idesc) {
-  asm volatile(
-      "{\n.reg .pred p, e;\n.reg .b64 db;\nsetp.ne.b32 p, %4, 0;\nelect.sync _|e, 0xffffffff;\n"
-      "mov.b64 db, {%2, %5};\n"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n}"
-      ::"r"(tmem_d), "r"(tmem_a), "r"(b_lo), "r"(idesc), "n"(kAcc), "r"(kDescHi)
-      : "memory");
-}
 // The same with an explicit high descriptor word: operands that are not in the 128-byte swizzle.
 template <int kAcc>
 __device__ __forceinline__ void umma_ss_hi(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
@@ -214,32 +221,46 @@ constexpr uint32_t kExtDescHi = (256u >> 4) | (1u << 14);            // SBO, ver
 constexpr uint32_t kExtDescLoLbo = (128u >> 4) << 16;                // LBO field of the low word
 __device__ __forceinline__ uint32_t ext_row_offset(int r) { return (uint32_t)((r >> 3) * 256 + (r & 7) * 16); }
 
-// Copies 128 rows x 32 bytes (one K = 16 slice of a K-major operand) from shared to tensor memory.
-__device__ __forceinline__ void tmem_cp_128x256b(uint32_t tmem_dst, uint64_t sdesc) {
-  asm volatile("{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n@e tcgen05.cp.cta_group::1.128x256b [%0], %1;\n}"
-               ::"r"(tmem_dst), "l"(sdesc) : "memory");
-}
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
                "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
                ::"r"(smem_u32(bar)) : "memory");
 }
-// Starts the load of 32 consecutive fp32 columns of this thread's TMEM lane; the registers
+// Starts the load of 16 consecutive fp32 columns of this thread's TMEM lane; the registers
 // are valid only after tmem_ld_wait on the same array.
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
 // Waits for the thread's outstanding TMEM loads.  The registers pass through the statement so
 // that no use of them can be scheduled before it.
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                :
                : "memory");
+}
+// Columns [lo, hi) of this thread's TMEM lane, 16 at a time: f(chunk) while the next chunk is on its way, so
+// that a warp has exponentials to issue all the time; `loaded` is called once all columns are in registers.
+template <typename F, typename L>
+__device__ __forceinline__ void for_columns(uint32_t taddr, int lo, int hi, F f, L loaded) {
+  uint32_t r0[16], r1[16];
+  tmem_ld16_issue(taddr + lo, r0);
+#pragma unroll 1
+  for (int c = lo; c < hi; c += 32) {
+    tmem_ld_wait(r0);
+    if (c + 16 < hi) tmem_ld16_issue(taddr + c + 16, r1);
+    else loaded();
+    f(r0);
+    if (c + 16 >= hi) break;
+    tmem_ld_wait(r1);
+    if (c + 32 < hi) tmem_ld16_issue(taddr + c + 32, r0);
+    else loaded();
+    f(r1);
+  }
 }
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -275,36 +296,31 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   return d;
 }
 
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes,
-// 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);          // start address
-  d |= (uint64_t)(1024u >> 4) << 32;                 // stride byte offset between 8-row groups
-  d |= (uint64_t)1 << 46;                            // descriptor version (sm_100)
-  d |= (uint64_t)2 << 61;                            // SWIZZLE_128B
-  return d;
-}
 // Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M x N tile.
 __device__ __forceinline__ uint32_t instr_desc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+// Rows that CTAs exchange carry the mark of the launch that wrote them, in the same 16 (or 8) bytes as the
+// data: they are written and read as one access each, so a reader that sees the mark has the data, and
+// neither side needs a fence, a counter or a second trip.
+__device__ __forceinline__ void st_row16(float4* p, float4 v) {
+  asm volatile("{\n.reg .b128 t;\n.reg .b64 lo, hi;\nmov.b64 lo, {%1, %2};\nmov.b64 hi, {%3, %4};\nmov.b128 t, {lo, hi};\n"
+               "st.relaxed.gpu.global.b128 [%0], t;\n}" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ float4 ld_row16(const void* p) {
+  float4 v;
+  asm volatile("{\n.reg .b128 t;\n.reg .b64 lo, hi;\nld.relaxed.gpu.global.b128 t, [%4];\nmov.b128 {lo, hi}, t;\n"
+               "mov.b64 {%0, %1}, lo;\nmov.b64 {%2, %3}, hi;\n}" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
   return v;
 }
-
-// Counters in shared memory that only grow, each written by one warp: a wait for "at least v"
-// cannot mistake one round for another, whoever waits and however late.
-__device__ __forceinline__ void smem_store_release(uint32_t* c, uint32_t v) {
-  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(c)), "r"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t smem_count_acquire(const uint32_t* c) {
-  uint32_t v;
-  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(c)) : "memory");
+__device__ __forceinline__ uint2 ld_row8(const uint2* p) {
+  uint2 v;
+  asm volatile("{\n.reg .b64 t;\nld.relaxed.gpu.global.b64 t, [%2];\nmov.b64 {%0, %1}, t;\n}" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ void st_row8(uint2* p, uint32_t a, uint32_t b) {
+  asm volatile("{\n.reg .b64 t;\nmov.b64 t, {%1, %2};\nst.relaxed.gpu.global.b64 [%0], t;\n}" ::"l"(p), "r"(a), "r"(b) : "memory");
 }
 
 struct Smem {
@@ -318,9 +334,7 @@ struct Smem {
   uint64_t* q_empty;   // [2]
   uint64_t* lse_full;  // [2]
   uint64_t* lse_free;  // [2]
-  uint64_t* parts;     // [2] direct merge: the pair's partial rows are all delivered
   uint32_t* tmem_holder;
-  uint32_t* a_done;    // [NSTATW] pass-A ops whose partial rows each statistics warp has written
   uint8_t* ext_a;      // the constant key-side operand of the extra K step of pass B
   uint8_t* ext_b;      // [2] its row-side operand: -lse/scale of the current / next pass-B op
   float4* xrow;        // [2][NWG][128] partial rows of a group: copies of a row in pass A, then (direct merge) the
@@ -347,9 +361,7 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   s.q_empty = (uint64_t*)p;   p += 16;
   s.lse_full = (uint64_t*)p;  p += 16;
   s.lse_free = (uint64_t*)p;  p += 16;
-  s.parts = (uint64_t*)p;     p += 16;
   s.tmem_holder = (uint32_t*)p; p += 8;
-  s.a_done = (uint32_t*)p;    p += 4 * 16;
   p = (uint8_t*)(((uintptr_t)p + 15) & ~(uintptr_t)15);
   p = (uint8_t*)(((uintptr_t)p + 127) & ~(uintptr_t)127);
   s.ext_a = p;                p += kExtBytes;
@@ -359,8 +371,27 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   return s;
 }
 
-// Merge of two partial softmax rows (m, z_all, z_win, w) with base-2 exponents;
-// w = sum over observed keys of e * (logit2 - m).
+// A partial softmax row (m, z_all, z_win, w) with base-2 exponents: sums of e = 2^(logit2 - m) over all keys of the
+// segment and over those of the window, and w = sum over the observed keys of e * (logit2 - m).  m is any reference: on
+// its way to other CTAs a row has the one that puts z_all into [1, 2) (a scaling by a power of two), and the
+// launch's mark takes the place of z_all's exponent.  No keys: m = -inf.  A sum that is not finite: m = inf,
+// which makes the merged row NaN.
+__device__ __forceinline__ float4 pack_part(float m, float z, float zwin, float w, uint32_t tag) {
+  const uint32_t zb = __float_as_uint(z);
+  const int k = (int)(zb >> 23) - 127;
+  const float f = __uint_as_float((uint32_t)(127 - k) << 23);
+  float4 o = make_float4(m + (float)k, __uint_as_float((zb & 0x7FFFFFu) | (tag << 23)), zwin * f, fmaf(-(float)k, z - zwin, w) * f);
+  if (m == -CUDART_INF_F) o = make_float4(m, __uint_as_float(tag << 23), 0.f, 0.f);
+  else if (!(z <= 1e38f) || k < -120) o.x = CUDART_INF_F;
+  return o;
+}
+__device__ __forceinline__ bool part_tagged(const float4& v, uint32_t want) { return (__float_as_uint(v.y) >> 23) == want; }
+__device__ __forceinline__ float4 unpack_part(float4 v) {
+  v.y = v.x == -CUDART_INF_F ? 0.f : __uint_as_float((__float_as_uint(v.y) & 0x7FFFFFu) | 0x3F800000u);
+  return v;
+}
+
+// Merge of two partial rows.
 __device__ __forceinline__ float4 merge_rows(float4 a, float4 b) {
   if (b.x == -CUDART_INF_F) return a;
   if (a.x == -CUDART_INF_F) return b;
@@ -392,6 +423,41 @@ __device__ __forceinline__ float4 merge_batch(float4 acc, const float4 (&v)[K]) 
 #pragma unroll
   for (int u = 0; u < K; ++u) term(v[u], o);
   return o;
+}
+
+// Loads up to K partial rows per lane, at `stride` from one another, `count` of them in this lane (0 or less: none),
+// and waits until all have come, by the whole warp.  The first of every lane's is waited for alone, so that a
+// long wait costs the memory system little.  False (and the status set) if they do not come.
+template <int K>
+__device__ __forceinline__ bool wait_parts(const float4* p, int64_t stride, int count, uint32_t want, float4 (&v)[K],
+                                           int32_t* status, long long limit) {
+  const long long t0 = clock64();
+  uint32_t missing = 0;
+#pragma unroll
+  for (int u = 0; u < K; ++u) {
+    v[u] = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
+    missing |= u < count ? 1u << u : 0u;
+  }
+  for (bool first = true;; ) {
+    const uint32_t get = first ? missing & 1u : missing;
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+      if (get >> u & 1u) v[u] = ld_row16(p + u * stride);
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+      if ((get >> u & 1u) && part_tagged(v[u], want)) { v[u] = unpack_part(v[u]); missing &= ~(1u << u); }
+    const bool open = first ? (missing & 1u) != 0 : missing != 0;
+    if (!__any_sync(0xffffffffu, open)) {
+      if (!first) return true;
+      first = false;
+      continue;
+    }
+    if (__any_sync(0xffffffffu, clock64() - t0 > limit)) {
+      atomicCAS(status, 0, CAKE_ERR_TIMEOUT);
+      return false;
+    }
+    if (first) __nanosleep(40);
+  }
 }
 
 // -lse / scale as three bf16 terms (24 bits) in columns 0..2 of the rows' operand of the extra K step.
@@ -435,8 +501,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     for (int i = 0; i < STAGES; ++i) { mbar_init(&S.full[i], 1); mbar_init(&S.empty[i], 1); }
     for (int i = 0; i < NBUF; ++i) { mbar_init(&S.acc_full[i], 1); mbar_init(&S.acc_empty[i], 4); }
     for (int i = 0; i < 2; ++i) { mbar_init(&S.q_full[i], 1); mbar_init(&S.q_empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&S.lse_full[i], kDirect ? 4 : 1); mbar_init(&S.lse_free[i], 1); mbar_init(&S.parts[i], 1); }
-    for (int i = 0; i < NSTATW; ++i) S.a_done[i] = 0;
+    for (int i = 0; i < 2; ++i) { mbar_init(&S.lse_full[i], kDirect ? 4 : 1); mbar_init(&S.lse_free[i], 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // the program of this CTA: a global read per op would put an L2 round trip on every op
@@ -465,6 +530,13 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *S.tmem_holder;
+  if (warp == WARP_TMA && op_lo < op_hi) {
+    // The first key tiles start on their way to L2 while the kernel before this one ends.  (A prefetch reads nothing: if
+    // that kernel still writes K, its stores go to the same L2 lines.)
+    const ScoreOp op = get_op(op_lo);
+    const int n = min(STAGES, (op.nkeys + TILE - 1) / TILE);
+    for (int it = 0; it < n; ++it) tma_prefetch_3d(&k_map, 0, (int)(op.base + op.key0) + it * TILE, 0);
+  }
   // Up to here nothing was read that the kernel before this one in the stream may write (the op tables
   // come with the batch): a CTA starts as soon as an SM is free, while that kernel's last CTAs still run.
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -483,8 +555,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       bool ok = true;
       for (int oi = op_lo; oi < op_hi && ok; ++oi) {
         const ScoreOp op = get_op(oi);
-        if (op.nkeys <= 0) continue;
-        const uint64_t pol = (op.phase || !P.pair_done) ? drop : keep;
+        const uint64_t pol = (op.phase || !P.both) ? drop : keep;
         const int qb = qn & 1;
         // the MMAs of the op that used this query buffer two ops ago must be done
         ok = mbar_wait(&S.q_empty[qb], ((qn >> 1) & 1) ^ 1, P.status, P.spin_limit);
@@ -529,7 +600,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       bool ok = true;
       for (int oi = op_lo; oi < op_hi && ok; ++oi) {
         const ScoreOp op = get_op(oi);
-        if (op.nkeys <= 0) continue;
         const uint32_t idesc = op.phase ? instr_desc(128, rows_pad) : instr_desc(128, TILE);
         const int eslot = kbm & 1;
         const uint32_t ext_b_lo = ((smem_u32(S.ext_b + eslot * kExtBytes) & 0x3FFFFu) >> 4) | kExtDescLoLbo;
@@ -539,18 +609,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         if (!ok) break;
         const uint32_t qaddr = smem_u32(S.q + qb * kQBytes);
         const uint32_t q_lo = (qaddr & 0x3FFFFu) >> 4;      // address field of the descriptors
-        const uint32_t tmem_q = tmem_base + (uint32_t)TMEM_Q_COL;
-        if (!op.phase) {
-          // pass A multiplies every key tile by the same queries: hold them in tensor memory, so
-          // that an MMA reads only the key tile from shared memory.  The copies run in issue
-          // order behind the previous op's MMAs and ahead of this op's.
-          tc_fence_after();
-          for (int sl = 0; sl < n_slab; ++sl)
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              tmem_cp_128x256b(tmem_q + (uint32_t)((sl * 4 + ks) * 8),
-                               smem_desc(qaddr + sl * SLAB_BYTES + ks * 32));
-        }
         if (op.phase) {
           // the rows' -lse/scale operand of this op (written by the denominator warp)
           ok = mbar_wait(&S.lse_full[eslot], (kbm >> 1) & 1, P.status, P.spin_limit);
@@ -581,17 +639,17 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
             umma_ss_hi<1>(tmem_d, ext_a_lo, ext_b_lo, idesc, kExtDescHi);      // ... - lse/scale
           } else {
-            // D[row][key] = Q K^T, queries from tensor memory
-            umma_ts<0>(tmem_d, tmem_q, k_lo, idesc);
-            umma_ts<1>(tmem_d, tmem_q + 8, k_lo + 2, idesc);
-            umma_ts<1>(tmem_d, tmem_q + 16, k_lo + 4, idesc);
-            umma_ts<1>(tmem_d, tmem_q + 24, k_lo + 6, idesc);
+            // D[row][key] = Q K^T
+            umma_ss<0>(tmem_d, q_lo, k_lo, idesc);
+            umma_ss<1>(tmem_d, q_lo + 2, k_lo + 2, idesc);
+            umma_ss<1>(tmem_d, q_lo + 4, k_lo + 4, idesc);
+            umma_ss<1>(tmem_d, q_lo + 6, k_lo + 6, idesc);
             if (n_slab == 2) {
               constexpr uint32_t o = SLAB_BYTES >> 4;
-              umma_ts<1>(tmem_d, tmem_q + 32, k_lo + o, idesc);
-              umma_ts<1>(tmem_d, tmem_q + 40, k_lo + o + 2, idesc);
-              umma_ts<1>(tmem_d, tmem_q + 48, k_lo + o + 4, idesc);
-              umma_ts<1>(tmem_d, tmem_q + 56, k_lo + o + 6, idesc);
+              umma_ss<1>(tmem_d, q_lo + o, k_lo + o, idesc);
+              umma_ss<1>(tmem_d, q_lo + o + 2, k_lo + o + 2, idesc);
+              umma_ss<1>(tmem_d, q_lo + o + 4, k_lo + o + 4, idesc);
+              umma_ss<1>(tmem_d, q_lo + o + 6, k_lo + o + 6, idesc);
             }
           }
           umma_commit(&S.empty[s]);
@@ -606,183 +664,69 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
   } else if (warp == WARP_MERGE) {
     // ------------------------------------------------ row merger
-    // Every (pair, row) is merged by one CTA of the grid: once all partials of the pair have
-    // been delivered, the warp loads the row's partials in one round trip, merges them in a
-    // fixed order and publishes the row's base-2 log-sum-exp and entropy term.
-    if (P.pair_done) {
+    // Every (pair, row) is merged by one CTA of the grid: row r of pair p by CTA (p * rows + r) % grid, so that with
+    // many short pairs every CTA gets a few rows.  The warp waits for the row's partials, merges them in a
+    // fixed order and publishes the row's base-2 log-sum-exp and entropy term.  Short pairs (a ragged batch,
+    // MHA) have few partials per row: the rows of `ways` consecutive pairs are merged side by side, by
+    // 32 / ways lanes each.
+    if (P.both && !kDirect) {
+      constexpr int kBatch = 12;                     // loads per lane in flight: the 384 partials of a row at 128 CTAs
+      const int ways = P.merge_ways, lpr = 32 / ways;         // lanes per row
+      const int sub = lane / lpr, l8 = lane % lpr;
       bool ok = true;
-      // Publishes, in program order, every pass-A op of this CTA whose twelve partial row sets
-      // are written: one fence, then the op's count goes to its pair.
-      int pub_oi = op_lo;
-      uint32_t pub = 0;
-      auto publish = [&]() -> bool {               // true once every pass-A op is published
-        while (pub_oi < op_hi) {
-          const ScoreOp o = get_op(pub_oi);
-          if (o.nkeys <= 0 || o.phase) { ++pub_oi; continue; }
-          // every statistics warp counts its own finished pass-A ops: a warp whose group has
-          // no tile in an op runs ahead of the others, so a single shared count of arrivals
-          // could be reached before the slowest warp has written this op's rows
-          const uint32_t mine = lane < NSTATW ? smem_count_acquire(&S.a_done[lane]) : 0xFFFFFFFFu;
-          if (!__all_sync(0xffffffffu, mine >= pub + 1u)) return false;
-          __threadfence();
-          if (lane == 0) atomicAdd(&P.pair_cnt[o.req * P.Hkv + o.g], (uint32_t)NSTATW);
-          ++pub;
-          ++pub_oi;
-        }
-        return true;
-      };
-      if constexpr (kDirect) {
-        // nothing to merge here: the statistics warps do it
-      } else if (P.merge_ways > 1) {
-        // Short pairs (a ragged batch, MHA): a wave holds several pairs whose rows have few
-        // partials each, so the rows of `ways` (2 to 32) consecutive pairs are merged side by side,
-        // by 32 / ways lanes each, and the wave's denominators are ready that much sooner.
-        const int ways = P.merge_ways, lpr = 32 / ways;         // lanes per row
-        const int sub = lane / lpr, l8 = lane % lpr;
-        for (int gi = 0; gi < P.n_groups && ok; ++gi) {
-          const int pair = (P.group_begin ? P.group_begin[gi] : gi * ways) + sub;
-          const bool have = pair < (P.group_begin ? P.group_begin[gi + 1] : P.n_pairs);
-          const int s_lo = have ? P.pair_aseg[pair] * NWG : 0, s_hi = have ? P.pair_aseg[pair + 1] * NWG : 0;
-          const int r0 = have ? (int)((blockIdx.x + gridDim.x - (unsigned)(((long long)pair * P.rows) % gridDim.x)) % gridDim.x)
-                              : P.rows;
-          bool waited = false;
-          for (int r = r0;; r += gridDim.x) {
-            const bool active = have && r < P.rows;
-            if (!__any_sync(0xffffffffu, active)) break;
-            if (!waited) {
-              const uint32_t want = (uint32_t)(s_hi - s_lo) * 4u * P.epoch;
-              const long long t0 = clock64();
-              for (;;) {
-                const bool ready = !active || ld_acquire(&P.pair_cnt[pair]) >= want;
-                if (__all_sync(0xffffffffu, ready)) break;
-                publish();
-                if (clock64() - t0 > P.spin_limit) { atomicCAS(P.status, 0, CAKE_ERR_TIMEOUT); ok = false; break; }
-                __nanosleep(100);
-              }
-              if (!ok) break;
-              waited = true;
-            }
-            float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-            if (active) {
-              for (int base = s_lo; base < s_hi; base += 8 * lpr) {
-                float4 pv[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                  const int sg = base + u * lpr + l8;
-                  pv[u] = sg < s_hi ? __ldcg(&P.rowpart[(size_t)sg * 128 + r])
-                                    : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) acc = merge_rows(acc, pv[u]);
-              }
-            }
-            for (int o = lpr >> 1; o > 0; o >>= 1) {           // inside the lanes of a row
-              float4 other;
-              other.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
-              other.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
-              other.z = __shfl_xor_sync(0xffffffffu, acc.z, o);
-              other.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
-              acc = (lane & o) ? merge_rows(other, acc) : merge_rows(acc, other);
-            }
-            if (active && l8 == 0) {
-              const float lz = log2f(acc.y);
-              __stcg(&P.lse2[(size_t)pair * 128 + r], acc.x + lz);
-              __stcg(&P.hrow[(size_t)pair * 128 + r], (acc.w - lz * (acc.y - acc.z)) / acc.y);
-              __threadfence();
-              atomicAdd(&P.pair_done[pair], 1u);
-            }
-          }
-        }
-      } else
-      for (int pair = 0; pair < P.n_pairs && ok; ++pair) {
-        const int s_lo = P.pair_aseg[pair] * NWG, s_hi = P.pair_aseg[pair + 1] * NWG;
-        bool waited = false;
-        // row r of pair p belongs to CTA (p * rows + r) % grid: with many short pairs every CTA
-        // gets a few (pair, row) items instead of the first `rows` CTAs getting all of them
-        const int r0 = (int)((blockIdx.x + gridDim.x - (unsigned)(((long long)pair * P.rows) % gridDim.x)) % gridDim.x);
-        for (int r = r0; r < P.rows; r += gridDim.x) {
-          if (!waited) {
-            const uint32_t want = (uint32_t)(s_hi - s_lo) * 4u * P.epoch;   // one per warp
-            const long long t0 = clock64();
-            while (ld_acquire(&P.pair_cnt[pair]) < want) {
-              publish();
-              if (clock64() - t0 > P.spin_limit) { atomicCAS(P.status, 0, CAKE_ERR_TIMEOUT); ok = false; break; }
-              __nanosleep(40);
-            }
-            if (!ok) break;
-            waited = true;
-          }
+      for (int gi = 0; gi < P.n_groups && ok; ++gi) {
+        const int pair = (P.group_begin ? P.group_begin[gi] : gi * ways) + sub;
+        const bool have = pair < (P.group_begin ? P.group_begin[gi + 1] : P.n_pairs);
+        const int s_lo = have ? P.pair_aseg[pair] * NWG : 0, s_hi = have ? P.pair_aseg[pair + 1] * NWG : 0;
+        const int r0 = have ? (int)((blockIdx.x + gridDim.x - (unsigned)(((long long)pair * P.rows) % gridDim.x)) % gridDim.x)
+                            : P.rows;
+        for (int r = r0; ok; r += gridDim.x) {
+          const bool active = have && r < P.rows;
+          if (!__any_sync(0xffffffffu, active)) break;
           float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-          // 12 loads per lane in flight: the 384 partials of a row at 128 CTAs come in one round trip
-          for (int base = s_lo; base < s_hi; base += 32 * 12) {
-            float4 pv[12];
-#pragma unroll
-            for (int u = 0; u < 12; ++u) {
-              const int sg = base + u * 32 + lane;
-              pv[u] = sg < s_hi ? __ldcg(&P.rowpart[(size_t)sg * 128 + r])
-                                : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < 12; ++u) acc = merge_rows(acc, pv[u]);
+          for (int base = s_lo;; base += kBatch * lpr) {
+            if (!__any_sync(0xffffffffu, active && base < s_hi)) break;
+            const int left = s_hi - base - l8;         // partials base + l8, base + l8 + lpr, ...
+            float4 pv[kBatch];
+            ok = wait_parts(&P.rowpart[(size_t)(base + l8) * 128 + (active ? r : 0)], (int64_t)lpr * 128,
+                            active ? (left + lpr - 1) / lpr : 0, P.want, pv, P.status, P.spin_limit);
+            if (!ok) break;
+            acc = merge_batch(acc, pv);
           }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            float4 other;
-            other.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
-            other.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
-            other.z = __shfl_xor_sync(0xffffffffu, acc.z, o);
-            other.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
-            // the lower lane's partial always goes first, so every lane gets the same result
-            acc = (lane & o) ? merge_rows(other, acc) : merge_rows(acc, other);
+          if (!ok) break;
+          // over the lanes of a row: the largest reference, then the sums
+          float mx = acc.x;
+          for (int o = lpr >> 1; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          const float d = acc.x == -CUDART_INF_F ? 0.f : acc.x - mx, f = acc.x == -CUDART_INF_F ? 0.f : exp2f(d);
+          float w = f * fmaf(d, acc.y - acc.z, acc.w), z = acc.y * f, zwin = acc.z * f;
+          for (int o = lpr >> 1; o > 0; o >>= 1) {
+            z += __shfl_xor_sync(0xffffffffu, z, o);
+            zwin += __shfl_xor_sync(0xffffffffu, zwin, o);
+            w += __shfl_xor_sync(0xffffffffu, w, o);
           }
-          if (lane == 0) {
-            const float lz = log2f(acc.y);
-            __stcg(&P.lse2[(size_t)pair * 128 + r], acc.x + lz);
+          if (active && l8 == 0) {
+            const float lz = log2f(z);
+            st_row8(&P.lse2[((size_t)pair * 128 + r) * kLseStride], __float_as_uint(mx + lz), P.tag);
             // sum_j p log2 p over the observed keys = (w - log2(z) * z_obs) / z
-            __stcg(&P.hrow[(size_t)pair * 128 + r], (acc.w - lz * (acc.y - acc.z)) / acc.y);
-            __threadfence();
-            atomicAdd(&P.pair_done[pair], 1u);
+            __stcg(&P.hrow[(size_t)pair * 128 + r], (w - lz * (z - zwin)) / z);
           }
         }
-      }
-      // ops that finish after this warp's last merge
-      const long long t0 = clock64();
-      while (ok && !publish()) {
-        if (clock64() - t0 > P.spin_limit) { atomicCAS(P.status, 0, CAKE_ERR_TIMEOUT); break; }
-        __nanosleep(100);
       }
     }
   } else if (warp == WARP_LSE) {
     // ------------------------------------------------ denominator fetcher
-    // For every pass-B op of this CTA, in program order: wait until all rows of the op's pair
-    // are merged, copy the pair's 128 denominators into a two-slot shared-memory ring.
+    // For every pass-B op of this CTA, in program order: wait until all rows of the op's pair are
+    // merged, write the pair's -lse/scale operand into a two-slot shared-memory ring.
     uint32_t kb = 0;
     bool ok = true;
-    for (int oi = op_lo; oi < op_hi && ok; ++oi) {
+    for (int oi = op_lo; oi < op_hi && ok && !kDirect; ++oi) {
       const ScoreOp op = get_op(oi);
-      if (op.nkeys <= 0 || !op.phase) continue;
+      if (!op.phase) continue;
       const int slot = kb & 1;
       const int pair = op.req * P.Hkv + op.g;
-      if (lane == 0) {
-        ok = mbar_wait(&S.lse_free[slot], ((kb >> 1) & 1) ^ 1, P.status, P.spin_limit);
-        if (ok && P.pair_done) {
-          const uint32_t want = kDirect ? (uint32_t)(P.pair_aseg[pair + 1] - P.pair_aseg[pair]) * (uint32_t)NSTATW * P.epoch
-                                        : (uint32_t)P.rows * P.epoch;
-          const uint32_t* count = kDirect ? &P.pair_cnt[pair] : &P.pair_done[pair];
-          const long long t0 = clock64();
-          while (ld_acquire(count) < want) {
-            if (clock64() - t0 > P.spin_limit) { atomicCAS(P.status, 0, CAKE_ERR_TIMEOUT); ok = false; break; }
-            __nanosleep(32);
-          }
-        }
-      }
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      ok = mbar_wait(&S.lse_free[slot], ((kb >> 1) & 1) ^ 1, P.status, P.spin_limit);
+      ok = __all_sync(0xffffffffu, ok) != 0;
       if (!ok) break;
-      if constexpr (kDirect) {                       // the statistics warps take it from here
-        if (lane == 0) mbar_arrive(&S.parts[slot]);
-        ++kb;
-        continue;
-      }
       float4 v;
       if (P.lse_ext) {
         // the caller's natural-log values [req][H_q][S_w]: tile row r' = i*G + h, base 2
@@ -794,7 +738,32 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         v = make_float4(x[0], x[1], x[2], x[3]);
       } else {
-        v = __ldcg(reinterpret_cast<const float4*>(P.lse2 + (size_t)pair * 128) + lane);
+        const uint2* at = P.lse2 + ((size_t)pair * 128 + 4 * lane) * kLseStride;      // rows 4 * lane ..
+        const bool mine = 4 * lane < P.rows;           // (rows is a multiple of 32)
+        const long long t0 = clock64();
+        // A CTA waits for one row, another one than its neighbours, before it asks for all: 128 CTAs that poll the
+        // same lines delay the stores they wait for.
+        const int probe = (int)(blockIdx.x % (unsigned)P.rows);
+        uint2 x[4];
+        for (bool all = false;;) {
+          if (!all) {
+            uint2 p = make_uint2(0u, 0u);
+            if (lane == 0) p = ld_row8(P.lse2 + ((size_t)pair * 128 + probe) * kLseStride);
+            all = __any_sync(0xffffffffu, p.y == P.want);
+          }
+          bool got = all;
+          if (all) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = mine ? ld_row8(at + e * kLseStride) : make_uint2(0u, P.want);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) got = got && x[e].y == P.want;
+          }
+          if (__all_sync(0xffffffffu, got)) break;
+          if (__any_sync(0xffffffffu, clock64() - t0 > P.spin_limit)) { atomicCAS(P.status, 0, CAKE_ERR_TIMEOUT); ok = false; break; }
+          __nanosleep(32);
+        }
+        if (!ok) break;
+        v = make_float4(__uint_as_float(x[0].x), __uint_as_float(x[1].x), __uint_as_float(x[2].x), __uint_as_float(x[3].x));
       }
       {
         const float vv[4] = {v.x, v.y, v.z, v.w};
@@ -811,16 +780,12 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // Every warp owns TMEM lanes 32*quad.. of the tiles its group takes and writes its own partial
     // results.  It waits for other statistics warps only where rows are exchanged: with kCopies for its
     // group at the end of a pass-A op, with kDirect for all of them at the start of a pass-B op.
-    // Group wg takes the tiles t with t % NWG == wg; with as many buffers as groups that is
-    // always buffer wg, whose "ready" barrier the group then meets in consecutive phases.
+    // Group wg takes the tiles t with t % NWG == wg, from buffer t % NBUF.
     const int wg = warp >> 2;
     const int quad = warp & 3;                      // TMEM lane quadrant this warp may read
     const int lane_row = quad * 32 + lane;          // accumulator lane (row in pass A, key in pass B)
-    const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(wg * 128);
-    uint64_t* const my_full = &S.acc_full[wg];
-    uint64_t* const my_empty = &S.acc_empty[wg];
-    uint32_t tmod = 0;                              // tiles of the ops so far, modulo NWG
-    uint32_t fpar = 0;                              // phase parity of my_full
+    const uint32_t taddr0 = tmem_base + ((uint32_t)(quad * 32) << 16);
+    uint32_t t = wg, t_op = 0;                      // the group's next tile, the first tile of the op
     uint32_t n_a_done = 0;                          // pass-A ops this warp has delivered
     uint32_t kbs = 0;                               // pass-B ops so far
     // pass A: the window row of this lane, and the columns its copy of the rows sums
@@ -828,32 +793,26 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const int i_row = (kCopies ? lane_row - copy * P.rows : lane_row) / G;
     const int c_lo = kCopies ? copy * (TILE / P.reps) : 0, c_hi = kCopies ? c_lo + TILE / P.reps : TILE;
     bool ok = true;
+    const float inv_sw = 1.f / (float)P.Sw, inv_g = 1.f / (float)G;
     for (int oi = op_lo; oi < op_hi; ++oi) {
       const ScoreOp op = get_op(oi);
-      if (op.nkeys <= 0) continue;
       const int ntiles = (op.nkeys + TILE - 1) / TILE;
-      const int it0 = (int)((wg + NWG - tmod) % NWG);            // the group's first tile of the op
-      tmod = (tmod + (uint32_t)ntiles) % NWG;
-      if (op.phase) {
+      const int it0 = (int)(t - t_op);                           // the group's first tile of the op
+      t_op += (uint32_t)ntiles;
+      if (kEntropyB || op.phase) {
         // ---------------- pass B: thread = key, columns = rows r' = i*G + h
         if constexpr (kDirect) {
           // One thread per row and group; every CTA adds in the same order.
           const int slot = kbs & 1, xslot = xrow_slot(n_a_done, kbs), pair = op.req * P.Hkv + op.g;
-          const int s_lo = P.pair_aseg[pair];        // read before the wait
-          int s_hi = P.pair_aseg[pair + 1];
-          if (ok) ok = mbar_wait(&S.parts[slot], (kbs >> 1) & 1, P.status, P.spin_limit);
-          if (!ok) s_hi = s_lo;
+          const int s_lo = P.pair_aseg[pair], s_hi = P.pair_aseg[pair + 1];
+          const uint32_t free_par = ((kbs >> 1) & 1) ^ 1;
           ++kbs;
           float4 acc = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-          if (lane_row < P.rows) {
-            for (int sg = s_lo; sg < s_hi; sg += 8) {
-              float4 pv[8];
-#pragma unroll
-              for (int u = 0; u < 8; ++u)
-                pv[u] = sg + u < s_hi ? __ldcg(&P.rowpart[((size_t)(sg + u) * NWG + wg) * 128 + lane_row])
-                                      : make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-              acc = merge_batch(acc, pv);
-            }
+          for (int sg = s_lo; sg < s_hi && ok; sg += 8) {
+            float4 pv[8];
+            ok = wait_parts(&P.rowpart[((size_t)sg * NWG + wg) * 128 + lane_row], (int64_t)NWG * 128,
+                            lane_row < P.rows ? s_hi - sg : 0, P.want, pv, P.status, P.spin_limit);
+            if (ok) acc = merge_batch(acc, pv);
           }
           S.xrow[(xslot * NWG + wg) * 128 + lane_row] = acc;
           asm volatile("bar.sync 1, %0;" ::"n"(STAT_THREADS) : "memory");
@@ -865,6 +824,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               for (int q = 0; q < NWG; ++q) pv[q] = S.xrow[(xslot * NWG + q) * 128 + lane_row];
               acc = merge_batch(acc, pv);
             }
+            // the MMAs of the op that used this slot two ops ago must be done
+            if (ok) ok = mbar_wait(&S.lse_free[slot], free_par, P.status, P.spin_limit);
             const float lz = log2f(acc.y);
             put_ext_row(S.ext_b + slot * kExtBytes, lane_row, P.rows, acc.x + lz, P.inv_scale2);
             if (op.key0 == 0 && lane_row < P.rows)
@@ -877,11 +838,11 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         float vacc[G], hs[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) { vacc[h] = 0.f; hs[h] = 0.f; }
-        const float inv_sw = 1.f / (float)P.Sw, inv_g = 1.f / (float)G;
-        for (int it = it0; it < ntiles; it += NWG) {
-          if (ok) ok = mbar_wait(my_full, fpar, P.status, P.spin_limit);
-          fpar ^= 1u;
+        for (int it = it0; it < ntiles; it += NWG, t += NWG) {
+          if (ok) ok = mbar_wait(&S.acc_full[t % NBUF], (t / NBUF) & 1, P.status, P.spin_limit);
           if (!ok) continue;
+          uint64_t* const my_empty = &S.acc_empty[t % NBUF];
+          const uint32_t taddr = taddr0 + (t % NBUF) * 128u;
           tc_fence_after();
           float s1[G], s2[G], hk[G], a2 = 0.f;
 #pragma unroll
@@ -889,21 +850,18 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           f32x2 s1p[(G + 1) / 2], s2p[(G + 1) / 2], hkp[(G + 1) / 2];   // the same, two heads per register
 #pragma unroll
           for (int hp = 0; hp < (G + 1) / 2; ++hp) { s1p[hp] = 0ull; s2p[hp] = 0ull; hkp[hp] = 0ull; }
-          for (int c0 = 0; c0 < P.rows; c0 += 32) {
-            uint32_t r[32];
-            tmem_ld32_issue(taddr + c0, r);
-            tmem_ld_wait(r);
-            if (c0 + 32 >= P.rows) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(my_empty);
-            }
-            // 32 columns = 32/G window rows x G heads; the accumulator is q.k - lse/scale
+          auto release = [&]() {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(my_empty);
+          };
+          for_columns(taddr, 0, P.rows, [&](const uint32_t (&r)[16]) {
+            // 16 columns = 16/G window rows x G heads; the accumulator is q.k - lse/scale
             if constexpr (G % 2 == 0) {
               // two heads per instruction
               const f32x2 sc2 = pack2(P.scale2, P.scale2);
 #pragma unroll
-              for (int ii = 0; ii < 32 / G; ++ii) {
+              for (int ii = 0; ii < 16 / G; ++ii) {
                 f32x2 asum = 0ull;
 #pragma unroll
                 for (int hp = 0; hp < G / 2; ++hp) {
@@ -924,7 +882,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               }
             } else {
 #pragma unroll
-              for (int ii = 0; ii < 32 / G; ++ii) {
+              for (int ii = 0; ii < 16 / G; ++ii) {
                 float a = 0.f;
 #pragma unroll
                 for (int h = 0; h < G; ++h) {
@@ -938,7 +896,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 a2 = fmaf(a, a, a2);
               }
             }
-          }
+          }, release);
           if constexpr (G % 2 == 0) {
 #pragma unroll
             for (int hp = 0; hp < G / 2; ++hp) {
@@ -979,108 +937,106 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
       } else {
         // ---------------- pass A: thread = window row r' = i*G + h, columns = keys
-        const int last = op.n + i_row;                 // last key this row may attend to
         float m = -CUDART_INF_F, z = 0.f, zwin = 0.f, w = 0.f;
-        for (int it = it0; it < ntiles; it += NWG) {
-          if (ok) ok = mbar_wait(my_full, fpar, P.status, P.spin_limit);
-          fpar ^= 1u;
+        for (int it = it0; it < ntiles; it += NWG, t += NWG) {
+          if (ok) ok = mbar_wait(&S.acc_full[t % NBUF], (t / NBUF) & 1, P.status, P.spin_limit);
           if (!ok) continue;
+          uint64_t* const my_empty = &S.acc_empty[t % NBUF];
+          const uint32_t taddr = taddr0 + (t % NBUF) * 128u;
           tc_fence_after();
-          const int key0 = op.key0 + it * TILE;
-          const bool interior = key0 + TILE <= op.n && it * TILE + TILE <= op.nkeys;
+          // columns of observed keys (every row sees them), and of keys at all
+          const int c_key = op.nkeys - it * TILE, c_obs = min(op.n - op.key0 - it * TILE, c_key);
+          const int c_fast = c_obs >= c_hi ? c_hi : max(c_lo, c_obs & ~15);
           if (!kCopies && quad * 32 >= P.rows) {       // these TMEM lanes hold padding rows
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(my_empty);
             continue;
           }
-#pragma unroll 1
-          for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
-            uint32_t r[32];
-            tmem_ld32_issue(taddr + c0, r);
-            tmem_ld_wait(r);
-            if (c0 + 32 >= c_hi) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(my_empty);
+          bool again = false;
+          if (c_fast > c_lo) {
+            // Whole chunks of observed keys.  The exponentials are taken against the row's running reference m
+            // without looking for the tile's maximum first (an op's first tile: that of its first chunk).
+            // Afterwards the reference moves up by the binary exponent of a sum that is far above 1; only where the
+            // sum nears the end of fp32's range is the tile taken again, from its maxima.
+            if (m == -CUDART_INF_F) {
+              uint32_t r[16];
+              tmem_ld16_issue(taddr + c_lo, r);
+              tmem_ld_wait(r);
+              float cm = __uint_as_float(r[0]);
+#pragma unroll
+              for (int e = 1; e < 16; ++e) cm = fmaxf(cm, __uint_as_float(r[e]));
+              m = cm * P.scale2;
             }
-            if (interior) {
-              // Every key is visible and observed.  The exponentials are taken against the row's
-              // running reference m without looking for the chunk's maximum first; a chunk whose
-              // sum comes out beyond kChunkSumMax (or not finite: m still -inf) holds a logit far
-              // above m and is done once more after m has moved to the chunk's maximum.  That is
-              // rare after the first tiles, and any reference within reach of the fp32 exponent
-              // range gives the same sums.
-              const f32x2 sc2 = pack2(P.scale2, P.scale2);
-              float zs, ws;
+            // two keys per instruction: four partial sums in two packed accumulators
+            const f32x2 sc2 = pack2(P.scale2, P.scale2), nm2 = pack2(-m, -m);
+            f32x2 zc[2] = {0ull, 0ull}, wc[2] = {0ull, 0ull};
+            for_columns(taddr, c_lo, c_fast, [&](const uint32_t (&r)[16]) {
+#pragma unroll
+              for (int e = 0; e < 16; e += 2) {
+                const f32x2 tt2 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, nm2);
+                float t0, t1;
+                unpack2(tt2, t0, t1);
+                const f32x2 ee2 = pack2(ex2(t0), ex2(t1));
+                zc[(e >> 1) & 1] = add2(zc[(e >> 1) & 1], ee2);
+                wc[(e >> 1) & 1] = fma2(ee2, tt2, wc[(e >> 1) & 1]);
+              }
+            }, []() {});
+            float z0, z1, w0, w1;
+            unpack2(add2(zc[0], zc[1]), z0, z1);
+            unpack2(add2(wc[0], wc[1]), w0, w1);
+            const float zs = z0 + z1;
+            again = zs > kTileSumMax;                  // (a NaN is added and stays)
+            if (!again) {
+              z += zs;
+              w += w0 + w1;
+              if (zs > kShiftSum) {
+                const int k = (int)(__float_as_uint(z) >> 23) - 127;
+                const float f = __uint_as_float((uint32_t)(127 - k) << 23);
+                m += (float)k;
+                w = fmaf(-(float)k, z - zwin, w) * f;
+                z *= f; zwin *= f;
+              }
+            }
+          }
+          // The chunks at the end of the prompt (window keys, which a row sees up to its own and which are not
+          // observed) and those of a tile taken again, from the chunk's maximum.
+          const int c_slow = __any_sync(0xffffffffu, again) ? c_lo : c_fast;
 #pragma unroll 1
-              for (int pass = 0;; ++pass) {
-                // two keys per instruction: four partial sums in two packed accumulators
-                const f32x2 nm2 = pack2(-m, -m);
-                f32x2 zc[2] = {0ull, 0ull}, wc[2] = {0ull, 0ull};
+          for (int c0 = c_slow; c0 < c_hi && c0 < c_key; c0 += 16) {
+            uint32_t r[16];
+            tmem_ld16_issue(taddr + c0, r);
+            tmem_ld_wait(r);
+            const int n_obs = c_obs - c0;                                        // observed keys of the chunk
+            const int n_vis = c0 < c_fast && !again ? 0 : min(c_key - c0, n_obs + i_row + 1);   // visible ones
+            float cm = -CUDART_INF_F;
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                  const f32x2 tt2 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sc2, nm2);
-                  float t0, t1;
-                  unpack2(tt2, t0, t1);
-                  const f32x2 ee2 = pack2(ex2(t0), ex2(t1));
-                  zc[(e >> 1) & 1] = add2(zc[(e >> 1) & 1], ee2);
-                  wc[(e >> 1) & 1] = fma2(ee2, tt2, wc[(e >> 1) & 1]);
-                }
-                float z0, z1, w0, w1;
-                unpack2(add2(zc[0], zc[1]), z0, z1);
-                unpack2(add2(wc[0], wc[1]), w0, w1);
-                zs = z0 + z1;
-                ws = w0 + w1;
-                if (zs <= kChunkSumMax || pass > 0) break;
-                float cm = __uint_as_float(r[0]);
-#pragma unroll
-                for (int e = 1; e < 32; ++e) cm = fmaxf(cm, __uint_as_float(r[e]));
-                const float mn = cm * P.scale2;
+            for (int e = 0; e < 16; ++e) cm = e < n_vis ? fmaxf(cm, __uint_as_float(r[e])) : cm;
+            if (cm != -CUDART_INF_F) {
+              cm *= P.scale2;
+              if (cm > m) {
+                const float mn = cm;
                 const float f = ex2(m - mn);                  // 0 while m = -inf
                 const float dm = (m == -CUDART_INF_F) ? 0.f : (m - mn);
                 w = f * fmaf(dm, z - zwin, w);
                 z *= f; zwin *= f;
                 m = mn;
               }
-              z += zs;
-              w += ws;
-            } else {
-              float cm = -CUDART_INF_F;
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                const int j = key0 + c0 + e;
-                const bool vis = (it * TILE + c0 + e < op.nkeys) && j <= last;
-                cm = vis ? fmaxf(cm, __uint_as_float(r[e])) : cm;
-              }
-              if (cm != -CUDART_INF_F) {
-                cm *= P.scale2;
-                if (cm > m) {
-                  const float mn = cm;
-                  const float f = ex2(m - mn);
-                  const float dm = (m == -CUDART_INF_F) ? 0.f : (m - mn);
-                  w = f * fmaf(dm, z - zwin, w);
-                  z *= f; zwin *= f;
-                  m = mn;
-                }
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                  const int j = key0 + c0 + e;
-                  const bool vis = (it * TILE + c0 + e < op.nkeys) && j <= last;
-                  const bool obs = j < op.n;
-                  const float tt = fmaf(__uint_as_float(r[e]), P.scale2, -m);
-                  const float ee = vis ? ex2(tt) : 0.f;
-                  z += ee;
-                  zwin += obs ? 0.f : ee;
-                  w = (vis && obs) ? fmaf(ee, tt, w) : w;
-                }
+              for (int e = 0; e < 16; ++e) {
+                const float tt = fmaf(__uint_as_float(r[e]), P.scale2, -m);
+                const float ee = e < n_vis ? ex2(tt) : 0.f;
+                z += ee;
+                zwin += e < n_obs ? 0.f : ee;
+                w = e < n_obs && e < n_vis ? fmaf(ee, tt, w) : w;
               }
             }
           }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(my_empty);
         }
-        // Deliver this warp's 32 partial rows of the segment.  Making them visible to the other
-        // CTAs takes a fence of a few thousand cycles; the merger warp pays it once per op for all
-        // twelve warps, which only tell it, inside the CTA, that their rows are written.
+        // Deliver this warp's 32 partial rows of the segment.
         float4 part = make_float4(m, z, zwin, w);
         if constexpr (kCopies) {
           // the group's copies of a row become one partial
@@ -1090,10 +1046,9 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
           if (copy == 0)
             for (int c = 1; c < P.reps; ++c) part = merge_rows(part, x[c * P.rows + lane_row]);
         }
-        if (!kCopies || copy == 0) __stcg(&P.rowpart[((size_t)op.seg * NWG + wg) * 128 + lane_row], part);
-        __syncwarp();
+        if (!kCopies || copy == 0)
+          st_row16(&P.rowpart[((size_t)op.seg * NWG + wg) * 128 + lane_row], pack_part(part.x, part.y, part.z, part.w, P.tag));
         ++n_a_done;
-        if (lane == 0) smem_store_release(&S.a_done[warp], n_a_done);
       }
     }
   }
@@ -1162,12 +1117,10 @@ int tc_reps(int rows) { return rows == 32 ? 4 : rows == 64 ? 2 : 1; }
 
 // Cuts the `tiles` tiles of one (request, head) pair, which start at flat tile index `flat`
 // of a wave of `W` tiles shared by `n_cta` CTAs (slot c owns flat tiles
-// [c*W/n_cta, (c+1)*W/n_cta)), into per-slot segments; slot c belongs to CTA (c+rot)%n_cta.
-// With `split`, a slot's segment of two or more tiles becomes two ops (pad = 1: first half,
-// pad = 2: second half) that the program builder may place apart.
+// [c*W/n_cta, (c+1)*W/n_cta)), into per-slot segments; slot c belongs to CTA (c+rot) of all, modulo their number.
 void cut_pair(std::vector<std::vector<ScoreOp>>& per_cta, int rot, int n_cta, int64_t W, int64_t flat,
               int tiles, int keys, int req, int g, int phase, int32_t& seg_counter, int64_t base,
-              int n_obs, bool split = false) {
+              int n_obs) {
   int t0 = 0;
   while (t0 < tiles) {
     const int64_t f = flat + t0;
@@ -1176,20 +1129,14 @@ void cut_pair(std::vector<std::vector<ScoreOp>>& per_cta, int rot, int n_cta, in
     while (c > 0 && (int64_t)c * W / n_cta > f) --c;
     const int64_t share_end = (int64_t)(c + 1) * W / n_cta;
     const int t1 = (int)((share_end - flat) < tiles ? (share_end - flat) : tiles);
-    const int parts = (split && t1 - t0 >= 2) ? 2 : 1;
-    const int tm = t0 + (t1 - t0 + 1) / 2;
-    for (int part = 0; part < parts; ++part) {
-      const int a = part == 0 ? t0 : tm, b = (parts == 2 && part == 0) ? tm : t1;
-      ScoreOp op;
-      op.base = base; op.n = n_obs;
-      op.pad = parts == 2 ? part + 1 : 0;
-      op.req = req; op.g = g; op.key0 = a * TILE;
-      const int kend = b * TILE < keys ? b * TILE : keys;
-      op.nkeys = kend - a * TILE;
-      op.phase = phase;
-      op.seg = seg_counter++;
-      per_cta[(c + rot) % n_cta].push_back(op);
-    }
+    ScoreOp op;
+    op.base = base; op.n = n_obs;
+    op.pad = 0;
+    op.req = req; op.g = g; op.key0 = t0 * TILE;
+    op.nkeys = (t1 * TILE < keys ? t1 * TILE : keys) - t0 * TILE;
+    op.phase = phase;
+    op.seg = seg_counter++;
+    per_cta[(c + rot) % (int)per_cta.size()].push_back(op);
     t0 = t1;
   }
 }
@@ -1215,6 +1162,14 @@ std::vector<int> tc_waves(const ReqInfo* reqs, int n_req, int Hkv, int head_dim)
 
 }  // namespace
 
+// Exchanged rows of the current batch: merged rows of every pair, then the partial rows of every pass-A segment.
+size_t tc_exchange_bytes(int64_t pairs, int64_t segs) {
+  return (size_t)pairs * 128 * kLseStride * sizeof(uint2) + (size_t)segs * NWG * 128 * sizeof(float4);
+}
+static_assert(CAKE_MAX_LAYERS < 512, "a launch's mark has 9 bits");
+
+size_t tc_index_size(int64_t pairs, int n_sm) { return 3 * (size_t)(pairs + 1) + 2 * (size_t)(n_sm + 1); }
+
 bool tc_path_supported(const cake_config& c) {
   const int G = c.n_q_heads / c.n_kv_heads;
   const int rows = G * c.window;
@@ -1230,11 +1185,13 @@ int64_t tc_max_segments(const cake_config& c, int n_sm) {
   const int64_t bytes = (int64_t)c.n_kv_heads * c.max_total_tokens * c.head_dim * 2;
   int64_t waves = 2 * (bytes / kWaveBytes) + 2;
   if (waves > pairs) waves = pairs;
-  return pairs + (waves + 2) * n_sm;          // + the two waves whose ops are halved
+  return pairs + waves * n_sm;
 }
 
-// Builds the per-CTA programs of the batch in ctx->h_req[0..n_req): `full` = both passes
-// interleaved by wave, `bonly` = pass B alone (denominators supplied by the caller).
+inline int op_tiles(const ScoreOp& op) { return (op.nkeys + TILE - 1) / TILE; }
+
+// Builds the per-CTA programs of the batch in ctx->h_req[0..n_req): one with both passes, and one with
+// pass B alone (denominators supplied by the caller).
 int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
   const cake_config& c = ctx->cfg;
   const int Hkv = c.n_kv_heads;
@@ -1271,27 +1228,31 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     n_cta = best_n;
     ctx->n_tc_ctas = n_cta;
   }
-  // Program of a CTA, by waves:  A0 A1 B0 A2 B1 ... A(n-1) B(n-2) B(n-1).  Pass B of a wave waits
-  // for the wave's merged denominators, which trail the slowest CTA's pass A by some 7 us; in
-  // the steady state the pass A in between covers that.  At the two ends it does not, so there
-  // (when the waves are single pairs, and there are at least four) one op is halved and its halves
-  // placed apart: A2's first half goes before B0, and B(n-3)'s second half goes after A(n-1).
-  std::vector<std::vector<std::vector<ScoreOp>>> was(n_waves), wbs(n_waves);   // [wave][CTA]
-  std::vector<std::vector<ScoreOp>> full(n_cta), bonly(n_cta);
+  // A single wave with no more pairs than CTAs: if a tile more per CTA allows it, every CTA works for one pair.  A
+  // second pair is another row-pass op, another wait for denominators and another column-pass op in a row
+  // (8 heads of 7919 keys on 124 CTAs: most CTAs were done after 18.7 us, the four with two pairs after 23.4).
+  std::vector<int> pair_cta;                         // first CTA of every pair, and their number
+  if (n_waves == 1 && n_pairs <= ctx->n_sm_score) {
+    int64_t W = 0;
+    for (int p = 0; p < n_pairs; ++p) W += (ctx->h_req[p / Hkv].N + TILE - 1) / TILE;
+    const int64_t steps = (W + n_cta - 1) / n_cta;
+    for (int64_t most = steps; most <= steps + 1 && pair_cta.empty(); ++most) {
+      std::vector<int> first(1, 0);
+      for (int p = 0; p < n_pairs; ++p)
+        first.push_back(first.back() + (int)(((ctx->h_req[p / Hkv].N + TILE - 1) / TILE + most - 1) / most));
+      if (first.back() <= ctx->n_sm_score) pair_cta = first;
+    }
+    if (!pair_cta.empty()) ctx->n_tc_ctas = n_cta = pair_cta.back();
+  }
+  std::vector<std::vector<ScoreOp>> a_ops(n_cta), b_ops(n_cta);
   int32_t aseg = 0, bseg = 0;
   int32_t* pair_aseg = ctx->h_tc_index;                    // [pairs+1]
   int32_t* pair_bseg = ctx->h_tc_index + (n_pairs + 1);    // [pairs+1]
-  const bool ends = kWaveDepth == 1 && n_waves >= 4;
-  auto single = [&](int wv) { return wave_begin[wv + 1] - wave_begin[wv] == 1; };
-  const int split_a = ends && single(2) ? 2 : -1;
-  const int split_b = ends && single(n_waves - 3) ? n_waves - 3 : -1;
   int rot = 0;
   for (int wv = 0; wv < n_waves; ++wv) {
     int64_t WA = 0;
     for (int p = wave_begin[wv]; p < wave_begin[wv + 1]; ++p)
       WA += (ctx->h_req[p / Hkv].N + TILE - 1) / TILE;
-    was[wv].assign(n_cta, {});
-    wbs[wv].assign(n_cta, {});
     int64_t fa = 0;
     for (int p = wave_begin[wv]; p < wave_begin[wv + 1]; ++p) {
       const int r = p / Hkv, g = p % Hkv;
@@ -1300,65 +1261,21 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
       pair_aseg[p] = aseg;
       pair_bseg[p] = bseg;
       const int64_t base = (int64_t)g * T + rq.cu;
-      cut_pair(was[wv], rot, n_cta, WA, fa, ta, rq.N, r, g, 0, aseg, base, rq.n, wv == split_a);
+      const bool own = !pair_cta.empty();
+      const int c0 = own ? pair_cta[p] : rot, nc = own ? pair_cta[p + 1] - c0 : n_cta;
+      const int64_t w = own ? ta : WA, f = own ? 0 : fa;
+      cut_pair(a_ops, c0, nc, w, f, ta, rq.N, r, g, 0, aseg, base, rq.n);
       // pass B walks the same flat tile positions, so a CTA re-reads the tiles it brought in
-      if (tb > 0) cut_pair(wbs[wv], rot, n_cta, WA, fa, tb, rq.n, r, g, 1, bseg, base, rq.n, wv == split_b);
+      if (tb > 0) cut_pair(b_ops, c0, nc, w, f, tb, rq.n, r, g, 1, bseg, base, rq.n);
       fa += ta;
     }
     // a wave's remainder tiles land on different CTAs each time (golden-ratio stride)
     rot = (rot + (int)(n_cta * 0.381966) + 1) % n_cta;
   }
-  // which = 0: every op, 1: first halves and unsplit ops, 2: second halves
-  auto put = [&](std::vector<ScoreOp>& dst, const std::vector<ScoreOp>& src, int which) {
-    for (const ScoreOp& op : src)
-      if (which == 0 || (which == 1 && op.pad != 2) || (which == 2 && op.pad == 2)) dst.push_back(op);
-  };
-  for (int cta = 0; cta < n_cta; ++cta) {
-    for (int wv = 0; wv < n_waves; ++wv) {
-      // pass A of this wave
-      if (wv == split_a) {
-        put(full[cta], was[wv][cta], 1);                       // A2 first half
-        put(full[cta], wbs[wv - 2][cta], 0);                   // B0 (held back one slot)
-        put(full[cta], was[wv][cta], 2);                       // A2 second half
-      } else {
-        put(full[cta], was[wv][cta], 0);
-      }
-      // pass B of the wave kWaveDepth behind
-      if (split_b >= 0 && wv == split_b + 2) put(full[cta], wbs[split_b][cta], 2);   // B(n-3) second half, after A(n-1)
-      const int bw = wv - kWaveDepth;
-      if (bw >= 0 && !(split_a >= 0 && bw == split_a - 2 && wv == split_a - 1)) {
-        if (bw == split_b) put(full[cta], wbs[bw][cta], 1);    // B(n-3) first half in its usual place
-        else put(full[cta], wbs[bw][cta], 0);
-      }
-      put(bonly[cta], wbs[wv][cta], 0);
-    }
-    for (int wv = n_waves > kWaveDepth ? n_waves - kWaveDepth : 0; wv < n_waves; ++wv)
-      put(full[cta], wbs[wv][cta], 0);
-  }
   pair_aseg[n_pairs] = aseg;
   pair_bseg[n_pairs] = bseg;
   if (aseg > ctx->max_tc_segs || bseg > ctx->max_tc_segs) return CAKE_ERR_CAPACITY;
 
-  int32_t* cta_full = ctx->h_tc_index + 3 * (n_pairs + 1);   // [n_sm+1]
-  int32_t* cta_b = cta_full + (ctx->n_sm + 1);               // [n_sm+1]
-  int64_t total = 0;
-  for (int cta = 0; cta < n_cta; ++cta) total += (int64_t)(full[cta].size() + bonly[cta].size());
-  if (total > ctx->max_tc_ops) return CAKE_ERR_CAPACITY;
-  int32_t o = 0;
-  for (int cta = 0; cta < n_cta; ++cta) {
-    cta_full[cta] = o;
-    for (const ScoreOp& op : full[cta]) ctx->h_tc_ops[o++] = op;
-  }
-  cta_full[n_cta] = o;
-  ctx->n_tc_ops_full = o;
-  for (int cta = 0; cta < n_cta; ++cta) {
-    cta_b[cta] = o;
-    for (const ScoreOp& op : bonly[cta]) ctx->h_tc_ops[o++] = op;
-  }
-  cta_b[n_cta] = o;
-  ctx->n_tc_ops_b = o - ctx->n_tc_ops_full;
-  ctx->n_tc_asegs = aseg;
-  ctx->n_tc_bsegs = bseg;
   // several rows at a time when there are pairs to take them from and a row has few partials
   {
     int max_segs = 0;
@@ -1369,17 +1286,12 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     while (ways < 32 && 2 * ways <= n_pairs && partials * 2 * ways <= 512) ways *= 2;
     if (n_pairs < 4) ways = 1;
     ctx->tc_merge_ways = ways;
-    // The merger handles up to `ways` consecutive pairs at once and waits for the pass A of all of them.  A
-    // group that reaches from wave w into w+1 makes B(w) wait for the end of A(w+1), which comes right
-    // before it, and for the way from there to the denominators; one that reaches into w+2 would make it
-    // wait for an A that comes after it.  So a group lies inside a wave (8 requests of 8K to 64K, groups of
-    // 2 pairs: 10.28 ms against 10.87 with groups across two waves), except in the last two: their pass B
-    // follows all of pass A, and every group less is 2 us less between the two (47.8 against 50.4 us for 8
-    // pairs in two waves).
+    // The merger handles up to `ways` consecutive pairs at once and waits for the pass A of all of them, and
+    // pass B of a pair for the whole group: a group lies inside a wave.
     int32_t* group_begin = ctx->h_tc_index + 2 * (n_pairs + 1);
     int ng = 0;
     for (int wv = 0, p0 = 0; wv < n_waves; ++wv) {
-      const int p1 = wv + 2 >= n_waves ? n_pairs : wave_begin[wv + 1];
+      const int p1 = wave_begin[wv + 1];
       for (; p0 < p1; p0 += std::min(ways, p1 - p0)) group_begin[ng++] = p0;
     }
     group_begin[ng] = n_pairs;
@@ -1393,6 +1305,36 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
     for (int p = 0; p < n_pairs; ++p) all_b = all_b && pair_bseg[p + 1] > pair_bseg[p];
     ctx->tc_direct = n_waves == 1 && all_b && max_segs <= kDirectSegs;
   }
+  // Program of a CTA, by waves:  A0 A1 B0 A2 B1 ... A(n-1) B(n-2) B(n-1).  Pass B of a wave waits for the wave's merged
+  // denominators, which trail the slowest CTA's pass A by some 4 us; the pass A in between covers that.  (Tiles of
+  // A(w+1) and B(w) in turn, so that DRAM is never idle, and a lead of pass A of 4 to 16 tiles beyond the wave were
+  // each no faster alone and 2 to 4 % slower in a long run, where the power cap sets the clock.)
+  const int64_t n_full = (int64_t)aseg + bseg, total = n_full + bseg;
+  if (total > ctx->max_tc_ops) return CAKE_ERR_CAPACITY;
+  int32_t* cta_full = ctx->h_tc_index + 3 * (n_pairs + 1);   // [n_sm+1]
+  int32_t* cta_b = cta_full + (ctx->n_sm + 1);               // [n_sm+1]
+  int32_t o = 0, ob = (int32_t)n_full;
+  auto wave_of = [&](const ScoreOp& op) {
+    return (int)(std::upper_bound(wave_begin.begin(), wave_begin.end(), op.req * Hkv + op.g) - wave_begin.begin()) - 1;
+  };
+  for (int cta = 0; cta < n_cta; ++cta) {
+    cta_full[cta] = o;
+    cta_b[cta] = ob;
+    size_t ib = 0;
+    for (const ScoreOp& a : a_ops[cta]) {
+      for (const int w = wave_of(a); ib < b_ops[cta].size() && wave_of(b_ops[cta][ib]) < w - 1; ++ib)
+        ctx->h_tc_ops[o++] = b_ops[cta][ib];
+      ctx->h_tc_ops[o++] = a;
+    }
+    for (; ib < b_ops[cta].size(); ++ib) ctx->h_tc_ops[o++] = b_ops[cta][ib];
+    for (const ScoreOp& b : b_ops[cta]) ctx->h_tc_ops[ob++] = b;
+  }
+  cta_full[n_cta] = o;
+  cta_b[n_cta] = ob;
+  ctx->n_tc_ops_full = (int32_t)n_full;
+  ctx->n_tc_ops_b = bseg;
+  ctx->n_tc_asegs = aseg;
+  ctx->n_tc_bsegs = bseg;
   return CAKE_OK;
 }
 
@@ -1404,7 +1346,7 @@ int32_t tc_build_plan(cake_ctx* ctx, int32_t n_req) {
 //   2  inside every CTA's program the pass-B ops come in non-decreasing wave order and every
 //      pass-A op of a wave w' <= w precedes the first pass-B op of wave w (so a wave's pass B can
 //      only ever wait for pass-A ops that wait for nothing themselves)
-//   3  the pairs the merger warps handle side by side lie in one wave or in the last two
+//   3  the pairs the merger warps handle side by side lie in one wave
 //   4  op counts and segment numbers stay inside the tables the context would allocate
 //   5  no statistics warp writes a slot of the exchange rows that another may still read (xrow_slot)
 int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_req, const int64_t* cu,
@@ -1428,7 +1370,7 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
   x.max_tc_segs = (int32_t)tc_max_segments(c, n_sm);
   x.max_tc_ops = 3 * x.max_tc_segs + 8;
   std::vector<ScoreOp> ops((size_t)x.max_tc_ops);
-  std::vector<int32_t> index(3 * (size_t)(n_pairs + 1) + 2 * (size_t)(n_sm + 1));
+  std::vector<int32_t> index(tc_index_size(n_pairs, n_sm));
   x.h_tc_ops = ops.data();
   x.h_tc_index = index.data();
   const int32_t rc = tc_build_plan(&x, n_req);
@@ -1511,8 +1453,8 @@ int32_t tc_plan_check(const cake_config& c, int n_sm, int reserved, int32_t n_re
   if (group_begin[0] != 0 || group_begin[x.n_tc_groups] != n_pairs) return fail(3);
   for (int gi = 0; gi < x.n_tc_groups; ++gi) {
     const int p0 = group_begin[gi], p1 = group_begin[gi + 1] - 1;
-    if (p1 < p0 || p1 - p0 >= x.tc_merge_ways || (wave_of[p1] != wave_of[p0] && wave_of[p0] + 2 < x.n_tc_waves)) return fail(3);
-    if (x.n_tc_waves <= 2 && p0 != gi * x.tc_merge_ways) return fail(3);
+    if (p1 < p0 || p1 - p0 >= x.tc_merge_ways || wave_of[p1] != wave_of[p0]) return fail(3);
+    if (x.n_tc_waves == 1 && p0 != gi * x.tc_merge_ways) return fail(3);
   }
   return CAKE_OK;
 }
@@ -1555,14 +1497,13 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   TcParams P;
   P.ops = ctx->d_tc_ops;
   P.reqs = ctx->d_req;
-  // with one or two waves the groups are those of the plain rule, which spares the merger a read per group
-  P.group_begin = ctx->n_tc_waves > 2 ? ctx->d_tc_index + 2 * (n_pairs + 1) : nullptr;
+  // with one wave the groups are those of the plain rule, which spares the merger a read per group
+  P.group_begin = ctx->n_tc_waves > 1 ? ctx->d_tc_index + 2 * (n_pairs + 1) : nullptr;
   P.n_groups = ctx->n_tc_groups;
   P.pair_aseg = ctx->d_tc_index;
-  P.pair_cnt = ctx->d_tc_sync;
-  P.lse2 = ctx->d_lse2_tc;
+  P.lse2 = (uint2*)ctx->d_tc_exch;
   P.lse_ext = lse;
-  P.rowpart = ctx->d_tc_rowpart;
+  P.rowpart = (float4*)(ctx->d_tc_exch + (size_t)n_pairs * 128 * kLseStride * sizeof(uint2));
   P.raw = ctx->d_raw[layer % ctx->score_depth];
   P.colpart = ctx->d_colpart[layer % ctx->score_depth];
   P.hrow = ctx->d_hrow[layer % ctx->score_depth];
@@ -1580,18 +1521,18 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.bessel = c.var_ddof ? (float)c.window / (float)(c.window - 1) : 1.f;
 
   const int sp = prof_begin(ctx, CAKE_PROF_SCORE, st);
-  const int32_t* cta_full = ctx->d_tc_index + 3 * (n_pairs + 1);
+  P.cta_op = ctx->d_tc_index + 3 * (n_pairs + 1);
   if (lse) {
     // denominators supplied: pass B alone, entropy from its columns
     ctx->hhead_from_rows = false;
-    P.cta_op = cta_full + (ctx->n_sm + 1);
-    P.pair_done = nullptr;
-    P.epoch = 0;
+    P.cta_op += ctx->n_sm + 1;
+    P.both = 0;
+    P.tag = P.want = 0;
   } else {
     ctx->hhead_from_rows = true;
-    P.cta_op = cta_full;
-    P.pair_done = ctx->d_tc_sync + ctx->max_pairs;
-    P.epoch = ++ctx->tc_epoch + (uint32_t)ctx->debug_epoch_skew;
+    P.both = 1;
+    P.tag = ++ctx->tc_tag;
+    P.want = P.tag + (uint32_t)ctx->debug_epoch_skew;
   }
   cudaError_t e;
   const bool eb = lse != nullptr;

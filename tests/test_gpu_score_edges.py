@@ -1,0 +1,59 @@
+"""Scores where the row pass can go wrong: prompts whose window starts at every place in a chunk of 16 keys, a tile of
+128 and a CTA's share, and rows whose largest logit lies far above those of their first keys (the running reference
+moves up, or the tile is taken again from its maxima).  Indicators and preferences against the float64 oracle
+with the tolerance of the parity tests (1e-3 relative: bf16 inputs, fp32 accumulation)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cake_oracle as O
+from paper_2503_12491_b200 import harness, synth
+
+pytestmark = pytest.mark.gpu
+
+RTOL = 1e-3
+
+
+def check(w, qs, ks):
+    cake = harness.cake_for(w)
+    cake.begin(w.cu_seqlens)
+    cake.score_layer(0, qs[0], ks[0])
+    ind = cake.get_indicators(0).cpu().numpy()
+    P = cake.get_preferences()[2].cpu().numpy()
+    cu = w.cu_seqlens
+    for r, N in enumerate(w.seq_lens):
+        ref = O.score_layer(qs[0][r].float().cpu().numpy().astype(np.float64),
+                            ks[0][:, cu[r]:cu[r + 1]].float().cpu().numpy().astype(np.float64),
+                            gamma=w.gamma, pool_kernel=w.pool_kernel)
+        got, want = ind[:, cu[r]:cu[r] + N - w.window], ref["indicator"]
+        assert (np.abs(got - want) <= RTOL * np.abs(want) + 1e-30).all(), (r, N)
+        assert abs(P[r, 0] - ref["P"]) <= RTOL * abs(ref["P"]) + 1e-30
+    assert cake.status() == 0
+    cake.destroy()
+
+
+@pytest.mark.parametrize("hq,hkv,window,d", [(8, 2, 32, 128), (2, 2, 32, 64), (4, 2, 32, 128), (8, 1, 16, 64)])
+@pytest.mark.parametrize("first", [33, 128, 143, 160, 239, 1024])
+def test_windows_at_every_place_of_a_chunk(hq, hkv, window, d, first):
+    lens = tuple(first + i for i in range(0, 18, 1 if first < 200 else 5))
+    w = synth.scaled(synth.workload(3), n_layers=1, n_q_heads=hq, n_kv_heads=hkv, head_dim=d, window=window, seq_lens=lens,
+                     total_budget=window + 20)
+    qs, ks, _ = harness.device_inputs(w)
+    check(w, qs, ks)
+
+
+@pytest.mark.parametrize("jump", [8.0, 45.0, 65.0, 90.0, 300.0])
+@pytest.mark.parametrize("hq,hkv", [(8, 2), (2, 2)])
+def test_a_logit_far_above_the_first_keys(hq, hkv, jump):
+    """Window queries and one key share a direction: that key's logits are `jump` nats above the others, which
+    are of the order of one, for the rows of even index; it lies in a later tile of its CTA's share."""
+    w = synth.scaled(synth.workload(3), n_layers=1, n_q_heads=hq, n_kv_heads=hkv, seq_lens=(20000, 700), total_budget=60)
+    gen = torch.Generator().manual_seed(7)
+    d = w.head_dim
+    q = torch.randn(2, hq, w.window, d, generator=gen)
+    k = torch.randn(hkv, w.total_tokens, d, generator=gen)
+    q[..., 0] = 0.0
+    q[:, :, ::2, 0] = 4.0
+    k[..., 0] = 0.0
+    k[:, [130, 390, 517, 9001, 15555, 20000 + 400], 0] = jump * d ** 0.5 / 4.0
+    check(w, [q.bfloat16().cuda()], [k.bfloat16().cuda()])
