@@ -368,8 +368,9 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
     }
     ctx->n_units = nu;
     {
+      // a team per KV head where a head has more than a warp's partial sums, else one per request
       const int64_t partials = ctx->use_tc ? (int64_t)ctx->n_tc_bsegs * kScoreWarps : (int64_t)nu * c.n_kv_heads;
-      ctx->n_fin_parts = partials > 512 * (int64_t)n_req * c.n_kv_heads ? c.n_kv_heads : 1;
+      ctx->n_fin_parts = partials > 32 * (int64_t)n_req * c.n_kv_heads ? c.n_kv_heads : 1;
     }
     ctx->packed_rows_bound = bound;
     memcpy(ctx->h_cu, cu, sizeof(int64_t) * (n_req + 1));

@@ -119,7 +119,7 @@ struct cake_ctx {
   int32_t arrived_budgets; // stage whose budgets were computed when its layer was scored (-1: none, or a
                            // preference was set since)
   int32_t max_n_tokens;    // longest prompt of the batch
-  int32_t n_fin_parts;     // CTAs that share the preference of a request
+  int32_t n_fin_parts;     // teams that share the preference of a request
   int64_t packed_rows_bound;
   int64_t* h_cu;           // host copy of cu_seqlens [max_requests+1]
   // ---- pinned staging ----
