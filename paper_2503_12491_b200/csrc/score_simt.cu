@@ -102,6 +102,8 @@ scores_simt(const T* __restrict__ q_win, const T* __restrict__ k, const ScoreArg
 #pragma unroll
   for (int r = 0; r < 8; ++r) mz[r * NT] = make_float2(-CUDART_INF_F, 0.f);
   float acc[8][KPT];
+  // up to here nothing was read or written that the kernel before this one, which may still run, has to do with
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   fetch(0);
 #pragma unroll 1
   for (int st = 0; st < steps; ++st) {
@@ -174,6 +176,8 @@ scores_simt(const T* __restrict__ q_win, const T* __restrict__ k, const ScoreArg
       mz[r * NT] = make_float2(mn, e);
     }
   }
+  // The column pass may take its places; it waits for this kernel's end before it reads.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!A.rowpart) return;
   // over the threads of a row group, in a fixed order: maxima, then sums against them
   const int lane = tid & 31, warp = tid >> 5;
@@ -267,18 +271,24 @@ struct ColArgs {
 
 // One CTA per (unit, KV head): 64 keys at a time, a lane per key, and four quarters of the window rows
 // on two warps each.  Bound: the latency of the loads: 14 us for 4 heads of 6K keys and 128 rows at 30 % of the
-// issue slots and 7 % of the special-function unit.
+// issue slots and 7 % of the special-function unit, with two window rows in flight.  A thread now has 16 logits in
+// flight (8 where a KV head has one query head), as many as the registers of three CTAs per SM allow: eight layers
+// take 402 us with two rows at a time and 381 so, where the next kernel starts early; where it does not, 432 and 429.
 constexpr int COL_KEYS = 64;
 template <int GM>          // query heads per KV head, at most
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, 3)
 colstats_simt(const ColArgs A) {
   __shared__ float s_lse[kMaxRows];
   __shared__ float s_part[4][2 + 2 * GM][COL_KEYS];
   __shared__ float s_red[NT / 32][2 * GM];
+  constexpr int COL_BATCH = GM <= 2 ? 8 : 16 / GM;        // window rows of a thread whose loads are in flight together
   const int G = A.Hq / A.Hkv, rows = G * A.Sw;
   const int g = blockIdx.y, unit = A.u0 + (int)blockIdx.x;
   const ScoreUnit u = A.units[unit];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // the logits and the denominators come from the kernel before this one, which may still run
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int quarter = warp >> 1, key_l = (warp & 1) * 32 + lane;
   const float* sc = A.scores + ((size_t)blockIdx.x * A.Hkv + g) * rows * A.unit_keys;
   for (int r = tid; r < rows; r += NT) s_lse[r] = A.lse2[((size_t)u.req * A.Hkv + g) * rows + r];
@@ -295,24 +305,32 @@ colstats_simt(const ColArgs A) {
     float s1[GM], s2[GM], a1 = 0.f, a2 = 0.f;
 #pragma unroll
     for (int h = 0; h < GM; ++h) { s1[h] = 0.f; s2[h] = 0.f; }
-#pragma unroll 2
-    for (int i = quarter; i < A.Sw; i += 4) {
-      float v[GM], a = 0.f;
+    for (int i0 = quarter; i0 < A.Sw; i0 += 4 * COL_BATCH) {
+      float x[COL_BATCH][GM];
 #pragma unroll
-      for (int h = 0; h < GM; ++h) v[h] = h < G ? __ldcg(&col[(size_t)(h * A.Sw + i) * A.unit_keys]) - s_lse[h * A.Sw + i] : 0.f;
+      for (int e = 0; e < COL_BATCH; ++e)
 #pragma unroll
-      for (int h = 0; h < GM; ++h) {
-        if (h < G) {
-          const float p = exp2f(v[h]);
-          hs[h] = fmaf(valid ? p : 0.f, v[h], hs[h]);
-          s1[h] += p;
-          s2[h] = fmaf(p, p, s2[h]);
-          a += p;
+        for (int h = 0; h < GM; ++h)
+          x[e][h] = h < G && i0 + 4 * e < A.Sw ? __ldcg(&col[(size_t)(h * A.Sw + i0 + 4 * e) * A.unit_keys]) : 0.f;
+#pragma unroll
+      for (int e = 0; e < COL_BATCH; ++e) {
+        const int i = i0 + 4 * e;
+        if (i >= A.Sw) break;
+        float a = 0.f;
+#pragma unroll
+        for (int h = 0; h < GM; ++h) {
+          if (h < G) {
+            const float v = x[e][h] - s_lse[h * A.Sw + i], p = exp2f(v);
+            hs[h] = fmaf(valid ? p : 0.f, v, hs[h]);
+            s1[h] += p;
+            s2[h] = fmaf(p, p, s2[h]);
+            a += p;
+          }
         }
+        a *= inv_g;
+        a1 += a;
+        a2 = fmaf(a, a, a2);
       }
-      a *= inv_g;
-      a1 += a;
-      a2 = fmaf(a, a, a2);
     }
     s_part[quarter][0][key_l] = a1;
     s_part[quarter][1][key_l] = a2;
@@ -352,6 +370,25 @@ colstats_simt(const ColArgs A) {
   }
 }
 
+// A launch whose CTAs may take their places while the kernel before it ends (both kernels wait for that end before
+// they touch what others do).  Without it a layer's two kernels and the next layer's each stood 2 to 3 us apart: eight
+// layers of 6K keys 429 -> 381 us, four of 512 keys 100 -> 82.  scores_simt lets the column pass in once its logits are
+// out; from its start on it is slower (389 us), since the waiting CTAs hold registers.
+template <typename... Params, typename... Args>
+cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <typename T, int TY>
 cudaError_t launch_scores(int device, dim3 grid, cudaStream_t st, const void* q, const void* k, const ScoreArgs& A) {
   static PerDeviceOnce attr;
@@ -360,9 +397,9 @@ cudaError_t launch_scores(int device, dim3 grid, cudaStream_t st, const void* q,
     if (e != cudaSuccess) return e;
     attr.mark(device);
   }
-  scores_simt<T, TY><<<grid, NT, Shape<T, TY>::kSmem, st>>>((const T*)q, (const T*)k, A);
+  const cudaError_t e = launch_early(scores_simt<T, TY>, grid, Shape<T, TY>::kSmem, st, (const T*)q, (const T*)k, A);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 template <typename T>
@@ -410,10 +447,7 @@ int32_t run(cake_ctx* ctx, int32_t layer, const void* q_win, const void* k, cons
     if (lse || !whole) CAKE_CUDA_TRY(scores(u0, n, false, true));
     B.u0 = u0;
     const dim3 grid(n, c.n_kv_heads);
-    if (G == 1) colstats_simt<1><<<grid, NT, 0, st>>>(B);
-    else if (G == 2) colstats_simt<2><<<grid, NT, 0, st>>>(B);
-    else if (G <= 4) colstats_simt<4><<<grid, NT, 0, st>>>(B);
-    else colstats_simt<8><<<grid, NT, 0, st>>>(B);
+    CAKE_CUDA_TRY(launch_early(G == 1 ? colstats_simt<1> : G == 2 ? colstats_simt<2> : G <= 4 ? colstats_simt<4> : colstats_simt<8>, grid, 0, st, B));
     count_launch();
   }
   prof_end(ctx, sp, st);

@@ -1,4 +1,4 @@
-"""Scores where the row pass can go wrong: prompts whose window starts at every place in a chunk of 16 keys, a tile of
+"""Scores where the passes can go wrong: prompts whose window starts at every place in a chunk of 16 keys, a tile of
 128 and a CTA's share, and rows whose largest logit lies far above those of their first keys (the running reference
 moves up, or the tile is taken again from its maxima).  Indicators and preferences against the float64 oracle
 with the tolerance of the parity tests (1e-3 relative: bf16 inputs, fp32 accumulation)."""
@@ -57,3 +57,30 @@ def test_a_logit_far_above_the_first_keys(hq, hkv, jump):
     k[..., 0] = 0.0
     k[:, [130, 390, 517, 9001, 15555, 20000 + 400], 0] = jump * d ** 0.5 / 4.0
     check(w, [q.bfloat16().cuda()], [k.bfloat16().cuda()])
+
+
+@pytest.mark.parametrize("hq,hkv,window", [(2, 2, 3), (2, 2, 33), (4, 2, 31), (4, 2, 33), (6, 2, 13), (8, 2, 17), (16, 2, 7), (16, 2, 9)])
+def test_fp32_windows_around_a_batch_of_rows(hq, hkv, window):
+    """The column pass of fp32 inputs takes a quarter of the window rows in batches of 2 to 8.  Three layers in a row,
+    on other inputs each: a layer's kernels start while the ones before them end."""
+    w = synth.scaled(synth.workload(1), n_layers=3, n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=(window + 1, 150, 700),
+                     total_budget=3 * (window + 20))
+    qs, ks, _ = harness.device_inputs(w)
+    cake = harness.cake_for(w)
+    cake.begin(w.cu_seqlens)
+    ind = []
+    for l in range(w.n_layers):
+        cake.score_layer(l, qs[l], ks[l])
+        ind.append(cake.get_indicators(l))
+        cake.allocate(l)
+        cake.evict(l)
+    P, cu = cake.get_preferences()[2].cpu().numpy(), w.cu_seqlens
+    for l in range(w.n_layers):
+        for r, N in enumerate(w.seq_lens):
+            ref = O.score_layer(qs[l][r].cpu().numpy().astype(np.float64), ks[l][:, cu[r]:cu[r + 1]].cpu().numpy().astype(np.float64),
+                                gamma=w.gamma, pool_kernel=w.pool_kernel)
+            got, want = ind[l].cpu().numpy()[:, cu[r]:cu[r] + N - w.window], ref["indicator"]
+            assert (np.abs(got - want) <= RTOL * np.abs(want) + 1e-30).all(), (l, r)
+            assert abs(P[r, l] - ref["P"]) <= RTOL * abs(ref["P"]) + 1e-30
+    assert cake.status() == 0
+    cake.destroy()
