@@ -7,7 +7,7 @@ import pytest
 import torch
 
 from oracle import cake_oracle as O
-from paper_2503_12491_b200 import harness, synth
+from paper_2503_12491_b200 import binding, harness, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -83,4 +83,47 @@ def test_fp32_windows_around_a_batch_of_rows(hq, hkv, window):
             assert (np.abs(got - want) <= RTOL * np.abs(want) + 1e-30).all(), (l, r)
             assert abs(P[r, l] - ref["P"]) <= RTOL * abs(ref["P"]) + 1e-30
     assert cake.status() == 0
+    cake.destroy()
+
+
+@pytest.mark.parametrize("hq,hkv,window,dtype", [(8, 2, 32, "bf16"), (2, 2, 32, "bf16"), (4, 2, 32, "bf16"), (8, 2, 32, "fp32")])
+@pytest.mark.parametrize("tokens", [300, 700, 6100])
+def test_infinite_logits_are_reported(hq, hkv, window, dtype, tokens):
+    """A channel of some keys is infinite (an overflow): a run of 16 or 40 keys at the start of the prompt or of every
+    tile, seen by queries of one sign or of both, so that a row's first logits of a tile are all -inf while its
+    neighbours' are finite or inf.  The status says so, and the next batch of the context is not touched by it.  One
+    request, at 6100 tokens with several tiles per warp, and two."""
+    lens = (tokens,) if tokens != 700 else (tokens, 450)
+    w = synth.scaled(synth.workload(3), n_layers=1, n_q_heads=hq, n_kv_heads=hkv, window=window, seq_lens=lens,
+                     total_budget=window + 20, dtype=dtype)
+    if tokens == 6100:                               # more pairs than the device has SMs for: several tiles per CTA
+        w = synth.scaled(w, seq_lens=(tokens,) * 24)
+    (q0,), (k0,), _ = harness.device_inputs(w)
+    q0[..., 0] = q0[..., 0].abs() + 0.5
+    cake = harness.cake_for(w)
+
+    def score(q, k):
+        cake.begin(w.cu_seqlens)
+        cake.score_layer(0, q, k)
+        out = cake.get_indicators(0), *cake.get_preferences()
+        return cake.status(), out
+
+    status, fresh = score(q0, k0)
+    assert status == 0
+    for sign in ("one", "both"):
+        q = q0.clone()
+        if sign == "both":
+            q[:, :, ::2, 0] *= -1
+        for run in (16, 40):
+            for where in ("start", "tiles"):
+                for value in (float("inf"), float("-inf")):
+                    k = k0.clone()
+                    for r, N in enumerate(w.seq_lens):
+                        rows = torch.arange(N - window, device="cuda")
+                        rows = rows[(rows % 128 if where == "tiles" else rows) < run] + w.cu_seqlens[r]
+                        k[:, rows, 0] = value
+                    status, _ = score(q, k)
+                    assert status == binding.CAKE_ERR_NONFINITE, (sign, run, where, value)
+                    status, again = score(q0, k0)
+                    assert status == 0 and all(torch.equal(a, b) for a, b in zip(fresh, again))
     cake.destroy()
