@@ -262,6 +262,11 @@ __device__ __forceinline__ void for_columns(uint32_t taddr, int lo, int hi, F f,
     f(r1);
   }
 }
+__device__ __forceinline__ float max_or_nan(float a, float b) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -374,15 +379,16 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
 // A partial softmax row (m, z_all, z_win, w) with base-2 exponents: sums of e = 2^(logit2 - m) over all keys of the
 // segment and over those of the window, and w = sum over the observed keys of e * (logit2 - m).  m is any reference: on
 // its way to other CTAs a row has the one that puts z_all into [1, 2) (a scaling by a power of two), and the
-// launch's mark takes the place of z_all's exponent.  No keys: m = -inf.  A sum that is not finite: m = inf,
-// which makes the merged row NaN.
+// launch's mark takes the place of z_all's exponent.  No keys: m = -inf and z_all = 0.  A sum that is not finite
+// (whatever m): m = inf, which makes the merged row NaN.
 __device__ __forceinline__ float4 pack_part(float m, float z, float zwin, float w, uint32_t tag) {
   const uint32_t zb = __float_as_uint(z);
   const int k = (int)(zb >> 23) - 127;
   const float f = __uint_as_float((uint32_t)(127 - k) << 23);
   float4 o = make_float4(m + (float)k, __uint_as_float((zb & 0x7FFFFFu) | (tag << 23)), zwin * f, fmaf(-(float)k, z - zwin, w) * f);
-  if (m == -CUDART_INF_F) o = make_float4(m, __uint_as_float(tag << 23), 0.f, 0.f);
-  else if (!(z <= 1e38f) || k < -120) o.x = CUDART_INF_F;
+  if (!(z <= 1e38f)) o.x = CUDART_INF_F;
+  else if (m == -CUDART_INF_F) o = make_float4(m, __uint_as_float(tag << 23), 0.f, 0.f);
+  else if (k < -120) o.x = CUDART_INF_F;
   return o;
 }
 __device__ __forceinline__ bool part_tagged(const float4& v, uint32_t want) { return (__float_as_uint(v.y) >> 23) == want; }
@@ -393,8 +399,8 @@ __device__ __forceinline__ float4 unpack_part(float4 v) {
 
 // Merge of two partial rows.
 __device__ __forceinline__ float4 merge_rows(float4 a, float4 b) {
-  if (b.x == -CUDART_INF_F) return a;
-  if (a.x == -CUDART_INF_F) return b;
+  if (b.x == -CUDART_INF_F && b.y == 0.f) return a;
+  if (a.x == -CUDART_INF_F && a.y == 0.f) return b;
   const float mn = fmaxf(a.x, b.x);
   const float fa = exp2f(a.x - mn), fb = exp2f(b.x - mn);
   float4 o;
@@ -1013,8 +1019,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             const int n_vis = c0 < c_fast && !again ? 0 : min(c_key - c0, n_obs + i_row + 1);   // visible ones
             float cm = -CUDART_INF_F;
 #pragma unroll
-            for (int e = 0; e < 16; ++e) cm = e < n_vis ? fmaxf(cm, __uint_as_float(r[e])) : cm;
-            if (cm != -CUDART_INF_F) {
+            for (int e = 0; e < 16; ++e) cm = e < n_vis ? max_or_nan(cm, __uint_as_float(r[e])) : cm;
+            if (cm != -CUDART_INF_F) {                        // (a NaN goes into z, where it stays)
               cm *= P.scale2;
               if (cm > m) {
                 const float mn = cm;

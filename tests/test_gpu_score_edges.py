@@ -127,3 +127,19 @@ def test_infinite_logits_are_reported(hq, hkv, window, dtype, tokens):
                     status, again = score(q0, k0)
                     assert status == 0 and all(torch.equal(a, b) for a, b in zip(fresh, again))
     cake.destroy()
+
+
+@pytest.mark.parametrize("hq,hkv", [(8, 2), (2, 2), (4, 2)])
+@pytest.mark.parametrize("first", [16, 128, 144, 149, 2096])
+def test_nan_in_the_window_is_reported(hq, hkv, first):
+    """Window keys that are NaN: the rows of a chunk at the end of the prompt may see nothing but NaN in it."""
+    w = synth.scaled(synth.workload(3), n_layers=1, n_q_heads=hq, n_kv_heads=hkv, seq_lens=(first + 32,), total_budget=32 + 5)
+    (q,), (k0,), _ = harness.device_inputs(w)
+    cake = harness.cake_for(w)
+    for lo, hi in ((0, 32), (0, 16), (16, 32), (31, 32), (0, 0)):
+        k = k0.clone()
+        k[:, first + lo:first + hi] = float("nan")
+        cake.begin(w.cu_seqlens)
+        cake.score_layer(0, q, k)
+        assert cake.status() == (binding.CAKE_ERR_NONFINITE if hi > lo else 0), (lo, hi)
+    cake.destroy()
