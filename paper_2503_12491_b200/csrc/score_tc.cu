@@ -965,16 +965,16 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             // without looking for the tile's maximum first (an op's first tile: that of its first chunk).
             // Afterwards the reference moves up by the binary exponent of a sum that is far above 1; only where the
             // sum nears the end of fp32's range is the tile taken again, from its maxima.
-            // The load is the whole warp's, so the vote decides; and a row whose first keys all have logits of -inf takes a
-            // finite reference, so that the -inf reach its entropy term as 0 * -inf and its other logits are summed.
-            if (__any_sync(0xffffffffu, m == -CUDART_INF_F)) {
+            // (All rows of the warp at once: the load is a collective.  A row whose first keys all have logits of -inf takes
+            // a finite reference, so that the -inf reach its entropy term as 0 * -inf and its other logits are summed.)
+            if (it == it0) {
               uint32_t r[16];
               tmem_ld16_issue(taddr + c_lo, r);
               tmem_ld_wait(r);
               float cm = __uint_as_float(r[0]);
 #pragma unroll
               for (int e = 1; e < 16; ++e) cm = fmaxf(cm, __uint_as_float(r[e]));
-              if (m == -CUDART_INF_F) m = cm > -CUDART_INF_F ? cm * P.scale2 : 0.f;
+              m = cm > -CUDART_INF_F ? cm * P.scale2 : 0.f;
             }
             // two keys per instruction: four partial sums in two packed accumulators
             const f32x2 sc2 = pack2(P.scale2, P.scale2), nm2 = pack2(-m, -m);
