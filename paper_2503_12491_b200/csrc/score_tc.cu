@@ -127,13 +127,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: false (and the sticky status set) if the phase never completes.
+// Bounded wait of a whole warp: false (and the sticky status set) if the phase never completes.  Its lanes agree: what
+// follows (TMEM loads, votes, elected issue) is the whole warp's, and a phase may complete just as the limit is reached.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int32_t* status,
                                           long long limit) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > limit) {
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if (__any_sync(0xffffffffu, clock64() - t0 > limit)) {
       atomicCAS(status, 0, CAKE_ERR_TIMEOUT);
       return false;
     }
@@ -731,7 +732,6 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const int slot = kb & 1;
       const int pair = op.req * P.Hkv + op.g;
       ok = mbar_wait(&S.lse_free[slot], ((kb >> 1) & 1) ^ 1, P.status, P.spin_limit);
-      ok = __all_sync(0xffffffffu, ok) != 0;
       if (!ok) break;
       float4 v;
       if (P.lse_ext) {
