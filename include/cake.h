@@ -26,7 +26,8 @@
  *     and cake_status first make the stream they are given wait for that
  *     internal work.  Hence: results are ordered into the caller's stream by
  *     the call that hands them out, not by cake_allocate / cake_evict
- *     themselves, and the stream arguments of those two calls are unused.
+ *     themselves, and the stream arguments of those two calls are unused.  What a call has
+ *     still to read on its stream (budgets) is not overwritten by a later one before.
  *     Q and K of a layer are read only by cake_score_layer's kernels (caller's
  *     stream); K and V are read again by cake_compact.
  *   - A context serves one batch of requests at a time and is not thread-safe.

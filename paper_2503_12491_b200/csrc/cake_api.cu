@@ -92,6 +92,7 @@ void free_ctx(cake_ctx* c) {
   if (c->h_units) cudaFreeHost(c->h_units);
   if (c->upload_done) cudaEventDestroy(c->upload_done);
   if (c->ev_main) cudaEventDestroy(c->ev_main);
+  for (BudgetRead& r : c->budget_read) if (r.done) cudaEventDestroy(r.done);
   for (int i = 0; i < kScoreDepth; ++i) {
     if (c->ev_score[i]) cudaEventDestroy(c->ev_score[i]);
     if (c->ev_pool[i]) cudaEventDestroy(c->ev_pool[i]);
@@ -119,6 +120,28 @@ cudaError_t side_after(cake_ctx* c, cudaStream_t st) {
 cudaError_t main_after_side(cake_ctx* c, cudaStream_t st) {
   cudaError_t e = cudaEventRecord(c->ev_pool_side, c->pool_st);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_pool_side, 0);
+  return e;
+}
+
+// The budgets of a stage are read on the caller's stream by whoever hands results out, and written on the internal one, two
+// stages later into the same buffer: the write waits for the reads.  (An event can be waited for inside the capture
+// that recorded it, or outside if none did; elsewhere the order is the caller's, who launches the graph.)
+cudaError_t before_budget_write(cake_ctx* c, int32_t stage) {
+  BudgetRead& r = c->budget_read[stage & 1];
+  if (!r.pending) return cudaSuccess;
+  r.pending = false;
+  return step_place(c->pool_st).capture == r.at.capture ? cudaStreamWaitEvent(c->pool_st, r.done, 0) : cudaSuccess;
+}
+cudaError_t after_budget_read(cake_ctx* c, int32_t stage, cudaStream_t st) {
+  BudgetRead& r = c->budget_read[stage & 1];
+  const StepPlace here = step_place(st);
+  // an earlier read on another stream: the event is needed for this one
+  if (r.pending && (here.stream == 0 || here.stream != r.at.stream || here.capture != r.at.capture)) {
+    const cudaError_t e = before_budget_write(c, stage);
+    if (e != cudaSuccess) return e;
+  }
+  const cudaError_t e = cudaEventRecord(r.done, st);
+  if (e == cudaSuccess) { r.pending = true; r.at = here; }
   return e;
 }
 
@@ -197,6 +220,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && cudaStreamCreateWithFlags(&x->pool_st, cudaStreamNonBlocking) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_pool_side, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&x->ev_main, cudaEventDisableTiming) == cudaSuccess;
+  for (BudgetRead& r : x->budget_read) ok = ok && cudaEventCreateWithFlags(&r.done, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < kScoreDepth; ++i) {
     ok = ok && cudaEventCreateWithFlags(&x->ev_score[i], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&x->ev_pool[i], cudaEventDisableTiming) == cudaSuccess;
@@ -324,8 +348,14 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
       if (cu[r + 1] - cu[r] < c.window) return CAKE_ERR_ARG;
     if (cu[n_req] > c.max_total_tokens) return CAKE_ERR_CAPACITY;
   }
-  // the previous batch's cascade must be done before its state is reset or overwritten
+  // the previous batch's cascade, and the reads of its results, must be done before its state is reset or overwritten
   CAKE_CUDA_TRY(main_after_side(ctx, st));
+  for (BudgetRead& r : ctx->budget_read) {
+    const StepPlace here = r.pending ? step_place(st) : r.at;
+    if (r.pending && r.at.capture == here.capture && (here.stream == 0 || here.stream != r.at.stream))
+      CAKE_CUDA_TRY(cudaStreamWaitEvent(st, r.done, 0));
+    r.pending = false;
+  }
   const int64_t T = n_req > 0 ? cu[n_req] : 0;
   const bool same = ctx->n_req == n_req && n_req > 0 &&
                     memcmp(ctx->h_cu, cu, sizeof(int64_t) * (n_req + 1)) == 0;
@@ -439,6 +469,7 @@ int32_t cake_score_layer(cake_ctx* ctx, int32_t layer, const void* q_win, const 
   CAKE_CUDA_TRY(cudaStreamWaitEvent(ctx->pool_st, ctx->ev_score[place], 0));
   const int sp = prof_begin(ctx, CAKE_PROF_FINALIZE, ctx->pool_st);
   const bool budgets = ctx->last_alloc < layer;      // nobody has asked for a later stage's before
+  if (budgets) CAKE_CUDA_TRY(before_budget_write(ctx, layer));
   rc = launch_arrive(ctx, layer, true, true, budgets, ctx->pool_st);
   prof_end(ctx, sp, ctx->pool_st);
   if (rc != CAKE_OK) return rc;
@@ -459,6 +490,7 @@ int32_t cake_allocate(cake_ctx* ctx, int32_t stage, void* stream) {
   // since; any other stage is computed here, behind the budgets of stage - 1, which it falls back to.
   if (ctx->arrived_budgets != stage) {
     cudaStream_t ast = ctx->pool_st;
+    CAKE_CUDA_TRY(before_budget_write(ctx, stage));
     const int sp = prof_begin(ctx, CAKE_PROF_ALLOCATE, ast);
     const int32_t rc = launch_allocate(ctx, stage, ast);
     prof_end(ctx, sp, ast);
@@ -509,6 +541,7 @@ int32_t cake_compact(cake_ctx* ctx, int32_t layer_lo, int32_t layer_hi, const vo
   const int32_t rc = launch_compact(ctx, layer_lo, layer_hi, ptrs, k_out, v_out, row_offsets_out,
                                     positions_out, (cudaStream_t)stream);
   prof_end(ctx, sp, (cudaStream_t)stream);
+  CAKE_CUDA_TRY(after_budget_read(ctx, ctx->n_evicted - 1, (cudaStream_t)stream));
   return rc;
 }
 
@@ -541,6 +574,7 @@ int32_t cake_compact_int4(cake_ctx* ctx, int32_t layer_lo, int32_t layer_hi, con
                                          v_scale, v_zero, row_offsets_out, kgroup_offsets_out, positions_out,
                                          (cudaStream_t)stream);
   prof_end(ctx, sp, (cudaStream_t)stream);
+  CAKE_CUDA_TRY(after_budget_read(ctx, ctx->n_evicted - 1, (cudaStream_t)stream));
   return rc;
 }
 
@@ -625,7 +659,8 @@ int32_t cake_get_budgets(cake_ctx* ctx, int32_t* out, void* stream) {
       ctx->d_budget[ctx->last_alloc & 1], out, ctx->n_req, ctx->cfg.n_layers, ctx->last_alloc + 1,
       ctx->cfg.window);
   count_launch();
-  return cuda_status(cudaGetLastError());
+  CAKE_CUDA_TRY(cudaGetLastError());
+  return cuda_status(after_budget_read(ctx, ctx->last_alloc, (cudaStream_t)stream));
 }
 
 int32_t cake_get_positions(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* out, int64_t capacity,
@@ -635,7 +670,9 @@ int32_t cake_get_positions(cake_ctx* ctx, int32_t req, int32_t layer, int32_t* o
   if (req < 0 || req >= ctx->n_req || layer < 0 || layer >= ctx->cfg.n_layers) return CAKE_ERR_ARG;
   if (layer >= ctx->n_evicted || ctx->last_alloc != ctx->n_evicted - 1) return CAKE_ERR_STATE;
   CAKE_CUDA_TRY(main_after_side(ctx, (cudaStream_t)stream));
-  return launch_get_positions(ctx, req, layer, out, capacity, (cudaStream_t)stream);
+  const int32_t rc = launch_get_positions(ctx, req, layer, out, capacity, (cudaStream_t)stream);
+  CAKE_CUDA_TRY(after_budget_read(ctx, ctx->n_evicted - 1, (cudaStream_t)stream));
+  return rc;
 }
 
 int32_t cake_status(cake_ctx* ctx, int32_t* device_status_out, void* stream) {
@@ -726,6 +763,7 @@ int32_t cake_decode_begin(cake_ctx* ctx, const void* const* k_layers, const void
     }
   }
   const int32_t rc = launch_decode_begin(ctx, ptrs, k_cache, v_cache, row_offsets_out, st);
+  CAKE_CUDA_TRY(after_budget_read(ctx, c.n_layers - 1, st));
   if (rc != CAKE_OK) return rc;
   ctx->dec_update_mode = update_mode;
   ctx->dec_last_layer = -1;

@@ -64,10 +64,16 @@ struct ScoreOp {
   int32_t pad;
 };
 
-// Where a decode step was enqueued: the stream, by its unique id or in a capture by its handle (0:
+// Where a call was enqueued: the stream, by its unique id or in a capture by its handle (0:
 // unknown), and the stream capture that recorded it (0: none, the step ran).
 struct StepPlace {
   unsigned long long stream, capture;
+};
+// A read of a budget buffer on a caller's stream that the next write of the buffer has to wait for.
+struct BudgetRead {
+  cudaEvent_t done;
+  bool pending;
+  StepPlace at;
 };
 
 struct LayerPtrs {
@@ -115,6 +121,7 @@ struct cake_ctx {
   int32_t n_pref;          // layers whose preference is known
   int32_t n_evicted;       // stages completed
   int32_t alloc_of_buf[2]; // stage whose budgets live in budget buffer 0/1 (-1 none)
+  cake::BudgetRead budget_read[2];   // newest read of either buffer on a caller's stream
   int32_t last_alloc;      // most recent stage passed to cake_allocate
   int32_t arrived_budgets; // stage whose budgets were computed when its layer was scored (-1: none, or a
                            // preference was set since)

@@ -57,3 +57,55 @@ def test_positions_of_a_budget(kind, lens):
             assert np.array_equal(got[g], want), (r, g)
     assert cake.status() == 0
     cake.destroy()
+
+
+@pytest.mark.parametrize("reader", ["compact", "int4", "positions", "budgets"])
+@pytest.mark.parametrize("streams", ["one", "two"])
+def test_budgets_are_read_before_they_are_written_again(reader, streams):
+    """The buffer of a stage's budgets is written again two stages later, on the internal stream: results handed out
+    behind a long wait of the caller's stream are still those of their stage, also where another stream reads after it."""
+    w = synth.scaled(synth.workload(1), n_layers=3, n_q_heads=2, n_kv_heads=2, window=WINDOW, seq_lens=(3000,), total_budget=900)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    k = [torch.randn(2, 3000, w.head_dim, generator=gen, device="cuda") for _ in range(3)]
+    x = torch.rand(2, 3000, generator=gen, device="cuda")
+    cake = harness.cake_for(w)
+
+    def read():
+        if reader == "compact":
+            rows = cake.packed_rows_bound()
+            out = cake.compact(k, k, layer_hi=1, k_out=torch.zeros(rows, w.head_dim, device="cuda"),
+                               v_out=torch.zeros(rows, w.head_dim, device="cuda"), positions=torch.zeros(rows, dtype=torch.int32, device="cuda"))
+            return list(out)
+        if reader == "budgets":
+            return [cake.get_budgets()]
+        return [cake.get_positions(0, 0, 896)]
+
+    def run(wait):
+        cake.begin(w.cu_seqlens)
+        cake.set_preferences(torch.ones(1, 3, dtype=torch.float64, device="cuda"))
+        for l in range(3 if reader == "int4" else 1):
+            cake.set_indicators(l, x)
+            cake.allocate(l)
+            cake.evict(l)
+        torch.cuda.synchronize()
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side if streams == "two" else torch.cuda.current_stream()):
+            if wait:
+                torch.cuda._sleep(20_000_000)        # about ten milliseconds
+            if reader == "int4":
+                out = cake.compact_int4(k, k)
+                out = [out["row_offsets"], out["positions"][:1800], out["k_codes"][:1800]]
+            else:
+                out = read()
+        if streams == "two":
+            cake.get_budgets()
+        if wait:
+            for stage in (0,) if reader == "int4" else (1, 2):      # (INT4 compaction has read the budgets of stage 2)
+                cake.allocate(stage)
+        torch.cuda.synchronize()
+        return out
+
+    want, got = run(False), run(True)
+    assert all(torch.equal(a, b) for a, b in zip(want, got))
+    assert cake.status() == 0
+    cake.destroy()
