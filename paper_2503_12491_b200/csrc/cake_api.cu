@@ -207,10 +207,9 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     // packed rows: H_kv * sum_r min(B_total, L * N_r) <= H_kv * min(R * B_total, L * T)
     const int64_t a = R * c.total_budget, b = (int64_t)c.n_layers * T;
     x->pos_packed_cap = (int64_t)c.n_kv_heads * (a < b ? a : b);
-    // a request longer than the shared-memory bitmap orders its positions in global scratch:
-    // one bitmap of ceil((n + 3)/32) words per (request, layer, head)
+    // a batch with a request longer than the shared-memory bitmap orders its positions in global scratch
     x->bitmap_words = T + 3 > (int64_t)kBitmapSmemWords * 32
-                          ? (int64_t)c.n_layers * c.n_kv_heads * (T / 32 + 2 * R + 1) : 0;
+                          ? (int64_t)c.n_layers * c.n_kv_heads * bitmap_words_before(T, R) : 0;
   }
   x->h_cu = (int64_t*)calloc((size_t)R + 1, sizeof(int64_t));
   bool ok = x->h_cu != nullptr;

@@ -256,6 +256,11 @@ inline float* layer_store(const cake_ctx* ctx, int32_t layer) {
   return ctx->d_store + (size_t)layer * ctx->cfg.n_kv_heads * ctx->total_tokens;
 }
 
+// Global scratch of the selection, for requests whose bitmap does not fit shared memory: words of a (layer, KV head)'s
+// bitmaps before request r of a batch, which starts at token cu.  A request of N tokens needs at most
+// (N - 1 + 3 + 31) / 32 <= N / 32 + 2 words, so that any requests fit between their neighbours.
+__host__ __device__ inline int64_t bitmap_words_before(int64_t cu, int64_t r) { return cu / 32 + 2 * r; }
+
 // Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
 __device__ __forceinline__ uint32_t ordered_key(float v) {
   uint32_t b = __float_as_uint(v);

@@ -131,7 +131,7 @@ template <int POS_THREADS>
 __global__ void __launch_bounds__(POS_THREADS, 1024 / POS_THREADS)
 sorted_positions(const float* __restrict__ store, const int32_t* __restrict__ prefix_all, const ReqInfo* __restrict__ reqs, const int32_t* __restrict__ budget,
                  const int64_t* __restrict__ offsets, int32_t* __restrict__ out, uint32_t* __restrict__ scratch,
-                 int64_t scratch_words, int req0, int lo, int L, int Hkv, int Sw, int smem_words, int cap, int64_t T,
+                 int req0, int lo, int L, int Hkv, int Sw, int smem_words, int cap, int64_t T,
                  int64_t capacity) {
   extern __shared__ __align__(16) uint32_t sh_dyn[];
   __shared__ SelectSmem S;
@@ -166,8 +166,7 @@ sorted_positions(const float* __restrict__ store, const int32_t* __restrict__ pr
   uint2* const list = reinterpret_cast<uint2*>(sh_dyn + smem_words);
   uint32_t* bits = sh_dyn;
   if (words > smem_words) {
-    const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    bits = scratch + cta * (size_t)scratch_words;
+    bits = scratch + (size_t)(gridDim.x * gridDim.y) * bitmap_words_before(rq.cu, req) + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * words;
   }
   // the bucket with prefix[d] < b <= prefix[d + 1]
   const int32_t* pf = prefix_all + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
@@ -443,8 +442,6 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
     attr.mark(ctx->device);
   }
   const int64_t ctas = (int64_t)c.n_kv_heads * (hi - lo) * n_req;
-  if (need_words > kBitmapSmemWords &&
-      (!ctx->d_bitmap || ctas * (int64_t)need_words > ctx->bitmap_words)) return CAKE_ERR_CAPACITY;
   const dim3 grid(c.n_kv_heads, hi - lo, n_req);
   // A list is a chain of scans and short passes: with more lists than the device holds CTAs of 1024
   // threads, smaller ones keep more chains in flight (1024 lists of 4K tokens: 42 us with 1024 threads).
@@ -461,7 +458,7 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
 #define CAKE_POSITIONS(NT)                                                                                                \
   cfg.blockDim = dim3(NT);                                                                                                \
   e = cudaLaunchKernelEx(&cfg, sorted_positions<NT>, (const float*)ctx->d_store, (const int32_t*)ctx->d_prefix,           \
-                         (const ReqInfo*)ctx->d_req, budget, offsets, out, ctx->d_bitmap, (int64_t)need_words, req0, lo,  \
+                         (const ReqInfo*)ctx->d_req, budget, offsets, out, ctx->d_bitmap, req0, lo,                       \
                          c.n_layers, c.n_kv_heads, c.window, smem_words, cap, ctx->total_tokens, capacity)
   if (ctas <= ctx->n_sm) { CAKE_POSITIONS(1024); }
   else if (ctas <= 2 * ctx->n_sm) { CAKE_POSITIONS(512); }

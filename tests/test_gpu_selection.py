@@ -109,3 +109,34 @@ def test_budgets_are_read_before_they_are_written_again(reader, streams):
     assert all(torch.equal(a, b) for a, b in zip(want, got))
     assert cake.status() == 0
     cake.destroy()
+
+
+@pytest.mark.parametrize("lens", [(1_600_003,), (1_600_003, 3001, 90_007), (517, 1_580_000, 1_600_001)])
+@pytest.mark.parametrize("kind", ["spread", "one bucket", "ties"])
+def test_prompts_beyond_the_shared_memory_bitmap(kind, lens):
+    """Requests of more than 1.57 M tokens, alone and beside short ones: their bitmaps lie in global scratch, which is
+    sized by the sum of the tokens."""
+    w = synth.scaled(synth.workload(1), n_layers=1, n_q_heads=1, n_kv_heads=1, window=WINDOW, seq_lens=lens,
+                     total_budget=WINDOW + 100_001, dtype="bf16")
+    rng = np.random.default_rng(len(kind) + len(lens))
+    cu = w.cu_seqlens
+    ind = np.zeros((1, w.total_tokens), dtype=np.float32)
+    for r, N in enumerate(lens):
+        ind[0, cu[r]:cu[r] + N - WINDOW] = values(kind, N - WINDOW, rng)
+    cake = harness.cake_for(w)
+    cake.begin(cu)
+    cake.set_preferences(torch.ones(len(lens), 1, dtype=torch.float64, device="cuda"))
+    cake.set_indicators(0, torch.from_numpy(ind).cuda())
+    cake.allocate(0)
+    cake.evict(0)
+    k = torch.zeros(1, w.total_tokens, w.head_dim, dtype=torch.bfloat16, device="cuda")
+    _, _, off, pos = cake.compact([k], [k])
+    off, pos = off.tolist(), pos.cpu().numpy()
+    for r, N in enumerate(lens):
+        n = N - WINDOW
+        b = min(n, 100_001)
+        want = np.concatenate([O.topk_keep(ind[0, cu[r]:cu[r] + n].astype(np.float64), b), np.arange(n, N)])
+        assert np.array_equal(pos[off[r]:off[r + 1]], want), r
+        assert np.array_equal(cake.get_positions(r, 0, b + WINDOW).cpu().numpy()[0], want), r
+    assert cake.status() == 0
+    cake.destroy()
