@@ -164,8 +164,9 @@ int32_t cake_allocate(cake_ctx* ctx, int32_t stage, void* stream);
  * and stages in order.
  * Budgets only shrink, so the set that a TopK on the surviving pairs would leave
  * is the first entries of all of the layer's stored pairs, as many as the budget
- * says: it is found where it is read (cake_compact, the getters), and this call
- * enqueues no work of its own. */
+ * says: it is found where it is read, and this call enqueues no work of its own.
+ * Every read of a layer's set (cake_compact, cake_compact_int4, cake_decode_begin,
+ * cake_get_positions) is a pass over two bytes per token and KV head of it. */
 int32_t cake_evict(cake_ctx* ctx, int32_t stage, void* stream);
 
 /* Gathers the retained rows of layers [layer_lo, layer_hi) (Eq. 12: K^ = K[D,:],

@@ -78,7 +78,7 @@ void free_ctx(cake_ctx* c) {
   cudaFree(c->d_req); cudaFree(c->d_units); cudaFree(c->d_H); cudaFree(c->d_V); cudaFree(c->d_P);
   cudaFree(c->d_budget[0]); cudaFree(c->d_budget[1]); cudaFree(c->d_status);
   cudaFree(c->d_ring);
-  cudaFree(c->d_store); cudaFree(c->d_prefix); cudaFree(c->d_hist); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
+  cudaFree(c->d_store); cudaFree(c->d_codes); cudaFree(c->d_prefix); cudaFree(c->d_hist); cudaFree(c->d_arrivals); cudaFree(c->d_headsum);
   cudaFree(c->d_pos_packed); cudaFree(c->d_bitmap); cudaFree(c->d_lse2);
   cudaFree(c->d_scores); cudaFree(c->d_simt_arrivals);
   cudaFree(c->d_rowpart);
@@ -208,7 +208,7 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
     const int64_t a = R * c.total_budget, b = (int64_t)c.n_layers * T;
     x->pos_packed_cap = (int64_t)c.n_kv_heads * (a < b ? a : b);
     // a batch with a request longer than the shared-memory bitmap orders its positions in global scratch
-    x->bitmap_words = T + 3 > (int64_t)kBitmapSmemWords * 32
+    x->bitmap_words = T > (int64_t)kBitmapSmemWords * 32
                           ? (int64_t)c.n_layers * c.n_kv_heads * bitmap_words_before(T, R) : 0;
   }
   x->h_cu = (int64_t*)calloc((size_t)R + 1, sizeof(int64_t));
@@ -232,8 +232,8 @@ int32_t cake_create(const cake_config* cfg, cake_ctx** out) {
   ok = ok && dev_alloc(&x->d_budget[0], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_budget[1], R * c.n_layers) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_status, 1) == cudaSuccess;
-  // (vector loads of a row's end may reach seven values beyond the last row)
-  ok = ok && dev_alloc(&x->d_store, (size_t)c.n_layers * c.n_kv_heads * T + 8) == cudaSuccess;
+  ok = ok && dev_alloc(&x->d_store, (size_t)c.n_layers * c.n_kv_heads * T) == cudaSuccess;
+  ok = ok && dev_alloc(&x->d_codes, (size_t)c.n_layers * c.n_kv_heads * code_tokens(T, R)) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_prefix, (size_t)x->max_lists * (kBins + 1)) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_hist, (size_t)R * c.n_kv_heads * kBins) == cudaSuccess;
   ok = ok && dev_alloc(&x->d_arrivals, (size_t)R * c.n_kv_heads + R) == cudaSuccess;

@@ -16,12 +16,10 @@ constexpr int kSimtMinUnit = 64;      // fewest keys of a score unit of the SIMT
 constexpr int kSimtMaxUnit = 1024;
 constexpr int64_t kMaxScoreElems = 64ll << 20;   // logits the SIMT kernels keep between their two steps (256 MB)
 constexpr int kSimtThreads = 256;
-constexpr int kBinBits = 12;         // buckets of the indicators: their top bits
-constexpr int kBins = 1 << kBinBits;
+constexpr int kBins = 4096;          // buckets of the indicators, see bucket_of
 constexpr int kChunkKeys = 4096;     // granularity of the token ranges of the pooling
-constexpr int kBitmapSmemWords = 48 * 1024;   // positions of up to 1.5 M tokens are ordered in shared memory
-
-constexpr int kSelectSmemWords = 50 * 1024;   // dynamic shared memory of the selection: bitmap and list of candidates
+constexpr int kBitmapSmemWords = 36 * 1024;   // positions of up to 1.1 M tokens are ordered in a CTA's shared memory
+constexpr int kSelectSmemWords = 50 * 1024;   // dynamic shared memory of the selection: queues, bitmap and list of candidates
 constexpr int kScoreDepth = 8;        // layers whose score outputs may wait for their pooling, where memory allows
 constexpr int kScoreGroups = 3;      // statistics warp groups per CTA of the tensor-core score kernel
 constexpr int kScoreWarps = 4 * kScoreGroups;   // statistics warps: one column-pass partial each
@@ -146,6 +144,7 @@ struct cake_ctx {
   uint8_t* d_ring;         // one allocation for the places of d_raw, d_colpart and d_hrow
   float* d_raw[cake::kScoreDepth];     // [H_kv][max_total_tokens] un-pooled indicator, by layer % score_depth
   float* d_store;          // [L][H_kv][tokens of the batch] pooled indicators of every layer, +inf on the windows
+  uint16_t* d_codes;       // [L][H_kv][code_tokens(n_req)] upper half of every indicator's ordered key, see code_row
   int64_t max_lists;       // (request, layer, head) triples
   int32_t* d_prefix;       // [max_lists][kBins+1] bucket offsets of every (request, layer, head)
   uint32_t* d_hist;        // [max_pairs][kBins] bucket histogram of the arriving layer (zero at rest)
@@ -256,16 +255,70 @@ inline float* layer_store(const cake_ctx* ctx, int32_t layer) {
   return ctx->d_store + (size_t)layer * ctx->cfg.n_kv_heads * ctx->total_tokens;
 }
 
+// Codes of a layer of the current batch: a request's start on a multiple of eight, so that they are written and read in
+// vectors whatever the prompts' lengths.
+__host__ __device__ inline int64_t code_row(int64_t cu, int64_t r) { return (cu & ~(int64_t)7) + 8 * r; }
+inline int64_t code_tokens(int64_t tokens, int64_t n_req) { return code_row(tokens, n_req) + 8; }
+inline uint16_t* layer_codes(const cake_ctx* ctx, int32_t layer) {
+  return ctx->d_codes + (size_t)layer * ctx->cfg.n_kv_heads * code_tokens(ctx->total_tokens, ctx->n_req);
+}
+
 // Global scratch of the selection, for requests whose bitmap does not fit shared memory: words of a (layer, KV head)'s
 // bitmaps before request r of a batch, which starts at token cu.  A request of N tokens needs at most
-// (N - 1 + 3 + 31) / 32 <= N / 32 + 2 words, so that any requests fit between their neighbours.
-__host__ __device__ inline int64_t bitmap_words_before(int64_t cu, int64_t r) { return cu / 32 + 2 * r; }
+// (N - 1 + 31) / 32 <= N / 32 + 1 words, so that any requests fit between their neighbours.
+__host__ __device__ inline int64_t bitmap_words_before(int64_t cu, int64_t r) { return cu / 32 + r; }
 
 // Order-preserving integer image of a float; -0 and +0 compare equal, as they do as floats.
 __device__ __forceinline__ uint32_t ordered_key(float v) {
   uint32_t b = __float_as_uint(v);
   b = b == 0x80000000u ? 0u : b;
   return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+
+// A key's bucket, counted from the top (bucket 0 holds the largest values): four to a power of two, and 64 to one between
+// 2^-27 and 2^5, where the indicators of prompts of up to millions of tokens lie.  (There every 17th bucket is empty.)
+constexpr uint32_t kFineFirst = 0x80000000u | (127u - 27u) << 23, kFineEnd = kFineFirst + (32u << 23);
+static_assert((0xFFFFFFFFu >> 21) + ((kFineEnd - kFineFirst) >> 17) == kBins - 1, "every key has a bucket");
+__device__ __forceinline__ int bucket_of(uint32_t key) {
+  return (int)((kBins - 1) + (kFineFirst >> 17)) - (int)(key >> 21) - (int)(min(max(key, kFineFirst), kFineEnd) >> 17);
+}
+// (0 beyond the last key: its predecessor ends the topmost buckets)
+__device__ __forceinline__ uint32_t bucket_first_key(int bucket) {
+  const int bin = kBins - 1 - bucket, fine = bin - (int)(kFineFirst >> 21), steps = (int)((kFineEnd - kFineFirst) >> 17);
+  if (fine < 0) return (uint32_t)bin << 21;
+  if (fine >= steps + steps / 16) return bin - steps > 2047 ? 0u : (uint32_t)(bin - steps) << 21;
+  const int sixteen = fine / 17;
+  return kFineFirst + (uint32_t)(16 * sixteen + min(fine - 17 * sixteen, 16)) * (1u << 17);
+}
+__device__ __forceinline__ uint32_t bucket_last_key(int bucket) { return bucket > 0 ? bucket_first_key(bucket - 1) - 1u : 0xFFFFFFFFu; }
+
+__device__ __forceinline__ void copy_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// ---- clusters: the rank, barriers, and what a peer has at the place of `p` in its shared memory
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ uint32_t ld_peer(const void* p, uint32_t rank) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(peer_addr(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 ld_peer2(const void* p, uint32_t rank) {
+  uint2 v;
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(peer_addr(p, rank)) : "memory");
+  return v;
 }
 
 // The eviction indicator of one key from the mean and variance of its window attention

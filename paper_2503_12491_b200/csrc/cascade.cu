@@ -21,10 +21,8 @@ __device__ inline double warp_sum_f64(double v) {
 }
 
 // --------------------------------------------------------------- pool + bins
-// A key's (ordered_key's) bucket is its top kBinBits bits, counted from the top (bucket 0 holds the largest values).
 // When a layer arrives, its pooled indicators are histogrammed: "the top b" are then all values of the buckets
 // before the one that contains the b-th, and the best part of that bucket.
-__device__ inline int bucket_of(uint32_t key) { return (kBins - 1) - (int)(key >> (32 - kBinBits)); }
 
 // Token ranges of the pooling items: a request's tokens in at most `want` equal runs, a
 // multiple of kChunkKeys long.
@@ -70,9 +68,6 @@ __device__ inline int team_excl_scan(int v, int* warp_tot, int* total) {
 
 constexpr int PH_PER = 4;                            // consecutive tokens per thread and pass
 constexpr int kTileTok = 4096;                       // tokens of a run on their way to shared memory at a time
-__device__ __forceinline__ void copy_async4(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
 
 struct AllocArgs {           // budgets of one stage
   const double* dP;          // [req][L]
@@ -220,12 +215,13 @@ __device__ void finalize_heads(const FinalizeArgs& F, const AllocArgs& A, const 
 struct ArriveArgs {
   const float* raw;
   float* store;
+  uint16_t* codes;
   const ReqInfo* reqs;
   uint32_t* hist;
   uint32_t* arrivals;
   int32_t* prefix;
   int n_req, want, layer, L, Hkv, kp, mode, do_pool;
-  int64_t T;
+  int64_t T, code_T;
 };
 struct alignas(16) ArriveSmem {   // of a team
   union { uint32_t sh[kBins]; AllocSmem alloc; };
@@ -260,6 +256,7 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
     team_sync();
     const float* src = raw + (size_t)g * T + rq.cu;
     float* dst = Q.store + (size_t)g * T + rq.cu;
+    uint16_t* code = Q.codes + (size_t)g * Q.code_T + code_row(rq.cu, req);
     const int t0 = split * span, t1 = min(rq.N, t0 + span);
     // Writes four tokens and counts their buckets.  Neighbours often share a bucket, so a run is counted
     // once, at its first token; without branches (with them a warp issued some 300 instructions for its
@@ -275,9 +272,14 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
             for (int e = 0; e < PH_PER; ++e) dst[j0 + e] = out[e];
           }
         }
+        uint32_t key[PH_PER];
         int q[PH_PER];
 #pragma unroll
-        for (int e = 0; e < PH_PER; ++e) q[e] = bucket_of(ordered_key(out[e]));
+        for (int e = 0; e < PH_PER; ++e) {
+          key[e] = ordered_key(out[e]);
+          q[e] = bucket_of(key[e]);
+        }
+        *reinterpret_cast<uint2*>(code + j0) = make_uint2(__byte_perm(key[0], key[1], 0x7632), __byte_perm(key[2], key[3], 0x7632));
         const bool s1 = q[1] != q[0], s2 = q[2] != q[1], s3 = q[3] != q[2];
         atomicAdd(&sh[q[0]], s1 ? 1u : s2 ? 2u : s3 ? 3u : 4u);
         if (s1) atomicAdd(&sh[q[1]], s2 ? 1u : s3 ? 2u : 3u);
@@ -290,8 +292,10 @@ arrive_layer(const ArriveArgs Q, const FinalizeArgs F, const AllocArgs B) {
           if (j < t1 && j >= rq.n) {
             dst[j] = CUDART_INF_F;
           } else if (j < t1) {
+            const uint32_t key = ordered_key(out[e]);
             if (do_pool) dst[j] = out[e];
-            atomicAdd(&sh[bucket_of(ordered_key(out[e]))], 1u);
+            code[j] = (uint16_t)(key >> 16);
+            atomicAdd(&sh[bucket_of(key)], 1u);
           }
         }
       }
@@ -671,6 +675,7 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
   ArriveArgs Q;
   Q.raw = ctx->d_raw[layer % ctx->score_depth];
   Q.store = layer_store(ctx, layer);
+  Q.codes = layer_codes(ctx, layer);
   Q.reqs = ctx->d_req;
   Q.hist = ctx->d_hist;
   Q.arrivals = ctx->d_arrivals;
@@ -678,6 +683,7 @@ int32_t launch_arrive(cake_ctx* ctx, int32_t layer, bool do_pool, bool finalize,
   Q.n_req = ctx->n_req; Q.layer = layer; Q.L = c.n_layers; Q.Hkv = c.n_kv_heads;
   Q.kp = c.pool_kernel; Q.mode = c.pool_mode; Q.do_pool = do_pool ? 1 : 0;
   Q.T = ctx->total_tokens;
+  Q.code_T = code_tokens(ctx->total_tokens, ctx->n_req);
   int grid;
   cascade_shape(ctx, layer, finalize ? ctx->n_req * F.parts : 0, &Q.want, &grid);
   const AllocArgs B = alloc_args(ctx, layer);

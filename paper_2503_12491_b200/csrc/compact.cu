@@ -63,85 +63,103 @@ block_offsets(const int32_t* __restrict__ budget, int64_t* __restrict__ row_off,
   }
 }
 
-constexpr int kTieCap = 512;                         // entries of equal rank but for their position that are ranked one by one
+constexpr int kTieCap = 512;                         // entries that can be ranked one by one
 constexpr int kFewEntries = 64;                      // entries that are ranked without another histogram
 constexpr int SP_BINS = 1024;                        // (22 - clz in the code is 32 - clz - log2 of this)
 constexpr int SP_BATCH = 4;                          // groups of 32 entries a warp has in flight
+constexpr int SP_UNLISTED = 8;                       // the same of values, where it goes over them again
+constexpr int SP_GROUPS = 4;                         // 16-byte groups of values a lane has in flight
+constexpr int SP_QUEUE_WORDS = 64 * 5;               // a warp's queue
+constexpr int kSelectCluster = kPortableCluster;     // most CTAs that share a list
 
 struct SelectSmem {
-  uint32_t hist[SP_BINS];
+  uint32_t hist[2][SP_BINS];                         // in turn: peers read one while the next is counted
   uint2 ties[kTieCap];                               // (key, position)
   int warp_tot[32];
-  int total, count, tie_count;
-  int bucket, start, n_in;
+  int total;
+  int count, tie_count, ones, before;
   uint32_t sel_bin, sel_rem, sel_cnt;
 };
+static_assert(sizeof(uint2) * kTieCap <= sizeof(uint32_t) * 2 * SP_BINS, "the cluster's ties take the histograms' place");
 
-// Bins of the histogram from the top: the one that holds the krem-th entry, how many of its entries are wanted,
-// and its size.
-__device__ inline void find_bin(uint32_t krem, SelectSmem& S) {
+// Bins of the histogram, summed over the list's CTAs, from the top: the one that holds the krem-th entry, how many of
+// its entries are wanted, and its size.
+__device__ inline void find_bin(uint32_t krem, const uint32_t* hist, int csize, SelectSmem& S) {
+  constexpr int MOST = SP_BINS / 256;                // bins of a thread
   const int per = max(1, SP_BINS / (int)blockDim.x);
-  int mine = 0;
-  for (int q = 0; q < per; ++q) mine += (int)S.hist[SP_BINS - 1 - (threadIdx.x * per + q)];
-  int above = block_excl_scan(mine, S.warp_tot, &S.total);
-  for (int q = 0; q < per; ++q) {
-    const int bin = SP_BINS - 1 - (threadIdx.x * per + q), h = (int)S.hist[bin];
-    if ((uint32_t)above < krem && (uint32_t)(above + h) >= krem) {
-      S.sel_bin = (uint32_t)bin;
-      S.sel_rem = krem - (uint32_t)above;
-      S.sel_cnt = (uint32_t)h;
+  int h[MOST], mine = 0;
+#pragma unroll
+  for (int q = 0; q < MOST; ++q) {
+    h[q] = 0;
+    if (q < per) {
+      const uint32_t* at = &hist[SP_BINS - 1 - (threadIdx.x * per + q)];
+      if (csize == 1) h[q] = (int)*at;
+      else for (int r = 0; r < csize; ++r) h[q] += (int)ld_peer(at, (uint32_t)r);
     }
-    above += h;
+    mine += h[q];
   }
-  __syncthreads();
-}
-__device__ inline void clear_hist(SelectSmem& S) {
-  for (int i = threadIdx.x; i < SP_BINS; i += blockDim.x) S.hist[i] = 0;
+  int above = block_excl_scan(mine, S.warp_tot, &S.total);
+#pragma unroll
+  for (int q = 0; q < MOST; ++q) {
+    if ((uint32_t)above < krem && (uint32_t)(above + h[q]) >= krem) {
+      S.sel_bin = (uint32_t)(SP_BINS - 1 - (threadIdx.x * per + q));
+      S.sel_rem = krem - (uint32_t)above;
+      S.sel_cnt = (uint32_t)h[q];
+    }
+    above += h[q];
+  }
   __syncthreads();
 }
 // Counts a bin for every lane that has one (>= 0).  Pooled values repeat: a run of equal bins in
 // neighbouring lanes is counted once.  Called by whole warps.
-__device__ __forceinline__ void count_bin(int bin, SelectSmem& S) {
+__device__ __forceinline__ void count_bin(int bin, uint32_t* hist) {
   if (!__any_sync(0xffffffffu, bin >= 0)) return;
   const int lane = threadIdx.x & 31, before = __shfl_up_sync(0xffffffffu, bin, 1);
   const bool first = lane == 0 || bin != before;
   const uint32_t firsts = __ballot_sync(0xffffffffu, first);
   if (first && bin >= 0) {
     const uint32_t later = lane < 31 ? firsts >> (lane + 1) : 0u;
-    atomicAdd(&S.hist[bin], later ? (uint32_t)__ffs(later) : 32u - lane);
+    atomicAdd(&hist[bin], later ? (uint32_t)__ffs(later) : 32u - lane);
   }
 }
 
-// One CTA per (head, layer in [lo, hi), request): which positions the current budget b keeps, then these in ascending
-// order, then the window, written at out[base + g*len ...].
+// `csize` CTAs (a cluster) per (head, layer in [lo, hi), request): which positions the current budget b keeps, then
+// these in ascending order, then the window, written at out[base + g*len ...].  A CTA owns a run of the values.
 //   1. The bucket offsets say which bucket holds the b-th largest value, and how many of its entries are wanted.
-//   2. One pass over the values, eight to a lane: the bits of those in the buckets before are set, those inside go
-//      to a list in shared memory, as (key, position).  If there are too many for it, the steps below go over all values.
-//   3. Histograms of SP_BINS equal parts of the bucket's keys narrow it to the bin that holds the b-th value, until that
-//      has few entries (usually at once); these are ranked by (key, position).
+//   2. One pass over the values' codes (upper halves of their keys): the bits of those in the buckets before are set, those
+//      inside go to the CTA's list in shared memory, as (value, position).  A CTA whose list overflows goes over its
+//      values again in the steps below.
+//   3. Histograms of SP_BINS equal parts of the bucket's keys, and of the positions where the keys are equal, narrow it to
+//      the bin that holds the b-th entry, until that has few entries (usually at once); these are ranked by (key, position).
 //   4. Ranks of the bits, positions.
-// Bound: the pass over the values, and between the steps the latency of the chain, which other lists' CTAs on the SM
-// hide: 46 us for 256 lists of 131 040 values (134 MB), 29 for 512 of 26 000, 20 for 1024 of 4064.  Placing every layer's
-// values in bucket order when it arrived made this step 31, 27 and 22 us, for a launch of 7 to 76 us per layer.
-// Without the bucket offsets three digit histograms of all values took 300 us in the first case and 137 in the
-// second (run lengths, and atomics on few hot bins), and a sample in their place 129 and 133, since the candidates
-// on either side of the cut are many where a layer keeps much.  `bits` is shared memory when the request's n
-// bits fit, else a slice of global scratch.
+// Bound: the pass over the codes, and between the steps the latency of the chain, which other lists' CTAs on the SM
+// hide.  A retained set may be read after every stage, and by layers, so what counts is few lists as much as many, and
+// values that share a bucket: 8 lists of 131 040 values 16 us, 80 20, 256 33, 256 of 32 736 17, 1024 of 4064 21; 256 lists whose
+// values all share a bucket 206, all equal 370.  With one CTA per list, a pass over the values themselves (lanes 32
+// bytes apart, every sector fetched twice), eight buckets to a power of two everywhere and a bisection among equal
+// values these took 23, 25, 42, 19, 21, 447 and 2620 us, and ordinary indicators (log-normal, sigma 0.15) overflowed the
+// list: 50 us instead of 36 at 256 lists.  Without the bucket offsets three digit histograms of all values took 300 us.
+// `bits` is shared memory when a CTA's bits fit, else a slice of global scratch.
 template <int POS_THREADS>
 __global__ void __launch_bounds__(POS_THREADS, 1024 / POS_THREADS)
-sorted_positions(const float* __restrict__ store, const int32_t* __restrict__ prefix_all, const ReqInfo* __restrict__ reqs, const int32_t* __restrict__ budget,
+sorted_positions(const float* __restrict__ store, const uint16_t* __restrict__ codes, const int32_t* __restrict__ prefix_all, const ReqInfo* __restrict__ reqs, const int32_t* __restrict__ budget,
                  const int64_t* __restrict__ offsets, int32_t* __restrict__ out, uint32_t* __restrict__ scratch,
-                 int req0, int lo, int L, int Hkv, int Sw, int smem_words, int cap, int64_t T,
-                 int64_t capacity) {
+                 int req0, int lo, int L, int Hkv, int Sw, int csize, int smem_words, int cap, int64_t T,
+                 int64_t code_T, int64_t capacity) {
   extern __shared__ __align__(16) uint32_t sh_dyn[];
   __shared__ SelectSmem S;
-  const int g = blockIdx.x, layer = lo + blockIdx.y, req = req0 + blockIdx.z;
+  const int g = blockIdx.x / csize, rank = blockIdx.x - g * csize, layer = lo + blockIdx.y, req = req0 + blockIdx.z;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int WARPS = POS_THREADS / 32;
+  const bool split = csize > 1;
+  auto meet = [&]() { if (split) cluster_sync(); else __syncthreads(); };
   const ReqInfo rq = reqs[req];
   const int n = rq.n;
   const int b = budget[(size_t)req * L + layer];
   const int len = b + Sw;
+  constexpr int PER = kBins / 32, EACH = PER / 32;
+  const int32_t* pf = prefix_all + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
+  const int coarse = __ldg(&pf[PER * lane]);         // (for step 1, on its way with the budget)
   // without row offsets the caller gave a capacity: never write past it
   const int64_t room = offsets ? (int64_t)len : capacity - (int64_t)g * len;
   // The offsets are written by the kernel before this one, which may still run; nothing else that is read here is.
@@ -152,77 +170,81 @@ sorted_positions(const float* __restrict__ store, const int32_t* __restrict__ pr
   };
   if (b <= 0 || b >= n) {
     int32_t* dst = row_start();
-    for (int t = threadIdx.x; t < (b <= 0 ? 0 : n); t += POS_THREADS)
+    const int t0 = rank * POS_THREADS + threadIdx.x, step = csize * POS_THREADS;
+    for (int t = t0; t < (b <= 0 ? 0 : n); t += step)
       if (t < room) dst[t] = t;
-    for (int t = threadIdx.x; t < Sw; t += POS_THREADS)
+    for (int t = t0; t < Sw; t += step)
       if (b + t < room) dst[b + t] = n + t;
     return;
   }
-  // Element q = a + i of the row, counted from the 16-byte boundary at or before its start, is value i: lanes load
-  // whole groups of four, and bits and positions count in elements until they are written out.
   const float* const v = store + ((size_t)layer * Hkv + g) * T + rq.cu;
-  const int a = (int)((reinterpret_cast<uintptr_t>(v) >> 2) & 3), end = a + n;
-  const int words = (end + 31) >> 5;
-  uint2* const list = reinterpret_cast<uint2*>(sh_dyn + smem_words);
-  uint32_t* bits = sh_dyn;
-  if (words > smem_words) {
-    bits = scratch + (size_t)(gridDim.x * gridDim.y) * bitmap_words_before(rq.cu, req) + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * words;
-  }
-  // the bucket with prefix[d] < b <= prefix[d + 1]
-  const int32_t* pf = prefix_all + (((size_t)req * L + layer) * Hkv + g) * (kBins + 1);
+  // this CTA's words of 32 values, [w_lo, w_hi)
+  const int words = (n + 31) >> 5, share = (words + csize - 1) / csize;
+  const int w_lo = min(words, rank * share), w_hi = min(words, w_lo + share);
+  uint4* const queue = reinterpret_cast<uint4*>(sh_dyn) + warp * 64;             // octets of the warp that are to be taken,
+  int* const queue_at = reinterpret_cast<int*>(sh_dyn) + WARPS * 256 + warp * 64;   //   up to 63, and their numbers
+  uint32_t* bits = sh_dyn + SP_QUEUE_WORDS * WARPS;
+  uint2* const list = reinterpret_cast<uint2*>(bits + smem_words);
+  if (share > smem_words)
+    bits = scratch + (size_t)(Hkv * gridDim.y) * bitmap_words_before(rq.cu, req) + (size_t)(blockIdx.y * Hkv + g) * words + w_lo;
+  // octets (groups of eight values) of this CTA; the last one's codes beyond the prompt are not looked at
+  const int o_lo = 4 * w_lo, o_hi = max(o_lo, min((n + 7) >> 3, 4 * w_hi));
+  const int o_first = o_lo + warp * 32 * SP_GROUPS + lane;
+  const uint4* const c8 = reinterpret_cast<const uint4*>(codes + ((size_t)layer * Hkv + g) * code_T + code_row(rq.cu, req));
+  uint4 next[SP_GROUPS];                             // octets of the lane on their way
+  auto fetch = [&](int o0) {
+#pragma unroll
+    for (int u = 0; u < SP_GROUPS; ++u) next[u] = o0 + 32 * u < o_hi ? __ldcg(c8 + o0 + 32 * u) : make_uint4(0, 0, 0, 0);
+  };
+  fetch(o_first);
+  if (threadIdx.x == 0) S.count = S.tie_count = S.ones = S.before = 0;
+  for (int wi = threadIdx.x; wi < w_hi - w_lo; wi += POS_THREADS) bits[wi] = 0;
+  // The bucket with prefix[d] < b <= prefix[d + 1], by every warp for itself: the 128 that hold it, then the one.
+  int bucket, start, n_in;
   {
-    constexpr int PER = kBins / POS_THREADS;
-    int at[PER + 1];
+    const int from = 31 - __clz((int)__ballot_sync(0xffffffffu, coarse < b));          // (prefix[0] = 0 < b)
+    int at[EACH], below = 0;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) at[q] = __ldg(&pf[q * POS_THREADS + threadIdx.x]);
-    at[PER] = 0;
+    for (int q = 0; q < EACH; ++q) at[q] = __ldg(&pf[PER * from + 32 * q + lane + 1]);
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      const int next = __ldg(&pf[q * POS_THREADS + threadIdx.x + 1]);
-      if (at[q] < b && next >= b) { S.bucket = q * POS_THREADS + threadIdx.x; S.start = at[q]; S.n_in = next - at[q]; }
+    for (int q = 0; q < EACH; ++q) below += __popc(__ballot_sync(0xffffffffu, at[q] < b));
+    start = __shfl_sync(0xffffffffu, coarse, from);
+    int next = 0;
+#pragma unroll
+    for (int q = 0; q < EACH; ++q) {
+      const int before = __shfl_sync(0xffffffffu, at[q], (below - 1) & 31), after = __shfl_sync(0xffffffffu, at[q], below & 31);
+      if (below > 0 && (below - 1) >> 5 == q) start = before;
+      if (below >> 5 == q) next = after;
     }
+    bucket = PER * from + below;
+    n_in = next - start;
   }
-  if (threadIdx.x == 0) { S.count = 0; S.tie_count = 0; }
+  uint32_t krem = (uint32_t)(b - start);             // entries of the bucket that are kept
+  uint32_t klo = bucket_first_key(bucket), khi = bucket_last_key(bucket);
+  const uint32_t in_lo = klo, in_hi = khi;
+  __threadfence_block();
   __syncthreads();
-  const int d = S.bucket, n_in = S.n_in;
-  uint32_t krem = (uint32_t)(b - S.start);           // entries of the bucket that are kept
-  uint32_t klo = (uint32_t)(kBins - 1 - d) << (32 - kBinBits), khi = klo | ((1u << (32 - kBinBits)) - 1u);
-  const bool listed = n_in <= cap;
-  if (listed) {
-    // In buckets above zero the bits of a float are compared as they are: as signed integers they have the order of
-    // the keys there, and everything else lies below.
-    const bool plain = klo > 0x80000000u;
-    const int ilo = (int)(klo ^ 0x80000000u), ihi = (int)(khi ^ 0x80000000u);
-    const uint4* const v4 = reinterpret_cast<const uint4*>(v - a);
-    const int n_oct = (end + 7) >> 3;                // (up to seven elements beyond the row are loaded, and not looked at)
-    uint4 next[2];
-    auto fetch = [&](int o) {
-      next[0] = next[1] = make_uint4(0, 0, 0, 0);
-      if (o < n_oct) { next[0] = __ldcg(v4 + 2 * o); next[1] = __ldcg(v4 + 2 * o + 1); }
-    };
-    fetch(warp * 32 + lane);
-    for (int o0 = warp * 32; o0 < n_oct; o0 += POS_THREADS) {
-      const int o = o0 + lane;
-      uint32_t x[8] = {next[0].x, next[0].y, next[0].z, next[0].w, next[1].x, next[1].y, next[1].z, next[1].w};
-      fetch(o + POS_THREADS);
-      if (!plain) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = ordered_key(__uint_as_float(x[e])) ^ 0x80000000u;
-      }
+  {
+    // One pass over the upper halves of the keys: those above the bucket's are kept, those of the bucket are listed.  Few
+    // octets have either; they are gathered in the warp's queue and taken 32 at a time.
+    const uint32_t c_lo = klo >> 16, c_hi = khi >> 16;
+    auto take = [&](int i, bool have) {
+      const int o = queue_at[i & 63];
+      const uint4 c = queue[i & 63];
+      const uint32_t x[4] = {c.x, c.y, c.z, c.w};
       uint32_t above = 0, in = 0;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        above |= (int)x[e] > ihi ? 1u << e : 0u;
-        in |= (int)x[e] >= ilo ? 1u << e : 0u;
+        const uint32_t code = e & 1 ? x[e >> 1] >> 16 : x[e >> 1] & 0xFFFFu;
+        above |= code > c_hi ? 1u << e : 0u;
+        in |= code >= c_lo ? 1u << e : 0u;
       }
-      // elements of the row among the eight
-      const int lo_e = max(0, a - 8 * o), hi_e = min(8, max(0, end - 8 * o));
-      const uint32_t row = (0xFFu << lo_e) & (0xFFu >> (8 - hi_e));
+      const uint32_t row = have ? 0xFFu >> (8 - min(8, n - 8 * o)) : 0u;         // those of the prompt
       above &= row;
       in &= row & ~above;
-      if (o < n_oct) reinterpret_cast<uint8_t*>(bits)[o] = (uint8_t)above;
-      if (!__any_sync(0xffffffffu, in != 0)) continue;
+      if (above) reinterpret_cast<uint8_t*>(bits)[o - o_lo] = (uint8_t)above;
       const int mine = __popc(in);
+      if (!__any_sync(0xffffffffu, mine)) return;
       int inc = mine;
 #pragma unroll
       for (int s = 1; s < 32; s <<= 1) {
@@ -232,115 +254,169 @@ sorted_positions(const float* __restrict__ store, const int32_t* __restrict__ pr
       int at = 0;
       if (lane == 31) at = atomicAdd(&S.count, inc);
       at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
+      while (in) {
+        const int e = __ffs(in) - 1;
+        in &= in - 1;
+        if (at < cap) {
+          list[at].y = (uint32_t)(8 * o + e);
+          copy_async4(&list[at].x, v + 8 * o + e);
+        }
+        ++at;
+      }
+    };
+    int head = 0, tail = 0;
+    constexpr int step = POS_THREADS * SP_GROUPS;
+    for (int o0 = o_first; o0 - lane < o_hi; o0 += step) {
+      uint4 now[SP_GROUPS];
 #pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (in >> e & 1u) list[at++] = make_uint2(x[e] ^ 0x80000000u, (uint32_t)(8 * o + e));
+      for (int u = 0; u < SP_GROUPS; ++u) now[u] = next[u];
+      fetch(o0 + step);
+#pragma unroll
+      for (int u = 0; u < SP_GROUPS; ++u) {
+        const uint32_t most = __vmaxu2(__vmaxu2(now[u].x, now[u].y), __vmaxu2(now[u].z, now[u].w));
+        const bool hit = max(most & 0xFFFFu, most >> 16) >= c_lo && o0 + 32 * u < o_hi;
+        const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+        if (hit) {
+          const int i = (tail + __popc(hits & ((1u << lane) - 1u))) & 63;
+          queue[i] = now[u];
+          queue_at[i] = o0 + 32 * u;
+        }
+        tail += __popc(hits);
+        if (tail - head >= 32) {
+          __syncwarp();
+          take(head + lane, true);
+          head += 32;
+          __syncwarp();
+        }
+      }
     }
-    if (threadIdx.x < 4 && n_oct + (int)threadIdx.x < 4 * words) reinterpret_cast<uint8_t*>(bits)[n_oct + threadIdx.x] = 0;
+    __syncwarp();
+    if (tail > head) take(head + lane, lane < tail - head);
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
   __threadfence_block();
   __syncthreads();
-  const int cnt = listed ? n_in : n;
-  // f(key, element, whether there is such an entry), whole warps
+  const int cnt = S.count;
+  const bool listed = cnt <= cap;
+  // f(key, position, whether there is such an entry) for the bucket's entries among this CTA's values, whole warps
   auto for_entries = [&](auto f) {
-    for (int i0 = warp * 32 * SP_BATCH; i0 < cnt; i0 += WARPS * 32 * SP_BATCH) {
-      uint2 x[SP_BATCH];
+    if (listed) {
+      for (int i0 = warp * 32 * SP_BATCH; i0 < cnt; i0 += WARPS * 32 * SP_BATCH) {
+        uint2 x[SP_BATCH];
 #pragma unroll
-      for (int u = 0; u < SP_BATCH; ++u) {
-        const int i = i0 + 32 * u + lane;
-        x[u] = make_uint2(0u, 0u);
-        if (i < cnt) x[u] = listed ? list[i] : make_uint2(ordered_key(__ldcg(v + i)), (uint32_t)(a + i));
+        for (int u = 0; u < SP_BATCH; ++u) x[u] = i0 + 32 * u + lane < cnt ? list[i0 + 32 * u + lane] : make_uint2(0u, 0u);
+#pragma unroll
+        for (int u = 0; u < SP_BATCH; ++u)
+          if (i0 + 32 * u < cnt) f(ordered_key(__uint_as_float(x[u].x)), (int)x[u].y, i0 + 32 * u + lane < cnt);
       }
+    } else {
+      const int hi_v = min(n, 32 * w_hi);
+      for (int i0 = 32 * w_lo + warp * 32 * SP_UNLISTED; i0 < hi_v; i0 += POS_THREADS * SP_UNLISTED) {
+        float x[SP_UNLISTED];
 #pragma unroll
-      for (int u = 0; u < SP_BATCH; ++u)
-        if (i0 + 32 * u < cnt) f(x[u].x, (int)x[u].y, i0 + 32 * u + lane < cnt);
+        for (int u = 0; u < SP_UNLISTED; ++u) x[u] = i0 + 32 * u + lane < hi_v ? __ldcg(v + i0 + 32 * u + lane) : 0.f;
+#pragma unroll
+        for (int u = 0; u < SP_UNLISTED; ++u) {
+          const uint32_t key = ordered_key(x[u]);
+          f(key, i0 + 32 * u + lane, i0 + 32 * u + lane < hi_v && key >= in_lo && key <= in_hi);
+        }
+      }
     }
   };
+  // The entries in question: n_bin of them with keys klo to khi and, where these are equal, positions plo to phi.  Those
+  // before (larger keys, or equal keys and lower positions) are kept, and krem of the n_bin.
   uint32_t n_bin = (uint32_t)n_in;
-  while (n_bin > (uint32_t)kFewEntries && klo < khi) {
-    const uint32_t width = khi - klo;
-    const int shift = width < SP_BINS ? 0 : 22 - __clz(width);
-    clear_hist(S);
-    for_entries([&](uint32_t key, int, bool have) {
-      count_bin(have && key >= klo && key <= khi ? (int)((key - klo) >> shift) : -1, S);
-    });
+  int plo = 0, phi = n - 1;
+  const uint32_t few = n_in <= cap ? kFewEntries : kTieCap;      // (a round is a pass over the values if a list has overflowed)
+  for (int round = 0; n_bin > few && (krem < n_bin || klo == 0); ++round) {
+    uint32_t* const hist = S.hist[round & 1];
+    for (int i = threadIdx.x; i < SP_BINS; i += POS_THREADS) hist[i] = 0;
     __syncthreads();
-    find_bin(krem, S);
-    klo += S.sel_bin << shift;
-    if (khi - klo >= 1u << shift) khi = klo + ((1u << shift) - 1u);
+    const bool by_key = klo < khi;
+    const uint32_t width = by_key ? khi - klo : (uint32_t)(phi - plo);
+    const int shift = width < SP_BINS ? 0 : 22 - __clz(width);
+    for_entries([&](uint32_t key, int pos, bool have) {
+      const bool in = have && key >= klo && key <= khi && pos >= plo && pos <= phi;
+      count_bin(in ? (int)((by_key ? key - klo : (uint32_t)(phi - pos)) >> shift) : -1, hist);
+    });
+    meet();
+    find_bin(krem, hist, csize, S);
     krem = S.sel_rem;
     n_bin = S.sel_cnt;
-    __syncthreads();
-  }
-  // every entry above the bin, and krem of its n_bin entries
-  int pos_cut = -1;                                  // more than kTieCap are equal: up to this position
-  const bool few = n_bin <= (uint32_t)kTieCap;
-  if (!few) {
-    int plo = a, phi = end - 1;                      // smallest cut with count(pos <= cut) >= krem
-    while (plo < phi) {
-      const int mid = plo + ((phi - plo) >> 1);
-      int c = 0;
-      for_entries([&](uint32_t key, int pos, bool have) { c += have && key == klo && pos <= mid ? 1 : 0; });
-      block_excl_scan(c, S.warp_tot, &S.total);
-      const int tot = S.total;
-      __syncthreads();
-      if ((uint32_t)tot >= krem) phi = mid; else plo = mid + 1;
+    const uint32_t at = S.sel_bin << shift, last = (1u << shift) - 1u;
+    if (by_key) {
+      klo += at;
+      khi = min(khi, klo + min(last, 0xFFFFFFFFu - klo));
+    } else {
+      phi -= (int)at;
+      plo = max(plo, phi - (int)last);
     }
-    pos_cut = plo;
   }
-  if (!listed) {
-    for (int wi = threadIdx.x; wi < words; wi += POS_THREADS) bits[wi] = 0;
-    __threadfence_block();
-    __syncthreads();
+  if (krem == n_bin && klo > 0) {                    // all of them are kept
+    if (klo < khi) khi = klo - 1u;
+    else plo = phi + 1;
+    n_bin = 0;
   }
   for_entries([&](uint32_t key, int pos, bool have) {
-    if (have && (key > khi || (key == klo && pos <= pos_cut))) atomicOr(&bits[pos >> 5], 1u << (pos & 31));
-    if (few && have && key >= klo && key <= khi) S.ties[atomicAdd(&S.tie_count, 1)] = make_uint2(key, (uint32_t)pos);
+    const bool kept = key > khi || (key == khi && pos < plo);
+    if (have && kept) atomicOr(&bits[(pos >> 5) - w_lo], 1u << (pos & 31));
+    if (have && !kept && key >= klo && pos <= phi) S.ties[atomicAdd(&S.tie_count, 1)] = make_uint2(key, (uint32_t)pos);
   });
   __threadfence_block();
   __syncthreads();
-  if (few) {
-    for (int i = threadIdx.x; i < (int)n_bin; i += POS_THREADS) {
-      const uint2 e = S.ties[i];
-      uint32_t ahead = 0;
-      for (int o = 0; o < (int)n_bin; ++o) {
-        const uint2 x = S.ties[o];
-        ahead += x.x > e.x || (x.x == e.x && x.y < e.y) ? 1u : 0u;
-      }
-      if (ahead < krem) atomicOr(&bits[e.y >> 5], 1u << (e.y & 31));
+  // the cluster's ties, and the kept positions before this CTA's
+  uint2* all = S.ties;
+  int before = 0;
+  if (split) {
+    int ones = 0;
+    for (int wi = threadIdx.x; wi < w_hi - w_lo; wi += POS_THREADS) ones += __popc(bits[wi]);
+    ones = __reduce_add_sync(0xffffffffu, ones);
+    if (lane == 0 && ones) atomicAdd(&S.ones, ones);
+    meet();
+    all = reinterpret_cast<uint2*>(&S.hist[0][0]);
+    int at = 0;
+    for (int r = 0; r < csize; ++r) {
+      const int c = (int)ld_peer(&S.tie_count, (uint32_t)r);
+      if (r < rank) before += (int)ld_peer(&S.ones, (uint32_t)r);
+      for (int i = threadIdx.x; i < c; i += POS_THREADS) all[at + i] = ld_peer2(&S.ties[i], (uint32_t)r);
+      at += c;
     }
-    __threadfence_block();
+    cluster_arrive();                                // nothing of the peers is read from here on
     __syncthreads();
   }
-  int32_t* const dst = row_start();
-  for (int t = threadIdx.x; t < Sw; t += POS_THREADS)
-    if (b + t < room) dst[b + t] = n + t;
-  // Ranks of the bits: a warp takes a run of the words, 32 at a time, so that its lanes write close together.
-  const int run = (words + 32 * WARPS - 1) / (32 * WARPS) * 32, w0 = min(words, warp * run), w1 = min(words, w0 + run);
-  int ones = 0;
-  for (int wi = w0 + lane; wi < w1; wi += 32) ones += __popc(bits[wi]);
-  ones = __reduce_add_sync(0xffffffffu, ones);
-  if (lane == 0) S.warp_tot[warp] = ones;
-  __syncthreads();
-  int rank = __reduce_add_sync(0xffffffffu, lane < warp ? S.warp_tot[lane] : 0);
-  for (int wb = w0; wb < w1; wb += 32) {
-    uint32_t m = wb + lane < w1 ? bits[wb + lane] : 0u;
-    const int mine = __popc(m);
-    int inc = mine;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, inc, s);
-      if (lane >= s) inc += t;
+  for (int i = threadIdx.x; i < (int)n_bin; i += POS_THREADS) {
+    const uint2 e = all[i];
+    uint32_t ahead = 0;
+    for (int o = 0; o < (int)n_bin; ++o) {
+      const uint2 x = all[o];
+      ahead += x.x > e.x || (x.x == e.x && x.y < e.y) ? 1u : 0u;
     }
-    int at = rank + inc - mine;
-    while (m) {
-      const int bit = __ffs(m) - 1;
-      m &= m - 1;
-      if (at < b && at < room) dst[at] = ((wb + lane) << 5) + bit - a;
-      ++at;
-    }
-    rank += __shfl_sync(0xffffffffu, inc, 31);
+    const int wi = (int)(e.y >> 5);
+    if (ahead < krem && wi >= w_lo && wi < w_hi) atomicOr(&bits[wi - w_lo], 1u << (e.y & 31));
+    if (ahead < krem && wi < w_lo) atomicAdd(&S.before, 1);
   }
+  __threadfence_block();
+  __syncthreads();
+  before += S.before;
+  int32_t* const dst = row_start();
+  if (rank == 0)
+    for (int t = threadIdx.x; t < Sw; t += POS_THREADS)
+      if (b + t < room) dst[b + t] = n + t;
+  // Ranks of the bits: a thread takes a run of the words, or of their bytes where there are more threads than words.
+  const int limit = (int)min((int64_t)b, max(room, (int64_t)0));
+  auto place = [&](int width, auto unit) {
+    const int units = (w_hi - w_lo) * (32 / width), run = (units + POS_THREADS - 1) / POS_THREADS;
+    const int u0 = min(units, (int)threadIdx.x * run), u1 = min(units, u0 + run);
+    int ones = 0;
+    for (int u = u0; u < u1; ++u) ones += __popc(unit(u));
+    int to = before + block_excl_scan(ones, S.warp_tot, &S.total);
+    for (int u = u0; u < u1; ++u)
+      for (uint32_t m = unit(u); m; m &= m - 1, ++to)
+        if (to < limit) dst[to] = 32 * w_lo + width * u + __ffs(m) - 1;
+  };
+  if (w_hi - w_lo < POS_THREADS) place(8, [&](int u) { return (uint32_t)reinterpret_cast<const uint8_t*>(bits)[u]; });
+  else place(32, [&](int u) { return bits[u]; });
+  if (split) cluster_wait();                         // a peer may still read this CTA's ties
 }
 
 constexpr int GA_THREADS = 128;
@@ -430,10 +506,6 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
   const int32_t* budget = ctx->d_budget[(ctx->n_evicted - 1) & 1];
   int max_n = 0;
   for (int r = req0; r < req0 + n_req; ++r) max_n = ctx->h_req[r].n > max_n ? ctx->h_req[r].n : max_n;
-  const int need_words = (max_n + 3 + 31) / 32;
-  const int smem_words = need_words <= kBitmapSmemWords ? (need_words + 1) / 2 * 2 : 0;
-  // list of a bucket's entries, 8 bytes each: a sixteenth of the values, or all of a short prompt's
-  const int cap = std::min(std::max(2048, max_n / 16), (kSelectSmemWords - smem_words) / 2);
   static PerDeviceOnce attr;
   if (attr.need(ctx->device)) {
     CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelectSmemWords * 4));
@@ -441,29 +513,41 @@ int32_t run_sorted_positions(cake_ctx* ctx, int req0, int n_req, int lo, int hi,
     CAKE_CUDA_TRY(cudaFuncSetAttribute(sorted_positions<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelectSmemWords * 4));
     attr.mark(ctx->device);
   }
-  const int64_t ctas = (int64_t)c.n_kv_heads * (hi - lo) * n_req;
-  const dim3 grid(c.n_kv_heads, hi - lo, n_req);
-  // A list is a chain of scans and short passes: with more lists than the device holds CTAs of 1024
-  // threads, smaller ones keep more chains in flight (1024 lists of 4K tokens: 42 us with 1024 threads).
+  const int64_t lists = (int64_t)c.n_kv_heads * (hi - lo) * n_req;
+  // Threads per list: as many as the device holds at 1024 per SM, and no more than leave a lane two octets: first in larger
+  // CTAs (256 lists of 131 040 values: 33 us with 512 threads, 39 with 256, 41 with 1024), then in more of them (8 lists:
+  // 21 us with one CTA of 1024, 16 with eight).
+  const int64_t most = std::max<int64_t>((int64_t)ctx->n_sm * 1024 / lists, 256), want = (max_n + 15) / 16;
+  int threads = 256, csize = 1;
+  while (threads < 1024 && 2 * threads <= most && threads < want) threads *= 2;
+  const int widest = widest_cluster(false, kSelectCluster);
+  while (2 * csize <= widest && (int64_t)2 * csize * threads <= most && csize * threads < want) csize *= 2;
+  // a CTA's bitmap, and its list of the bucket's entries, 8 bytes each: a sixteenth of the values, or all of a short prompt's
+  const int share = ((max_n + 31) / 32 + csize - 1) / csize, queue_words = SP_QUEUE_WORDS * threads / 32;
+  const int smem_words = share <= kBitmapSmemWords ? (share + 1) / 2 * 2 : 0;
+  const int cap = std::min(std::max(2048, 2 * share), (kSelectSmemWords - queue_words - smem_words) / 2);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.dynamicSmemBytes = (size_t)(smem_words + 2 * cap) * 4;
+  cfg.gridDim = dim3((unsigned)(c.n_kv_heads * csize), hi - lo, n_req);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = (size_t)(queue_words + smem_words + 2 * cap) * 4;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[2];
   cfg.attrs = at;
-  cfg.numAttrs = offsets ? 1 : 0;                    // behind run_offsets, which wrote them
-  cudaError_t e;
-#define CAKE_POSITIONS(NT)                                                                                                \
-  cfg.blockDim = dim3(NT);                                                                                                \
-  e = cudaLaunchKernelEx(&cfg, sorted_positions<NT>, (const float*)ctx->d_store, (const int32_t*)ctx->d_prefix,           \
-                         (const ReqInfo*)ctx->d_req, budget, offsets, out, ctx->d_bitmap, req0, lo,                       \
-                         c.n_layers, c.n_kv_heads, c.window, smem_words, cap, ctx->total_tokens, capacity)
-  if (ctas <= ctx->n_sm) { CAKE_POSITIONS(1024); }
-  else if (ctas <= 2 * ctx->n_sm) { CAKE_POSITIONS(512); }
-  else { CAKE_POSITIONS(256); }
-#undef CAKE_POSITIONS
+  cfg.numAttrs = 0;
+  if (offsets) {                                     // behind run_offsets, which wrote them
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (csize > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = (unsigned)csize;
+    at[cfg.numAttrs].val.clusterDim.y = 1;
+    at[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, threads == 1024 ? sorted_positions<1024> : threads == 512 ? sorted_positions<512> : sorted_positions<256>,
+                                           (const float*)ctx->d_store, (const uint16_t*)ctx->d_codes, (const int32_t*)ctx->d_prefix, (const ReqInfo*)ctx->d_req, budget, offsets,
+                                           out, ctx->d_bitmap, req0, lo, c.n_layers, c.n_kv_heads, c.window, csize, smem_words, cap,
+                                           ctx->total_tokens, code_tokens(ctx->total_tokens, ctx->n_req), capacity);
   count_launch();
   return cuda_status(e);
 }

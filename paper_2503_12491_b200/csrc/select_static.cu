@@ -18,26 +18,8 @@ constexpr int SEL_WIDE_CTAS = 128;             // CTAs (one per SM) up to which 
 constexpr int kSelShare = 2048;                // values per CTA below which a head is spread no further
 constexpr int kSelSmemKeys = 40 * 1024;        // keys a CTA holds in shared memory; a larger share is read again
 
-__device__ __forceinline__ uint32_t sel_cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t sel_remote(const void* p, uint32_t rank) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ uint2 sel_ld_remote(const void* p, uint32_t rank) {
-  uint2 v;
-  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(sel_remote(p, rank)) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sel_st_remote(const void* p, uint32_t rank, uint2 v) {
-  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(sel_remote(p, rank)), "r"(v.x), "r"(v.y) : "memory");
-}
-__device__ __forceinline__ void sel_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+__device__ __forceinline__ void st_peer2(const void* p, uint32_t rank, uint2 v) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(peer_addr(p, rank)), "r"(v.x), "r"(v.y) : "memory");
 }
 
 // A cluster of `csize` CTAs per head keeps the `keep` entries that come first in the order (value
@@ -61,7 +43,7 @@ select_positions_static(const float* __restrict__ values, int n, int keep, int32
   __shared__ uint2 s_warp2[SEL_WARPS];
   __shared__ uint32_t s_digit, s_rem;
   __shared__ uint2 x_count[SEL_CLUSTER_WIDE];        // (above, equal) of every CTA of the cluster
-  const int rank = (int)sel_cluster_rank();
+  const int rank = (int)cluster_rank();
   const int head = blockIdx.x / csize;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lo = min(n, rank * share), cnt = min(n, lo + share) - lo;
@@ -100,10 +82,10 @@ select_positions_static(const float* __restrict__ values, int n, int keep, int32
     const uint32_t* sum = h;
     if (csize > 1) {
       sum = sums;
-      sel_cluster_sync();
+      cluster_sync();
       const int pairs = SEL_BINS / 2 / csize;        // pairs of bins in a section
       for (int i = threadIdx.x; i < SEL_BINS / 2; i += SEL_THREADS)
-        parts[i] = sel_ld_remote(&h[2 * (rank * pairs + i % pairs)], (uint32_t)(i / pairs));
+        parts[i] = ld_peer2(&h[2 * (rank * pairs + i % pairs)], (uint32_t)(i / pairs));
       __syncthreads();
       if ((int)threadIdx.x < pairs) {
         uint2 t = make_uint2(0, 0);
@@ -112,8 +94,8 @@ select_positions_static(const float* __restrict__ values, int n, int keep, int32
       }
       __syncthreads();
       for (int i = threadIdx.x; i < SEL_BINS / 2; i += SEL_THREADS)
-        sel_st_remote(&sums[2 * (rank * pairs + i % pairs)], (uint32_t)(i / pairs), parts[i % pairs]);
-      sel_cluster_sync();
+        st_peer2(&sums[2 * (rank * pairs + i % pairs)], (uint32_t)(i / pairs), parts[i % pairs]);
+      cluster_sync();
     } else {
       __syncthreads();
     }
@@ -181,8 +163,8 @@ select_positions_static(const float* __restrict__ values, int n, int keep, int32
   before = make_uint2(__shfl_sync(0xffffffffu, total.x, warp) - mine.x, __shfl_sync(0xffffffffu, total.y, warp) - mine.y);
   total = make_uint2(__shfl_sync(0xffffffffu, total.x, 31), __shfl_sync(0xffffffffu, total.y, 31));
   if (csize > 1) {
-    if ((int)threadIdx.x < csize) sel_st_remote(&x_count[rank], threadIdx.x, total);
-    sel_cluster_sync();               // also: nobody leaves while its histograms may still be read
+    if ((int)threadIdx.x < csize) st_peer2(&x_count[rank], threadIdx.x, total);
+    cluster_sync();               // also: nobody leaves while its histograms may still be read
     for (int p = 0; p < rank; ++p) { before.x += x_count[p].x; before.y += x_count[p].y; }
   }
   int32_t* dst = out + (size_t)head * keep;

@@ -26,6 +26,8 @@ def values(kind, n, rng):
         return np.where(rng.random(n) < 0.33, np.float32(1.0), np.exp(x))
     if kind == "negative":
         return -np.exp(x)
+    if kind == "bucket edges":                       # around the powers of two where fine buckets begin and end
+        return (np.exp2(rng.choice([-30, -28, -27, -26, 4, 5, 6], size=n)) * (1 + rng.integers(-2, 3, size=n) / 64)).astype(np.float32)
     x[rng.random(n) < 0.1] = np.inf                  # "extremes"
     x[rng.random(n) < 0.3] = np.finfo(np.float32).min
     return x
@@ -57,6 +59,14 @@ def test_positions_of_a_budget(kind, lens):
             assert np.array_equal(got[g], want), (r, g)
     assert cake.status() == 0
     cake.destroy()
+
+
+@pytest.mark.parametrize("kind", ["bucket edges", "spread", "one bucket", "all equal"])
+@pytest.mark.parametrize("lens", [(33, 70_001, 517, 131_072), (32_739, 32_770), (16_418,), (8_225, 3)])
+def test_lists_that_several_ctas_share(kind, lens):
+    """Few lists are spread over clusters: runs of values that end inside a word, CTAs without any, candidates of one
+    bucket in all of them, and buckets on either side of the range with finer ones."""
+    test_positions_of_a_budget(kind, lens)
 
 
 @pytest.mark.parametrize("reader", ["compact", "int4", "positions", "budgets"])
@@ -113,9 +123,11 @@ def test_budgets_are_read_before_they_are_written_again(reader, streams):
 
 @pytest.mark.parametrize("lens", [(1_600_003,), (1_600_003, 3001, 90_007), (517, 1_580_000, 1_600_001)])
 @pytest.mark.parametrize("kind", ["spread", "one bucket", "ties"])
-def test_prompts_beyond_the_shared_memory_bitmap(kind, lens):
-    """Requests of more than 1.57 M tokens, alone and beside short ones: their bitmaps lie in global scratch, which is
-    sized by the sum of the tokens."""
+@pytest.mark.parametrize("cluster", ["8", "1"])
+def test_prompts_beyond_the_shared_memory_bitmap(kind, lens, cluster, monkeypatch):
+    """Requests of more than 1.2 M tokens, alone and beside short ones: a CTA's bitmap does not fit its shared memory
+    (with one CTA per list) and lies in global scratch, which is sized by the sum of the tokens."""
+    monkeypatch.setenv("CAKE_MAX_CLUSTER", cluster)
     w = synth.scaled(synth.workload(1), n_layers=1, n_q_heads=1, n_kv_heads=1, window=WINDOW, seq_lens=lens,
                      total_budget=WINDOW + 100_001, dtype="bf16")
     rng = np.random.default_rng(len(kind) + len(lens))
