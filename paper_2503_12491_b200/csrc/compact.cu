@@ -428,8 +428,8 @@ constexpr int GA_BATCH = 8;                          // passes of K and of V loa
 //
 // Bound: memory; rows of 256 bytes at random places.  One lookup (a binary search and a 64-bit division) per
 // row and four rows in flight took 210 us for 1.05 M rows of 256 bytes in K and V (5.1 TB/s).
-// Its CTAs take their places while the positions are written out (2 us less per call: four layers of 512 tokens
-// 82 -> 80 us); offsets and positions are read behind the wait, so they are not declared read-only here.
+// A short gather's CTAs take their places while the positions are written out (see run_gather); offsets and positions are
+// read behind the wait, so they are not declared read-only here.
 template <int CPR, bool kDecode>
 __global__ void __launch_bounds__(GA_THREADS)
 gather_rows(const LayerPtrs ptrs, const int64_t* offsets, const int64_t* dec_off,
@@ -566,7 +566,11 @@ int32_t run_gather(cake_ctx* ctx, const LayerPtrs& ptrs, const int64_t* row_off,
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  // An early start spares 2 us (four layers of 512 tokens 81.4 -> 78.6 us), but the CTAs then lie where the kernel before had
+  // left room and not evenly, which a long gather pays for: 1.05 M rows behind 256 lists of 131 040 values 187 -> 200 us for
+  // both, the 128K prefill 4110 -> 4145, a ragged batch 9346 -> 9384; between 131 K and 1 M rows of shorter prompts it is
+  // even.  So it is for gathers of up to four runs of 32 rows a warp.
+  cfg.numAttrs = ctx->packed_rows_bound <= (int64_t)grid * GA_THREADS ? 1 : 0;
   cudaError_t e;
 #define CAKE_GATHER(CPR)                                                                                                 \
   e = cudaLaunchKernelEx(&cfg, dec_off ? gather_rows<CPR, true> : gather_rows<CPR, false>, ptrs, row_off, dec_off, budget, pos,  \
