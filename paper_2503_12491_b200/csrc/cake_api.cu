@@ -421,8 +421,12 @@ int32_t cake_begin(cake_ctx* ctx, int32_t n_req, const int64_t* cu, void* stream
   if (n_req == 0) { ctx->n_units = 0; ctx->packed_rows_bound = 0; ctx->n_tc_ctas = 0; }
   if (ctx->use_tc) {
     ctx->tc_tag = 0;
-    if (ctx->n_tc_ctas > 0)
-      CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_tc_exch, 0, tc_exchange_bytes((int64_t)n_req * c.n_kv_heads, ctx->n_tc_asegs), st));
+    if (ctx->n_tc_ctas > 0) {
+      // (a plan that merges in every CTA has no merged rows, which come first)
+      const int64_t pairs = (int64_t)n_req * c.n_kv_heads;
+      const size_t skip = ctx->tc_direct ? tc_exchange_bytes(pairs, 0) : 0;
+      CAKE_CUDA_TRY(cudaMemsetAsync(ctx->d_tc_exch + skip, 0, tc_exchange_bytes(pairs, ctx->n_tc_asegs) - skip, st));
+    }
   }
   ctx->n_req = n_req;
   ctx->total_tokens = T;
