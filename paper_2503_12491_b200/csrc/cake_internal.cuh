@@ -59,7 +59,6 @@ struct ScoreOp {
   int32_t phase;
   int32_t seg;
   int32_t n;       // non-window keys of the request
-  int32_t pad;
 };
 
 // Where a call was enqueued: the stream, by its unique id or in a capture by its handle (0:

@@ -78,7 +78,6 @@ struct TcParams {
   const int32_t* cta_op;        // [n_cta + 1]
   const int32_t* group_begin;   // [n_groups + 1] first pair of every merge group; null: every merge_ways pairs
   int n_groups;
-  const ReqInfo* reqs;
   const int32_t* pair_aseg;     // [pairs + 1] pass-A segment ranges per pair
   int both;                     // 0: pass B alone
   uint32_t tag, want;           // mark of this launch's exchanged rows, and the one that readers wait for
@@ -90,7 +89,6 @@ struct TcParams {
   float* colpart;               // pass B out: [B-segment][statistics warp][G][2]
   float* hrow;                  // [pair][128] sum_j p log2 p of every window row
   int32_t* status;
-  int64_t T;
   long long spin_limit;         // cycles after which a wait gives up and raises CAKE_ERR_TIMEOUT
   int n_pairs;
   int Hkv, Hq, Sw, rows, d;
@@ -1139,7 +1137,6 @@ void cut_pair(std::vector<std::vector<ScoreOp>>& per_cta, int rot, int n_cta, in
     const int t1 = (int)((share_end - flat) < tiles ? (share_end - flat) : tiles);
     ScoreOp op;
     op.base = base; op.n = n_obs;
-    op.pad = 0;
     op.req = req; op.g = g; op.key0 = t0 * TILE;
     op.nkeys = (t1 * TILE < keys ? t1 * TILE : keys) - t0 * TILE;
     op.phase = phase;
@@ -1195,8 +1192,6 @@ int64_t tc_max_segments(const cake_config& c, int n_sm) {
   if (waves > pairs) waves = pairs;
   return pairs + waves * n_sm;
 }
-
-inline int op_tiles(const ScoreOp& op) { return (op.nkeys + TILE - 1) / TILE; }
 
 // Builds the per-CTA programs of the batch in ctx->h_req[0..n_req): one with both passes, and one with
 // pass B alone (denominators supplied by the caller).
@@ -1504,7 +1499,6 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   const int n_pairs = ctx->n_req * c.n_kv_heads;
   TcParams P;
   P.ops = ctx->d_tc_ops;
-  P.reqs = ctx->d_req;
   // with one wave the groups are those of the plain rule, which spares the merger a read per group
   P.group_begin = ctx->n_tc_waves > 1 ? ctx->d_tc_index + 2 * (n_pairs + 1) : nullptr;
   P.n_groups = ctx->n_tc_groups;
@@ -1517,7 +1511,6 @@ int32_t launch_score_tc(cake_ctx* ctx, int32_t layer, const void* q_win, const v
   P.hrow = ctx->d_hrow[layer % ctx->score_depth];
   P.n_pairs = n_pairs;
   P.status = ctx->d_status;
-  P.T = ctx->total_tokens;
   P.Hkv = c.n_kv_heads; P.Hq = c.n_q_heads; P.Sw = c.window; P.rows = ctx->rows; P.d = c.head_dim;
   P.scale2 = kLog2e / sqrtf((float)c.head_dim);
   P.inv_scale2 = 1.f / P.scale2;
