@@ -30,9 +30,8 @@
 // Bound.  A key tile of 128 keys and 128 rows is 16 384 exponentials per pass: 1024 cycles of the special-function
 // unit.  A statistics warp takes 3400 to 3700 cycles for its share of three tiles (3072 at the unit's rate) with the
 // next TMEM columns on their way during the arithmetic; with a load, a wait and a check per 32 columns it
-// took 3800 (pass B) and 4600 (pass A).  128K layer, 128 CTAs: 120 us per launch before, 111 now: long
-// prompts run into the device's power limit, of which the MMAs take the largest part (610 W above idle
-// at this kernel's rate, whatever the operands' source or the tile's width; the statistics 235 W).
+// took 3800 (pass B) and 4600 (pass A).  128K layer, 128 CTAs: 206 k cycles per launch before, 198 k now.  Long
+// prompts run into the device's power limit (1.75 instead of 1.965 GHz).
 //
 // Warp roles in a CTA of 512 threads: warps 0..11 are "statistics" warps in three groups of
 // four (a group takes every third accumulator tile, a warp owns 32 of its TMEM lanes and writes
