@@ -274,9 +274,11 @@ struct ColArgs {
 // issue slots and 7 % of the special-function unit, with two window rows in flight.  A thread now has 16 logits in
 // flight (8 where a KV head has one query head), as many as the registers of three CTAs per SM allow: eight layers
 // take 402 us with two rows at a time and 381 so, where the next kernel starts early; where it does not, 432 and 429.
+// With more than four query heads per KV head these registers do not hold a thread's sums and logits, and it is two CTAs
+// per SM: eight layers of 6K keys with 16 heads on 2 take 344 us so and 363 with three, which spilled; 32 on 4 400 and 404.
 constexpr int COL_KEYS = 64;
 template <int GM>          // query heads per KV head, at most
-__global__ void __launch_bounds__(NT, 3)
+__global__ void __launch_bounds__(NT, GM > 4 ? 2 : 3)
 colstats_simt(const ColArgs A) {
   __shared__ float s_lse[kMaxRows];
   __shared__ float s_part[4][2 + 2 * GM][COL_KEYS];
