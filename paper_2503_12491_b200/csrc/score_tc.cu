@@ -584,9 +584,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
       }
       // The next kernel of the stream may start once every CTA has issued its last loads; in shorter
-      // launches (one wave, column pass alone) once it is done with its statistics.  Earlier the next kernel's CTAs take the SMs that are left to those kernels: when they
-      // could start with this kernel, layers of the 4K MHA and 32K GQA prompts took 10 % longer, and with the
-      // last op 8 %; as it is, 1 to 7 % less than without an early start (1465 -> 1385 us at 32K GQA).
+      // launches (one wave, column pass alone) once it is done with its statistics.  Earlier the next kernel's CTAs take
+      // the SMs that are left to the cascade's.  (Measured when an eviction still had a launch of its own there: a start with
+      // this kernel made layers of the 4K MHA and 32K GQA prompts 10 % slower, one with the last op 8 %, and this one
+      // 1 to 7 % faster than none.)
       if constexpr (!kDirect && !kEntropyB) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       // do not leave the CTA while a bulk copy may still be writing its shared memory
       const uint32_t issued = t;
